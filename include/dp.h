@@ -80,16 +80,20 @@ typedef struct dp_model dp_model;
 typedef struct dp_ctx dp_ctx;
 
 /* Precision modes of a context. */
-#define DP_PREC_FP64  0   /* every step with float64 accuracy; the dense products
-                             (the fitting-net GEMMs and, for 3-layer doubling
-                             embedding nets with s_1 in {16, 25, 32}, the last
-                             embedding layer and layer 1 with their s-tangents)
-                             run on the tensor cores as exact products of BF16
-                             digit expansions of
-                             the FP64 operands (every partial sum an integer
-                             below 2^24, held exactly by the FP32 accumulators),
-                             the rest on the FP64 units; other shapes run as
-                             FP64_SIMT */
+#define DP_PREC_FP64  0   /* every step with float64 accuracy; the embedding nets,
+                             functions of the one number s(r), as Chebyshev
+                             series in s made on the device (in double-double
+                             arithmetic) whenever the parameters change: the
+                             terms kept leave less than 2^-55 of the net's size.
+                             Nets that 44 terms do not resolve are evaluated as
+                             written, for 3-layer doubling nets with s_1 in
+                             {16, 25, 32} with their last two layers and the
+                             s-tangents as exact products (below).  The
+                             fitting-net GEMMs run on the tensor cores as exact
+                             products of BF16 digit expansions of the FP64
+                             operands (every partial sum an integer below 2^24,
+                             held exactly by the FP32 accumulators), the rest
+                             on the FP64 units. */
 #define DP_PREC_FP64_SIMT 2  /* every step in float64 on the FP64 units */
 #define DP_PREC_MIXED 1   /* embedding- and fitting-net GEMMs on the tensor cores
                              (BF16 operands, FP32 accumulation, FP32 tanh); the
@@ -174,6 +178,8 @@ void dp_ctx_free(dp_ctx *ctx);
  * s_1 in {16, 25, 32}: the back-propagation of Sec. 2 (Eq. embedding through
  * the chain rule of the environment matrix, Sec. 3.2) needs, for every real
  * neighbour row, G and its derivative dG/ds with respect to the row's s(r).
+ * (FP64 contexts need neither while their nets run as Chebyshev series, see
+ * DP_PREC_FP64; the store then serves the nets that are not resolved.)
  * With the store on, the forward computes both once and keeps them in device
  * memory (natoms_max * N_m * 2 * M values, FP64 or FP32 as the context
  * computes them: 86.8 / 43.4 GB for 393,216 water atoms with N_m = 138,

@@ -9,6 +9,7 @@
 #include <string>
 #include <vector>
 
+#include "cheb.cuh"
 #include "dp_internal.cuh"
 
 namespace {
@@ -149,6 +150,13 @@ struct dp_ctx {
     bool use_ex;
     unsigned char *d_ex_w;
     int64_t ex_version;
+    // FP64 embedding nets as Chebyshev series in s (cheb.n == 0: not resolved,
+    // the kernels above run): made from the parameters of version cheb_version
+    bool use_cheb;
+    ChebModel cheb;
+    ChebBuffers cb;
+    double *h_cheb_mx;  // pinned host copy of cb.mx
+    int64_t cheb_version;
     // mixed precision: BF16 / FP32 copies of the parameters
     MixedModel mx;
     float *d_p32;
@@ -547,6 +555,25 @@ dp_status ensure_ex(dp_ctx *c)
     return DP_OK;
 }
 
+// Series of the embedding nets, again whenever the model's parameters changed.
+dp_status ensure_cheb(dp_ctx *c)
+{
+    if (c->cheb_version == c->model->version) return DP_OK;
+    GroupTimer tm(c, G_EMBED_FWD);
+    cudaError_t e = cudaSuccess;
+    if (c->cheb_version < 0) e = dp_launch_cheb_setup(c->stream, c->cb, &c->launches);
+    if (e == cudaSuccess) e = dp_launch_cheb_build(c->stream, c->m, c->cb, &c->launches);
+    if (e != cudaSuccess) return cuda_fail(e, "embedding series");
+    const size_t bytes = sizeof(double) * dp_cheb_elems(c->m, 3);
+    DP_CUDA(cudaMemcpyAsync(c->h_cheb_mx, c->cb.mx, bytes, cudaMemcpyDeviceToHost, c->stream), "embedding series");
+    DP_CUDA(cudaStreamSynchronize(c->stream), "embedding series");
+    c->cheb.n = dp_cheb_terms(c->m, c->h_cheb_mx);
+    c->cheb.C = c->cb.C;
+    c->cheb.Ct = c->cb.Ct;
+    c->cheb_version = c->model->version;
+    return DP_OK;
+}
+
 dp_status enqueue_eval(dp_ctx *c, const double *coords, const int32_t *types, const Box3 &b, int64_t N,
                        int64_t nloc, double *energy, double *force, double *virial, double *atom_energy)
 {
@@ -557,10 +584,14 @@ dp_status enqueue_eval(dp_ctx *c, const double *coords, const int32_t *types, co
     const int n = (int)nloc;  // the centres
     if (n > 0) {
         if ((s = enqueue_format(c, coords, types, b, nloc))) return s;
-        if (!mixed && c->use_ex && (s = ensure_ex(c))) return s;
+        if (c->use_cheb && (s = ensure_cheb(c))) return s;
+        const bool cheb = c->use_cheb && c->cheb.n > 0;
+        if (!mixed && !cheb && c->use_ex && (s = ensure_ex(c))) return s;
         {
             GroupTimer tm(c, G_EMBED_FWD);
-            e = mixed && c->eb.Gmx
+            e = cheb ? dp_launch_cheb_fwd(c->stream, c->m, c->cheb, coords, types, b, n, c->fb, c->nb, c->eb,
+                                          &c->launches)
+                : mixed && c->eb.Gmx
                     ? dp_launch_embed_tan_mx(c->stream, c->m, c->mx, coords, types, b, n, c->fb, c->nb, c->eb,
                                              c->num_sms, c->d_status, &c->launches)
                 : mixed     ? dp_launch_embed_fwd_mx(c->stream, c->m, c->mx, coords, types, b, n, c->fb, c->nb,
@@ -586,7 +617,8 @@ dp_status enqueue_eval(dp_ctx *c, const double *coords, const int32_t *types, co
         }
         {
             GroupTimer tm(c, G_EMBED_BWD);
-            e = mixed && c->eb.Gmx
+            e = cheb ? dp_launch_cheb_bwd(c->stream, c->m, c->cheb, types, n, c->fb, c->nb, c->eb, &c->launches)
+                : mixed && c->eb.Gmx
                     ? dp_launch_embed_bwd_stmx(c->stream, c->m, coords, types, b, n, c->fb, c->eb, c->num_sms,
                                                &c->launches)
                 : mixed     ? dp_launch_embed_bwd_mx(c->stream, c->m, c->mx, coords, types, b, n, c->fb, c->nb,
@@ -913,6 +945,7 @@ void dp_ctx_free(dp_ctx *c)
     dev_free(c->d_retry);
     if (c->h_status) cudaFreeHost(c->h_status);
     if (c->h_mass_stage) cudaFreeHost(c->h_mass_stage);
+    if (c->h_cheb_mx) cudaFreeHost(c->h_cheb_mx);
     void *bufs[] = {c->nb.cand, c->nb.ncand, c->nb.xref, c->nb.cell_count, c->nb.cell_start,
                     c->nb.cell_cursor, c->nb.cell_atoms, c->nb.cell_sorted, c->nb.atom_cell,
                     c->nb.type_perm, c->nb.type_start, c->fb.nlist, c->fb.keys, c->fb.nreal,
@@ -921,7 +954,7 @@ void dp_ctx_free(dp_ctx *c)
                     c->eb.fit_t, c->eb.fit_h, c->d_p32, c->d_emb_ops, c->d_fit_fwd, c->d_fit_bwd,
                     c->pb.dT, c->pb.dD, c->pb.Db, c->pb.dDb, c->pb.fit_scr, c->pb.rowscr, c->pb.slices,
                     c->d_oz_w, c->d_oz_e, c->ob.a, c->ob.aexp, c->ob.t, c->ob.h, c->ob.g, c->d_dtile, c->d_ex_w,
-                    c->eb.Gst, c->eb.Gmx};
+                    c->eb.Gst, c->eb.Gmx, c->cb.C, c->cb.Ct, c->cb.y, c->cb.mx, c->cb.trig};
     for (void *p : bufs) dev_free(p);
     delete c;
 }
@@ -1008,6 +1041,17 @@ dp_status dp_ctx_create(const dp_model *model, int64_t natoms_max, int32_t cand_
             }
         }
         cudaGetLastError();
+    }
+    c->cheb_version = -1;
+    if (precision == DP_PREC_FP64 && dp_cheb_supported(c->m)) {
+        double **bufs[] = {&c->cb.C, &c->cb.Ct, &c->cb.y, &c->cb.mx, &c->cb.trig};
+        for (int q = 0; q < 5; ++q) ALLOC(*bufs[q], dp_cheb_elems(c->m, q));
+        if (!s && cudaMallocHost((void **)&c->h_cheb_mx, sizeof(double) * dp_cheb_elems(c->m, 3)) != cudaSuccess) {
+            c->h_cheb_mx = nullptr;
+            cudaGetLastError();
+            s = fail(DP_ERR_NOMEM, "pinned allocation failed");
+        }
+        c->use_cheb = true;
     }
     // G and dG/ds (FP32) stored by the mixed forward (plain BF16 operands), on the same rule
     if (!s && precision == DP_PREC_MIXED) {

@@ -1,0 +1,760 @@
+// embed_cheb.cu -- FP64 environment matrix, embedding net and descriptor
+// (Algorithm 2; Eqs. embedding, embedding-first, embedding-rest, descrpt) and
+// their backward, with every embedding net as a Chebyshev series in its one
+// input s(r).
+//
+// An embedding net is M functions of the single number s.  They are analytic
+// (tanh of affine maps), so their Chebyshev series on s in [0, S] converge
+// geometrically: the water, copper and student nets reach 1e-17 of their size
+// with 17 to 20 terms.  The series turn the two contractions of the path inside
+// out:
+//   T_cf  = scale sum_b sum_n P^b_nc C^b_nf,   P^b_nc = sum_rows R~_c T_n(t),
+//   dE/dR~_c + ... per row from  U^b_nc = sum_f C^b_nf gT_cf:
+//   sum_f G_f gT_cf = sum_n U_nc T_n(t),  sum_f (dG_f/ds) gT_cf = sum_n V_nc T_n(t),
+// V the coefficients of the derivative (Mason and Handscomb, Chebyshev
+// Polynomials, 2003, sec. 2.4).  A row costs 4 n (forward) and 8 n (backward)
+// FMAs instead of a net with its s-derivative and 12 M FMAs; what depends on M
+// is done once per atom.  G is never formed.
+//
+// The coefficients are made on the device when a context first evaluates a set
+// of parameters: k_cheb_nodes evaluates the nets at the NN Chebyshev nodes in
+// double-double arithmetic (Dekker 1971, Knuth's two-sum), k_cheb_coef the discrete
+// transform, also in double-double, so the stored coefficients are the series'
+// rounded to FP64.  dp_cheb_terms keeps the terms until the derivative of what
+// is left is below 2^-55 of the net's size; a net that 44 terms do not resolve
+// makes the context use the kernels of embed_x.cu / embed.cu instead.  Rows
+// with s > S (r < 0.75 A) evaluate the net itself, one row at a time.
+//
+// What bounds the kernels: the FP64 pipe (16 cycles per warp instruction and SM).
+// One 128-thread CTA per atom, several per SM, so that the phases of different
+// atoms overlap; rows one per thread, then the per-atom products over (term,
+// component) and (component, feature) items.  Measured per evaluation of 139,968
+// water atoms (20 terms): forward 159 -> 13.0 ms, backward 25.0 -> 16.7 ms against
+// the kernels of embed_x.cu that evaluate the nets and keep G and dG/ds; 32,000
+// copper atoms: 79 -> 3.0 and 12.8 -> 4.6 ms; 192 water atoms: 0.37 -> 0.04 and
+// 0.17 -> 0.05 ms.  Errors against extended precision are the same (forces
+// 1e-15 of their norm on water, 2e-14 on copper, both ways).
+#include <cmath>
+
+#include "cheb.cuh"
+
+namespace {
+
+constexpr int NN = DP_CHEB_NN;
+constexpr int CT = 128;       // threads of a CTA = rows of a chunk
+constexpr int LDT = CT + 1;   // row pitch of the T_n(t) table (odd: lanes on n hit different banks)
+constexpr unsigned FULL = 0xffffffffu;
+
+// ------------------------------------------------------- double-double ------
+
+struct dd {
+    double h, l;
+};
+
+__device__ __forceinline__ dd two_sum(double a, double b)
+{
+    const double s = __dadd_rn(a, b), v = __dsub_rn(s, a);
+    return {s, __dadd_rn(__dsub_rn(a, __dsub_rn(s, v)), __dsub_rn(b, v))};
+}
+__device__ __forceinline__ dd quick_sum(double a, double b)
+{
+    const double s = __dadd_rn(a, b);
+    return {s, __dsub_rn(b, __dsub_rn(s, a))};
+}
+__device__ __forceinline__ dd dd_add(dd a, dd b)
+{
+    dd s = two_sum(a.h, b.h);
+    const dd t = two_sum(a.l, b.l);
+    s = quick_sum(s.h, __dadd_rn(s.l, t.h));
+    return quick_sum(s.h, __dadd_rn(s.l, t.l));
+}
+__device__ __forceinline__ dd dd_mul(dd a, dd b)
+{
+    const double p = __dmul_rn(a.h, b.h);
+    double e = __fma_rn(a.h, b.h, -p);
+    e = __fma_rn(a.h, b.l, e);
+    e = __fma_rn(a.l, b.h, e);
+    return quick_sum(p, e);
+}
+__device__ __forceinline__ dd dd_neg(dd a) { return {-a.h, -a.l}; }
+__device__ __forceinline__ dd dd_div(dd a, dd b)
+{
+    const double q = __ddiv_rn(a.h, b.h);
+    dd r = dd_add(a, dd_neg(dd_mul(b, {q, 0.0})));
+    const double q2 = __ddiv_rn(r.h, b.h);
+    r = dd_add(r, dd_neg(dd_mul(b, {q2, 0.0})));
+    return dd_add(quick_sum(q, q2), {__ddiv_rn(r.h, b.h), 0.0});
+}
+
+// sin (odd = 1) or cos (odd = 0) of |x| <= pi / 4 by Taylor's series
+__device__ dd dd_trig(dd x, int odd)
+{
+    const dd x2 = dd_neg(dd_mul(x, x));
+    dd term = odd ? x : dd{1.0, 0.0}, sum = term;
+    for (int k = odd + 1; k < 32; k += 2) {
+        term = dd_div(dd_mul(term, x2), {(double)k * (double)(k + 1), 0.0});
+        sum = dd_add(sum, term);
+    }
+    return sum;
+}
+
+// tanh of |x| <= 1/64: the odd Taylor series (remainder below 1e-25)
+__device__ __forceinline__ dd dd_tanh_small(dd x)
+{
+    const double u = x.h * x.h;
+    double p = 21844.0 / 6081075.0;
+    p = fma(p, u, -1382.0 / 155925.0);
+    p = fma(p, u, 62.0 / 2835.0);
+    p = fma(p, u, -17.0 / 315.0);
+    p = fma(p, u, 2.0 / 15.0);
+    p = fma(p, u, -1.0 / 3.0);
+    return dd_add(x, {x.h * (u * p), 0.0});
+}
+
+__global__ void k_cheb_setup(double *__restrict__ trig)
+{
+    const int q = blockIdx.x * blockDim.x + threadIdx.x;
+    const dd pi = {3.141592653589793116, 1.2246467991473532e-16};
+    if (q < 4 * NN) {
+        // cos(pi q / (2 NN)) through the symmetries of the cosine
+        int j = q > 2 * NN ? 4 * NN - q : q;
+        const bool neg = j > NN;
+        if (neg) j = 2 * NN - j;
+        const bool s = 2 * j > NN;
+        const dd th = dd_div(dd_mul(pi, {(double)(s ? NN - j : j), 0.0}), {2.0 * NN, 0.0});
+        dd v = dd_trig(th, s ? 1 : 0);
+        if (neg) v = dd_neg(v);
+        trig[2 * q] = v.h;
+        trig[2 * q + 1] = v.l;
+    } else if (q < 4 * NN + DP_CHEB_NTANH) {
+        // tanh(k / 32): the series at k / 32 / 2^m <= 1/2048 (remainder 1e-38), doubled m times
+        const int k = q - 4 * NN;
+        double v = k / 32.0;
+        int m = 0;
+        for (; v > 1.0 / 2048.0; ++m) v *= 0.5;
+        const dd z = {v, 0.0}, u = dd_mul(z, z);
+        const double c[7] = {1.0, -1.0, 2.0, -17.0, 62.0, -1382.0, 21844.0};
+        const double d[7] = {1.0, 3.0, 15.0, 315.0, 2835.0, 155925.0, 6081075.0};
+        dd p = dd_div({c[6], 0.0}, {d[6], 0.0});
+        for (int i = 5; i >= 0; --i) p = dd_add(dd_mul(p, u), dd_div({c[i], 0.0}, {d[i], 0.0}));
+        dd t = dd_mul(z, p);
+        for (; m > 0; --m) t = dd_div(dd_add(t, t), dd_add({1.0, 0.0}, dd_mul(t, t)));
+        trig[2 * q] = t.h;
+        trig[2 * q + 1] = t.l;
+    }
+}
+
+// tanh(x) to about 1e-21: tanh(k/32 + t) = (A + B) / (1 + A B); 1 beyond 22
+// (1 - tanh(22) = 1.6e-19)
+__device__ dd dd_tanh(dd x, const double *__restrict__ tab)
+{
+    if (!(fabs(x.h) < 22.0)) return x.h != x.h ? x : dd{copysign(1.0, x.h), 0.0};
+    const bool neg = x.h < 0.0;
+    if (neg) x = dd_neg(x);
+    const int k = (int)rint(x.h * 32.0);
+    const dd A = {tab[2 * k], tab[2 * k + 1]};
+    const dd B = dd_tanh_small(dd_add(x, {-k / 32.0, 0.0}));
+    const dd t = dd_div(dd_add(A, B), dd_add({1.0, 0.0}, dd_mul(A, B)));
+    return neg ? dd_neg(t) : t;
+}
+
+// One CTA per (net, node): the net at s_k = S/2 (1 + cos(pi (2k+1) / (2 NN))),
+// thread o on output o of each layer.
+__global__ void __launch_bounds__(CT) k_cheb_nodes(DevModel m, const double *__restrict__ trig, double *__restrict__ y)
+{
+    __shared__ dd h[2][DP_MAX_EMB_W];
+    const int net = blockIdx.x / NN, k = blockIdx.x % NN, o = threadIdx.x;
+    const double *W = m.params + m.emb_base[net];
+    const int q = 2 * k + 1;
+    dd s = dd_add({1.0, 0.0}, {trig[2 * q], trig[2 * q + 1]});
+    s = dd_div(s, {DP_CHEB_SCALE, 0.0});
+    const double *tab = trig + 2 * 4 * NN;
+    int win = m.emb[0], cur = 0;
+    if (o < win) h[0][o] = dd_tanh(dd_add(dd_mul(s, {W[o], 0.0}), {W[win + o], 0.0}), tab);
+    W += 2 * win;
+    for (int l = 1; l < m.n_emb; ++l) {
+        __syncthreads();
+        const int wout = m.emb[l], sk = dp_skip_kind(win, wout);
+        if (o < wout) {
+            dd z = {W[win * wout + o], 0.0};
+            for (int p = 0; p < win; ++p) z = dd_add(z, dd_mul(h[cur][p], {W[p * wout + o], 0.0}));
+            z = dd_tanh(z, tab);
+            if (sk) z = dd_add(z, h[cur][o < win ? o : o - win]);
+            h[cur ^ 1][o] = z;
+        }
+        W += win * wout + wout;
+        win = wout;
+        cur ^= 1;
+    }
+    if (o < m.M) {
+        double *out = y + ((size_t)blockIdx.x * m.M + o) * 2;
+        out[0] = h[cur][o].h;   // each thread reads what it wrote
+        out[1] = h[cur][o].l;
+    }
+}
+
+// One CTA per (net, n): C_n = (2 - [n = 0]) / NN sum_k cos(pi n (2k+1) / (2 NN)) y_k
+__global__ void __launch_bounds__(CT) k_cheb_coef(DevModel m, const double *__restrict__ trig,
+                                                  const double *__restrict__ y, double *__restrict__ C,
+                                                  double *__restrict__ Ct, double *__restrict__ mx)
+{
+    __shared__ double wm[CT / 32];
+    const int net = blockIdx.x / NN, n = blockIdx.x % NN, f = threadIdx.x, M = m.M, T = m.ntypes;
+    double v = 0.0;
+    if (f < M) {
+        dd acc = {0.0, 0.0};
+        for (int k = 0; k < NN; ++k) {
+            const int j = (n * (2 * k + 1)) % (4 * NN);
+            const double *yk = y + ((size_t)(net * NN + k) * M + f) * 2;
+            acc = dd_add(acc, dd_mul({trig[2 * j], trig[2 * j + 1]}, {yk[0], yk[1]}));
+        }
+        acc = dd_div(acc, {n == 0 ? (double)NN : 0.5 * NN, 0.0});
+        v = acc.h;
+        C[(size_t)blockIdx.x * M + f] = v;
+        Ct[((size_t)(net / T) * M + f) * (T * NN) + (net % T) * NN + n] = v;
+    }
+    v = fabs(v);
+    bool bad = !(v <= 1e300);
+    for (int s = 16; s > 0; s >>= 1) v = fmax(v, __shfl_xor_sync(FULL, v, s));
+    if ((f & 31) == 0) wm[f >> 5] = v;
+    bad = __syncthreads_or(bad);
+    if (f == 0) {
+        for (int w = 1; w < CT / 32; ++w) v = fmax(v, wm[w]);
+        mx[blockIdx.x] = bad ? 1e301 : v;
+    }
+}
+
+// ---------------------------------------------------------- rows beyond S ---
+
+// The net with its s-derivative at s, by the whole CTA (rows with s > S only):
+// G in ga[0..M), dG/ds in da.  ga, da, gb, db: DP_MAX_EMB_W doubles each.
+__device__ void net_direct(const DevModel &m, int net, double s, double *&ga, double *&da, double *&gb, double *&db)
+{
+    const int o = threadIdx.x;
+    const double *W = m.params + m.emb_base[net];
+    int win = m.emb[0];
+    __syncthreads();
+    if (o < win) {
+        const double w0 = W[o], t = dp_tanh64(fma(s, w0, W[win + o]), m.tanh_tab);
+        ga[o] = t;
+        da[o] = fma(-t, t, 1.0) * w0;
+    }
+    W += 2 * win;
+    for (int l = 1; l < m.n_emb; ++l) {
+        __syncthreads();
+        const int wout = m.emb[l], sk = dp_skip_kind(win, wout);
+        if (o < wout) {
+            double z = W[win * wout + o], dz = 0.0;
+            for (int p = 0; p < win; ++p) {
+                const double w = W[p * wout + o];
+                z = fma(ga[p], w, z);
+                dz = fma(da[p], w, dz);
+            }
+            const double t = dp_tanh64(z, m.tanh_tab);
+            const int os = o < win ? o : o - win;
+            gb[o] = t + (sk ? ga[os] : 0.0);
+            db[o] = fma(fma(-t, t, 1.0), dz, sk ? da[os] : 0.0);
+        }
+        double *u = ga;
+        ga = gb;
+        gb = u;
+        u = da;
+        da = db;
+        db = u;
+        W += win * wout + wout;
+        win = wout;
+    }
+    __syncthreads();
+}
+
+// Type block of row q of the atom (rows of all blocks one after the other);
+// start[b] is the first row of block b, start[T] the number of rows.
+__device__ __forceinline__ int row_block(const int *start, int T, int q)
+{
+    int b = 0;
+    while (b + 1 < T && q >= start[b + 1]) ++b;
+    return b;
+}
+
+// ---------------------------------------------------------------- forward ---
+
+__global__ void __launch_bounds__(CT) k_cheb_fwd(DevModel m, ChebModel cm, const double *__restrict__ x,
+                                                 const int32_t *__restrict__ types, Box3 box,
+                                                 const int32_t *__restrict__ type_perm,
+                                                 const int32_t *__restrict__ nlist, const int32_t *__restrict__ nreal,
+                                                 double *__restrict__ pair_d, double *__restrict__ Tout,
+                                                 double *__restrict__ Dout)
+{
+    extern __shared__ __align__(16) double sm[];
+    const int nc = cm.n, M = m.M, T = m.ntypes, nm = m.nm, tid = threadIdx.x;
+    double *R4 = sm;                       // [CT][4] rows of R~
+    double *part = R4 + CT * 4;            // [2][CT][4] moment partials of the row slices
+    double *Mom = part + 2 * CT * 4;       // [T nc][4]
+    double *Ts = Mom + T * nc * 4;         // [4][M]
+    double *Tch = Ts + 4 * M;              // [nc][LDT] T_n(t) of the chunk's rows
+    __shared__ int start[DP_MAX_TYPES + 1];
+    __shared__ double fbuf[4][DP_MAX_EMB_W];  // rows beyond S
+    const int i = type_perm[blockIdx.x];
+    const int a = types[i];
+    const bool a_ok = (unsigned)a < (unsigned)T;
+    if (tid == 0) {
+        int r = 0;
+        for (int b = 0; b < T; ++b) {
+            start[b] = r;
+            r += a_ok ? nreal[(size_t)i * T + b] : 0;
+        }
+        start[T] = r;
+    }
+    for (int p = tid; p < T * nc * 4; p += CT) Mom[p] = 0.0;
+    __syncthreads();
+    const int R = start[T];
+    const double xi[3] = {x[3 * i], x[3 * i + 1], x[3 * i + 2]};
+    const int ns = CT / nc;                    // row slices of the moment sums
+    const int mn = tid % nc, msl = tid / nc;   // this thread's term and slice
+    bool any_far = false;
+    int seg = 0;
+    for (int c0 = 0; c0 < R; c0 += CT) {
+        const int q = c0 + tid;
+        bool far = false;
+        if (q < R) {
+            const int b = row_block(start, T, q);
+            const size_t slot = (size_t)i * nm + m.sel_off[b] + (q - start[b]);
+            const int j = nlist[slot];
+            const double xj[3] = {x[3 * j], x[3 * j + 1], x[3 * j + 2]};
+            double d[3], s, ds;
+            const double r = dp_pinned_dist(xi, xj, box, d);
+            dp_switch(r, m.rcut_smth, m.rcut, s, ds);
+            pair_d[slot * 3] = d[0];
+            pair_d[slot * 3 + 1] = d[1];
+            pair_d[slot * 3 + 2] = d[2];
+            const double sr = s / r;
+            far = !(s <= DP_CHEB_S);
+            double *Rq = R4 + tid * 4;
+            Rq[0] = far ? 0.0 : s;
+            Rq[1] = far ? 0.0 : sr * d[0];
+            Rq[2] = far ? 0.0 : sr * d[1];
+            Rq[3] = far ? 0.0 : sr * d[2];
+            const double t = far ? 0.0 : fma(s, DP_CHEB_SCALE, -1.0), t2 = t + t;
+            double p0 = 1.0, p1 = t;
+            Tch[tid] = 1.0;
+            for (int n = 1; n < nc; ++n) {
+                Tch[n * LDT + tid] = p1;
+                const double p2 = fma(t2, p1, -p0);
+                p0 = p1;
+                p1 = p2;
+            }
+        }
+        any_far = __syncthreads_or(far) || any_far;
+        for (int b = 0; b < T; ++b) {
+            const int lo = max(start[b] - c0, 0), hi = min(start[b + 1] - c0, CT);
+            if (lo >= hi) continue;
+            double *pt = part + (seg & 1) * CT * 4;
+            if (msl < ns) {
+                double acc[4] = {0.0, 0.0, 0.0, 0.0};
+                const double *tn = Tch + mn * LDT;
+                for (int r = lo + msl; r < hi; r += ns) {
+                    const double tv = tn[r];
+                    const double2 u = *reinterpret_cast<const double2 *>(R4 + r * 4);
+                    const double2 w = *reinterpret_cast<const double2 *>(R4 + r * 4 + 2);
+                    acc[0] = fma(tv, u.x, acc[0]);
+                    acc[1] = fma(tv, u.y, acc[1]);
+                    acc[2] = fma(tv, w.x, acc[2]);
+                    acc[3] = fma(tv, w.y, acc[3]);
+                }
+#pragma unroll
+                for (int c = 0; c < 4; ++c) pt[tid * 4 + c] = acc[c];
+            }
+            __syncthreads();
+            for (int p = tid; p < nc * 4; p += CT) {
+                double v = Mom[b * nc * 4 + p];
+                for (int u = 0; u < ns; ++u) v += pt[u * nc * 4 + p];
+                Mom[b * nc * 4 + p] = v;
+            }
+            ++seg;
+        }
+        __syncthreads();
+    }
+    // T = scale sum_k P_k C_k, items (c, f)
+    {
+        const double *C = cm.C + (size_t)(a_ok ? a : 0) * T * NN * M;
+        for (int p0 = tid; p0 < 4 * M; p0 += 4 * CT) {
+            double acc[4] = {0.0, 0.0, 0.0, 0.0};
+            int c[4], f[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int p = p0 + u * CT;
+                c[u] = p / M;
+                f[u] = p - c[u] * M;
+            }
+            for (int b = 0; b < T; ++b) {
+                if (start[b] == start[b + 1]) continue;
+                const double *Cb = C + (size_t)b * NN * M, *mo = Mom + b * nc * 4;
+#pragma unroll 4
+                for (int n = 0; n < nc; ++n)
+#pragma unroll
+                    for (int u = 0; u < 4; ++u)
+                        if (p0 + u * CT < 4 * M) acc[u] = fma(mo[n * 4 + c[u]], Cb[n * M + f[u]], acc[u]);
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+                if (p0 + u * CT < 4 * M) Ts[p0 + u * CT] = acc[u] * m.desc_scale;
+        }
+    }
+    __syncthreads();
+    if (any_far) {
+        double *ga = fbuf[0], *da = fbuf[1], *gb = fbuf[2], *db = fbuf[3];
+        for (int q = 0; q < R; ++q) {
+            const int b = row_block(start, T, q);
+            const double *d = pair_d + ((size_t)i * nm + m.sel_off[b] + (q - start[b])) * 3;
+            const double dv[3] = {d[0], d[1], d[2]};
+            const double r = __dsqrt_rn(__dadd_rn(__dadd_rn(__dmul_rn(dv[0], dv[0]), __dmul_rn(dv[1], dv[1])),
+                                                  __dmul_rn(dv[2], dv[2])));
+            double s, ds;
+            dp_switch(r, m.rcut_smth, m.rcut, s, ds);
+            if (s <= DP_CHEB_S) continue;  // uniform: every thread has the same row
+            net_direct(m, a * T + b, s, ga, da, gb, db);
+            const double sr = s / r;
+            for (int p = tid; p < 4 * M; p += CT) {
+                const int c = p / M;
+                Ts[p] += (c == 0 ? s : sr * dv[c - 1]) * ga[p - c * M] * m.desc_scale;
+            }
+            __syncthreads();
+        }
+    }
+    for (int p = tid; p < 4 * M; p += CT) Tout[(size_t)i * 4 * M + p] = Ts[p];
+    const int nd = m.m2 * M;
+    for (int q = tid; q < nd; q += CT) {
+        const int a2 = q / M, b2 = q - a2 * M;
+        double acc = Ts[a2] * Ts[b2];
+        acc = fma(Ts[M + a2], Ts[M + b2], acc);
+        acc = fma(Ts[2 * M + a2], Ts[2 * M + b2], acc);
+        acc = fma(Ts[3 * M + a2], Ts[3 * M + b2], acc);
+        Dout[(size_t)i * nd + q] = acc;
+    }
+}
+
+// --------------------------------------------------------------- backward ---
+
+__global__ void __launch_bounds__(CT) k_cheb_bwd(DevModel m, ChebModel cm, const int32_t *__restrict__ types,
+                                                 const int32_t *__restrict__ type_perm,
+                                                 const int32_t *__restrict__ nreal, const double *__restrict__ Tin,
+                                                 const double *__restrict__ gD, double *__restrict__ pair_g,
+                                                 double *__restrict__ f_own, double *__restrict__ vir_part)
+{
+    extern __shared__ __align__(16) double sm[];
+    const int nc = cm.n, M = m.M, m2 = m.m2, T = m.ntypes, nm = m.nm, tid = threadIdx.x;
+    const int Kt = T * nc, LDG = M | 1;
+    double *UV = sm;                        // [Kt][8]: U_nc, V_nc
+    double *g4 = UV + Kt * 8;               // [M][4]: gT_cf
+    double *Ts = g4 + M * 4;                // [4][M]
+    double *lp = Ts + 4 * M;                // [2][4][m2] partial long sums
+    double *gs = lp + 8 * m2;               // [m2][LDG] dE/dD, then [slices][Kt][4] partials of U
+    __shared__ int start[DP_MAX_TYPES + 1];
+    __shared__ double fbuf[4][DP_MAX_EMB_W];
+    __shared__ double fsum[CT / 32][8], wsum[CT / 32][16];
+    __shared__ unsigned farbits[(DP_MAX_NM + CT) / 32];
+    const int i = type_perm[blockIdx.x];
+    const int a = types[i];
+    const bool a_ok = (unsigned)a < (unsigned)T;
+    if (tid == 0) {
+        int r = 0;
+        for (int b = 0; b < T; ++b) {
+            start[b] = r;
+            r += a_ok ? nreal[(size_t)i * T + b] : 0;
+        }
+        start[T] = r;
+    }
+    for (int p = tid; p < 4 * M; p += CT) Ts[p] = Tin[(size_t)i * 4 * M + p];
+    {
+        const double *g = gD + (size_t)i * m2 * M;
+        for (int p = tid; p < m2 * M; p += CT) gs[(p / M) * LDG + p % M] = g[p];
+    }
+    __syncthreads();
+    const int R = start[T];
+    // gT[c][x] = scale ([x < m2] sum_b gD[x][b] T[c][b] + sum_{a < m2} gD[a][x] T[c][a]);
+    // the m2 4 long sums two threads each first
+    for (int p = tid; p < 8 * m2; p += CT) {
+        const int h = p / (4 * m2), e = p - h * 4 * m2, c = e / m2, xx = e - c * m2;
+        const double *gr = gs + xx * LDG, *tr = Ts + c * M;
+        double v0 = 0.0, v1 = 0.0;
+        int b = h;
+        for (; b + 2 < M; b += 4) {
+            v0 = fma(gr[b], tr[b], v0);
+            v1 = fma(gr[b + 2], tr[b + 2], v1);
+        }
+        for (; b < M; b += 2) v0 = fma(gr[b], tr[b], v0);
+        lp[p] = v0 + v1;
+    }
+    __syncthreads();
+    for (int p = tid; p < 4 * M; p += CT) {
+        const int c = p / M, xx = p - c * M;
+        double v0 = 0.0, v1 = 0.0;
+        int a2 = 0;
+        for (; a2 + 1 < m2; a2 += 2) {
+            v0 = fma(gs[a2 * LDG + xx], Ts[c * M + a2], v0);
+            v1 = fma(gs[(a2 + 1) * LDG + xx], Ts[c * M + a2 + 1], v1);
+        }
+        if (a2 < m2) v0 = fma(gs[a2 * LDG + xx], Ts[c * M + a2], v0);
+        v0 += v1;
+        if (xx < m2) v0 += lp[c * m2 + xx] + lp[4 * m2 + c * m2 + xx];
+        g4[xx * 4 + c] = v0 * m.desc_scale;
+    }
+    __syncthreads();
+    // U_kc = sum_f C_kf gT_cf: thread = (term k of the centre's nets, feature slice)
+    {
+        const double *Ct = cm.Ct + (size_t)(a_ok ? a : 0) * M * T * NN;
+        const int nsl = Kt < CT ? CT / Kt : 1;
+        for (int p = tid; p < Kt * nsl; p += CT) {
+            const int fs = p / Kt, k = p - fs * Kt, b = k / nc;
+            const double *ck = Ct + b * NN + (k - b * nc);
+            double acc[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll 4
+            for (int f = fs; f < M; f += nsl) {
+                const double cv = ck[(size_t)f * T * NN];
+                const double2 u = *reinterpret_cast<const double2 *>(g4 + f * 4);
+                const double2 w = *reinterpret_cast<const double2 *>(g4 + f * 4 + 2);
+                acc[0] = fma(cv, u.x, acc[0]);
+                acc[1] = fma(cv, u.y, acc[1]);
+                acc[2] = fma(cv, w.x, acc[2]);
+                acc[3] = fma(cv, w.y, acc[3]);
+            }
+#pragma unroll
+            for (int c = 0; c < 4; ++c) gs[p * 4 + c] = acc[c];
+        }
+        __syncthreads();
+        for (int p = tid; p < Kt * 4; p += CT) {
+            double v = gs[p];
+            for (int u = 1; u < nsl; ++u) v += gs[u * Kt * 4 + p];
+            UV[(p >> 2) * 8 + (p & 3)] = v;
+        }
+    }
+    __syncthreads();
+    // V: the derivative's coefficients, d/ds = (2 / S) d/dt, v_n = (2 - [n = 0]) sum_{m = n+1, n+3, ..} m u_m
+    for (int p = tid; p < Kt * 4; p += CT) {
+        const int k = p >> 2, c = p & 3, b = k / nc, n = k - b * nc;
+        const double *u = UV + b * nc * 8 + c;
+        double v = 0.0;
+        for (int q = n + 1; q < nc; q += 2) v = fma((double)q, u[q * 8], v);
+        UV[k * 8 + 4 + c] = v * ((n == 0 ? 1.0 : 2.0) * DP_CHEB_SCALE);
+    }
+    __syncthreads();
+
+    double fo[3] = {0.0, 0.0, 0.0}, vir[9];
+#pragma unroll
+    for (int q = 0; q < 9; ++q) vir[q] = 0.0;
+    // pair gradient of a row from its sums P_c = sum_f G_f gT_cf and Q = sum_c R~_c sum_f (dG_f/ds) gT_cf
+    auto chain = [&](double *pg, const double *d, double inv, double s, double ds, const double *P, double Q) {
+        const double u[3] = {d[0] * inv, d[1] * inv, d[2] * inv};
+        const double dot = P[1] * u[0] + P[2] * u[1] + P[3] * u[2];
+        const double sr = s * inv;
+        const double coef = (P[0] + Q) * ds + ds * dot - sr * dot;
+#pragma unroll
+        for (int e = 0; e < 3; ++e) {
+            const double gv = fma(u[e], coef, sr * P[1 + e]);
+            pg[e] = gv;
+            fo[e] += gv;
+#pragma unroll
+            for (int f = 0; f < 3; ++f) vir[f * 3 + e] -= d[f] * gv;
+        }
+    };
+    auto radius = [](const double *d) {
+        return __dsqrt_rn(__dadd_rn(__dadd_rn(__dmul_rn(d[0], d[0]), __dmul_rn(d[1], d[1])), __dmul_rn(d[2], d[2])));
+    };
+    bool any_far = false;
+    for (int c0 = 0; c0 < R; c0 += CT) {
+        const int q = c0 + tid;
+        bool far = false;
+        if (q < R) {
+            const int b = row_block(start, T, q);
+            double *pg = pair_g + ((size_t)i * nm + m.sel_off[b] + (q - start[b])) * 3;
+            const double d[3] = {pg[0], pg[1], pg[2]};
+            const double r = radius(d);
+            double s, ds;
+            dp_switch(r, m.rcut_smth, m.rcut, s, ds);
+            far = !(s <= DP_CHEB_S);
+            if (!far) {
+                const double inv = 1.0 / r, sr = s * inv;
+                const double t = fma(s, DP_CHEB_SCALE, -1.0), t2 = t + t;
+                const double2 *uv = reinterpret_cast<const double2 *>(UV + b * nc * 8);
+                double P[4] = {uv[0].x, uv[0].y, uv[1].x, uv[1].y};
+                double Qc[4] = {uv[2].x, uv[2].y, uv[3].x, uv[3].y};
+                double p0 = 1.0, p1 = t;
+#pragma unroll 2
+                for (int n = 1; n < nc; ++n) {
+                    const double2 a0 = uv[n * 4], a1 = uv[n * 4 + 1], a2 = uv[n * 4 + 2], a3 = uv[n * 4 + 3];
+                    P[0] = fma(a0.x, p1, P[0]);
+                    P[1] = fma(a0.y, p1, P[1]);
+                    P[2] = fma(a1.x, p1, P[2]);
+                    P[3] = fma(a1.y, p1, P[3]);
+                    Qc[0] = fma(a2.x, p1, Qc[0]);
+                    Qc[1] = fma(a2.y, p1, Qc[1]);
+                    Qc[2] = fma(a3.x, p1, Qc[2]);
+                    Qc[3] = fma(a3.y, p1, Qc[3]);
+                    const double p2 = fma(t2, p1, -p0);
+                    p0 = p1;
+                    p1 = p2;
+                }
+                chain(pg, d, inv, s, ds, P, s * Qc[0] + sr * (d[0] * Qc[1] + d[1] * Qc[2] + d[2] * Qc[3]));
+            }
+        }
+        const unsigned bal = __ballot_sync(FULL, far);
+        if ((tid & 31) == 0) farbits[(c0 + tid) >> 5] = bal;
+        any_far |= far;
+    }
+    if (__syncthreads_or(any_far)) {
+        // rows beyond S in row order; their d is still in place
+        double *ga = fbuf[0], *da = fbuf[1], *gb = fbuf[2], *db = fbuf[3];
+        for (int q = 0; q < R; ++q) {
+            if (!((farbits[q >> 5] >> (q & 31)) & 1u)) continue;
+            const int b = row_block(start, T, q);
+            double *pg = pair_g + ((size_t)i * nm + m.sel_off[b] + (q - start[b])) * 3;
+            const double d[3] = {pg[0], pg[1], pg[2]};
+            const double r = radius(d);
+            double s, ds;
+            dp_switch(r, m.rcut_smth, m.rcut, s, ds);
+            net_direct(m, a * T + b, s, ga, da, gb, db);
+            double p[8];
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                p[c] = tid < M ? ga[tid] * g4[tid * 4 + c] : 0.0;
+                p[4 + c] = tid < M ? da[tid] * g4[tid * 4 + c] : 0.0;
+            }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+                for (int c = 0; c < 8; ++c) p[c] += __shfl_xor_sync(FULL, p[c], o);
+            if ((tid & 31) == 0)
+#pragma unroll
+                for (int c = 0; c < 8; ++c) fsum[tid >> 5][c] = p[c];
+            __syncthreads();
+            if (tid == 0) {
+#pragma unroll
+                for (int c = 0; c < 8; ++c)
+                    for (int w = 1; w < CT / 32; ++w) p[c] += fsum[w][c];
+                const double inv = 1.0 / r, sr = s * inv;
+                chain(pg, d, inv, s, ds, p, s * p[4] + sr * (d[0] * p[5] + d[1] * p[6] + d[2] * p[7]));
+            }
+            __syncthreads();
+        }
+    }
+    // own force and virial: a transposing shuffle tree (16 adds), then the four warps in order
+    {
+        double p[16];
+#pragma unroll
+        for (int q = 0; q < 3; ++q) p[q] = fo[q];
+#pragma unroll
+        for (int q = 0; q < 9; ++q) p[3 + q] = vir[q];
+#pragma unroll
+        for (int q = 12; q < 16; ++q) p[q] = 0.0;
+        const int lane = tid & 31;
+#pragma unroll
+        for (int w = 16, n = 8; w >= 2; w >>= 1, n >>= 1) {
+            const bool up = (lane & w) != 0;
+#pragma unroll
+            for (int k = 0; k < n; ++k) {
+                const double send = up ? p[k] : p[n + k];
+                const double keep = up ? p[n + k] : p[k];
+                p[k] = keep + __shfl_xor_sync(FULL, send, w);
+            }
+        }
+        p[0] += __shfl_xor_sync(FULL, p[0], 1);
+        if ((lane & 1) == 0) wsum[tid >> 5][lane >> 1] = p[0];
+        __syncthreads();
+        if (tid < 12) {
+            double v = wsum[0][tid];
+            for (int w = 1; w < CT / 32; ++w) v += wsum[w][tid];
+            if (tid < 3) f_own[(size_t)i * 3 + tid] = v;
+            else vir_part[(size_t)i * 9 + tid - 3] = v;
+        }
+    }
+}
+
+size_t fwd_smem(const DevModel &m, int nc)
+{
+    return sizeof(double) * (CT * 4 + 2 * CT * 4 + (size_t)m.ntypes * nc * 4 + 4 * m.M + (size_t)nc * LDT);
+}
+
+size_t bwd_smem(const DevModel &m, int nc)
+{
+    const size_t Kt = (size_t)m.ntypes * nc, nsl = Kt < CT ? CT / Kt : 1;
+    const size_t g = (size_t)m.m2 * (m.M | 1), u = Kt * nsl * 4;
+    return sizeof(double) * (Kt * 8 + 8 * (size_t)m.M + 8 * (size_t)m.m2 + (g > u ? g : u));
+}
+
+constexpr size_t SMEM_MAX = 220 * 1024;  // dynamic, next to ~7 KB of static shared memory
+
+}  // namespace
+
+bool dp_cheb_supported(const DevModel &m) { return bwd_smem(m, NN) <= SMEM_MAX && fwd_smem(m, NN) <= SMEM_MAX; }
+
+size_t dp_cheb_elems(const DevModel &m, int which)
+{
+    const size_t nets = (size_t)m.ntypes * m.ntypes;
+    switch (which) {
+    case 0:
+    case 1: return nets * NN * m.M;
+    case 2: return nets * NN * m.M * 2;
+    case 3: return nets * NN;
+    default: return 2 * (4 * NN + DP_CHEB_NTANH);
+    }
+}
+
+cudaError_t dp_launch_cheb_setup(cudaStream_t st, ChebBuffers cb, int64_t *launches)
+{
+    k_cheb_setup<<<(4 * NN + DP_CHEB_NTANH + 127) / 128, 128, 0, st>>>(cb.trig);
+    *launches += 1;
+    return cudaGetLastError();
+}
+
+cudaError_t dp_launch_cheb_build(cudaStream_t st, const DevModel &m, ChebBuffers cb, int64_t *launches)
+{
+    const int grid = m.ntypes * m.ntypes * NN;
+    k_cheb_nodes<<<grid, CT, 0, st>>>(m, cb.trig, cb.y);
+    k_cheb_coef<<<grid, CT, 0, st>>>(m, cb.trig, cb.y, cb.C, cb.Ct, cb.mx);
+    *launches += 2;
+    return cudaGetLastError();
+}
+
+int dp_cheb_terms(const DevModel &m, const double *mx)
+{
+    int need = 4;
+    for (int net = 0; net < m.ntypes * m.ntypes; ++net) {
+        const double *c = mx + net * NN;
+        double size = 0.0, tail = 0.0;
+        for (int n = 0; n < NN; ++n) size = c[n] > size ? c[n] : size;
+        if (!(size <= 1e300)) return 0;
+        // |d/ds of the terms n ..| <= (2 / S) sum n^2 |C_n|
+        int n = NN;
+        for (; n > 0; --n) {
+            tail += DP_CHEB_SCALE * (double)(n - 1) * (n - 1) * c[n - 1];
+            if (tail > 0x1p-55 * size) break;
+        }
+        need = n > need ? n : need;
+    }
+    need = (need + 3) / 4 * 4;
+    return need <= NN - 4 ? need : 0;
+}
+
+cudaError_t dp_launch_cheb_fwd(cudaStream_t st, const DevModel &m, const ChebModel &cm, const double *x,
+                               const int32_t *types, Box3 box, int N, const FormatBuffers &fb,
+                               const NlistBuffers &nb, EvalBuffers eb, int64_t *launches)
+{
+    const size_t smem = fwd_smem(m, cm.n);
+    cudaError_t e = cudaFuncSetAttribute(k_cheb_fwd, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_MAX);
+    if (e != cudaSuccess) return e;
+    k_cheb_fwd<<<N, CT, smem, st>>>(m, cm, x, types, box, nb.type_perm, fb.nlist, fb.nreal, eb.pair_g, eb.T, eb.D);
+    *launches += 1;
+    return cudaGetLastError();
+}
+
+cudaError_t dp_launch_cheb_bwd(cudaStream_t st, const DevModel &m, const ChebModel &cm, const int32_t *types, int N,
+                               const FormatBuffers &fb, const NlistBuffers &nb, EvalBuffers eb, int64_t *launches)
+{
+    const size_t smem = bwd_smem(m, cm.n);
+    cudaError_t e = cudaFuncSetAttribute(k_cheb_bwd, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_MAX);
+    if (e != cudaSuccess) return e;
+    k_cheb_bwd<<<N, CT, smem, st>>>(m, cm, types, nb.type_perm, fb.nreal, eb.T, eb.gD, eb.pair_g, eb.f_own,
+                                    eb.vir_part);
+    *launches += 1;
+    return cudaGetLastError();
+}
