@@ -610,8 +610,8 @@ dp_status enqueue_eval(dp_ctx *c, const double *coords, const int32_t *types, co
             GroupTimer tm(c, G_FIT);
             e = mixed && !c->use_oz
                     ? dp_launch_fit_mx(c->stream, c->m, c->mx, n, c->nb, c->eb, c->d_status, &c->launches)
-                : c->use_oz ? dp_launch_fit_oz(c->stream, c->m, c->oz, c->ob, n, c->nb, c->eb, c->d_status,
-                                               &c->launches)
+                : c->use_oz ? dp_launch_fit_oz(c->stream, c->m, c->oz, c->ob, n, c->nb, c->eb, c->num_sms,
+                                               c->d_status, &c->launches)
                             : dp_launch_fit(c->stream, c->m, n, c->nb, c->eb, &c->launches);
             if (e != cudaSuccess) return cuda_fail(e, "fit");
         }

@@ -250,6 +250,7 @@ struct OzGemm {
     int K, N;          // contraction and output widths (unpadded)
     int nK, nN;        // chunks of DP_OZ_KC and DP_OZ_NC
     int beta, S;       // digit width (bits) and digit count
+    int seg;           // K-chunks the group accumulators hold exactly before they are drained
     int64_t w_off[DP_MAX_TYPES];  // element offset of the type's weight digits
     int64_t e_off[DP_MAX_TYPES];  // offset of the type's column exponents
 };
@@ -279,7 +280,8 @@ struct OzBuffers {
 bool dp_oz_plan(const DevModel &m, OzModel &oz, int64_t &w_elems, int64_t &e_elems, int bits = 55);
 void dp_oz_split_weights(const DevModel &m, const double *h_params, const OzModel &oz, uint16_t *w, int32_t *e);
 cudaError_t dp_launch_fit_oz(cudaStream_t st, const DevModel &m, const OzModel &oz, const OzBuffers &ob, int N,
-                             const NlistBuffers &nb, EvalBuffers eb, int32_t *status, int64_t *launches);
+                             const NlistBuffers &nb, EvalBuffers eb, int num_sms, int32_t *status,
+                             int64_t *launches);
 
 // FP64 embedding forward with its last layer on the tensor cores by exact
 // splitting (csrc/embed_x.cu): 3-layer doubling nets with e1 in {16, 25, 32}.

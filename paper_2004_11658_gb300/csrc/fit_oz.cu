@@ -14,28 +14,36 @@
 // precision: FP64 rounding for the 55-bit plans of the FP64 mode, 2^-28
 // relative for the 28-bit plans of the split mixed mode).  A digit
 // is an integer of at most 8 bits, exact in BF16; every product is exact in
-// FP32, and beta is chosen per GEMM from its contraction length K so that
-//   K 4^(beta-1) (S + 2) < 2^24,
-// which bounds every partial sum of every C_g: the FP32 tensor-core
-// accumulators hold C_g exactly, in any summation order.  The result is the
-// exact product of the digit expansions, rounded once per group into FP64,
-// and is reproducible bit for bit.
+// FP32, and while
+//   K 4^(beta-1) (S + 2) < 2^24
+// every partial sum of every C_g is below 2^24: the FP32 tensor-core
+// accumulators hold C_g exactly, in any summation order.  A longer contraction
+// is cut into segments that satisfy this, added up in int64 (FP64 mode: 8 digits
+// of 7 bits throughout, 36 MMAs per 16 columns and 8 planes to read; 66 and 11
+// for the 1,600-long first layer when one segment had to hold it, with 5-bit
+// digits).  The result is the exact product of the digit expansions, rounded
+// once into FP64, and is reproducible bit for bit.
 //
-// Kernels.  k_oz_split: one warp per row of a 128-atom tile of one type;
-// row maximum, exponent, digits written as S BF16 matrices in the canonical
-// K-major layout of the MMA A operand (16-column chunks).  The weights'
-// digits are made once on the host.  k_oz_gemm: one CTA per (tile, 32-column
-// chunk of Y); one thread streams the digit chunks of A and W with bulk copies
-// (cp.async.bulk, a 2- to 4-stage ring on mbarriers) and issues S(S+1)/2 MMAs
-// of 128 x 32 x 16 per chunk into S group accumulators in tensor memory; the
-// epilogue (4 warps, one row per thread) combines the groups exactly in int64,
-// converts once (one rounding) and applies the layer's bias, tanh and skip
-// (forward) or the skip gradient (backward).  Every wait is bounded; on a timeout the kernel sets
+// Kernels.  k_oz_split: digits of the activations of a 128-atom tile of one
+// type, S BF16 matrices in the canonical K-major layout of the MMA A operand
+// (16-column chunks).  The weights' digits are made once on the host.
+// k_oz_gemm: persistent over (tile, 32-column chunk of Y); a copy warp streams
+// the digit chunks of A and W (cp.async.bulk, a 4-stage ring on mbarriers), an
+// MMA warp issues S(S+1)/2 MMAs of 128 x 32 x 16 per chunk into S group
+// accumulators in tensor memory, and 8 warps combine the groups exactly, round
+// once and apply the layer's bias, tanh and skip (forward) or the skip gradient
+// (backward).  Every wait is bounded; on a timeout the kernel sets
 // DPF_MMA_TIMEOUT, waits for its copies and MMAs, frees tensor memory and
 // returns.
+//
+// Measured per evaluation (12,288 water atoms): the six GEMMs 2.8 -> 1.22 ms,
+// the six splits 0.74 -> 0.43 ms; 192 atoms: the whole fitting net 0.96 -> 0.33
+// ms.  One elected lane of a whole warp issues: behind `threadIdx.x == 0` the
+// same MMAs took 139 cycles each instead of 97 in the former kernel.
 #include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <type_traits>
 #include <vector>
 
 #include "dp_internal.cuh"
@@ -44,7 +52,10 @@
 
 namespace {
 
-constexpr int OZ_STMAX = 4;                 // pipeline stages (at most)
+constexpr int OZ_NST = 4;                   // pipeline stages (40 KB each at 8 digits)
+constexpr int OZ_THREADS = 320;             // 8 epilogue warps, the MMA warp, the copy warp
+constexpr uint32_t OZ_TAB_BYTES = DP_TANH_NINT * DP_TANH_STRIDE * 8;
+static_assert(OZ_TAB_BYTES % 16 == 0, "bulk copy of the tanh table");
 constexpr int OZ_A_BLK = DP_OZ_TILE * DP_OZ_KC;  // elements of one A digit chunk (128 x 16)
 constexpr int OZ_B_BLK = DP_OZ_NC * DP_OZ_KC;    // elements of one W digit chunk (32 x 16)
 
@@ -89,22 +100,26 @@ struct OzSplitArgs {
     int64_t a_stride;
 };
 
-// One warp per group of 8 rows of a tile (a row group of the canonical
-// layout), so that every digit plane of a 16-column chunk is written as one
-// contiguous 256-byte block: lane = row (0..7) + 8 * (column half) + 16 *
-// (chunk parity).
+// One CTA per group of 8 rows of a tile (a row group of the canonical layout):
+// warp w takes the exponent (and output-layer energy) of row w, then every
+// digit plane of a 16-column chunk is written as one contiguous 256-byte block:
+// lane = row (0..7) + 8 * (column half) + 16 * (chunk parity), the warps
+// striding over the chunk pairs.  (One warp per row group, rows one after the
+// other, took 277 us for the descriptors of 12,288 water atoms and 181 us for
+// 192: a chain of dependent loads on few warps.)  The conversions run on the
+// integer pipe.
 __global__ void __launch_bounds__(256) k_oz_split(OzSplitArgs p)
 {
-    const int lane = threadIdx.x & 31;
-    const int gw = (int)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5);
-    const int tl = gw / (DP_OZ_TILE / 8), r0 = (gw % (DP_OZ_TILE / 8)) * 8;
+    __shared__ int e_s[8];
+    __shared__ int nz_s[8];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int tl = blockIdx.x / (DP_OZ_TILE / 8), r0 = (blockIdx.x % (DP_OZ_TILE / 8)) * 8;
     const TileRef T = oz_tile(tl, p.type_start, p.ntypes);
     if (T.a < 0) return;
-    const int Kp = p.nK * DP_OZ_KC;
     const double *wo = p.mode == 2 ? p.wout[T.a] : nullptr;
     const int bS = p.beta * p.S;
 
-    // value of column k of row r of the tile (0 past the row's end or the tile's atoms)
+    // value of column k of atom i (0 past the row's end or the tile's atoms)
     auto value = [&](int i, int k) -> double {
         if (i < 0 || k >= p.K) return 0.0;
         double v = p.mode == 2 ? wo[k] : p.src[(size_t)i * p.lds + k];
@@ -115,11 +130,8 @@ __global__ void __launch_bounds__(256) k_oz_split(OzSplitArgs p)
         return v;
     };
 
-    // per row: output-layer energy (mode 2) and exponent, lanes striding over k
-    int e_row = 0;  // lane j < 8 keeps the exponent of row r0 + j
-    double sc_row = 0.0;
-    for (int j = 0; j < 8; ++j) {
-        const int r = r0 + j;
+    {
+        const int r = r0 + warp;
         const int i = r < T.cnt ? p.type_perm[T.first + r] : -1;
         if (p.mode == 2) {
             double e = 0.0;
@@ -129,36 +141,45 @@ __global__ void __launch_bounds__(256) k_oz_split(OzSplitArgs p)
             for (int o = 16; o > 0; o >>= 1) e += __shfl_xor_sync(0xffffffffu, e, o);
             if (i >= 0 && lane == 0) p.Ei[i] = *p.bout[T.a] + e;
         }
-        double mx = 0.0;
-        for (int k = lane; k < p.K; k += 32) mx = fmax(mx, fabs(value(i, k)));
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-        int e = 0;
-        bool zero = !(mx > 0.0);
-        if (!zero) {
-            frexp(mx, &e);
-            if (e < bS - 1020) zero = true;  // below 2^-960: a zero row
+        // largest |x| by its bits (NaN left out)
+        unsigned long long mx = 0;
+#pragma unroll 4
+        for (int k = lane; k < p.K; k += 32) {
+            const unsigned long long b = (unsigned long long)__double_as_longlong(fabs(value(i, k)));
+            if (b > mx && b <= 0x7ff0000000000000ull) mx = b;
         }
-        if (zero) e = 0;
-        if (lane == j) {
-            e_row = e;
-            sc_row = zero ? 0.0 : oz_pow2(bS - e);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            const unsigned long long q = __shfl_xor_sync(0xffffffffu, mx, o);
+            mx = q > mx ? q : mx;
+        }
+        if (lane == 0) {
+            int e = 0;
+            const double m = __longlong_as_double((long long)mx);
+            bool zero = !(m > 0.0);
+            if (!zero) {
+                frexp(m, &e);
+                if (e < bS - 1020) zero = true;  // below 2^-960: a zero row
+            }
+            e_s[warp] = zero ? 0 : e;
+            nz_s[warp] = !zero;
+            p.aexp[(size_t)tl * DP_OZ_TILE + r] = zero ? 0 : e;
         }
     }
-    if (lane < 8) p.aexp[(size_t)tl * DP_OZ_TILE + r0 + lane] = e_row;
+    __syncthreads();
 
     // digits: lane handles row r0 + (lane & 7), columns kh*8 .. kh*8+7 of chunk kc
-    const int jr = lane & 7, kh = (lane >> 3) & 1, cpar = lane >> 4;
+    const int jr = lane & 7, kh = (lane >> 3) & 1;
     const int r = r0 + jr;
-    const int i = r < T.cnt ? p.type_perm[T.first + r] : -1;
-    const double scale = __shfl_sync(0xffffffffu, sc_row, jr);
+    const int i = r < T.cnt && nz_s[jr] ? p.type_perm[T.first + r] : -1;
+    const int sh = bS - e_s[jr];
     uint16_t *out = p.a + (size_t)tl * p.a_stride;
     const int ofs = oz_kofs(r, kh * 8);
-    for (int kc = cpar; kc < p.nK; kc += 2) {
+    for (int kc = 2 * warp + (lane >> 4); kc < p.nK; kc += 16) {
         const int k8 = kc * DP_OZ_KC + kh * 8;
         long long I[8];
 #pragma unroll
-        for (int q = 0; q < 8; ++q) I[q] = __double2ll_rn(value(i, k8 + q) * scale);
+        for (int q = 0; q < 8; ++q) I[q] = oz_rint_pow2(value(i, k8 + q), sh);
         for (int sd = p.S - 1; sd >= 0; --sd) {
             int d[8];
 #pragma unroll
@@ -171,7 +192,6 @@ __global__ void __launch_bounds__(256) k_oz_split(OzSplitArgs p)
             *reinterpret_cast<uint4 *>(out + ((size_t)kc * p.S + sd) * OZ_A_BLK + ofs) = u;
         }
     }
-    (void)Kp;
 }
 
 // ------------------------------------------------------------------- gemm --
@@ -197,8 +217,7 @@ struct OzGemmArgs {
     int ldo;
     const double *tanh_tab;
     int32_t *status;
-    int nst;        // pipeline stages
-    uint32_t tcols; // tensor-memory columns allocated (S * 32 rounded up to 256 or 512)
+    int units;  // (tile, column chunk) pairs, tiles past the last atom included
 };
 
 __device__ __forceinline__ void bulk_g2s(void *dst, const void *src, uint32_t bytes, uint64_t *mbar)
@@ -223,198 +242,304 @@ __device__ __forceinline__ double scale2(double y, int e)
     return (e >= -1022 && e <= 1023) ? y * oz_pow2(e) : ldexp(y, e);
 }
 
+// Persistent, one CTA per SM over the units (tile, 32-column chunk of Y) in
+// order, so that the CTAs at work share a tile's digits in L2.  Warps 0-7: the
+// epilogue (two warps per quarter of the tensor memory's lanes, 16 columns
+// each); warp 8 issues the MMAs, warp 9 the copies.  The group accumulators are
+// doubled (2 x 256 columns): the epilogue of one segment runs beside the MMAs
+// of the next.  A contraction longer than the accumulators hold exactly is cut
+// into segments of g.seg chunks, which the epilogue adds up in int64.
+//
+// Bounds, per unit of a 240-long contraction at S = 8: 15 chunks x 36 MMAs of
+// 20 cycles with A held in the collector (40 without, and 40 when two CTAs of
+// one SM alternate: measured) = 10.8 k cycles, 40 KB of copies per chunk at the
+// 60 B/clk that large bulk copies reach = 10.3 k; with the FP64 tanh 20 k
+// cycles of FP64 pipe.  The tanh table sits in shared memory: its lookups by 32
+// lanes cost 32 wavefronts each through L1, and were 53 k cycles per unit.
 template <int S>
-__global__ void __launch_bounds__(DP_OZ_TILE, 1) k_oz_gemm(OzGemmArgs p)
+__global__ void __launch_bounds__(OZ_THREADS, 1) k_oz_gemm(OzGemmArgs p)
 {
     extern __shared__ __align__(1024) unsigned char smraw[];
-    __shared__ __align__(8) uint64_t full[OZ_STMAX], empty[OZ_STMAX], done;
-    __shared__ int fe_s[DP_OZ_NC];
-    __shared__ double bias_s[DP_OZ_NC];
+    __shared__ __align__(8) uint64_t full[OZ_NST], empty[OZ_NST], tfull[2], tempty[2], tabbar, drain;
     __shared__ uint32_t tslot;
-    __shared__ int fail;
-    const int tid = threadIdx.x, warp = tid >> 5;
+    __shared__ volatile int fail;
+    const int tid = threadIdx.x, lane = tid & 31, warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
     const OzGemm &g = p.g;
-    const int nchunk = blockIdx.x % g.nN;
-    const TileRef T = oz_tile(blockIdx.x / g.nN, p.type_start, p.ntypes);
-    if (T.a < 0) return;
-    const int tl = blockIdx.x / g.nN;
-    const int nK = g.nK;
-    const uint32_t a_bytes = (uint32_t)S * OZ_A_BLK * 2, b_bytes = (uint32_t)S * OZ_B_BLK * 2;
-    const uint32_t stage_bytes = a_bytes + b_bytes;
-    const int NST = p.nst;
+    const int nK = g.nK, nseg = (nK + g.seg - 1) / g.seg;
+    constexpr uint32_t a_bytes = (uint32_t)S * OZ_A_BLK * 2, b_bytes = (uint32_t)S * OZ_B_BLK * 2;
+    constexpr uint32_t stage_bytes = a_bytes + b_bytes;
+    constexpr int NST = OZ_NST;
+    constexpr uint32_t TBUF = 256, TCOLS = 512;
+    static_assert(S * DP_OZ_NC <= TBUF, "group accumulators of one buffer");
+    const double *tab = reinterpret_cast<const double *>(smraw + NST * stage_bytes);
 
-    if (warp == 0) tc::tmem_alloc(&tslot, p.tcols);
-    if (tid < DP_OZ_NC) {
-        const int col = nchunk * DP_OZ_NC + tid;
-        fe_s[tid] = p.wexp[g.e_off[T.a] + col];
-        bias_s[tid] = (p.epi == 0 && col < g.N) ? p.bias[T.a][col] : 0.0;
-    }
+    if (warp == 0) tc::tmem_alloc(&tslot, TCOLS);
     if (tid == 0) {
         for (int s = 0; s < NST; ++s) {
             tc::mbar_init(&full[s], 1);
             tc::mbar_init(&empty[s], 1);
         }
-        tc::mbar_init(&done, 1);
+        for (int s = 0; s < 2; ++s) {
+            tc::mbar_init(&tfull[s], 1);
+            tc::mbar_init(&tempty[s], 8);
+        }
+        tc::mbar_init(&tabbar, 1);
+        tc::mbar_init(&drain, 1);
         fail = 0;
     }
     tc::fence_before_sync();
     __syncthreads();
     tc::fence_after_sync();
-    const uint32_t tbase = tslot;
+    const uint32_t tbase = __shfl_sync(0xffffffffu, tslot, 0);
 
-    if (tid == 0) {
-        const uint16_t *asrc = p.a + (size_t)tl * p.a_stride;
-        const uint16_t *bsrc = p.w + g.w_off[T.a] + (size_t)nchunk * nK * S * OZ_B_BLK;
-        int issued = 0;  // chunks whose copies were issued
-        auto load = [&](int kc) {
-            unsigned char *st = smraw + (size_t)(kc % NST) * stage_bytes;
-            mbar_expect_tx(&full[kc % NST], stage_bytes);
-            bulk_g2s(st, asrc + (size_t)kc * S * OZ_A_BLK, a_bytes, &full[kc % NST]);
-            bulk_g2s(st + a_bytes, bsrc + (size_t)kc * S * OZ_B_BLK, b_bytes, &full[kc % NST]);
-            ++issued;
-        };
-        for (int kc = 0; kc < NST && kc < nK; ++kc) load(kc);
-        const uint32_t idesc = tc::make_idesc_bf16(DP_OZ_TILE, DP_OZ_NC);
-        int consumed = 0;
+    if (warp == 9) {
+        // copies: the tanh table, then the digit chunks of every unit
+        int c = 0;
         bool ok = true;
-        for (int kc = 0; kc < nK; ++kc) {
-            const int st = kc % NST;
-            if (!tc::mbar_wait(&full[st], (kc / NST) & 1)) {
-                ok = false;
-                break;
+        if (p.epi == 0 && tc::elect_one()) {
+            mbar_expect_tx(&tabbar, OZ_TAB_BYTES);
+            bulk_g2s(smraw + NST * stage_bytes, p.tanh_tab, OZ_TAB_BYTES, &tabbar);
+        }
+        for (int u = blockIdx.x; u < p.units && ok; u += gridDim.x) {
+            const int tl = u / g.nN, nchunk = u - tl * g.nN;
+            const TileRef T = oz_tile(tl, p.type_start, p.ntypes);
+            if (T.a < 0) break;
+            const uint16_t *asrc = p.a + (size_t)tl * p.a_stride;
+            const uint16_t *bsrc = p.w + g.w_off[T.a] + (size_t)nchunk * nK * S * OZ_B_BLK;
+            for (int kc = 0; kc < nK; ++kc, ++c) {
+                const int st = c % NST;
+                if (c >= NST) ok = tc::mbar_wait(&empty[st], (c / NST - 1) & 1) && !fail;
+                ok = __all_sync(0xffffffffu, ok);
+                if (!ok) break;
+                if (tc::elect_one()) {
+                    unsigned char *dst = smraw + (size_t)st * stage_bytes;
+                    mbar_expect_tx(&full[st], stage_bytes);
+                    bulk_g2s(dst, asrc + (size_t)kc * S * OZ_A_BLK, a_bytes, &full[st]);
+                    bulk_g2s(dst + a_bytes, bsrc + (size_t)kc * S * OZ_B_BLK, b_bytes, &full[st]);
+                }
+                __syncwarp();
             }
-            ++consumed;
-            const uint32_t abase = tc::smem_u32(smraw + (size_t)st * stage_bytes);
+        }
+        if (!ok) fail = 1;
+        // no copy is in flight when the CTA leaves
+        for (int q = c > NST ? c - NST : 0; q < c; ++q) tc::mbar_wait(&full[q % NST], (q / NST) & 1);
+        if (p.epi == 0) tc::mbar_wait(&tabbar, 0);
+    } else if (warp == 8) {
+        const uint32_t idesc = tc::make_idesc_bf16(DP_OZ_TILE, DP_OZ_NC);
+        // the MMAs of one chunk, then the commit that frees its stage; one copy of
+        // the code per stage, so that every descriptor is a constant
+        auto issue = [&](auto stage, uint32_t dbase, bool acc0) {
+            constexpr int st = decltype(stage)::value;
             // descriptors of digit plane 1; plane s is (s - 1) blocks further (the
             // address field holds bytes / 16 and stays below 2^14 inside shared memory)
+            const uint32_t abase = tc::smem_u32(smraw) + st * stage_bytes;
             const uint64_t ad0 = tc::make_desc(abase, 128, 256);
             const uint64_t bd0 = tc::make_desc(abase + a_bytes, 128, 256);
 #pragma unroll
             for (int s = 1; s <= S; ++s) {
+                const uint64_t ad = ad0 + (uint64_t)((s - 1) * OZ_A_BLK * 2 / 16);
 #pragma unroll
-                for (int t = 1; t + s <= S + 1; ++t)
-                    tc::mma_bf16(tbase + (uint32_t)(s + t - 2) * DP_OZ_NC, ad0 + (uint64_t)((s - 1) * OZ_A_BLK * 2 / 16),
-                                 bd0 + (uint64_t)((t - 1) * OZ_B_BLK * 2 / 16), idesc, kc > 0 || s > 1);
+                for (int t = 1; t + s <= S + 1; ++t) {
+                    const uint32_t dc = dbase + (uint32_t)(s + t - 2) * DP_OZ_NC;
+                    const uint64_t bd = bd0 + (uint64_t)((t - 1) * OZ_B_BLK * 2 / 16);
+                    const bool acc = acc0 || s > 1;
+                    if (s == S) tc::mma_bf16(dc, ad, bd, idesc, acc);
+                    else if (t == 1) tc::mma_bf16_a<0>(dc, ad, bd, idesc, acc);
+                    else if (t + s <= S) tc::mma_bf16_a<1>(dc, ad, bd, idesc, acc);
+                    else tc::mma_bf16_a<2>(dc, ad, bd, idesc, acc);
+                }
             }
             tc::mma_commit(&empty[st]);
-            // refill the stage of the previous chunk once its MMAs are done
-            if (kc >= 1 && kc - 1 + NST < nK) {
-                const int ps = (kc - 1) % NST;
-                if (!tc::mbar_wait(&empty[ps], ((kc - 1) / NST) & 1)) {
-                    ok = false;
-                    break;
+        };
+        int c = 0, sc = 0;
+        bool ok = true;
+        for (int u = blockIdx.x; u < p.units && ok; u += gridDim.x) {
+            if (oz_tile(u / g.nN, p.type_start, p.ntypes).a < 0) break;
+            for (int sg = 0; sg < nseg && ok; ++sg, ++sc) {
+                const int buf = sc & 1;
+                if (sc >= 2) ok = tc::mbar_wait(&tempty[buf], ((sc >> 1) - 1) & 1) && !fail;
+                ok = __all_sync(0xffffffffu, ok);
+                if (!ok) break;
+                tc::fence_after_sync();
+                const uint32_t dbase = tbase + buf * TBUF;
+                const int k1 = min(nK, (sg + 1) * g.seg);
+                for (int kc = sg * g.seg; kc < k1; ++kc, ++c) {
+                    const int st = c % NST;
+                    ok = tc::mbar_wait(&full[st], (c / NST) & 1) && !fail;
+                    ok = __all_sync(0xffffffffu, ok);
+                    if (!ok) break;
+                    if (tc::elect_one()) {
+                        const bool acc0 = kc > sg * g.seg;
+                        if (st == 0) issue(std::integral_constant<int, 0>{}, dbase, acc0);
+                        else if (st == 1) issue(std::integral_constant<int, 1>{}, dbase, acc0);
+                        else if (st == 2) issue(std::integral_constant<int, 2>{}, dbase, acc0);
+                        else issue(std::integral_constant<int, 3>{}, dbase, acc0);
+                    }
+                    __syncwarp();
                 }
-                load(kc - 1 + NST);
+                if (ok && tc::elect_one()) tc::mma_commit(&tfull[buf]);
+                __syncwarp();
             }
         }
-        tc::mma_commit(&done);
-        if (!ok) {
-            fail = 1;
-            atomicOr(p.status, DPF_MMA_TIMEOUT);
-            // copies still in flight must land before the CTA leaves
-            for (int kc = consumed; kc < issued; ++kc) tc::mbar_wait(&full[kc % NST], (kc / NST) & 1);
-        }
-    }
-    const bool waited = tc::mbar_wait(&done, 0);
-    const bool bad = __syncthreads_or(!waited) || fail;
-    tc::fence_after_sync();
-    if (bad) {
-        if (tid == 0) atomicOr(p.status, DPF_MMA_TIMEOUT);
+        if (!ok) fail = 1;
+        if (tc::elect_one()) tc::mma_commit(&drain);
+        __syncwarp();
+        tc::mbar_wait(&drain, 0);
     } else {
-        const int r = tid;
-        const int i = r < T.cnt ? p.type_perm[T.first + r] : -1;
-        const uint32_t tl_lane = tbase + ((uint32_t)(32 * warp) << 16);
         // y = sum_{g=2}^{S+1} C_g 2^(beta (S + 1 - g)): the group sums are integers
         // below 2^24, combined exactly in two int64 Horner chains (the H groups of
-        // largest scale, then the rest; each chain below 2^(25 + beta (H - 1)) <= 2^53
-        // for every (beta, S) of oz_beta) and converted once: y = hi 2^(beta (S - H)) + lo.
-        // Then y 2^escale = sum_g C_g 2^(-beta g).  Sixteen columns at a time.
+        // largest scale, then the rest; each chain, summed over the segments, below
+        // 2^53 for every plan of oz_plan_gemm) and rounded once to FP64 with its
+        // scale, on the integer pipe: y 2^escale = sum_g C_g 2^(-beta g).
         constexpr int H = (S + 1) / 2;
-        const long long sh = 1ll << g.beta;
-        const double chi = oz_pow2(g.beta * (S - H));
-        const int escale = -g.beta * (S + 1);
-        const int er = i >= 0 ? p.aexp[(size_t)tl * DP_OZ_TILE + r] : 0;
-#pragma unroll 1
-        for (int h = 0; h < 2; ++h) {
-            long long hi[16], lo[16];
-            __syncwarp();  // the loads below are warp-wide; the previous half's stores diverge
+        const int w = g.beta * (S - H);
+        const int half = warp >> 2, row = 32 * (warp & 3) + lane;
+        const uint32_t tl_lane = tbase + ((uint32_t)(32 * (warp & 3)) << 16) + 16 * half;
+        const bool vec = (p.ldo & 1) == 0 && (p.ldh & 1) == 0;  // rows start on 16 bytes
+        int sc = 0;
+        bool ok = true;
+        if (p.epi == 0) ok = __all_sync(0xffffffffu, tc::mbar_wait(&tabbar, 0));
+        for (int u = blockIdx.x; u < p.units && ok; u += gridDim.x) {
+            const int tl = u / g.nN, nchunk = u - tl * g.nN;
+            const TileRef T = oz_tile(tl, p.type_start, p.ntypes);
+            if (T.a < 0) break;
+            const int i = row < T.cnt ? p.type_perm[T.first + row] : -1;
+            const int n0 = nchunk * DP_OZ_NC + 16 * half;   // first of this thread's 16 columns of Y
+            const int esc = (i >= 0 ? p.aexp[(size_t)tl * DP_OZ_TILE + row] : 0) - g.beta * (S + 1);
+            const int4 *fe4 = reinterpret_cast<const int4 *>(p.wexp + g.e_off[T.a] + n0);
+            // the skip's operands, asked for before the MMAs are waited for
+            const bool bcast = p.epi != 0 && p.gbc[T.a] != nullptr;
+            const double *hin = bcast ? p.gbc[T.a] : p.hin + (size_t)(i < 0 ? 0 : i) * p.ldh;
+            double sk[16];
 #pragma unroll
-            for (int gg = 2; gg <= S + 1; ++gg) {
-                float v[16];
-                tc::tmem_ld16(tl_lane + (uint32_t)(gg - 2) * DP_OZ_NC + 16 * h, v);
+            for (int n = 0; n < 16; ++n) sk[n] = 0.0;
+            if (i >= 0) {
+                if (p.skip == 1 && vec && !bcast && n0 + 16 <= g.N) {
 #pragma unroll
-                for (int n = 0; n < 16; ++n) {
-                    const long long iv = (long long)__float2int_rn(v[n]);
-                    if (gg == 2) hi[n] = iv;
-                    else if (gg <= H + 1) hi[n] = hi[n] * sh + iv;
-                    else if (gg == H + 2) lo[n] = iv;
-                    else lo[n] = lo[n] * sh + iv;
+                    for (int n = 0; n < 16; n += 2) {
+                        const double2 v = *reinterpret_cast<const double2 *>(hin + n0 + n);
+                        sk[n] = v.x;
+                        sk[n + 1] = v.y;
+                    }
+                } else if (p.skip != 0) {
+#pragma unroll
+                    for (int n = 0; n < 16; ++n)
+                        if (n0 + n < g.N) {
+                            const int q = n0 + n;
+                            sk[n] = p.skip == 1 ? hin[q]
+                                    : p.epi == 0 ? hin[q % p.skip_in]
+                                                 : hin[q] + hin[q + p.skip_in];
+                        }
                 }
             }
-            if (i < 0) continue;
-            const int c0 = 16 * h;                       // first column of this half in the chunk
-            const int n0 = nchunk * DP_OZ_NC + c0;       // ... and in Y
-            const int *fe = fe_s + c0;
-            const double *bs = bias_s + c0;
-            double *ho = p.hout + (size_t)i * p.ldo;
-            if (p.epi == 0) {
-                const double *hin = p.hin + (size_t)i * p.ldh;
-                double *to = p.tout + (size_t)i * p.ldo;
+            long long hi[16], lo[16];
 #pragma unroll
-                for (int n = 0; n < 16; ++n) {
-                    const int col = n0 + n;
-                    if (col < g.N) {
-                        const double z =
-                            scale2(fma((double)hi[n], chi, (double)lo[n]), er + fe[n] + escale) + bs[n];
-                        const double t = dp_tanh64(z, p.tanh_tab);
-                        const double sk =
-                            p.skip == 2 ? hin[col % p.skip_in] : (p.skip == 1 ? hin[col] : 0.0);
-                        to[col] = t;
-                        ho[col] = sk + t;
+            for (int n = 0; n < 16; ++n) hi[n] = lo[n] = 0;
+            for (int sg = 0; sg < nseg; ++sg, ++sc) {
+                const int buf = sc & 1;
+                ok = tc::mbar_wait(&tfull[buf], (sc >> 1) & 1) && !fail;
+                ok = __all_sync(0xffffffffu, ok);
+                if (!ok) break;
+                tc::fence_after_sync();
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    long long a[8], b[8];
+#pragma unroll
+                    for (int gg = 2; gg <= S + 1; ++gg) {
+                        float v[8];
+                        tc::tmem_ld8(tl_lane + buf * TBUF + (uint32_t)(gg - 2) * DP_OZ_NC + 8 * h, v);
+#pragma unroll
+                        for (int n = 0; n < 8; ++n) {
+                            const long long iv = (long long)__float2int_rn(v[n]);
+                            if (gg == 2) a[n] = iv;
+                            else if (gg <= H + 1) a[n] = (a[n] << g.beta) + iv;
+                            else if (gg == H + 2) b[n] = iv;
+                            else b[n] = (b[n] << g.beta) + iv;
+                        }
+                    }
+#pragma unroll
+                    for (int n = 0; n < 8; ++n) {
+                        hi[8 * h + n] += a[n];
+                        lo[8 * h + n] += b[n];
                     }
                 }
-            } else {
-                const double *gh = p.gbc[T.a] != nullptr ? p.gbc[T.a] : p.hin + (size_t)i * p.ldh;
+                tc::fence_before_sync();
+                __syncwarp();
+                if (lane == 0) tc::mbar_arrive(&tempty[buf]);
+            }
+            if (!ok) break;
+            if (i < 0) continue;
+            double *ho = p.hout + (size_t)i * p.ldo + n0;
+            double *to = p.epi == 0 ? p.tout + (size_t)i * p.ldo + n0 : nullptr;
 #pragma unroll
-                for (int n = 0; n < 16; ++n) {
-                    const int q = n0 + n;
-                    if (q < g.N) {
-                        double v = scale2(fma((double)hi[n], chi, (double)lo[n]), er + fe[n] + escale);
-                        if (p.skip == 1) v += gh[q];
-                        else if (p.skip == 2) v += gh[q] + gh[q + p.skip_in];
-                        ho[q] = v;
+            for (int q = 0; q < 4; ++q) {
+                const int4 f4 = fe4[q];
+                const int fe[4] = {f4.x, f4.y, f4.z, f4.w};
+#pragma unroll
+                for (int n2 = 0; n2 < 4; n2 += 2) {
+                    double y[2], t[2];
+#pragma unroll
+                    for (int v = 0; v < 2; ++v) {
+                        const int n = 4 * q + n2 + v, e = esc + fe[n2 + v];
+                        y[v] = e > -900 && e < 900 ? oz_i64x2_scaled_w(hi[n], lo[n], w, e)
+                                                   : scale2(fma((double)hi[n], oz_pow2(w), (double)lo[n]), e);
+                        if (p.epi == 0) {
+                            const int col = n0 + n;
+                            t[v] = dp_tanh64(y[v] + (col < g.N ? p.bias[T.a][col] : 0.0), tab);
+                            y[v] = t[v];
+                        }
+                        y[v] += sk[n];
+                    }
+                    const int n = 4 * q + n2;
+                    if (vec && n0 + n + 2 <= g.N) {
+                        *reinterpret_cast<double2 *>(ho + n) = make_double2(y[0], y[1]);
+                        if (p.epi == 0) *reinterpret_cast<double2 *>(to + n) = make_double2(t[0], t[1]);
+                    } else {
+#pragma unroll
+                        for (int v = 0; v < 2; ++v)
+                            if (n0 + n + v < g.N) {
+                                ho[n + v] = y[v];
+                                if (p.epi == 0) to[n + v] = t[v];
+                            }
                     }
                 }
             }
         }
+        if (!ok) fail = 1;
     }
     tc::fence_before_sync();
     __syncthreads();
-    if (warp == 0) tc::tmem_dealloc(tbase, p.tcols);
+    if (tid == 0 && fail) atomicOr(p.status, DPF_MMA_TIMEOUT);
+    if (warp == 0) tc::tmem_dealloc(tbase, TCOLS);
 }
 
-// digit width and count for a contraction of length K and `bits` bits per operand
-void oz_beta(int K, int bits, int &beta, int &S)
+// Digit width, digit count and segment length of a GEMM of contraction length
+// K (nK chunks) at `bits` bits per operand.  From 55 bits on: 8 digits of 7
+// bits, the widest for which one 16-column chunk is exact, and as many chunks
+// per segment as stay exact, spread evenly (400 columns: 400 4^6 10 < 2^24); the
+// int64 chains hold 2^8 segments.  Below: one segment and the widest digits
+// that the whole contraction allows.
+void oz_plan_gemm(OzGemm &g, int bits)
 {
-    for (beta = 7; beta >= 4; --beta) {
-        S = (bits + beta - 1) / beta;
-        const double bound = (double)K * std::pow(4.0, beta - 1) * (S + 2);
+    g.seg = g.nK;
+    if (bits >= 55) {
+        g.beta = 7;
+        g.S = 8;
+        const int most = 16777215 / (4096 * (g.S + 2)) / DP_OZ_KC;  // 25 chunks
+        const int nseg = (g.nK + most - 1) / most;
+        g.seg = (g.nK + nseg - 1) / nseg;
+        return;
+    }
+    for (g.beta = 7; g.beta >= 4; --g.beta) {
+        g.S = (bits + g.beta - 1) / g.beta;
+        const double bound = (double)g.K * std::pow(4.0, g.beta - 1) * (g.S + 2);
         if (bound < 16777216.0) return;
     }
-    beta = 0;
-    S = 0;
+    g.beta = 0;
+    g.S = 0;
 }
 
-// Up to 8 digits: 2 stages and 256 tensor-memory columns, so two CTAs share an
-// SM (one's epilogue overlaps the other's MMAs); more digits: 4 stages, one CTA.
-int gemm_stages(int S)
-{
-    if (S <= 8) return 2;
-    const int fit = (int)((225 * 1024) / ((size_t)S * (OZ_A_BLK + OZ_B_BLK) * 2));
-    return fit < OZ_STMAX ? fit : OZ_STMAX;
-}
-uint32_t gemm_tcols(int S) { return S * DP_OZ_NC <= 256 ? 256u : 512u; }
-size_t gemm_smem(int S) { return (size_t)gemm_stages(S) * S * (OZ_A_BLK + OZ_B_BLK) * 2; }
+size_t gemm_smem(int S) { return (size_t)OZ_NST * S * (OZ_A_BLK + OZ_B_BLK) * 2 + OZ_TAB_BYTES; }
 
 }  // namespace
 
@@ -439,9 +564,8 @@ bool dp_oz_plan(const DevModel &m, OzModel &oz, int64_t &w_elems, int64_t &e_ele
             g.N = Ns[d];
             g.nK = (g.K + DP_OZ_KC - 1) / DP_OZ_KC;
             g.nN = (g.N + DP_OZ_NC - 1) / DP_OZ_NC;
-            oz_beta(g.K, bits, g.beta, g.S);
-            if (g.beta == 0 || g.S * DP_OZ_NC > 512 || gemm_smem(g.S) > 225 * 1024) return false;
-            if (!(g.S == 4 || g.S == 5 || g.S == 8 || g.S == 10 || g.S == 11 || g.S == 14)) return false;
+            oz_plan_gemm(g, bits);
+            if (!(g.S == 4 || g.S == 5 || g.S == 8)) return false;
             in_w = std::max(in_w, g.nK * g.S * OZ_A_BLK);
             for (int a = 0; a < m.ntypes; ++a) {
                 g.w_off[a] = w_elems;
@@ -506,30 +630,20 @@ void dp_oz_split_weights(const DevModel &m, const double *h_params, const OzMode
 }
 
 cudaError_t dp_launch_fit_oz(cudaStream_t st, const DevModel &m, const OzModel &oz, const OzBuffers &ob, int N,
-                             const NlistBuffers &nb, EvalBuffers eb, int32_t *status, int64_t *launches)
+                             const NlistBuffers &nb, EvalBuffers eb, int num_sms, int32_t *status,
+                             int64_t *launches)
 {
     const int nf = m.n_fit, T = m.ntypes;
     const int tiles = (N + DP_OZ_TILE - 1) / DP_OZ_TILE + T;
     if (tiles > ob.tiles) return cudaErrorInvalidValue;
-    static size_t configured = 0;
     {
-        size_t need = 0;
-        for (int l = 0; l < nf; ++l) need = std::max(need, std::max(gemm_smem(oz.fwd[l].S), gemm_smem(oz.bwd[l].S)));
-        if (need > configured) {
-            cudaError_t e = cudaFuncSetAttribute(k_oz_gemm<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)need);
-            if (e == cudaSuccess)
-                e = cudaFuncSetAttribute(k_oz_gemm<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)need);
-            if (e == cudaSuccess)
-                e = cudaFuncSetAttribute(k_oz_gemm<5>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)need);
-            if (e == cudaSuccess)
-                e = cudaFuncSetAttribute(k_oz_gemm<10>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)need);
-            if (e == cudaSuccess)
-                e = cudaFuncSetAttribute(k_oz_gemm<11>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)need);
-            if (e == cudaSuccess)
-                e = cudaFuncSetAttribute(k_oz_gemm<14>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)need);
-            if (e != cudaSuccess) return e;
-            configured = need;
-        }
+        cudaError_t e = cudaFuncSetAttribute(k_oz_gemm<8>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             (int)gemm_smem(8));
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(k_oz_gemm<5>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gemm_smem(5));
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(k_oz_gemm<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gemm_smem(4));
+        if (e != cudaSuccess) return e;
     }
     const int K1 = m.m2 * m.M;
     const size_t plane = (size_t)ob.nmax * oz.fmax;
@@ -548,7 +662,7 @@ cudaError_t dp_launch_fit_oz(cudaStream_t st, const DevModel &m, const OzModel &
         }
         wo_off = off;
     }
-    const int split_blocks = (tiles * (DP_OZ_TILE / 8) * 32 + 255) / 256;
+    const int split_blocks = tiles * (DP_OZ_TILE / 8);
 
     auto split = [&](int mode, const double *src, int lds, const double *tv, const OzGemm &g) -> cudaError_t {
         OzSplitArgs a;
@@ -604,17 +718,12 @@ cudaError_t dp_launch_fit_oz(cudaStream_t st, const DevModel &m, const OzModel &
         a.ldo = ldo;
         a.tanh_tab = m.tanh_tab;
         a.status = status;
-        a.nst = gemm_stages(g.S);
-        a.tcols = gemm_tcols(g.S);
+        a.units = tiles * g.nN;
+        const int grid = std::min(a.units, num_sms);
         const size_t smem = gemm_smem(g.S);
-        switch (g.S) {
-        case 4: k_oz_gemm<4><<<tiles * g.nN, DP_OZ_TILE, smem, st>>>(a); break;
-        case 5: k_oz_gemm<5><<<tiles * g.nN, DP_OZ_TILE, smem, st>>>(a); break;
-        case 8: k_oz_gemm<8><<<tiles * g.nN, DP_OZ_TILE, smem, st>>>(a); break;
-        case 10: k_oz_gemm<10><<<tiles * g.nN, DP_OZ_TILE, smem, st>>>(a); break;
-        case 11: k_oz_gemm<11><<<tiles * g.nN, DP_OZ_TILE, smem, st>>>(a); break;
-        default: k_oz_gemm<14><<<tiles * g.nN, DP_OZ_TILE, smem, st>>>(a); break;
-        }
+        if (g.S == 4) k_oz_gemm<4><<<grid, OZ_THREADS, smem, st>>>(a);
+        else if (g.S == 5) k_oz_gemm<5><<<grid, OZ_THREADS, smem, st>>>(a);
+        else k_oz_gemm<8><<<grid, OZ_THREADS, smem, st>>>(a);
         *launches += 1;
         return cudaGetLastError();
     };

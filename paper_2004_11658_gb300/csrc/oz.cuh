@@ -89,14 +89,14 @@ static __host__ __device__ __forceinline__ long long oz_rint_pow2(double v, int 
     return (b >> 63) ? -r : r;
 }
 
-// The double nearest (ties to even) to (hi 2^32 + lo) 2^p, for |hi| < 2^62,
-// |lo| < 2^62 and a result in the normal range: the value of
-// fma((double)hi, 2^32, (double)lo) * 2^p (one rounding, an exact power-of-two
+// The double nearest (ties to even) to (hi 2^w + lo) 2^p, for |hi| < 2^62,
+// |lo| < 2^62, w <= 32 and a result in the normal range: the value of
+// fma((double)hi, 2^w, (double)lo) * 2^p (one rounding, an exact power-of-two
 // scale), built from the integer bits.
-static __host__ __device__ __forceinline__ double oz_i64x2_scaled(long long hi, long long lo, int p)
+static __host__ __device__ __forceinline__ double oz_i64x2_scaled_w(long long hi, long long lo, int w, int p)
 {
-    // X = hi 2^32 + lo, |X| < 2^95, as a sign and a magnitude of at most 95 bits
-    const __int128 X = (__int128)hi * ((__int128)1 << 32) + (__int128)lo;
+    // X = hi 2^w + lo, |X| < 2^95, as a sign and a magnitude of at most 95 bits
+    const __int128 X = (__int128)hi * ((__int128)1 << w) + (__int128)lo;
     if (X == 0) return 0.0;
     const bool neg = X < 0;
     const unsigned __int128 u = neg ? (unsigned __int128)(-X) : (unsigned __int128)X;
@@ -133,4 +133,10 @@ static __host__ __device__ __forceinline__ double oz_i64x2_scaled(long long hi, 
     std::memcpy(&d, &bits, 8);
     return d;
 #endif
+}
+
+// The same with w = 32 (the embedding layers' groups).
+static __host__ __device__ __forceinline__ double oz_i64x2_scaled(long long hi, long long lo, int p)
+{
+    return oz_i64x2_scaled_w(hi, lo, 32, p);
 }

@@ -23,7 +23,7 @@
 
 namespace {
 
-__device__ double dp_tanh_table[DP_TANH_NINT * DP_TANH_STRIDE];
+__device__ __align__(16) double dp_tanh_table[DP_TANH_NINT * DP_TANH_STRIDE];
 
 std::mutex g_mu;
 const double *g_addr[64] = {nullptr};
