@@ -251,6 +251,7 @@ dp_status read_box(const double *box, Box3 &b)
         b.L[a] = box[4 * a];
         if (!(b.L[a] > 0.0) || !std::isfinite(b.L[a])) return fail(DP_ERR_BOX, "cell edges must be positive");
     }
+    dp_make_box(b);
     return DP_OK;
 }
 
@@ -947,7 +948,7 @@ void dp_ctx_free(dp_ctx *c)
     if (c->h_mass_stage) cudaFreeHost(c->h_mass_stage);
     if (c->h_cheb_mx) cudaFreeHost(c->h_cheb_mx);
     void *bufs[] = {c->nb.cand, c->nb.ncand, c->nb.xref, c->nb.cell_count, c->nb.cell_start,
-                    c->nb.cell_cursor, c->nb.cell_atoms, c->nb.cell_sorted, c->nb.atom_cell,
+                    c->nb.cell_cursor, c->nb.cell_atoms, c->nb.cell_sorted, c->nb.cell_pos, c->nb.atom_cell,
                     c->nb.type_perm, c->nb.type_start, c->fb.nlist, c->fb.keys, c->fb.nreal,
                     c->eb.T, c->eb.D, c->eb.gD, c->eb.Ei, c->eb.pair_g, c->eb.f_own, c->eb.vir_part,
                     c->d_energy, c->d_virial, c->md_force, c->ke_part, c->d_inv_mass_conv, c->d_mass,
@@ -999,6 +1000,7 @@ dp_status dp_ctx_create(const dp_model *model, int64_t natoms_max, int32_t cand_
     ALLOC(c->nb.xref, 3 * N);
     ALLOC(c->nb.cell_atoms, N);
     ALLOC(c->nb.cell_sorted, N);
+    ALLOC(c->nb.cell_pos, N);
     ALLOC(c->nb.atom_cell, N);
     ALLOC(c->nb.type_perm, N);
     ALLOC(c->nb.type_start, T + 1);
@@ -1319,7 +1321,7 @@ dp_status dp_md_kick_drift(dp_ctx *c, double *coords, double *vel, const double 
     if (box) {
         if ((s = read_box(box, b))) return s;
     } else {
-        b.L[0] = b.L[1] = b.L[2] = 0.0;   // no wrapping
+        b = Box3{};   // no wrapping
     }
     if ((s = upload_masses(c, mass_per_type))) return s;
     if (N > 0) {

@@ -2,8 +2,10 @@
 // of the GB300 Deep Potential library (not part of the public ABI).
 #pragma once
 
+#include <cmath>
 #include <cuda_runtime.h>
 #include <stdint.h>
+#include <string.h>
 
 #include "../../include/dp.h"
 
@@ -36,32 +38,74 @@ struct DevModel {
     int64_t fit_base[DP_MAX_TYPES];
 };
 
+// Cell edges, and for dp_min_image_1 the high words of 0.4999 L, 0.5001 L
+// (rounded up) and 1.4999 L (dp_make_box).
 struct Box3 {
     double L[3];
+    int lo[3], hi[3], hi2[3];
 };
+
+inline int dp_hiword(double v)
+{
+    int64_t b;
+    memcpy(&b, &v, 8);
+    return (int)(b >> 32);
+}
+
+inline void dp_make_box(Box3 &b)
+{
+    for (int a = 0; a < 3; ++a) {
+        b.lo[a] = dp_hiword(0.4999 * b.L[a]);
+        b.hi[a] = dp_hiword(0.5001 * b.L[a]) + 1;
+        b.hi2[a] = dp_hiword(1.4999 * b.L[a]);
+    }
+}
+
+// The bits of the largest r^2 whose correctly rounded square root is <= R:
+// r <= R, decided on r^2 (as unsigned bits: a NaN compares above).
+inline uint64_t dp_r2_bits(double R)
+{
+    double q = R * R;
+    while (std::sqrt(q) > R) q = std::nextafter(q, 0.0);
+    for (double n = std::nextafter(q, INFINITY); std::sqrt(n) <= R; n = std::nextafter(n, INFINITY)) q = n;
+    uint64_t b;
+    memcpy(&b, &q, 8);
+    return b;
+}
 
 // ---------------------------------------------------------------------------
 // Pinned distance arithmetic.  Candidate sets and sort keys must be identical
 // to the CPU reference bit for bit, so the minimum image and |r| are computed
 // with explicitly rounded operations (no FMA contraction):
 //   d = xj - xi; d -= L * rint(d / L); r = sqrt((dx*dx + dy*dy) + dz*dz).
+// n = rint(d / L) is 0 or +-1 for almost every pair and is then decided by the
+// high word of |d| (the quotient is away from the ties), which leaves two
+// subtractions instead of a division, a rint and a product; the FP64 pipe, which
+// every distance kernel is bound by, has 16 cycles per warp instruction.
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ double dp_min_image_1(double xj, double xi, double L)
+__device__ __forceinline__ double dp_min_image_1(double xj, double xi, const Box3 &b, int a)
 {
-    double v = __dsub_rn(xj, xi);
-    double n = rint(__ddiv_rn(v, L));
-    return __dsub_rn(v, __dmul_rn(L, n));
+    const double v = __dsub_rn(xj, xi), L = b.L[a];
+    const int h = __double2hiint(v) & 0x7fffffff;
+    const bool in = h < b.lo[a];
+    if (in || (h >= b.hi[a] && h < b.hi2[a])) return __dsub_rn(v, in ? 0.0 : copysign(L, v));
+    return __dsub_rn(v, __dmul_rn(L, rint(__ddiv_rn(v, L))));
+}
+
+// r^2 of the minimum image d of xj - xi.
+__device__ __forceinline__ double dp_pinned_r2(const double *xi, const double *xj, const Box3 &b, double d[3])
+{
+    d[0] = dp_min_image_1(xj[0], xi[0], b, 0);
+    d[1] = dp_min_image_1(xj[1], xi[1], b, 1);
+    d[2] = dp_min_image_1(xj[2], xi[2], b, 2);
+    const double r2 = __dadd_rn(__dmul_rn(d[0], d[0]), __dmul_rn(d[1], d[1]));
+    return __dadd_rn(r2, __dmul_rn(d[2], d[2]));
 }
 
 __device__ __forceinline__ double dp_pinned_dist(const double *xi, const double *xj, const Box3 &b,
                                                  double d[3])
 {
-    d[0] = dp_min_image_1(xj[0], xi[0], b.L[0]);
-    d[1] = dp_min_image_1(xj[1], xi[1], b.L[1]);
-    d[2] = dp_min_image_1(xj[2], xi[2], b.L[2]);
-    double r2 = __dadd_rn(__dmul_rn(d[0], d[0]), __dmul_rn(d[1], d[1]));
-    r2 = __dadd_rn(r2, __dmul_rn(d[2], d[2]));
-    return __dsqrt_rn(r2);
+    return __dsqrt_rn(dp_pinned_r2(xi, xj, b, d));
 }
 
 // Packed sort key of Algorithm 1: (type, floor(|r| * 1e8), j) as
@@ -151,6 +195,7 @@ struct NlistBuffers {
     int32_t *cell_cursor; // [ncell]
     int32_t *cell_atoms;  // [N]
     int32_t *cell_sorted; // [N]
+    float4 *cell_pos;     // [N] wrapped positions in cell order, for the candidates' first test
     int32_t *atom_cell;   // [N]
     int32_t *type_perm;   // [N]
     int32_t *type_start;  // [ntypes + 1]

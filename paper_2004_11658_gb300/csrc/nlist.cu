@@ -120,10 +120,11 @@ __global__ void k_cell_fill(const int32_t *__restrict__ atom_cell, int N,
 }
 
 // Order each cell's atoms by index (rank sort; cells hold ~10^2 atoms), so the
-// candidate order does not depend on the atomics of k_cell_fill.
-__global__ void k_cell_sort(const int32_t *__restrict__ cell_start, int ncell,
+// candidate order does not depend on the atomics of k_cell_fill, with their
+// wrapped positions beside them.
+__global__ void k_cell_sort(const double *__restrict__ x, Box3 box, const int32_t *__restrict__ cell_start, int ncell,
                             const int32_t *__restrict__ cell_atoms, int32_t *__restrict__ cell_sorted,
-                            const int32_t *gate)
+                            float4 *__restrict__ cell_pos, const int32_t *gate)
 {
     DP_GATED(gate);
     int c = blockIdx.x;
@@ -133,6 +134,8 @@ __global__ void k_cell_sort(const int32_t *__restrict__ cell_start, int ncell,
         int v = cell_atoms[b + p], rank = 0;
         for (int q = 0; q < n; ++q) rank += cell_atoms[b + q] < v;
         cell_sorted[b + rank] = v;
+        cell_pos[b + rank] = make_float4((float)wrap1(x[3 * v], box.L[0]), (float)wrap1(x[3 * v + 1], box.L[1]),
+                                         (float)wrap1(x[3 * v + 2], box.L[2]), 0.0f);
     }
 }
 
@@ -145,44 +148,91 @@ __device__ __forceinline__ void append_candidate(bool take, int j, int lane, int
     n += __popc(bal);
 }
 
-// One warp per atom: scan the 27 cells around the atom's cell.
+// One warp per atom: scan the 27 cells around the atom's cell (the three cells
+// along x at once where they are adjacent in memory).  One pair in seven is a
+// candidate, so the atoms first pass an FP32 test with a margin (rlo2, covering
+// the rounding of the wrapped FP32 positions) on coalesced loads; the survivors
+// are collected in order and take the exact test 32 at a time, on r^2.
+// 98,304 water atoms: 17.1 -> 0.76 ms (before: the FP64 test of every pair,
+// with a division per component and a square root).
 __global__ void __launch_bounds__(128) k_cand_cells(
     const double *__restrict__ x, int N, Box3 box, int nx, int ny, int nz,
     const int32_t *__restrict__ atom_cell, const int32_t *__restrict__ cell_start,
-    const int32_t *__restrict__ cell_sorted, double rlist, int cap, int32_t *__restrict__ cand,
-    int32_t *__restrict__ ncand, double *__restrict__ xref, int32_t *status, const int32_t *gate)
+    const int32_t *__restrict__ cell_sorted, const float4 *__restrict__ cell_pos, uint64_t r2max, float rlo2, int cap,
+    int32_t *__restrict__ cand, int32_t *__restrict__ ncand, double *__restrict__ xref, int32_t *status,
+    const int32_t *gate)
 {
     DP_GATED(gate);
+    __shared__ int32_t buf[4][64];
     const int lane = threadIdx.x & 31;
     const int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     if (i >= N) return;
+    int32_t *bw = buf[threadIdx.x >> 5];
     const double xi[3] = {x[3 * i], x[3 * i + 1], x[3 * i + 2]};
+    const float L[3] = {(float)box.L[0], (float)box.L[1], (float)box.L[2]};
+    const float iL[3] = {1.0f / L[0], 1.0f / L[1], 1.0f / L[2]};
+    const float fi[3] = {(float)wrap1(xi[0], box.L[0]), (float)wrap1(xi[1], box.L[1]), (float)wrap1(xi[2], box.L[2])};
     const int ci = atom_cell[i];
     const int cx = ci % nx, cy = (ci / nx) % ny, cz = ci / (nx * ny);
     int32_t *row = cand + (size_t)i * cap;
-    int n = 0;
-    for (int dz = -1; dz <= 1; ++dz)
-        for (int dy = -1; dy <= 1; ++dy)
-            for (int dx = -1; dx <= 1; ++dx) {
-                int qx = (cx + dx + nx) % nx, qy = (cy + dy + ny) % ny, qz = (cz + dz + nz) % nz;
-                int c = (qz * ny + qy) * nx + qx;
-                int b = cell_start[c], e = cell_start[c + 1];
-                for (int p0 = b; p0 < e; p0 += 32) {
-                    int p = p0 + lane;
-                    bool take = false;
-                    int j = -1;
-                    if (p < e) {
-                        j = cell_sorted[p];
-                        if (j != i) {
-                            double d[3];
-                            const double xj[3] = {x[3 * j], x[3 * j + 1], x[3 * j + 2]};
-                            double r = dp_pinned_dist(xi, xj, box, d);
-                            take = r <= rlist;
-                        }
-                    }
-                    append_candidate(take, j, lane, n, cap, row);
+    int n = 0, have = 0;
+    auto exact = [&](int m) {  // the first m survivors of the buffer
+        bool take = false;
+        int j = -1;
+        if (lane < m) {
+            j = bw[lane];
+            double d[3];
+            const double xj[3] = {x[3 * j], x[3 * j + 1], x[3 * j + 2]};
+            take = (uint64_t)__double_as_longlong(dp_pinned_r2(xi, xj, box, d)) <= r2max;
+        }
+        append_candidate(take, j, lane, n, cap, row);
+    };
+    auto range = [&](int b, int e) {
+        for (int p0 = b; p0 < e; p0 += 32) {
+            const int p = p0 + lane;
+            bool near = false;
+            int j = -1;
+            if (p < e) {
+                const float4 q = cell_pos[p];
+                float dx = q.x - fi[0], dy = q.y - fi[1], dz = q.z - fi[2];
+                dx -= L[0] * rintf(dx * iL[0]);
+                dy -= L[1] * rintf(dy * iL[1]);
+                dz -= L[2] * rintf(dz * iL[2]);
+                // a NaN position passes on to the exact test
+                near = !(dx * dx + dy * dy + dz * dz > rlo2);
+                if (near) {
+                    j = cell_sorted[p];
+                    near = j != i;
                 }
             }
+            const unsigned bal = __ballot_sync(FULL, near);
+            if (near) bw[have + __popc(bal & ((1u << lane) - 1u))] = j;
+            have += __popc(bal);
+            __syncwarp();
+            if (have >= 32) {
+                exact(32);
+                const int rest = lane < have - 32 ? bw[32 + lane] : 0;
+                __syncwarp();
+                bw[lane] = rest;
+                have -= 32;
+                __syncwarp();
+            }
+        }
+    };
+    for (int dz = -1; dz <= 1; ++dz)
+        for (int dy = -1; dy <= 1; ++dy) {
+            const int qy = (cy + dy + ny) % ny, qz = (cz + dz + nz) % nz;
+            const int c0 = (qz * ny + qy) * nx;
+            if (cx > 0 && cx + 1 < nx) {
+                range(cell_start[c0 + cx - 1], cell_start[c0 + cx + 2]);
+            } else {
+                for (int dx = -1; dx <= 1; ++dx) {
+                    const int c = c0 + (cx + dx + nx) % nx;
+                    range(cell_start[c], cell_start[c + 1]);
+                }
+            }
+        }
+    exact(have);
     if (lane == 0) {
         if (n > cap) atomicOr(status, DPF_CAND_OVERFLOW);
         ncand[i] = min(n, cap);
@@ -194,7 +244,7 @@ __global__ void __launch_bounds__(128) k_cand_cells(
 
 // Small boxes (< 3 cells along an axis): every j, in index order.
 __global__ void __launch_bounds__(128) k_cand_brute(const double *__restrict__ x, int N, Box3 box,
-                                                    double rlist, int cap,
+                                                    uint64_t r2max, int cap,
                                                     int32_t *__restrict__ cand,
                                                     int32_t *__restrict__ ncand,
                                                     double *__restrict__ xref, int32_t *status,
@@ -213,7 +263,7 @@ __global__ void __launch_bounds__(128) k_cand_brute(const double *__restrict__ x
         if (j < N && j != i) {
             double d[3];
             const double xj[3] = {x[3 * j], x[3 * j + 1], x[3 * j + 2]};
-            take = dp_pinned_dist(xi, xj, box, d) <= rlist;
+            take = (uint64_t)__double_as_longlong(dp_pinned_r2(xi, xj, box, d)) <= r2max;
         }
         append_candidate(take, j, lane, n, cap, row);
     }
@@ -332,20 +382,22 @@ __device__ __forceinline__ void warp_bitonic_sort(uint64_t (&v)[KPL], int lane)
     }
 }
 
-// One warp per atom.  The candidates within rcut -- L(i) of Sec. 2 -- are
-// keyed and compacted into a per-warp shared buffer with ballots, then sorted
-// by a KPL*32-wide bitonic network in registers.  In the first pass (retry
+// One warp per atom.  The candidates within rcut -- L(i) of Sec. 2, decided on
+// r^2 -- are compacted into a per-warp shared buffer with ballots, then keyed
+// (the square root, on full lanes) and sorted by a KPL*32-wide bitonic network
+// in registers (98,304 water atoms: 2.54 -> 1.15 ms; the root of every candidate,
+// with divisions, before).  In the first pass (retry
 // list null) an atom with more than KPL*32 keys is appended to the retry list
 // and left to a second launch with a network as wide as the candidate cap.
 template <int KPL>
 __global__ void __launch_bounds__(128) k_format(
     DevModel m, const double *__restrict__ x, const int32_t *__restrict__ types, Box3 box, int N,
-    int cap, double stale2, const int32_t *__restrict__ cand, const int32_t *__restrict__ ncand,
+    int cap, uint64_t r2cut, double stale2, const int32_t *__restrict__ cand, const int32_t *__restrict__ ncand,
     const double *__restrict__ xref, int32_t *__restrict__ nlist, uint64_t *__restrict__ keys,
     int32_t *__restrict__ nreal, int32_t *status, int32_t *retry_count, int32_t *retry_list, int retry_pass)
 {
     constexpr int S = 32 * KPL;
-    __shared__ uint64_t kbuf[4][S];
+    __shared__ int32_t jbuf[4][S];
     const int lane = threadIdx.x & 31, wl = threadIdx.x >> 5;
     const int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     int i;
@@ -366,30 +418,26 @@ __global__ void __launch_bounds__(128) k_format(
         if (r * r > stale2) atomicOr(status, DPF_STALE);
     }
     const int32_t *row = cand + (size_t)i * cap;
-    uint64_t *kb = kbuf[wl];
+    int32_t *jb = jbuf[wl];
     int n = 0;
     for (int c0 = 0; c0 < ncnd; c0 += 32) {
         const int idx = c0 + lane;
         bool take = false;
-        uint64_t key = 0;
+        int j = 0;
         if (idx < ncnd) {
-            const int j = row[idx];
+            j = row[idx];
             const int tj = types[j];
             if ((unsigned)tj < (unsigned)T) {
                 double d[3];
                 const double xj[3] = {x[3 * j], x[3 * j + 1], x[3 * j + 2]};
-                const double r = dp_pinned_dist(xi, xj, box, d);
-                if (r <= m.rcut) {
-                    take = true;
-                    key = dp_pack_key(tj, r, j);
-                }
+                take = (uint64_t)__double_as_longlong(dp_pinned_r2(xi, xj, box, d)) <= r2cut;
             } else {
                 atomicOr(status, DPF_BAD_TYPE);
             }
         }
         const unsigned bal = __ballot_sync(FULL, take);
         const int pos = n + __popc(bal & ((1u << lane) - 1u));
-        if (take && pos < S) kb[pos] = key;
+        if (take && pos < S) jb[pos] = j;
         n += __popc(bal);
     }
     if (n > S) {  // cannot happen in the retry pass (S >= cap >= ncand)
@@ -404,7 +452,13 @@ __global__ void __launch_bounds__(128) k_format(
 #pragma unroll
     for (int e = 0; e < KPL; ++e) {
         const int p = lane * KPL + e;
-        v[e] = p < n ? kb[p] : DP_KEY_NONE;
+        v[e] = DP_KEY_NONE;
+        if (p < n) {
+            const int j = jb[p];
+            double d[3];
+            const double xj[3] = {x[3 * j], x[3 * j + 1], x[3 * j + 2]};
+            v[e] = dp_pack_key(types[j], dp_pinned_dist(xi, xj, box, d), j);
+        }
     }
     warp_bitonic_sort<KPL>(v, lane);
 
@@ -474,6 +528,7 @@ cudaError_t dp_launch_build(cudaStream_t st, const DevModel &m, const double *x,
     const int TB = 256;
     const bool cells = nc[0] >= 3 && nc[1] >= 3 && nc[2] >= 3;
     const int wblocks = (N + 3) / 4;  // 4 warps (atoms) per 128-thread CTA
+    const uint64_t r2max = dp_r2_bits(rlist);
     if (cells) {
         const int ncell = nc[0] * nc[1] * nc[2];
         k_zero_cells<<<(ncell + TB - 1) / TB, TB, 0, st>>>(nb.cell_count, ncell, gate);
@@ -482,13 +537,17 @@ cudaError_t dp_launch_build(cudaStream_t st, const DevModel &m, const double *x,
         k_cell_scan<<<1, 1024, 0, st>>>(nb.cell_count, ncell, nb.cell_start, nb.cell_cursor, gate);
         k_cell_fill<<<(N + TB - 1) / TB, TB, 0, st>>>(nb.atom_cell, N, nb.cell_start, nb.cell_cursor,
                                                       nb.cell_atoms, gate);
-        k_cell_sort<<<ncell, 128, 0, st>>>(nb.cell_start, ncell, nb.cell_atoms, nb.cell_sorted, gate);
-        k_cand_cells<<<wblocks, 128, 0, st>>>(x, N, box, nc[0], nc[1], nc[2], nb.atom_cell,
-                                              nb.cell_start, nb.cell_sorted, rlist, cap, nb.cand,
-                                              nb.ncand, nb.xref, status, gate);
+        k_cell_sort<<<ncell, 128, 0, st>>>(x, box, nb.cell_start, ncell, nb.cell_atoms, nb.cell_sorted, nb.cell_pos,
+                                           gate);
+        // FP32 margin: 1e-3 A, and 16 roundings of a coordinate below the longest edge
+        const double Lm = std::max(box.L[0], std::max(box.L[1], box.L[2]));
+        const float rlo = (float)(rlist * (1.0 + 1e-6) + 1e-3 + 16.0 * Lm * 0x1p-23);
+        k_cand_cells<<<wblocks, 128, 0, st>>>(x, N, box, nc[0], nc[1], nc[2], nb.atom_cell, nb.cell_start,
+                                              nb.cell_sorted, nb.cell_pos, r2max, rlo * rlo, cap, nb.cand, nb.ncand,
+                                              nb.xref, status, gate);
         *launches += 6;
     } else {
-        k_cand_brute<<<wblocks, 128, 0, st>>>(x, N, box, rlist, cap, nb.cand, nb.ncand, nb.xref,
+        k_cand_brute<<<wblocks, 128, 0, st>>>(x, N, box, r2max, cap, nb.cand, nb.ncand, nb.xref,
                                               status, gate);
         *launches += 1;
     }
@@ -520,9 +579,10 @@ cudaError_t dp_launch_format(cudaStream_t st, const DevModel &m, const double *x
 {
     const int blocks = (N + 3) / 4;
     const double stale2 = skin > 0.0 ? 0.25 * skin * skin : 0.0;
+    const uint64_t r2cut = dp_r2_bits(m.rcut);
     cudaMemsetAsync(retry, 0, sizeof(int32_t), st);
 #define DP_FMT(K, RP)                                                                                  \
-    k_format<K><<<blocks, 128, 0, st>>>(m, x, types, box, N, cap, stale2, nb.cand, nb.ncand, nb.xref,  \
+    k_format<K><<<blocks, 128, 0, st>>>(m, x, types, box, N, cap, r2cut, stale2, nb.cand, nb.ncand, nb.xref,  \
                                         fb.nlist, fb.keys, fb.nreal, status, retry, retry + 1, RP)
     // first pass: network of sort_small keys
     switch (sort_small) {

@@ -78,6 +78,7 @@ extern "C" dp_status dp_format_nlist_noalloc(const dp_model_desc *desc, const do
         b.L[a] = box[4 * a];
         if (!(b.L[a] >= 2.0 * rlist)) return fail(DP_ERR_BOX, "dp_format_nlist_noalloc: every cell edge must be >= 2 (rcut + skin)");
     }
+    dp_make_box(b);
 
     // One-time set-up per device, with that device current: the device
     // address of the scratch array.
