@@ -534,12 +534,9 @@ dp_status ensure_oz(dp_ctx *c)
         if ((s = dev_alloc(&ob.g, 2 * plane, "fitting activations"))) return s;
     }
     if (c->oz_version != c->model->version) {
-        std::vector<uint16_t> w((size_t)c->oz_w_elems, 0);
-        std::vector<int32_t> e((size_t)c->oz_e_elems, 0);
-        dp_oz_split_weights(c->m, c->model->h_params, c->oz, w.data(), e.data());
-        DP_CUDA(cudaStreamSynchronize(c->stream), "fitting digits");
-        DP_CUDA(cudaMemcpy(c->d_oz_w, w.data(), w.size() * 2, cudaMemcpyHostToDevice), "fitting digits");
-        DP_CUDA(cudaMemcpy(c->d_oz_e, e.data(), e.size() * 4, cudaMemcpyHostToDevice), "fitting digits");
+        GroupTimer tm(c, G_FIT);
+        cudaError_t e = dp_launch_oz_weights(c->stream, c->m, c->oz, c->d_oz_w, c->d_oz_e, &c->launches);
+        if (e != cudaSuccess) return cuda_fail(e, "fitting digits");
         c->oz_version = c->model->version;
     }
     return DP_OK;

@@ -513,6 +513,81 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_oz_gemm(OzGemmArgs p)
     if (warp == 0) tc::tmem_dealloc(tbase, TCOLS);
 }
 
+// Weight digits of every type, layer and direction, one CTA per 32 rows of a B
+// operand: row n of the forward operand is column n of W_l, row q of the
+// backward operand is row q of W_l.  (On the host this took most of a training
+// step on a small frame; the parameters change every step.)
+__global__ void __launch_bounds__(256) k_oz_wsplit(DevModel m, OzModel oz, uint16_t *__restrict__ w,
+                                                   int32_t *__restrict__ e)
+{
+    __shared__ unsigned long long mx_s[8][DP_OZ_NC];
+    int u = blockIdx.x, a = 0, l = 0, d = 0;
+    int kin = m.m2 * m.M;
+    int64_t off = 0;
+    for (;;) {
+        const OzGemm &t = d == 0 ? oz.fwd[l] : oz.bwd[l];
+        if (u < t.nN) break;
+        u -= t.nN;
+        if (++d == 2) {
+            d = 0;
+            off += (int64_t)kin * m.fit[l] + m.fit[l];
+            kin = m.fit[l];
+            if (++l == m.n_fit) {
+                l = 0;
+                ++a;
+                off = 0;
+                kin = m.m2 * m.M;
+            }
+        }
+    }
+    const OzGemm &g = d == 0 ? oz.fwd[l] : oz.bwd[l];
+    const double *W = m.params + m.fit_base[a] + off;
+    const int F = m.fit[l], rl = threadIdx.x & 31, sl = threadIdx.x >> 5, row = u * DP_OZ_NC + rl;
+    auto elem = [&](int k) -> double {
+        if (k >= g.K || row >= g.N) return 0.0;
+        return d == 0 ? W[(size_t)k * F + row] : W[(size_t)row * F + k];
+    };
+    unsigned long long mx = 0;  // parameters are finite
+#pragma unroll 4
+    for (int k = sl; k < g.K; k += 8) {
+        const unsigned long long b = (unsigned long long)__double_as_longlong(fabs(elem(k)));
+        mx = b > mx ? b : mx;
+    }
+    mx_s[sl][rl] = mx;
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < 8; ++q) mx = mx_s[q][rl] > mx ? mx_s[q][rl] : mx;
+    const double big = __longlong_as_double((long long)mx);
+    const int bS = g.beta * g.S;
+    int ex = 0;
+    bool zero = !(big > 0.0);
+    if (!zero) {
+        frexp(big, &ex);
+        if (ex < bS - 1020) zero = true;
+    }
+    if (zero) ex = 0;
+    if (sl == 0) e[g.e_off[a] + row] = ex;
+    uint16_t *out = w + g.w_off[a] + (size_t)u * g.nK * g.S * OZ_B_BLK;
+    for (int kb = sl; kb < 2 * g.nK; kb += 8) {
+        const int kc = kb >> 1, kh = kb & 1;
+        long long I[8];
+#pragma unroll
+        for (int q = 0; q < 8; ++q)
+            I[q] = zero ? 0 : oz_rint_pow2(elem(kc * DP_OZ_KC + kh * 8 + q), bS - ex);
+        for (int sd = g.S - 1; sd >= 0; --sd) {
+            int dg[8];
+#pragma unroll
+            for (int q = 0; q < 8; ++q) dg[q] = sd > 0 ? oz_digit_step(I[q], g.beta) : (int)I[q];
+            uint4 v;
+            v.x = (uint32_t)oz_bf16_int(dg[0]) | ((uint32_t)oz_bf16_int(dg[1]) << 16);
+            v.y = (uint32_t)oz_bf16_int(dg[2]) | ((uint32_t)oz_bf16_int(dg[3]) << 16);
+            v.z = (uint32_t)oz_bf16_int(dg[4]) | ((uint32_t)oz_bf16_int(dg[5]) << 16);
+            v.w = (uint32_t)oz_bf16_int(dg[6]) | ((uint32_t)oz_bf16_int(dg[7]) << 16);
+            *reinterpret_cast<uint4 *>(out + ((size_t)kc * g.S + sd) * OZ_B_BLK + oz_kofs(rl, kh * 8)) = v;
+        }
+    }
+}
+
 // Digit width, digit count and segment length of a GEMM of contraction length
 // K (nK chunks) at `bits` bits per operand.  From 55 bits on: 8 digits of 7
 // bits, the widest for which one 16-column chunk is exact, and as many chunks
@@ -582,51 +657,14 @@ bool dp_oz_plan(const DevModel &m, OzModel &oz, int64_t &w_elems, int64_t &e_ele
     return true;
 }
 
-void dp_oz_split_weights(const DevModel &m, const double *h_params, const OzModel &oz, uint16_t *w, int32_t *e)
+cudaError_t dp_launch_oz_weights(cudaStream_t st, const DevModel &m, const OzModel &oz, uint16_t *w, int32_t *e,
+                                 int64_t *launches)
 {
-    const int nf = m.n_fit;
-    for (int a = 0; a < m.ntypes; ++a) {
-        const double *W = h_params + m.fit_base[a];
-        int kin = m.m2 * m.M;
-        for (int l = 0; l < nf; ++l) {
-            const int F = m.fit[l];
-            // element (k, n) of W_l is W[k * F + n]; the forward GEMM's B operand is
-            // B[n][k] = W[k][n] (columns n), the backward's is B[q][n] = W[q][n] (rows q)
-            for (int d = 0; d < 2; ++d) {
-                const OzGemm &g = d == 0 ? oz.fwd[l] : oz.bwd[l];
-                auto elem = [&](int row, int k) -> double {  // B[row][k]
-                    if (d == 0) return (k < kin && row < F) ? W[(size_t)k * F + row] : 0.0;
-                    return (k < F && row < kin) ? W[(size_t)row * F + k] : 0.0;
-                };
-                const int Np = g.nN * DP_OZ_NC, Kp = g.nK * DP_OZ_KC;
-                for (int row = 0; row < Np; ++row) {
-                    double mx = 0.0;
-                    for (int k = 0; k < Kp; ++k) mx = std::max(mx, std::fabs(elem(row, k)));
-                    int ex = 0;
-                    bool zero = !(mx > 0.0);
-                    if (!zero) {
-                        std::frexp(mx, &ex);
-                        if (ex < g.beta * g.S - 1020) zero = true;
-                    }
-                    if (zero) ex = 0;
-                    e[g.e_off[a] + row] = ex;
-                    const double scale = zero ? 0.0 : std::ldexp(1.0, g.beta * g.S - ex);
-                    const int nc = row / DP_OZ_NC, rl = row % DP_OZ_NC;
-                    for (int k = 0; k < Kp; ++k) {
-                        long long I = std::llrint(elem(row, k) * scale);
-                        const int kc = k / DP_OZ_KC;
-                        uint16_t *blk = w + g.w_off[a] + ((size_t)nc * g.nK + kc) * g.S * OZ_B_BLK;
-                        for (int s = g.S - 1; s >= 0; --s) {
-                            const int dg = s > 0 ? oz_digit_step(I, g.beta) : (int)I;
-                            blk[(size_t)s * OZ_B_BLK + oz_kofs(rl, k % DP_OZ_KC)] = oz_bf16_int(dg);
-                        }
-                    }
-                }
-            }
-            W += (size_t)kin * F + F;
-            kin = F;
-        }
-    }
+    int grid = 0;
+    for (int l = 0; l < m.n_fit; ++l) grid += oz.fwd[l].nN + oz.bwd[l].nN;
+    k_oz_wsplit<<<grid * m.ntypes, 256, 0, st>>>(m, oz, w, e);
+    *launches += 1;
+    return cudaGetLastError();
 }
 
 cudaError_t dp_launch_fit_oz(cudaStream_t st, const DevModel &m, const OzModel &oz, const OzBuffers &ob, int N,
