@@ -39,3 +39,27 @@ cudaError_t dp_launch_cheb_fwd(cudaStream_t st, const DevModel &m, const ChebMod
                                const NlistBuffers &nb, EvalBuffers eb, int64_t *launches);
 cudaError_t dp_launch_cheb_bwd(cudaStream_t st, const DevModel &m, const ChebModel &cm, const int32_t *types, int N,
                                const FormatBuffers &fb, const NlistBuffers &nb, EvalBuffers eb, int64_t *launches);
+
+// Parameter gradient through the series (csrc/embed_cheb.cu): T, dT, D, dD of
+// every atom with the moments kept, then, from dPhi/dD and dPhi/d(dD), the
+// gradient of the embedding nets' parameters by way of the coefficients.
+struct ChebGradBuffers {
+    double *mom;    // [N][T n][8] moments and their tangents
+    double *part;   // [DP_CHEB_SPLITS][T T][NN][M] partial coefficient adjoints
+    double *node;   // [T T][NN][2][sum of widths] layer outputs and z adjoints at the nodes
+    int32_t *far;   // set when a row lies beyond S: the caller's other kernels run instead
+};
+constexpr int DP_CHEB_SPLITS = 64;
+// Terms the gradient keeps: the parameter derivatives' series converge as the
+// nets' with a polynomial factor, which 8 more terms cover.
+inline int dp_cheb_grad_terms(int n) { return n + 8 < DP_CHEB_NN ? n + 8 : DP_CHEB_NN; }
+size_t dp_cheb_grad_elems(const DevModel &m, int n, int64_t natoms, int which);  // doubles of mom, part, node
+bool dp_cheb_grad_supported(const DevModel &m, int n);
+cudaError_t dp_launch_chebpg_fwd(cudaStream_t st, const DevModel &m, const ChebModel &cm, const double *x,
+                                 const int32_t *types, Box3 box, int N, const double *lam, const FormatBuffers &fb,
+                                 const NlistBuffers &nb, EvalBuffers eb, PGradBuffers pb, ChebGradBuffers gb,
+                                 int64_t *launches);
+// Overwrites eb.T and pb.dT; writes grad[0 .. T T emb_net_size).
+cudaError_t dp_launch_chebpg_bwd(cudaStream_t st, const DevModel &m, const ChebModel &cm, int N,
+                                 const NlistBuffers &nb, EvalBuffers eb, PGradBuffers pb, ChebGradBuffers gb,
+                                 const double *trig, double *grad, int64_t *launches);

@@ -156,6 +156,7 @@ struct dp_ctx {
     ChebModel cheb;
     ChebBuffers cb;
     double *h_cheb_mx;  // pinned host copy of cb.mx
+    ChebGradBuffers cg; // parameter gradient (allocated on first use)
     int64_t cheb_version;
     // mixed precision: BF16 / FP32 copies of the parameters
     MixedModel mx;
@@ -952,7 +953,8 @@ void dp_ctx_free(dp_ctx *c)
                     c->eb.fit_t, c->eb.fit_h, c->d_p32, c->d_emb_ops, c->d_fit_fwd, c->d_fit_bwd,
                     c->pb.dT, c->pb.dD, c->pb.Db, c->pb.dDb, c->pb.fit_scr, c->pb.rowscr, c->pb.slices,
                     c->d_oz_w, c->d_oz_e, c->ob.a, c->ob.aexp, c->ob.t, c->ob.h, c->ob.g, c->d_dtile, c->d_ex_w,
-                    c->eb.Gst, c->eb.Gmx, c->cb.C, c->cb.Ct, c->cb.y, c->cb.mx, c->cb.trig};
+                    c->eb.Gst, c->eb.Gmx, c->cb.C, c->cb.Ct, c->cb.y, c->cb.mx, c->cb.trig, c->cg.mom,
+                    c->cg.part, c->cg.node, c->cg.far};
     for (void *p : bufs) dev_free(p);
     delete c;
 }
@@ -1383,21 +1385,34 @@ dp_status dp_param_grad(dp_ctx *c, const double *coords, const int32_t *types, c
     const size_t Nmax = (size_t)c->natoms_max, M = (size_t)c->m.M, nd = (size_t)c->m.m2 * M;
     if (!c->pb.slices) {
 #define ALLOCP(ptr, n) \
-    if (!s) s = dev_alloc(&(ptr), (n), #ptr)
+    if (!s && !(ptr)) s = dev_alloc(&(ptr), (n), #ptr)
         ALLOCP(c->pb.dT, Nmax * 4 * M);
         ALLOCP(c->pb.dD, Nmax * nd);
         ALLOCP(c->pb.Db, Nmax * nd);
         ALLOCP(c->pb.dDb, Nmax * nd);
         ALLOCP(c->pb.fit_scr, dp_pgrad_fit_scratch((int)Nmax));
         ALLOCP(c->pb.rowscr, dp_pgrad_row_scratch(c->num_sms));
-        ALLOCP(c->pb.slices, (size_t)c->num_sms * np);
+        if (c->use_cheb && dp_cheb_grad_supported(c->m, DP_CHEB_NN)) {
+            ALLOCP(c->cg.mom, dp_cheb_grad_elems(c->m, DP_CHEB_NN, c->natoms_max, 0));
+            ALLOCP(c->cg.part, dp_cheb_grad_elems(c->m, DP_CHEB_NN, c->natoms_max, 1));
+            ALLOCP(c->cg.node, dp_cheb_grad_elems(c->m, DP_CHEB_NN, c->natoms_max, 2));
+            ALLOCP(c->cg.far, 1);
+        }
+        ALLOCP(c->pb.slices, (size_t)c->num_sms * np);  // last: marks the set as complete
 #undef ALLOCP
         if (s) return s;
     }
     if ((s = ensure_perm(c, types, N))) return s;
     if ((s = enqueue_format(c, coords, types, b, N))) return s;
+    ChebModel cm;
+    if (c->use_cheb && (s = ensure_cheb(c))) return s;
+    const bool cheb = c->cg.far && c->cheb.n > 0;
+    if (cheb) {
+        cm = c->cheb;
+        cm.n = dp_cheb_grad_terms(cm.n);
+    }
     cudaError_t e = dp_launch_pgrad(c->stream, c->m, np, coords, types, b, (int)N, lambda, cE, c->fb, c->nb, c->eb,
-                                    c->pb, c->num_sms, grad, &c->launches);
+                                    c->pb, c->num_sms, cheb ? &cm : nullptr, &c->cg, c->cb.trig, grad, &c->launches);
     if (e != cudaSuccess) return cuda_fail(e, "dp_param_grad");
     return finish(c);
 }

@@ -377,7 +377,8 @@ cudaError_t dp_launch_embed_bwd_mx(cudaStream_t st, const DevModel &m, const Mix
 // true if the mixed-precision kernels support this model shape
 bool dp_mixed_supported(const DevModel &m);
 
-// Parameter gradient of cE E + sum lambda . F (pgrad.cu).
+// Parameter gradient of cE E + sum lambda . F (pgrad.cu); cm, cg, trig: the
+// embedding nets' series and their buffers, null to work through the nets.
 struct PGradBuffers {
     double *dT;       // [N][4][M] tangent of T
     double *dD;       // [N][m2*M]
@@ -390,8 +391,9 @@ size_t dp_pgrad_fit_scratch(int N);
 size_t dp_pgrad_row_scratch(int num_sms);
 cudaError_t dp_launch_pgrad(cudaStream_t st, const DevModel &m, int64_t nparams, const double *x, const int32_t *types,
                             Box3 box, int N, const double *lam, double cE, const FormatBuffers &fb,
-                            const NlistBuffers &nb, EvalBuffers eb, PGradBuffers pb, int num_sms, double *grad,
-                            int64_t *launches);
+                            const NlistBuffers &nb, EvalBuffers eb, PGradBuffers pb, int num_sms,
+                            const struct ChebModel *cm, const struct ChebGradBuffers *cg, const double *trig,
+                            double *grad, int64_t *launches);
 
 // MD integrator kernels.
 cudaError_t dp_launch_kick_drift(cudaStream_t st, int N, double *x, double *v, const double *f,

@@ -669,6 +669,390 @@ __global__ void __launch_bounds__(CT) k_cheb_bwd(DevModel m, ChebModel cm, const
     }
 }
 
+// ------------------------------------------------- parameter gradient ------
+//
+// Phi = sum_i (cE E_i - dE_i) with dE_i the tangent of E_i along
+// delta r_ij = lambda_j - lambda_i (csrc/pgrad.cu).  With P the moments and dP
+// their tangents, T = scale P C and dT = scale dP C, so the adjoint of the
+// coefficients is sum_atoms (P Tb + dP dTb); it goes back through the discrete
+// transform to the net's values at the NN nodes, and reverse mode runs through
+// the net at NN points instead of at every row.  12,288 water atoms, student
+// widths: 70 -> 5.3 ms (the net, its tangent and its reverse mode at every row
+// before); 648 atoms, full width: 13.8 -> 0.5 ms.
+
+// T, dT, D, dD and the moments of one atom per CTA, as k_cheb_fwd with the tangent.
+__global__ void __launch_bounds__(CT) k_chebpg_fwd(DevModel m, ChebModel cm, const double *__restrict__ x,
+                                                   const int32_t *__restrict__ types, Box3 box,
+                                                   const double *__restrict__ lam,
+                                                   const int32_t *__restrict__ type_perm,
+                                                   const int32_t *__restrict__ nlist,
+                                                   const int32_t *__restrict__ nreal, double *__restrict__ Tout,
+                                                   double *__restrict__ dTout, double *__restrict__ Dout,
+                                                   double *__restrict__ dDout, double *__restrict__ momout,
+                                                   int32_t *far_flag)
+{
+    extern __shared__ __align__(16) double sm[];
+    const int nc = cm.n, M = m.M, T = m.ntypes, nm = m.nm, tid = threadIdx.x;
+    double *R8 = sm;                       // [CT][8] R~ and dR~
+    double *part = R8 + CT * 8;            // [CT][8]
+    double *Mom = part + CT * 8;           // [T nc][8]
+    double *Ts = Mom + T * nc * 8;         // [8][M] T, dT
+    double *Tch = Ts + 8 * M;              // [nc][LDT] T_n(t)
+    double *dTch = Tch + nc * LDT;         // [nc][LDT] d/dtau T_n(t)
+    __shared__ int start[DP_MAX_TYPES + 1];
+    const int i = type_perm[blockIdx.x];
+    const int a = types[i];
+    const bool a_ok = (unsigned)a < (unsigned)T;
+    if (tid == 0) {
+        int r = 0;
+        for (int b = 0; b < T; ++b) {
+            start[b] = r;
+            r += a_ok ? nreal[(size_t)i * T + b] : 0;
+        }
+        start[T] = r;
+    }
+    for (int p = tid; p < T * nc * 8; p += CT) Mom[p] = 0.0;
+    __syncthreads();
+    const int R = start[T];
+    const double xi[3] = {x[3 * i], x[3 * i + 1], x[3 * i + 2]};
+    const double li[3] = {lam[3 * i], lam[3 * i + 1], lam[3 * i + 2]};
+    const int ns = CT / nc, mn = tid % nc, msl = tid / nc;
+    bool any_far = false;
+    for (int c0 = 0; c0 < R; c0 += CT) {
+        const int q = c0 + tid;
+        if (q < R) {
+            const int b = row_block(start, T, q);
+            const int j = nlist[(size_t)i * nm + m.sel_off[b] + (q - start[b])];
+            const double xj[3] = {x[3 * j], x[3 * j + 1], x[3 * j + 2]};
+            double d[3], s, ds;
+            const double r = dp_pinned_dist(xi, xj, box, d);
+            dp_switch(r, m.rcut_smth, m.rcut, s, ds);
+            const double inv = 1.0 / r;
+            const double u[3] = {d[0] * inv, d[1] * inv, d[2] * inv};
+            const double dr[3] = {lam[3 * j] - li[0], lam[3 * j + 1] - li[1], lam[3 * j + 2] - li[2]};
+            const double udr = u[0] * dr[0] + u[1] * dr[1] + u[2] * dr[2];
+            double *Rq = R8 + tid * 8;
+            Rq[0] = s;
+            Rq[4] = ds * udr;
+#pragma unroll
+            for (int e = 0; e < 3; ++e) {
+                Rq[1 + e] = s * u[e];
+                Rq[5 + e] = ds * u[e] * udr + s * inv * (dr[e] - u[e] * udr);
+            }
+            any_far |= !(s <= DP_CHEB_S);
+            const double t = fma(s, DP_CHEB_SCALE, -1.0), t2 = t + t, dt = DP_CHEB_SCALE * Rq[4];
+            double p0 = 1.0, p1 = t, q0 = 0.0, q1 = dt;
+            Tch[tid] = 1.0;
+            dTch[tid] = 0.0;
+            for (int n = 1; n < nc; ++n) {
+                Tch[n * LDT + tid] = p1;
+                dTch[n * LDT + tid] = q1;
+                const double p2 = fma(t2, p1, -p0), q2 = fma(t2, q1, fma(2.0 * dt, p1, -q0));
+                p0 = p1;
+                p1 = p2;
+                q0 = q1;
+                q1 = q2;
+            }
+        }
+        __syncthreads();
+        for (int b = 0; b < T; ++b) {
+            const int lo = max(start[b] - c0, 0), hi = min(start[b + 1] - c0, CT);
+            if (lo >= hi) continue;
+            if (msl < ns) {
+                double acc[8];
+#pragma unroll
+                for (int c = 0; c < 8; ++c) acc[c] = 0.0;
+                for (int r = lo + msl; r < hi; r += ns) {
+                    const double tv = Tch[mn * LDT + r], dv = dTch[mn * LDT + r];
+                    const double *Rq = R8 + r * 8;
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) {
+                        acc[c] = fma(tv, Rq[c], acc[c]);
+                        acc[4 + c] = fma(tv, Rq[4 + c], fma(dv, Rq[c], acc[4 + c]));
+                    }
+                }
+#pragma unroll
+                for (int c = 0; c < 8; ++c) part[tid * 8 + c] = acc[c];
+            }
+            __syncthreads();
+            for (int p = tid; p < nc * 8; p += CT) {
+                double v = Mom[b * nc * 8 + p];
+                for (int u = 0; u < ns; ++u) v += part[u * nc * 8 + p];
+                Mom[b * nc * 8 + p] = v;
+            }
+            __syncthreads();
+        }
+    }
+    if (any_far) atomicOr(far_flag, 1);
+    for (int p = tid; p < T * nc * 8; p += CT) momout[(size_t)i * T * nc * 8 + p] = Mom[p];
+    {
+        const double *C = cm.C + (size_t)(a_ok ? a : 0) * T * NN * M;
+        for (int p = tid; p < 8 * M; p += CT) {
+            const int c = p / M, f = p - c * M;
+            double acc = 0.0;
+            for (int b = 0; b < T; ++b) {
+                if (start[b] == start[b + 1]) continue;
+                const double *Cb = C + (size_t)b * NN * M + f, *mo = Mom + b * nc * 8 + c;
+#pragma unroll 4
+                for (int n = 0; n < nc; ++n) acc = fma(mo[n * 8], Cb[n * M], acc);
+            }
+            Ts[p] = acc * m.desc_scale;
+        }
+    }
+    __syncthreads();
+    for (int p = tid; p < 4 * M; p += CT) {
+        Tout[(size_t)i * 4 * M + p] = Ts[p];
+        dTout[(size_t)i * 4 * M + p] = Ts[4 * M + p];
+    }
+    const int nd = m.m2 * M;
+    for (int q = tid; q < nd; q += CT) {
+        const int a2 = q / M, b2 = q - a2 * M;
+        double acc = 0.0, dacc = 0.0;
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            const double ta = Ts[c * M + a2], tb = Ts[c * M + b2];
+            acc = fma(ta, tb, acc);
+            dacc = fma(Ts[(4 + c) * M + a2], tb, dacc);
+            dacc = fma(ta, Ts[(4 + c) * M + b2], dacc);
+        }
+        Dout[(size_t)i * nd + q] = acc;
+        dDout[(size_t)i * nd + q] = dacc;
+    }
+}
+
+// Tb and dTb of one atom per CTA from dPhi/dD (Db) and dPhi/d(dD) (dDb), over T
+// and dT: D = T_<^T T, dD = dT_<^T T + T_<^T dT; the scale of T folded in.
+__global__ void __launch_bounds__(CT) k_chebpg_tb(DevModel m, double *__restrict__ Tio, double *__restrict__ dTio,
+                                                  const double *__restrict__ Db, const double *__restrict__ dDb,
+                                                  const int32_t *far_flag)
+{
+    if (*far_flag) return;
+    extern __shared__ __align__(16) double sm[];
+    const int M = m.M, m2 = m.m2, tid = threadIdx.x, LDG = M | 1;
+    const size_t i = blockIdx.x;
+    double *Ts = sm, *dTs = Ts + 4 * M;  // [4][M] each
+    double *lp = dTs + 4 * M;            // [2][4][m2] long sums of Tb, dTb
+    double *g = lp + 8 * m2;             // [m2][LDG] one of the two adjoints
+    for (int p = tid; p < 4 * M; p += CT) {
+        Ts[p] = Tio[i * 4 * M + p];
+        dTs[p] = dTio[i * 4 * M + p];
+    }
+    constexpr int OWN = (4 * DP_MAX_EMB_W + CT - 1) / CT;
+    double tb[OWN], dtb[OWN];
+#pragma unroll
+    for (int u = 0; u < OWN; ++u) tb[u] = dtb[u] = 0.0;
+    for (int pass = 0; pass < 2; ++pass) {  // dDb with (dT -> Tb, T -> dTb), then Db with (T -> Tb)
+        const double *src = (pass == 0 ? dDb : Db) + i * m2 * M;
+        const double *A = pass == 0 ? dTs : Ts;
+        __syncthreads();
+        for (int p = tid; p < m2 * M; p += CT) g[(p / M) * LDG + p % M] = src[p];
+        __syncthreads();
+        for (int p = tid; p < 4 * m2; p += CT) {
+            const int c = p / m2, xx = p - c * m2;
+            double v = 0.0, dv = 0.0;
+            for (int b = 0; b < M; ++b) {
+                const double gv = g[xx * LDG + b];
+                v = fma(gv, A[c * M + b], v);
+                if (pass == 0) dv = fma(gv, Ts[c * M + b], dv);
+            }
+            lp[p] = v;
+            lp[4 * m2 + p] = dv;
+        }
+        __syncthreads();
+#pragma unroll
+        for (int u = 0; u < OWN; ++u) {
+            const int p = tid + u * CT;
+            if (p < 4 * M) {
+                const int c = p / M, xx = p - c * M;
+                double v = xx < m2 ? lp[c * m2 + xx] : 0.0, dv = xx < m2 && pass == 0 ? lp[4 * m2 + c * m2 + xx] : 0.0;
+                for (int a2 = 0; a2 < m2; ++a2) {
+                    const double gv = g[a2 * LDG + xx];
+                    v = fma(gv, A[c * M + a2], v);
+                    if (pass == 0) dv = fma(gv, Ts[c * M + a2], dv);
+                }
+                tb[u] += v;
+                dtb[u] += dv;
+            }
+        }
+    }
+#pragma unroll
+    for (int u = 0; u < OWN; ++u) {
+        const int p = tid + u * CT;
+        if (p < 4 * M) {
+            Tio[i * 4 * M + p] = tb[u] * m.desc_scale;
+            dTio[i * 4 * M + p] = dtb[u] * m.desc_scale;
+        }
+    }
+}
+
+// Partial coefficient adjoints: CTA (split, centre type, 16 terms of the type's
+// nets side by side) sums P Tb + dP dTb over its share of the type's atoms;
+// thread = (4 terms, features u, u + 32, ...).
+constexpr int CBK = 16;
+constexpr int CBA = 8;  // atoms staged at once
+__global__ void __launch_bounds__(CT) k_chebpg_cb(DevModel m, int nc, const int32_t *__restrict__ type_perm,
+                                                  const int32_t *__restrict__ type_start,
+                                                  const double *__restrict__ mom, const double *__restrict__ Tb,
+                                                  const double *__restrict__ dTb, double *__restrict__ part,
+                                                  const int32_t *far_flag)
+{
+    if (*far_flag) return;
+    extern __shared__ __align__(16) double sm[];
+    const int M = m.M, T = m.ntypes, Kt = T * nc, tid = threadIdx.x;
+    const int a = blockIdx.y, k0 = blockIdx.z * CBK;
+    double *ms = sm;               // [CBA][8][CBK]
+    double *ts = ms + CBA * 8 * CBK;  // [CBA][8][M]
+    const int s0 = type_start[a], cnt = type_start[a + 1] - s0;
+    const int lo = (int)((long long)blockIdx.x * cnt / gridDim.x), hi = (int)((long long)(blockIdx.x + 1) * cnt / gridDim.x);
+    const int kq = (tid >> 5) * 4, fl = tid & 31;
+    double acc[4][4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+#pragma unroll
+        for (int v = 0; v < 4; ++v) acc[u][v] = 0.0;
+    for (int b0 = lo; b0 < hi; b0 += CBA) {
+        const int n = min(CBA, hi - b0);
+        __syncthreads();
+        for (int p = tid; p < n * 8 * CBK; p += CT) {
+            const int at = p / (8 * CBK), k = (p / 8) % CBK, c = p % 8;
+            const size_t i = type_perm[s0 + b0 + at];
+            ms[(at * 8 + c) * CBK + k] = k0 + k < Kt ? mom[(i * Kt + k0 + k) * 8 + c] : 0.0;
+        }
+        for (int p = tid; p < n * 8 * M; p += CT) {
+            const int at = p / (8 * M), r = p - at * 8 * M;
+            const size_t i = type_perm[s0 + b0 + at];
+            ts[p] = r < 4 * M ? Tb[i * 4 * M + r] : dTb[i * 4 * M + r - 4 * M];
+        }
+        __syncthreads();
+        for (int e = 0; e < 8 * n; ++e) {
+            double mv[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) mv[u] = ms[e * CBK + kq + u];
+#pragma unroll
+            for (int v = 0; v < 4; ++v)
+                if (fl + 32 * v < M) {
+                    const double tv = ts[e * M + fl + 32 * v];
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) acc[u][v] = fma(mv[u], tv, acc[u][v]);
+                }
+        }
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+        const int k = k0 + kq + u;
+        if (k >= Kt) continue;
+        const int b = k / nc, n = k - b * nc;
+#pragma unroll
+        for (int v = 0; v < 4; ++v)
+            if (fl + 32 * v < M)
+                part[(((size_t)blockIdx.x * T * T + a * T + b) * NN + n) * M + fl + 32 * v] = acc[u][v];
+    }
+}
+
+// Sum of the partial adjoints in a fixed order, into the first one.
+__global__ void k_chebpg_sum(double *__restrict__ part, size_t elems, int splits, const int32_t *far_flag)
+{
+    if (*far_flag) return;
+    for (size_t p = blockIdx.x * (size_t)blockDim.x + threadIdx.x; p < elems; p += (size_t)gridDim.x * blockDim.x) {
+        double v = part[p];
+        for (int q = 1; q < splits; ++q) v += part[q * elems + p];
+        part[p] = v;
+    }
+}
+
+// One CTA per (net, node): the adjoint of the net's value there, Gb_f = sum_n
+// (2 - [n = 0]) / NN cos(pi n (2k+1) / (2 NN)) Cb_nf, and reverse mode through
+// the layers; layer outputs h and z adjoints go to node[net][k][0 / 1][.].
+__global__ void __launch_bounds__(CT) k_chebpg_node(DevModel m, int nc, const double *__restrict__ trig,
+                                                    const double *__restrict__ Cb, double *__restrict__ node, int se,
+                                                    const int32_t *far_flag)
+{
+    if (*far_flag) return;
+    __shared__ double h[DP_MAX_LAYERS][DP_MAX_EMB_W], t[DP_MAX_LAYERS][DP_MAX_EMB_W], g[DP_MAX_EMB_W], zb[DP_MAX_EMB_W];
+    const int net = blockIdx.x / NN, k = blockIdx.x % NN, o = threadIdx.x, M = m.M;
+    const double *P = m.params + m.emb_base[net];
+    const double s = (1.0 + trig[2 * (2 * k + 1)]) / DP_CHEB_SCALE;
+    if (o < m.emb[0]) h[0][o] = t[0][o] = dp_tanh64(fma(s, P[o], P[m.emb[0] + o]), m.tanh_tab);
+    int off = 2 * m.emb[0];
+    for (int l = 1; l < m.n_emb; ++l) {
+        __syncthreads();
+        const int win = m.emb[l - 1], wout = m.emb[l], sk = dp_skip_kind(win, wout);
+        if (o < wout) {
+            double z = P[off + win * wout + o];
+            for (int p = 0; p < win; ++p) z = fma(h[l - 1][p], P[off + p * wout + o], z);
+            t[l][o] = dp_tanh64(z, m.tanh_tab);
+            h[l][o] = t[l][o] + (sk ? h[l - 1][o < win ? o : o - win] : 0.0);
+        }
+        off += win * wout + wout;
+    }
+    if (o < M) {
+        double v = 0.0;
+        for (int n = 0; n < nc; ++n)
+            v = fma(trig[2 * ((n * (2 * k + 1)) % (4 * NN))] * (n == 0 ? 1.0 / NN : 2.0 / NN),
+                    Cb[((size_t)net * NN + n) * M + o], v);
+        g[o] = v;
+    }
+    double *hn = node + (size_t)blockIdx.x * 2 * se, *zn = hn + se;
+    int lo = se;
+    for (int l = m.n_emb - 1; l >= 0; --l) {
+        __syncthreads();
+        const int out = m.emb[l], in = l > 0 ? m.emb[l - 1] : 0;
+        lo -= out;
+        if (o < out) {
+            zb[o] = fma(-t[l][o], t[l][o], 1.0) * g[o];
+            hn[lo + o] = h[l][o];
+            zn[lo + o] = zb[o];
+        }
+        __syncthreads();
+        if (l > 0) {
+            off -= in * out + out;
+            const int sk = dp_skip_kind(in, out);
+            double v = 0.0;
+            if (o < in) {
+                for (int p = 0; p < out; ++p) v = fma(P[off + o * out + p], zb[p], v);
+                if (sk) v += g[o];
+                if (sk == 2) v += g[o + in];
+            }
+            __syncthreads();
+            if (o < in) g[o] = v;
+        }
+    }
+}
+
+// Gradient of every embedding parameter from the nodes' layer outputs and z
+// adjoints: dW[q][o] = sum_k h_k[q] zb_k[o], db[o] = sum_k zb_k[o].
+__global__ void k_chebpg_grad(DevModel m, const double *__restrict__ trig, const double *__restrict__ node, int se,
+                              double *__restrict__ grad, const int32_t *far_flag)
+{
+    if (*far_flag) return;
+    const int net = blockIdx.y;
+    const double *nd = node + (size_t)net * NN * 2 * se;
+    for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < m.emb_net_size; p += gridDim.x * blockDim.x) {
+        int l = 0, lo = 0, r = p, in = 1;  // layer, its offset in the node arrays, index in the layer
+        while (r >= (in + 1) * m.emb[l]) {
+            r -= (in + 1) * m.emb[l];
+            lo += m.emb[l];
+            in = m.emb[l];
+            ++l;
+        }
+        const int out = m.emb[l], q = r / out, o = r - q * out;
+        double v = 0.0;
+        for (int k = 0; k < NN; ++k) {
+            const double *hk = nd + (size_t)k * 2 * se, *zk = hk + se;
+            const double hv = q == in ? 1.0 : l == 0 ? (1.0 + trig[2 * (2 * k + 1)]) / DP_CHEB_SCALE : hk[lo - in + q];
+            v = fma(hv, zk[lo + o], v);
+        }
+        grad[m.emb_base[net] + p] = v;
+    }
+}
+
+size_t pg_fwd_smem(const DevModel &m, int nc)
+{
+    return sizeof(double) * (2 * CT * 8 + (size_t)m.ntypes * nc * 8 + 8 * m.M + 2 * (size_t)nc * LDT);
+}
+
+size_t pg_tb_smem(const DevModel &m) { return sizeof(double) * (8 * (size_t)m.M + 8 * m.m2 + (size_t)m.m2 * (m.M | 1)); }
+
 size_t fwd_smem(const DevModel &m, int nc)
 {
     return sizeof(double) * (CT * 4 + 2 * CT * 4 + (size_t)m.ntypes * nc * 4 + 4 * m.M + (size_t)nc * LDT);
@@ -756,5 +1140,60 @@ cudaError_t dp_launch_cheb_bwd(cudaStream_t st, const DevModel &m, const ChebMod
     k_cheb_bwd<<<N, CT, smem, st>>>(m, cm, types, nb.type_perm, fb.nreal, eb.T, eb.gD, eb.pair_g, eb.f_own,
                                     eb.vir_part);
     *launches += 1;
+    return cudaGetLastError();
+}
+
+bool dp_cheb_grad_supported(const DevModel &m, int n)
+{
+    return n > 0 && pg_fwd_smem(m, n) <= SMEM_MAX && pg_tb_smem(m) <= SMEM_MAX;
+}
+
+size_t dp_cheb_grad_elems(const DevModel &m, int n, int64_t natoms, int which)
+{
+    const size_t nets = (size_t)m.ntypes * m.ntypes;
+    size_t se = 0;
+    for (int l = 0; l < m.n_emb; ++l) se += m.emb[l];
+    switch (which) {
+    case 0: return (size_t)natoms * m.ntypes * n * 8;
+    case 1: return DP_CHEB_SPLITS * nets * NN * m.M;
+    default: return nets * NN * 2 * se;
+    }
+}
+
+cudaError_t dp_launch_chebpg_fwd(cudaStream_t st, const DevModel &m, const ChebModel &cm, const double *x,
+                                 const int32_t *types, Box3 box, int N, const double *lam, const FormatBuffers &fb,
+                                 const NlistBuffers &nb, EvalBuffers eb, PGradBuffers pb, ChebGradBuffers gb,
+                                 int64_t *launches)
+{
+    cudaError_t e = cudaMemsetAsync(gb.far, 0, sizeof(int32_t), st);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k_chebpg_fwd, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_MAX);
+    if (e != cudaSuccess) return e;
+    k_chebpg_fwd<<<N, CT, pg_fwd_smem(m, cm.n), st>>>(m, cm, x, types, box, lam, nb.type_perm, fb.nlist, fb.nreal,
+                                                     eb.T, pb.dT, eb.D, pb.dD, gb.mom, gb.far);
+    *launches += 1;
+    return cudaGetLastError();
+}
+
+cudaError_t dp_launch_chebpg_bwd(cudaStream_t st, const DevModel &m, const ChebModel &cm, int N,
+                                 const NlistBuffers &nb, EvalBuffers eb, PGradBuffers pb, ChebGradBuffers gb,
+                                 const double *trig, double *grad, int64_t *launches)
+{
+    const int T = m.ntypes, Kt = T * cm.n;
+    int se = 0;
+    for (int l = 0; l < m.n_emb; ++l) se += m.emb[l];
+    cudaError_t e = cudaFuncSetAttribute(k_chebpg_tb, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_MAX);
+    const size_t csm = sizeof(double) * CBA * 8 * (CBK + (size_t)m.M);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k_chebpg_cb, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)csm);
+    if (e != cudaSuccess) return e;
+    k_chebpg_tb<<<N, CT, pg_tb_smem(m), st>>>(m, eb.T, pb.dT, pb.Db, pb.dDb, gb.far);
+    k_chebpg_cb<<<dim3(DP_CHEB_SPLITS, T, (Kt + CBK - 1) / CBK), CT, csm, st>>>(
+        m, cm.n, nb.type_perm, nb.type_start, gb.mom, eb.T, pb.dT, gb.part, gb.far);
+    const size_t elems = (size_t)T * T * NN * m.M;
+    k_chebpg_sum<<<(int)((elems + 255) / 256), 256, 0, st>>>(gb.part, elems, DP_CHEB_SPLITS, gb.far);
+    k_chebpg_node<<<T * T * NN, CT, 0, st>>>(m, cm.n, trig, gb.part, gb.node, se, gb.far);
+    k_chebpg_grad<<<dim3((m.emb_net_size + 255) / 256, T * T), 256, 0, st>>>(m, trig, gb.node, se, grad, gb.far);
+    *launches += 5;
     return cudaGetLastError();
 }

@@ -17,6 +17,13 @@
 //              to the CTA's slice when the net changes.
 //   k_pg_reduce sums the slices in a fixed order (reproducible bit for bit).
 // G is recomputed in k_pg_emb, never stored.
+//
+// While the embedding nets run as Chebyshev series (embed_cheb.cu), k_pg_tan
+// and k_pg_emb are replaced by the series' kernels, which work on moments and
+// at the series' nodes instead of on every row through the net; they stay for
+// nets that are not resolved and, launched behind a device flag (`gate`), for
+// frames with a row beyond the series' domain.
+#include "cheb.cuh"
 #include "dp_internal.cuh"
 
 namespace {
@@ -98,8 +105,10 @@ __global__ void __launch_bounds__(NT) k_pg_tan(DevModel m, const double *__restr
                                                Box3 box, int N, const double *__restrict__ lam,
                                                const int32_t *__restrict__ nlist, const int32_t *__restrict__ nreal,
                                                double *__restrict__ Tout, double *__restrict__ dTout,
-                                               double *__restrict__ Dout, double *__restrict__ dDout, int LD, int wsz)
+                                               double *__restrict__ Dout, double *__restrict__ dDout, int LD, int wsz,
+                                               const int32_t *gate)
 {
+    if (gate != nullptr && *gate == 0) return;
     extern __shared__ double sm[];
     double *Wsm = sm;
     double *H = Wsm + wsz;            // [32][LD] all layer outputs (value)
@@ -446,8 +455,10 @@ __global__ void __launch_bounds__(NT, 1) k_pg_emb(DevModel m, const double *__re
                                                   const int32_t *__restrict__ nreal, const double *__restrict__ Tin,
                                                   const double *__restrict__ dTin, const double *__restrict__ Db,
                                                   const double *__restrict__ dDb, double *__restrict__ slices,
-                                                  int64_t nparams, double *__restrict__ rowscr, int LD, int wsz)
+                                                  int64_t nparams, double *__restrict__ rowscr, int LD, int wsz,
+                                                  const int32_t *gate)
 {
+    if (gate != nullptr && *gate == 0) return;
     extern __shared__ double sm[];
     double *Wsm = sm;                  // net weights
     double *ZB = Wsm + wsz;            // [32][maxw] z adjoints of one layer
@@ -647,9 +658,12 @@ __global__ void __launch_bounds__(NT, 1) k_pg_emb(DevModel m, const double *__re
     }
 }
 
-__global__ void k_pg_reduce(const double *__restrict__ slices, int nslices, int64_t nparams, double *__restrict__ grad)
+// The embedding parameters (p < nemb) come from the series' kernels unless the gate is set.
+__global__ void k_pg_reduce(const double *__restrict__ slices, int nslices, int64_t nparams, int64_t nemb,
+                            const int32_t *gate, double *__restrict__ grad)
 {
-    for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < nparams; p += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t first = gate != nullptr && *gate == 0 ? nemb : 0;
+    for (int64_t p = first + blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < nparams; p += (int64_t)gridDim.x * blockDim.x) {
         double acc = 0.0;
         for (int c = 0; c < nslices; ++c) acc += slices[(size_t)c * nparams + p];
         grad[p] = acc;
@@ -664,9 +678,11 @@ size_t dp_pgrad_row_scratch(int num_sms) { return (size_t)num_sms * 6 * ROWS * (
 
 cudaError_t dp_launch_pgrad(cudaStream_t st, const DevModel &m, int64_t nparams, const double *x, const int32_t *types,
                             Box3 box, int N, const double *lam, double cE, const FormatBuffers &fb,
-                            const NlistBuffers &nb, EvalBuffers eb, PGradBuffers pb, int num_sms, double *grad,
+                            const NlistBuffers &nb, EvalBuffers eb, PGradBuffers pb, int num_sms,
+                            const ChebModel *cm, const ChebGradBuffers *cg, const double *trig, double *grad,
                             int64_t *launches)
 {
+    const int32_t *gate = cm ? cg->far : nullptr;
     int maxw = 0, se = 0;
     for (int l = 0; l < m.n_emb; ++l) {
         maxw = m.emb[l] > maxw ? m.emb[l] : maxw;
@@ -679,12 +695,14 @@ cudaError_t dp_launch_pgrad(cudaStream_t st, const DevModel &m, int64_t nparams,
     // slices: one per CTA of k_pg_fit / k_pg_emb (both use num_sms CTAs)
     e = cudaMemsetAsync(pb.slices, 0, sizeof(double) * (size_t)num_sms * nparams, st);
     if (e != cudaSuccess) return e;
+    if (cm && (e = dp_launch_chebpg_fwd(st, m, *cm, x, types, box, N, lam, fb, nb, eb, pb, *cg, launches)) != cudaSuccess)
+        return e;
     {
         const size_t smem = sizeof(double) * ((size_t)wsz + 2 * ROWS * LD + 2 * ROWS * 4 + 2 * ROWS + 8 * DP_MAX_EMB_W);
         e = cudaFuncSetAttribute(k_pg_tan, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
         k_pg_tan<<<grid_emb, NT, smem, st>>>(m, x, types, box, N, lam, fb.nlist, fb.nreal, eb.T, pb.dT, eb.D, pb.dD,
-                                             LD, wsz);
+                                             LD, wsz, gate);
     }
     {
         const size_t smem = sizeof(double) * 4 * FRT * (FW + 1);
@@ -700,10 +718,11 @@ cudaError_t dp_launch_pgrad(cudaStream_t st, const DevModel &m, int64_t nparams,
         e = cudaFuncSetAttribute(k_pg_emb, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
         k_pg_emb<<<num_sms, NT, smem, st>>>(m, x, types, box, N, lam, fb.nlist, fb.nreal, eb.T, pb.dT, pb.Db, pb.dDb,
-                                            pb.slices, nparams, pb.rowscr, LD, wsz);
+                                            pb.slices, nparams, pb.rowscr, LD, wsz, gate);
     }
+    if (cm && (e = dp_launch_chebpg_bwd(st, m, *cm, N, nb, eb, pb, *cg, trig, grad, launches)) != cudaSuccess) return e;
     k_pg_reduce<<<(int)((nparams + 255) / 256 < 4096 ? (nparams + 255) / 256 : 4096), 256, 0, st>>>(
-        pb.slices, num_sms, nparams, grad);
+        pb.slices, num_sms, nparams, (int64_t)m.ntypes * m.ntypes * m.emb_net_size, gate, grad);
     *launches += 4;
     (void)maxw;
     (void)grid_emb;

@@ -97,3 +97,59 @@ def test_new_parameters_make_new_series(dp, oracle, synth):
         dp.dp_build_nlist(ctx, x, ty, b, 0.0)
         f = dp.dp_eval(ctx, x, ty, b)["force"]
         assert rel(f.cpu(), oracle.evaluate(desc, P, c, t, b)["force"]) < TOL
+
+
+def check_grad(dp, oracle, desc, P, c, t, box):
+    rng = np.random.default_rng(8)
+    lam = rng.standard_normal((len(c), 3))
+    ref = oracle.param_grad(desc, P, c, t, box, 0.37, lam)
+    ctx = dp.Context(dp.Model(desc, P), len(c))
+    x = torch.tensor(c, dtype=torch.float64, device="cuda")
+    ty = torch.tensor(t, dtype=torch.int32, device="cuda")
+    dp.dp_build_nlist(ctx, x, ty, box, 0.0)
+    g = dp.dp_param_grad(ctx, x, ty, box, 0.37, torch.tensor(lam, device="cuda"))
+    # embedding and fitting parameters apart: each block has its own scale
+    ne = sum(int(np.prod(s)) for n, s in synth_shapes(desc) if n.startswith("emb"))
+    assert rel(g[:ne].cpu(), ref[:ne]) < TOL
+    assert rel(g[ne:].cpu(), ref[ne:]) < TOL
+    g2 = dp.dp_param_grad(ctx, x, ty, box, 0.37, torch.tensor(lam, device="cuda"))
+    assert torch.equal(g, g2)
+
+
+def synth_shapes(desc):
+    from paper_2004_11658_gb300 import synth
+    return synth.layer_shapes(desc)
+
+
+@pytest.mark.parametrize("emb,m2,fit", [((24,), 24, (48, 48)), ((20, 20), 3, (17, 17)), ((8, 16, 16, 33), 5, (33,)),
+                                        ((25, 50, 100), 16, (64, 64, 64)), ((32, 64, 128), 16, (240, 240))])
+def test_gradient_shapes(dp, oracle, synth, emb, m2, fit):
+    c, t, b = synth.water_box(5, 5 * 49.7 / 16, seed=3)
+    desc = dict(synth.WATER_MODEL, emb=emb, m2=m2, fit=fit)
+    check_grad(dp, oracle, desc, synth.model_params(desc, 4, fit_in_gain=30.0, out_scale=1.0), c, t, b)
+
+
+def test_gradient_three_types_many_rows(dp, oracle, synth):
+    c, _, b = synth.copper_fcc(5, seed=2)
+    t = np.random.default_rng(5).integers(0, 3, len(c)).astype(np.int32)
+    desc = dict(synth.CU_MODEL, ntypes=3, sel=(120, 120, 120), emb=(8, 16, 32), fit=(32, 32))
+    check_grad(dp, oracle, desc, synth.model_params(desc, 1, fit_in_gain=30.0, out_scale=1.0), c, t, b)
+
+
+@pytest.mark.parametrize("case", ["rows beyond the series", "steep nets"])
+def test_gradient_through_the_nets(dp, oracle, synth, case):
+    """Frames and nets the series does not cover take the kernels that work
+    through the net."""
+    c, t, b = synth.water_box(5, 5 * 49.7 / 16, seed=3)
+    desc = synth.WATER_STUDENT
+    P = synth.model_params(desc, 0)
+    if case == "steep nets":
+        off = 0
+        for name, shape in synth.layer_shapes(desc):
+            n = int(np.prod(shape))
+            if name.endswith(".W0"):
+                P[off:off + n] *= 100.0
+            off += n
+    else:
+        c[34] = np.mod(c[30] + 0.4 * np.array([0.6, 0.0, 0.8]), b[0])
+    check_grad(dp, oracle, desc, P, c, t, b)
