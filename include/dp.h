@@ -343,11 +343,12 @@ dp_status dp_md_kick(dp_ctx *ctx, double *vel, const double *force, const int32_
  * at the current coordinates.  The force term is a mixed second derivative,
  * evaluated as forward tangents of the environment matrix, embedding,
  * descriptor and fitting nets along the neighbour displacements
- * lambda_j - lambda_i followed by reverse mode; G is recomputed, never
- * stored.  lambda: device [N][3]; grad: device [nparams] (flat layout of
+ * lambda_j - lambda_i followed by reverse mode; G is never stored (the
+ * embedding nets go through their series, DP_PREC_FP64, or are recomputed).
+ * lambda: device [N][3]; grad: device [nparams] (flat layout of
  * dp_model_nparams), overwritten.  FP64 contexts only (DP_ERR_UNSUPPORTED
  * otherwise).  Reproducible bit for bit.  Scratch of about
- * num_SMs * nparams doubles plus ~30 KB per atom is allocated on the first
+ * num_SMs * nparams doubles plus ~130 KB per atom is allocated on the first
  * call. */
 dp_status dp_param_grad(dp_ctx *ctx, const double *coords, const int32_t *types, const double box[9],
                         int64_t N, double cE, const double *lambda, double *grad);

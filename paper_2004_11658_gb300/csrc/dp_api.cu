@@ -143,6 +143,7 @@ struct dp_ctx {
     bool use_oz;
     OzModel oz;
     OzBuffers ob;
+    OzGradBuffers og;  // parameter gradient (allocated on first use)
     uint16_t *d_oz_w;
     int32_t *d_oz_e;
     int64_t oz_w_elems, oz_e_elems, oz_version;
@@ -954,7 +955,7 @@ void dp_ctx_free(dp_ctx *c)
                     c->pb.dT, c->pb.dD, c->pb.Db, c->pb.dDb, c->pb.fit_scr, c->pb.rowscr, c->pb.slices,
                     c->d_oz_w, c->d_oz_e, c->ob.a, c->ob.aexp, c->ob.t, c->ob.h, c->ob.g, c->d_dtile, c->d_ex_w,
                     c->eb.Gst, c->eb.Gmx, c->cb.C, c->cb.Ct, c->cb.y, c->cb.mx, c->cb.trig, c->cg.mom,
-                    c->cg.part, c->cg.node, c->cg.far};
+                    c->cg.part, c->cg.node, c->cg.far, c->og.a, c->og.b, c->og.exp, c->og.mx, c->og.x};
     for (void *p : bufs) dev_free(p);
     delete c;
 }
@@ -1398,6 +1399,13 @@ dp_status dp_param_grad(dp_ctx *c, const double *coords, const int32_t *types, c
             ALLOCP(c->cg.node, dp_cheb_grad_elems(c->m, DP_CHEB_NN, c->natoms_max, 2));
             ALLOCP(c->cg.far, 1);
         }
+        if (c->use_oz) {
+            ALLOCP(c->og.a, dp_oz_grad_elems(c->m, c->oz, c->natoms_max, 0));
+            ALLOCP(c->og.b, dp_oz_grad_elems(c->m, c->oz, c->natoms_max, 1));
+            ALLOCP(c->og.exp, dp_oz_grad_elems(c->m, c->oz, c->natoms_max, 2));
+            ALLOCP(c->og.mx, dp_oz_grad_elems(c->m, c->oz, c->natoms_max, 2));
+            ALLOCP(c->og.x, dp_oz_grad_elems(c->m, c->oz, c->natoms_max, 3));
+        }
         ALLOCP(c->pb.slices, (size_t)c->num_sms * np);  // last: marks the set as complete
 #undef ALLOCP
         if (s) return s;
@@ -1405,6 +1413,7 @@ dp_status dp_param_grad(dp_ctx *c, const double *coords, const int32_t *types, c
     if ((s = ensure_perm(c, types, N))) return s;
     if ((s = enqueue_format(c, coords, types, b, N))) return s;
     ChebModel cm;
+    if (c->use_oz && (s = ensure_oz(c))) return s;
     if (c->use_cheb && (s = ensure_cheb(c))) return s;
     const bool cheb = c->cg.far && c->cheb.n > 0;
     if (cheb) {
@@ -1412,7 +1421,8 @@ dp_status dp_param_grad(dp_ctx *c, const double *coords, const int32_t *types, c
         cm.n = dp_cheb_grad_terms(cm.n);
     }
     cudaError_t e = dp_launch_pgrad(c->stream, c->m, np, coords, types, b, (int)N, lambda, cE, c->fb, c->nb, c->eb,
-                                    c->pb, c->num_sms, cheb ? &cm : nullptr, &c->cg, c->cb.trig, grad, &c->launches);
+                                    c->pb, c->num_sms, cheb ? &cm : nullptr, &c->cg, c->cb.trig,
+                                    c->use_oz ? &c->oz : nullptr, &c->ob, &c->og, c->d_status, grad, &c->launches);
     if (e != cudaSuccess) return cuda_fail(e, "dp_param_grad");
     return finish(c);
 }

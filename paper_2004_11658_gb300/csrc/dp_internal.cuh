@@ -378,7 +378,8 @@ cudaError_t dp_launch_embed_bwd_mx(cudaStream_t st, const DevModel &m, const Mix
 bool dp_mixed_supported(const DevModel &m);
 
 // Parameter gradient of cE E + sum lambda . F (pgrad.cu); cm, cg, trig: the
-// embedding nets' series and their buffers, null to work through the nets.
+// embedding nets' series and their buffers, null to work through the nets;
+// oz, ob, og: null for the fitting net on the FP64 units.
 struct PGradBuffers {
     double *dT;       // [N][4][M] tangent of T
     double *dD;       // [N][m2*M]
@@ -387,12 +388,27 @@ struct PGradBuffers {
     double *rowscr;   // dp_pgrad_row_scratch(num_sms) doubles
     double *slices;   // [num_sms][nparams] per-CTA gradient partials
 };
+// Fitting-net part on the tensor cores (fit_oz.cu): forward with tangent, reverse
+// mode and the weight gradients; writes pb.Db, pb.dDb and the fitting
+// parameters' part of grad.
+struct OzGradBuffers {
+    uint16_t *a, *b;         // digits of the columns of X and Zb over the atoms
+    int32_t *exp;            // their exponents
+    unsigned long long *mx;  // their largest magnitudes
+    double *x;               // adjoints, 6 x [natoms][fmax]
+};
+size_t dp_oz_grad_elems(const DevModel &m, const OzModel &oz, int64_t natoms, int which);  // a, b, exp (= mx), x
+cudaError_t dp_launch_pgrad_fit_oz(cudaStream_t st, const DevModel &m, const OzModel &oz, const OzBuffers &ob,
+                                   const OzGradBuffers &og, const int32_t *types, int N, double cE,
+                                   const NlistBuffers &nb, EvalBuffers eb, PGradBuffers pb, int num_sms,
+                                   int32_t *status, double *grad, int64_t *launches);
 size_t dp_pgrad_fit_scratch(int N);
 size_t dp_pgrad_row_scratch(int num_sms);
 cudaError_t dp_launch_pgrad(cudaStream_t st, const DevModel &m, int64_t nparams, const double *x, const int32_t *types,
                             Box3 box, int N, const double *lam, double cE, const FormatBuffers &fb,
                             const NlistBuffers &nb, EvalBuffers eb, PGradBuffers pb, int num_sms,
                             const struct ChebModel *cm, const struct ChebGradBuffers *cg, const double *trig,
+                            const OzModel *oz, const OzBuffers *ob, const OzGradBuffers *og, int32_t *status,
                             double *grad, int64_t *launches);
 
 // MD integrator kernels.

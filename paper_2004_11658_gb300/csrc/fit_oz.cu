@@ -26,7 +26,7 @@
 //
 // Kernels.  k_oz_split: digits of the activations of a 128-atom tile of one
 // type, S BF16 matrices in the canonical K-major layout of the MMA A operand
-// (16-column chunks).  The weights' digits are made once on the host.
+// (16-column chunks); k_oz_wsplit: the weights', once per set of parameters.
 // k_oz_gemm: persistent over (tile, 32-column chunk of Y); a copy warp streams
 // the digit chunks of A and W (cp.async.bulk, a 4-stage ring on mbarriers), an
 // MMA warp issues S(S+1)/2 MMAs of 128 x 32 x 16 per chunk into S group
@@ -54,6 +54,8 @@ namespace {
 
 constexpr int OZ_NST = 4;                   // pipeline stages (40 KB each at 8 digits)
 constexpr int OZ_THREADS = 320;             // 8 epilogue warps, the MMA warp, the copy warp
+// chunks whose sums stay exact at 8 digits of 7 bits: 400 columns, 400 4^6 10 < 2^24
+constexpr int OZ_SEG = 16777215 / (4096 * 10) / DP_OZ_KC;
 constexpr uint32_t OZ_TAB_BYTES = DP_TANH_NINT * DP_TANH_STRIDE * 8;
 static_assert(OZ_TAB_BYTES % 16 == 0, "bulk copy of the tanh table");
 constexpr int OZ_A_BLK = DP_OZ_TILE * DP_OZ_KC;  // elements of one A digit chunk (128 x 16)
@@ -79,6 +81,22 @@ __device__ __forceinline__ TileRef oz_tile(int tl, const int32_t *__restrict__ t
         tl -= tiles;
     }
     return t;
+}
+
+// Exponent of a row or column from the bits of its largest |x|: 2^e > |x|.  zero: its
+// digits are 0 (nothing there, or below 2^-960).  An infinity or NaN gives OZ_NAN,
+// for which k_oz_gemm writes NaN.
+constexpr int OZ_NAN = 30000;
+__device__ __forceinline__ int oz_exponent(unsigned long long mx, int bS, bool &zero)
+{
+    zero = true;
+    if (mx == 0) return 0;
+    if (mx >= 0x7ff0000000000000ull) return OZ_NAN;
+    int e;
+    frexp(__longlong_as_double((long long)mx), &e);
+    if (e < bS - 1020) return 0;
+    zero = false;
+    return e;
 }
 
 // ------------------------------------------------------------------ split --
@@ -141,12 +159,12 @@ __global__ void __launch_bounds__(256) k_oz_split(OzSplitArgs p)
             for (int o = 16; o > 0; o >>= 1) e += __shfl_xor_sync(0xffffffffu, e, o);
             if (i >= 0 && lane == 0) p.Ei[i] = *p.bout[T.a] + e;
         }
-        // largest |x| by its bits (NaN left out)
+        // largest |x| by its bits; a row with an infinity or NaN gives NaN
         unsigned long long mx = 0;
 #pragma unroll 4
         for (int k = lane; k < p.K; k += 32) {
             const unsigned long long b = (unsigned long long)__double_as_longlong(fabs(value(i, k)));
-            if (b > mx && b <= 0x7ff0000000000000ull) mx = b;
+            mx = b > mx ? b : mx;
         }
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) {
@@ -154,16 +172,11 @@ __global__ void __launch_bounds__(256) k_oz_split(OzSplitArgs p)
             mx = q > mx ? q : mx;
         }
         if (lane == 0) {
-            int e = 0;
-            const double m = __longlong_as_double((long long)mx);
-            bool zero = !(m > 0.0);
-            if (!zero) {
-                frexp(m, &e);
-                if (e < bS - 1020) zero = true;  // below 2^-960: a zero row
-            }
-            e_s[warp] = zero ? 0 : e;
+            bool zero;
+            const int e = oz_exponent(mx, bS, zero);
+            e_s[warp] = e;
             nz_s[warp] = !zero;
-            p.aexp[(size_t)tl * DP_OZ_TILE + r] = zero ? 0 : e;
+            p.aexp[(size_t)tl * DP_OZ_TILE + r] = e;
         }
     }
     __syncthreads();
@@ -205,7 +218,7 @@ struct OzGemmArgs {
     OzGemm g;
     const int32_t *type_perm, *type_start;
     int ntypes;
-    int epi;      // 0: forward (bias, tanh, skip); 1: backward (skip gradient)
+    int epi;      // 0: forward (bias, tanh, skip); 1: backward (skip gradient); 2: tangent forward
     int skip;     // skip kind of the layer
     int skip_in;  // input width of the layer
     const double *bias[DP_MAX_TYPES];
@@ -218,6 +231,18 @@ struct OzGemmArgs {
     const double *tanh_tab;
     int32_t *status;
     int units;  // (tile, column chunk) pairs, tiles past the last atom included
+    const double *tin;  // epi 2: tanh values of the value pass
+    // weight gradients Y = X^T Z, contracted over the atoms of each type
+    int wg, rows, nq;                 // 1; rows of Y and their tiles
+    int64_t out_off[DP_MAX_TYPES];    // of a type's Y in hout
+};
+
+// One unit of k_oz_gemm: a 128-row tile of the A operand and a 32-column chunk of Y.
+struct OzUnit {
+    int a, tl, nchunk, nK, nseg, seg;
+    int first, cnt;             // atoms of the tile (not wg)
+    const uint16_t *as, *bs;    // digits of the first K-chunk
+    size_t astep, bstep;        // ... to the next
 };
 
 __device__ __forceinline__ void bulk_g2s(void *dst, const void *src, uint32_t bytes, uint64_t *mbar)
@@ -240,6 +265,43 @@ __device__ __forceinline__ void mbar_expect_tx(uint64_t *mbar, uint32_t bytes)
 __device__ __forceinline__ double scale2(double y, int e)
 {
     return (e >= -1022 && e <= 1023) ? y * oz_pow2(e) : ldexp(y, e);
+}
+
+template <int S>
+__device__ __forceinline__ bool oz_unit(const OzGemmArgs &p, int u, OzUnit &U)
+{
+    const OzGemm &g = p.g;
+    if (!p.wg) {
+        U.tl = u / g.nN;
+        U.nchunk = u - U.tl * g.nN;
+        const TileRef T = oz_tile(U.tl, p.type_start, p.ntypes);
+        U.a = T.a;
+        U.first = T.first;
+        U.cnt = T.cnt;
+        U.nK = g.nK;
+        U.seg = g.seg;
+        U.astep = (size_t)S * OZ_A_BLK;
+        U.bstep = (size_t)S * OZ_B_BLK;
+        U.as = p.a + (size_t)U.tl * p.a_stride;
+        U.bs = p.w + g.w_off[T.a < 0 ? 0 : T.a] + (size_t)U.nchunk * g.nK * U.bstep;
+    } else {
+        // chunks of 16 atoms, type after type; [chunk][tile or column chunk][S][block]
+        const int per = p.nq * g.nN;
+        U.a = u / per;
+        U.tl = (u - U.a * per) / g.nN;
+        U.nchunk = u - U.a * per - U.tl * g.nN;
+        int kb = 0;
+        for (int a = 0; a < U.a; ++a) kb += (p.type_start[a + 1] - p.type_start[a] + DP_OZ_KC - 1) / DP_OZ_KC;
+        U.nK = (p.type_start[U.a + 1] - p.type_start[U.a] + DP_OZ_KC - 1) / DP_OZ_KC;
+        U.seg = OZ_SEG;
+        U.first = U.cnt = 0;
+        U.astep = (size_t)p.nq * S * OZ_A_BLK;
+        U.bstep = (size_t)g.nN * S * OZ_B_BLK;
+        U.as = p.a + kb * U.astep + (size_t)U.tl * S * OZ_A_BLK;
+        U.bs = p.w + kb * U.bstep + (size_t)U.nchunk * S * OZ_B_BLK;
+    }
+    U.nseg = (U.nK + U.seg - 1) / U.seg;
+    return U.a >= 0;
 }
 
 // Persistent, one CTA per SM over the units (tile, 32-column chunk of Y) in
@@ -265,7 +327,6 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_oz_gemm(OzGemmArgs p)
     __shared__ volatile int fail;
     const int tid = threadIdx.x, lane = tid & 31, warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
     const OzGemm &g = p.g;
-    const int nK = g.nK, nseg = (nK + g.seg - 1) / g.seg;
     constexpr uint32_t a_bytes = (uint32_t)S * OZ_A_BLK * 2, b_bytes = (uint32_t)S * OZ_B_BLK * 2;
     constexpr uint32_t stage_bytes = a_bytes + b_bytes;
     constexpr int NST = OZ_NST;
@@ -301,12 +362,9 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_oz_gemm(OzGemmArgs p)
             bulk_g2s(smraw + NST * stage_bytes, p.tanh_tab, OZ_TAB_BYTES, &tabbar);
         }
         for (int u = blockIdx.x; u < p.units && ok; u += gridDim.x) {
-            const int tl = u / g.nN, nchunk = u - tl * g.nN;
-            const TileRef T = oz_tile(tl, p.type_start, p.ntypes);
-            if (T.a < 0) break;
-            const uint16_t *asrc = p.a + (size_t)tl * p.a_stride;
-            const uint16_t *bsrc = p.w + g.w_off[T.a] + (size_t)nchunk * nK * S * OZ_B_BLK;
-            for (int kc = 0; kc < nK; ++kc, ++c) {
+            OzUnit U;
+            if (!oz_unit<S>(p, u, U)) break;
+            for (int kc = 0; kc < U.nK; ++kc, ++c) {
                 const int st = c % NST;
                 if (c >= NST) ok = tc::mbar_wait(&empty[st], (c / NST - 1) & 1) && !fail;
                 ok = __all_sync(0xffffffffu, ok);
@@ -314,8 +372,8 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_oz_gemm(OzGemmArgs p)
                 if (tc::elect_one()) {
                     unsigned char *dst = smraw + (size_t)st * stage_bytes;
                     mbar_expect_tx(&full[st], stage_bytes);
-                    bulk_g2s(dst, asrc + (size_t)kc * S * OZ_A_BLK, a_bytes, &full[st]);
-                    bulk_g2s(dst + a_bytes, bsrc + (size_t)kc * S * OZ_B_BLK, b_bytes, &full[st]);
+                    bulk_g2s(dst, U.as + kc * U.astep, a_bytes, &full[st]);
+                    bulk_g2s(dst + a_bytes, U.bs + kc * U.bstep, b_bytes, &full[st]);
                 }
                 __syncwarp();
             }
@@ -354,22 +412,23 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_oz_gemm(OzGemmArgs p)
         int c = 0, sc = 0;
         bool ok = true;
         for (int u = blockIdx.x; u < p.units && ok; u += gridDim.x) {
-            if (oz_tile(u / g.nN, p.type_start, p.ntypes).a < 0) break;
-            for (int sg = 0; sg < nseg && ok; ++sg, ++sc) {
+            OzUnit U;
+            if (!oz_unit<S>(p, u, U)) break;
+            for (int sg = 0; sg < U.nseg && ok; ++sg, ++sc) {
                 const int buf = sc & 1;
                 if (sc >= 2) ok = tc::mbar_wait(&tempty[buf], ((sc >> 1) - 1) & 1) && !fail;
                 ok = __all_sync(0xffffffffu, ok);
                 if (!ok) break;
                 tc::fence_after_sync();
                 const uint32_t dbase = tbase + buf * TBUF;
-                const int k1 = min(nK, (sg + 1) * g.seg);
-                for (int kc = sg * g.seg; kc < k1; ++kc, ++c) {
+                const int k0 = sg * U.seg, k1 = min(U.nK, k0 + U.seg);
+                for (int kc = k0; kc < k1; ++kc, ++c) {
                     const int st = c % NST;
                     ok = tc::mbar_wait(&full[st], (c / NST) & 1) && !fail;
                     ok = __all_sync(0xffffffffu, ok);
                     if (!ok) break;
                     if (tc::elect_one()) {
-                        const bool acc0 = kc > sg * g.seg;
+                        const bool acc0 = kc > k0;
                         if (st == 0) issue(std::integral_constant<int, 0>{}, dbase, acc0);
                         else if (st == 1) issue(std::integral_constant<int, 1>{}, dbase, acc0);
                         else if (st == 2) issue(std::integral_constant<int, 2>{}, dbase, acc0);
@@ -395,21 +454,30 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_oz_gemm(OzGemmArgs p)
         const int w = g.beta * (S - H);
         const int half = warp >> 2, row = 32 * (warp & 3) + lane;
         const uint32_t tl_lane = tbase + ((uint32_t)(32 * (warp & 3)) << 16) + 16 * half;
-        const bool vec = (p.ldo & 1) == 0 && (p.ldh & 1) == 0;  // rows start on 16 bytes
+        const bool vec = !p.wg && (p.ldo & 1) == 0 && (p.ldh & 1) == 0;  // rows start on 16 bytes
         int sc = 0;
         bool ok = true;
         if (p.epi == 0) ok = __all_sync(0xffffffffu, tc::mbar_wait(&tabbar, 0));
         for (int u = blockIdx.x; u < p.units && ok; u += gridDim.x) {
-            const int tl = u / g.nN, nchunk = u - tl * g.nN;
-            const TileRef T = oz_tile(tl, p.type_start, p.ntypes);
-            if (T.a < 0) break;
-            const int i = row < T.cnt ? p.type_perm[T.first + row] : -1;
-            const int n0 = nchunk * DP_OZ_NC + 16 * half;   // first of this thread's 16 columns of Y
-            const int esc = (i >= 0 ? p.aexp[(size_t)tl * DP_OZ_TILE + row] : 0) - g.beta * (S + 1);
-            const int4 *fe4 = reinterpret_cast<const int4 *>(p.wexp + g.e_off[T.a] + n0);
+            OzUnit U;
+            if (!oz_unit<S>(p, u, U)) break;
+            const int n0 = U.nchunk * DP_OZ_NC + 16 * half;   // first of this thread's 16 columns of Y
+            int i, erow;
+            const int4 *fe4;
+            if (!p.wg) {
+                i = row < U.cnt ? p.type_perm[U.first + row] : -1;
+                erow = U.tl * DP_OZ_TILE + row;
+                fe4 = reinterpret_cast<const int4 *>(p.wexp + g.e_off[U.a] + n0);
+            } else {
+                i = U.tl * DP_OZ_TILE + row < p.rows ? U.tl * DP_OZ_TILE + row : -1;
+                erow = U.a * p.nq * DP_OZ_TILE + U.tl * DP_OZ_TILE + row;
+                fe4 = reinterpret_cast<const int4 *>(p.wexp + U.a * g.nN * DP_OZ_NC + n0);
+            }
+            const int esc = (i >= 0 ? p.aexp[erow] : 0) - g.beta * (S + 1);
+            double *hout = p.hout + (p.wg ? p.out_off[U.a] : 0);
             // the skip's operands, asked for before the MMAs are waited for
-            const bool bcast = p.epi != 0 && p.gbc[T.a] != nullptr;
-            const double *hin = bcast ? p.gbc[T.a] : p.hin + (size_t)(i < 0 ? 0 : i) * p.ldh;
+            const bool bcast = p.epi == 1 && p.gbc[U.a] != nullptr;
+            const double *hin = bcast ? p.gbc[U.a] : (p.wg ? hout : p.hin) + (size_t)(i < 0 ? 0 : i) * p.ldh;
             double sk[16];
 #pragma unroll
             for (int n = 0; n < 16; ++n) sk[n] = 0.0;
@@ -427,7 +495,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_oz_gemm(OzGemmArgs p)
                         if (n0 + n < g.N) {
                             const int q = n0 + n;
                             sk[n] = p.skip == 1 ? hin[q]
-                                    : p.epi == 0 ? hin[q % p.skip_in]
+                                    : p.epi != 1 ? hin[q % p.skip_in]
                                                  : hin[q] + hin[q + p.skip_in];
                         }
                 }
@@ -435,7 +503,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_oz_gemm(OzGemmArgs p)
             long long hi[16], lo[16];
 #pragma unroll
             for (int n = 0; n < 16; ++n) hi[n] = lo[n] = 0;
-            for (int sg = 0; sg < nseg; ++sg, ++sc) {
+            for (int sg = 0; sg < U.nseg; ++sg, ++sc) {
                 const int buf = sc & 1;
                 ok = tc::mbar_wait(&tfull[buf], (sc >> 1) & 1) && !fail;
                 ok = __all_sync(0xffffffffu, ok);
@@ -469,8 +537,9 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_oz_gemm(OzGemmArgs p)
             }
             if (!ok) break;
             if (i < 0) continue;
-            double *ho = p.hout + (size_t)i * p.ldo + n0;
-            double *to = p.epi == 0 ? p.tout + (size_t)i * p.ldo + n0 : nullptr;
+            double *ho = hout + (size_t)i * p.ldo + n0;
+            double *to = p.epi != 1 ? p.tout + (size_t)i * p.ldo + n0 : nullptr;
+            const double *ti = p.epi == 2 ? p.tin + (size_t)i * p.ldo + n0 : nullptr;
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
                 const int4 f4 = fe4[q];
@@ -483,23 +552,28 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_oz_gemm(OzGemmArgs p)
                         const int n = 4 * q + n2 + v, e = esc + fe[n2 + v];
                         y[v] = e > -900 && e < 900 ? oz_i64x2_scaled_w(hi[n], lo[n], w, e)
                                                    : scale2(fma((double)hi[n], oz_pow2(w), (double)lo[n]), e);
+                        if (e > 5000) y[v] = __longlong_as_double(0x7ff8000000000000ll);
+                        const int col = n0 + n;
                         if (p.epi == 0) {
-                            const int col = n0 + n;
-                            t[v] = dp_tanh64(y[v] + (col < g.N ? p.bias[T.a][col] : 0.0), tab);
+                            t[v] = dp_tanh64(y[v] + (col < g.N ? p.bias[U.a][col] : 0.0), tab);
                             y[v] = t[v];
+                        } else if (p.epi == 2) {
+                            const double tv = col < g.N ? ti[n] : 0.0;
+                            t[v] = y[v];
+                            y[v] *= fma(-tv, tv, 1.0);
                         }
                         y[v] += sk[n];
                     }
                     const int n = 4 * q + n2;
                     if (vec && n0 + n + 2 <= g.N) {
                         *reinterpret_cast<double2 *>(ho + n) = make_double2(y[0], y[1]);
-                        if (p.epi == 0) *reinterpret_cast<double2 *>(to + n) = make_double2(t[0], t[1]);
+                        if (p.epi != 1) *reinterpret_cast<double2 *>(to + n) = make_double2(t[0], t[1]);
                     } else {
 #pragma unroll
                         for (int v = 0; v < 2; ++v)
                             if (n0 + n + v < g.N) {
                                 ho[n + v] = y[v];
-                                if (p.epi == 0) to[n + v] = t[v];
+                                if (p.epi != 1) to[n + v] = t[v];
                             }
                     }
                 }
@@ -557,15 +631,9 @@ __global__ void __launch_bounds__(256) k_oz_wsplit(DevModel m, OzModel oz, uint1
     __syncthreads();
 #pragma unroll
     for (int q = 0; q < 8; ++q) mx = mx_s[q][rl] > mx ? mx_s[q][rl] : mx;
-    const double big = __longlong_as_double((long long)mx);
     const int bS = g.beta * g.S;
-    int ex = 0;
-    bool zero = !(big > 0.0);
-    if (!zero) {
-        frexp(big, &ex);
-        if (ex < bS - 1020) zero = true;
-    }
-    if (zero) ex = 0;
+    bool zero;
+    const int ex = oz_exponent(mx, bS, zero);
     if (sl == 0) e[g.e_off[a] + row] = ex;
     uint16_t *out = w + g.w_off[a] + (size_t)u * g.nK * g.S * OZ_B_BLK;
     for (int kb = sl; kb < 2 * g.nK; kb += 8) {
@@ -588,6 +656,127 @@ __global__ void __launch_bounds__(256) k_oz_wsplit(DevModel m, OzModel oz, uint1
     }
 }
 
+// --------------------------------------------- weight gradients' operands ---
+//
+// dPhi/dW_l = X^T Zb + dX^T dZb over the atoms of a type (the parameter gradient
+// of pgrad.cu: forward with tangent and reverse mode run on the same GEMMs):
+// digits of the columns of X (rows of the A operand) and of Zb (rows of the B
+// operand), scaled per column and type by its largest magnitude over the atoms.
+// The whole fitting part on the FP64 units, with per-CTA gradient slices, took 63
+// ms for 12,288 water atoms with the student's widths, now 4.0 ms; 648 atoms at
+// full width: 23 -> 0.8 ms (24 GEMMs and 14 splits, bound as k_oz_gemm).
+
+struct OzCols {
+    const double *src;   // [N][ld], columns 0 .. K-1
+    int ld, K, one;      // column `one` is 1 for every atom (-1: none)
+    int rb, nb;          // rows per block of the operand (128 or 32), blocks
+    uint16_t *out;       // [chunk of 16 atoms][nb][S][rb x 16]
+    int32_t *exp;        // [T][nb rb]
+    unsigned long long *mx;  // [T][nb rb] bits of the largest magnitude (zeroed)
+};
+struct OzColsPair {
+    OzCols c[2];
+};
+
+// Column maxima: threads on columns, CTAs on shares of the type-sorted atoms.
+__global__ void __launch_bounds__(128) k_oz_colmax(OzColsPair pr, const int32_t *__restrict__ type_perm,
+                                                   const int32_t *__restrict__ type_start, int N)
+{
+    const OzCols &o = pr.c[blockIdx.z];
+    const int q = blockIdx.x * 128 + threadIdx.x;
+    if (q >= o.K) return;
+    const int lo = (int)((long long)blockIdx.y * N / gridDim.y), hi = (int)((long long)(blockIdx.y + 1) * N / gridDim.y);
+    int a = 0;
+    for (int p = lo; p < hi;) {
+        while (p >= type_start[a + 1]) ++a;
+        const int e = min(hi, type_start[a + 1]);
+        unsigned long long mx = 0;
+#pragma unroll 4
+        for (; p < e; ++p) {
+            const unsigned long long b =
+                (unsigned long long)__double_as_longlong(fabs(o.src[(size_t)type_perm[p] * o.ld + q]));
+            mx = b > mx ? b : mx;
+        }
+        atomicMax(&o.mx[(size_t)a * o.nb * o.rb + q], mx);
+    }
+}
+
+// Digits of 16 atoms x 128 columns per CTA (thread: one column, 8 atoms).
+__global__ void __launch_bounds__(256) k_oz_tsplit(OzColsPair pr, const int32_t *__restrict__ type_perm,
+                                                   const int32_t *__restrict__ type_start, int ntypes)
+{
+    constexpr int S = 8, beta = 7;
+    const OzCols &o = pr.c[blockIdx.z];
+    const int q = blockIdx.y * 128 + (threadIdx.x & 127), kh = threadIdx.x >> 7;
+    if (q >= o.nb * o.rb) return;
+    int kc = blockIdx.x, a = 0;
+    for (;; ++a) {
+        if (a == ntypes) return;
+        const int nk = (type_start[a + 1] - type_start[a] + DP_OZ_KC - 1) / DP_OZ_KC;
+        if (kc < nk) break;
+        kc -= nk;
+    }
+    const int col = a * o.nb * o.rb + q;
+    bool zero;
+    const int ex = oz_exponent(q == o.one ? 0x3ff0000000000000ull : q < o.K ? o.mx[col] : 0, beta * S, zero);
+    if (kc == 0 && kh == 0) o.exp[col] = ex;
+    long long I[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+        const int p = type_start[a] + kc * DP_OZ_KC + kh * 8 + u;
+        double v = 0.0;
+        if (!zero && p < type_start[a + 1]) v = q == o.one ? 1.0 : o.src[(size_t)type_perm[p] * o.ld + q];
+        I[u] = oz_rint_pow2(v, beta * S - ex);
+    }
+    uint16_t *out = o.out + ((size_t)blockIdx.x * o.nb + q / o.rb) * S * o.rb * DP_OZ_KC + oz_kofs(q % o.rb, kh * 8);
+    for (int sd = S - 1; sd >= 0; --sd) {
+        int d[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) d[u] = sd > 0 ? oz_digit_step(I[u], beta) : (int)I[u];
+        uint4 v;
+        v.x = (uint32_t)oz_bf16_int(d[0]) | ((uint32_t)oz_bf16_int(d[1]) << 16);
+        v.y = (uint32_t)oz_bf16_int(d[2]) | ((uint32_t)oz_bf16_int(d[3]) << 16);
+        v.z = (uint32_t)oz_bf16_int(d[4]) | ((uint32_t)oz_bf16_int(d[5]) << 16);
+        v.w = (uint32_t)oz_bf16_int(d[6]) | ((uint32_t)oz_bf16_int(d[7]) << 16);
+        *reinterpret_cast<uint4 *>(out + (size_t)sd * o.rb * DP_OZ_KC) = v;
+    }
+}
+
+// Adjoints of the output layer: hb = cE w_out, dhb = -w_out of the atom's type,
+// and its z adjoints zb = cE, dzb = -1 (column 0).
+__global__ void k_oz_pg_out(DevModel m, const int32_t *__restrict__ types, int N, double cE, int F, int ld,
+                            int64_t wo_off, double *__restrict__ hb, double *__restrict__ dhb,
+                            double *__restrict__ zb, double *__restrict__ dzb)
+{
+    for (size_t q = blockIdx.x * (size_t)blockDim.x + threadIdx.x; q < (size_t)N * F;
+         q += (size_t)gridDim.x * blockDim.x) {
+        const size_t i = q / F;
+        const int n = (int)(q - i * F);
+        const int a = min(max(types[i], 0), m.ntypes - 1);  // as the type partition
+        const double w = m.params[m.fit_base[a] + wo_off + n];
+        hb[i * ld + n] = cE * w;
+        dhb[i * ld + n] = -w;
+        if (n == 0) {
+            zb[i * ld] = cE;
+            dzb[i * ld] = -1.0;
+        }
+    }
+}
+
+// z adjoints of a hidden layer: dzb = (1 - t^2) dhb, zb = (1 - t^2) (hb - 2 t dz dhb)
+__global__ void k_oz_pg_z(int N, int F, int ld, const double *__restrict__ t, const double *__restrict__ dz,
+                          const double *__restrict__ hb, const double *__restrict__ dhb, double *__restrict__ zb,
+                          double *__restrict__ dzb)
+{
+    for (size_t q = blockIdx.x * (size_t)blockDim.x + threadIdx.x; q < (size_t)N * F;
+         q += (size_t)gridDim.x * blockDim.x) {
+        const size_t i = q / F, e = i * ld + (q - i * F);
+        const double tv = t[e], one = fma(-tv, tv, 1.0), g = dhb[e];
+        dzb[e] = one * g;
+        zb[e] = one * fma(-2.0 * tv * dz[e], g, hb[e]);
+    }
+}
+
 // Digit width, digit count and segment length of a GEMM of contraction length
 // K (nK chunks) at `bits` bits per operand.  From 55 bits on: 8 digits of 7
 // bits, the widest for which one 16-column chunk is exact, and as many chunks
@@ -600,8 +789,7 @@ void oz_plan_gemm(OzGemm &g, int bits)
     if (bits >= 55) {
         g.beta = 7;
         g.S = 8;
-        const int most = 16777215 / (4096 * (g.S + 2)) / DP_OZ_KC;  // 25 chunks
-        const int nseg = (g.nK + most - 1) / most;
+        const int nseg = (g.nK + OZ_SEG - 1) / OZ_SEG;
         g.seg = (g.nK + nseg - 1) / nseg;
         return;
     }
@@ -667,32 +855,35 @@ cudaError_t dp_launch_oz_weights(cudaStream_t st, const DevModel &m, const OzMod
     return cudaGetLastError();
 }
 
-cudaError_t dp_launch_fit_oz(cudaStream_t st, const DevModel &m, const OzModel &oz, const OzBuffers &ob, int N,
-                             const NlistBuffers &nb, EvalBuffers eb, int num_sms, int32_t *status,
-                             int64_t *launches)
-{
-    const int nf = m.n_fit, T = m.ntypes;
-    const int tiles = (N + DP_OZ_TILE - 1) / DP_OZ_TILE + T;
-    if (tiles > ob.tiles) return cudaErrorInvalidValue;
-    {
-        cudaError_t e = cudaFuncSetAttribute(k_oz_gemm<8>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)gemm_smem(8));
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(k_oz_gemm<5>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gemm_smem(5));
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(k_oz_gemm<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gemm_smem(4));
-        if (e != cudaSuccess) return e;
-    }
-    const int K1 = m.m2 * m.M;
-    const size_t plane = (size_t)ob.nmax * oz.fmax;
-    double *H[2] = {ob.h, ob.h + plane};
-    double *G[2] = {ob.g, ob.g + plane};
+namespace {
+
+// The launches of one pass of the fitting net over N centres.
+struct OzRun {
+    cudaStream_t st;
+    const DevModel &m;
+    const OzModel &oz;
+    const OzBuffers &ob;
+    int N;
+    const NlistBuffers &nb;
+    double *Ei;
+    int num_sms;
+    int32_t *status;
+    int64_t *launches;
+    int T, nf, tiles, K1;
+    size_t plane;
     // parameter offsets of layer l (W_l, b_l) and of the output layer inside a type's block
-    int64_t boff[DP_MAX_LAYERS], wo_off = 0;
+    int64_t woff[DP_MAX_LAYERS], boff[DP_MAX_LAYERS], wo_off;
+
+    OzRun(cudaStream_t st_, const DevModel &m_, const OzModel &oz_, const OzBuffers &ob_, int N_,
+          const NlistBuffers &nb_, double *Ei_, int num_sms_, int32_t *status_, int64_t *launches_)
+        : st(st_), m(m_), oz(oz_), ob(ob_), N(N_), nb(nb_), Ei(Ei_), num_sms(num_sms_), status(status_),
+          launches(launches_), T(m_.ntypes), nf(m_.n_fit), tiles((N_ + DP_OZ_TILE - 1) / DP_OZ_TILE + m_.ntypes),
+          K1(m_.m2 * m_.M), plane((size_t)ob_.nmax * oz_.fmax)
     {
         int64_t off = 0;
         int kin = K1;
         for (int l = 0; l < nf; ++l) {
+            woff[l] = off;
             off += (int64_t)kin * m.fit[l];
             boff[l] = off;
             off += m.fit[l];
@@ -700,9 +891,21 @@ cudaError_t dp_launch_fit_oz(cudaStream_t st, const DevModel &m, const OzModel &
         }
         wo_off = off;
     }
-    const int split_blocks = tiles * (DP_OZ_TILE / 8);
 
-    auto split = [&](int mode, const double *src, int lds, const double *tv, const OzGemm &g) -> cudaError_t {
+    cudaError_t init() const
+    {
+        if (tiles > ob.tiles) return cudaErrorInvalidValue;
+        cudaError_t e = cudaFuncSetAttribute(k_oz_gemm<8>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             (int)gemm_smem(8));
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(k_oz_gemm<5>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gemm_smem(5));
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(k_oz_gemm<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gemm_smem(4));
+        return e;
+    }
+
+    cudaError_t split(int mode, const double *src, int lds, const double *tv, const OzGemm &g) const
+    {
         OzSplitArgs a;
         std::memset(&a, 0, sizeof(a));
         a.mode = mode;
@@ -714,7 +917,7 @@ cudaError_t dp_launch_fit_oz(cudaStream_t st, const DevModel &m, const OzModel &
             a.wout[t] = m.params + m.fit_base[t] + wo_off;
             a.bout[t] = m.params + m.fit_base[t] + wo_off + m.fit[nf - 1];
         }
-        a.Ei = eb.Ei;
+        a.Ei = Ei;
         a.K = g.K;
         a.nK = g.nK;
         a.beta = g.beta;
@@ -725,12 +928,31 @@ cudaError_t dp_launch_fit_oz(cudaStream_t st, const DevModel &m, const OzModel &
         a.a = ob.a;
         a.aexp = ob.aexp;
         a.a_stride = ob.a_stride;
-        k_oz_split<<<split_blocks, 256, 0, st>>>(a);
+        k_oz_split<<<tiles * (DP_OZ_TILE / 8), 256, 0, st>>>(a);
         *launches += 1;
         return cudaGetLastError();
-    };
-    auto gemm = [&](const OzGemm &g, int epi, int skip, int skip_in, int l, const double *hin, int ldh,
-                    bool bcast_wout, double *tout, double *hout, int ldo) -> cudaError_t {
+    }
+
+    cudaError_t launch(OzGemmArgs &a) const
+    {
+        a.type_perm = nb.type_perm;
+        a.type_start = nb.type_start;
+        a.ntypes = T;
+        a.tanh_tab = m.tanh_tab;
+        a.status = status;
+        const int grid = std::min(a.units, num_sms);
+        const size_t smem = gemm_smem(a.g.S);
+        if (a.g.S == 4) k_oz_gemm<4><<<grid, OZ_THREADS, smem, st>>>(a);
+        else if (a.g.S == 5) k_oz_gemm<5><<<grid, OZ_THREADS, smem, st>>>(a);
+        else k_oz_gemm<8><<<grid, OZ_THREADS, smem, st>>>(a);
+        *launches += 1;
+        return cudaGetLastError();
+    }
+
+    // epi as in OzGemmArgs; hin: the skip's operand (with bcast_wout the output weights)
+    cudaError_t gemm(const OzGemm &g, int epi, int skip, int skip_in, int l, const double *hin, int ldh,
+                     bool bcast_wout, const double *tin, double *tout, double *hout, int ldo) const
+    {
         OzGemmArgs a;
         std::memset(&a, 0, sizeof(a));
         a.a = ob.a;
@@ -739,9 +961,6 @@ cudaError_t dp_launch_fit_oz(cudaStream_t st, const DevModel &m, const OzModel &
         a.w = oz.w;
         a.wexp = oz.wexp;
         a.g = g;
-        a.type_perm = nb.type_perm;
-        a.type_start = nb.type_start;
-        a.ntypes = T;
         a.epi = epi;
         a.skip = skip;
         a.skip_in = skip_in;
@@ -751,35 +970,41 @@ cudaError_t dp_launch_fit_oz(cudaStream_t st, const DevModel &m, const OzModel &
         }
         a.hin = hin;
         a.ldh = ldh;
+        a.tin = tin;
         a.tout = tout;
         a.hout = hout;
         a.ldo = ldo;
-        a.tanh_tab = m.tanh_tab;
-        a.status = status;
         a.units = tiles * g.nN;
-        const int grid = std::min(a.units, num_sms);
-        const size_t smem = gemm_smem(g.S);
-        if (g.S == 4) k_oz_gemm<4><<<grid, OZ_THREADS, smem, st>>>(a);
-        else if (g.S == 5) k_oz_gemm<5><<<grid, OZ_THREADS, smem, st>>>(a);
-        else k_oz_gemm<8><<<grid, OZ_THREADS, smem, st>>>(a);
-        *launches += 1;
-        return cudaGetLastError();
-    };
+        return launch(a);
+    }
+};
 
-    cudaError_t e;
+}  // namespace
+
+cudaError_t dp_launch_fit_oz(cudaStream_t st, const DevModel &m, const OzModel &oz, const OzBuffers &ob, int N,
+                             const NlistBuffers &nb, EvalBuffers eb, int num_sms, int32_t *status,
+                             int64_t *launches)
+{
+    const OzRun r(st, m, oz, ob, N, nb, eb.Ei, num_sms, status, launches);
+    const int nf = r.nf, K1 = r.K1;
+    const size_t plane = r.plane;
+    double *H[2] = {ob.h, ob.h + plane};
+    double *G[2] = {ob.g, ob.g + plane};
+    cudaError_t e = r.init();
+    if (e != cudaSuccess) return e;
     // forward: h_l = skip(h_{l-1}) + tanh(h_{l-1} W_l + b_l), h_{-1} = D
     int kin = K1;
     for (int l = 0; l < nf; ++l) {
         const double *x = l == 0 ? eb.D : H[(l - 1) & 1];
         const int ldx = l == 0 ? K1 : oz.fmax;
-        if ((e = split(0, x, ldx, nullptr, oz.fwd[l])) != cudaSuccess) return e;
-        if ((e = gemm(oz.fwd[l], 0, dp_skip_kind(kin, m.fit[l]), kin, l, x, ldx, false,
-                      ob.t + (size_t)l * plane, H[l & 1], oz.fmax)) != cudaSuccess)
+        if ((e = r.split(0, x, ldx, nullptr, oz.fwd[l])) != cudaSuccess) return e;
+        if ((e = r.gemm(oz.fwd[l], 0, dp_skip_kind(kin, m.fit[l]), kin, l, x, ldx, false, nullptr,
+                        ob.t + (size_t)l * plane, H[l & 1], oz.fmax)) != cudaSuccess)
             return e;
         kin = m.fit[l];
     }
     // output layer (E_i) and dL/dz of the last layer (dL/dh = w_out)
-    if ((e = split(2, H[(nf - 1) & 1], oz.fmax, ob.t + (size_t)(nf - 1) * plane, oz.bwd[nf - 1])) != cudaSuccess)
+    if ((e = r.split(2, H[(nf - 1) & 1], oz.fmax, ob.t + (size_t)(nf - 1) * plane, oz.bwd[nf - 1])) != cudaSuccess)
         return e;
     // backward: dL/dh_{l-1} = (dL/dz_l) W_l^T + skip'(dL/dh_l)
     for (int l = nf - 1; l >= 0; --l) {
@@ -787,12 +1012,121 @@ cudaError_t dp_launch_fit_oz(cudaStream_t st, const DevModel &m, const OzModel &
         const bool last = l == nf - 1;
         double *out = l == 0 ? eb.gD : G[(l - 1) & 1];
         const int ldo = l == 0 ? K1 : oz.fmax;
-        if ((e = gemm(oz.bwd[l], 1, dp_skip_kind(kin_l, m.fit[l]), kin_l, l, last ? nullptr : G[l & 1], oz.fmax,
-                      last, nullptr, out, ldo)) != cudaSuccess)
+        if ((e = r.gemm(oz.bwd[l], 1, dp_skip_kind(kin_l, m.fit[l]), kin_l, l, last ? nullptr : G[l & 1], oz.fmax,
+                        last, nullptr, nullptr, out, ldo)) != cudaSuccess)
             return e;
         if (l > 0)
-            if ((e = split(1, G[(l - 1) & 1], oz.fmax, ob.t + (size_t)(l - 1) * plane, oz.bwd[l - 1])) != cudaSuccess)
+            if ((e = r.split(1, G[(l - 1) & 1], oz.fmax, ob.t + (size_t)(l - 1) * plane, oz.bwd[l - 1])) != cudaSuccess)
                 return e;
     }
     return cudaSuccess;
+}
+
+size_t dp_oz_grad_elems(const DevModel &m, const OzModel &oz, int64_t natoms, int which)
+{
+    const size_t K = (size_t)m.m2 * m.M > (size_t)oz.fmax ? (size_t)m.m2 * m.M : (size_t)oz.fmax;
+    const size_t nq = K / DP_OZ_TILE + 1, nn = (oz.fmax + DP_OZ_NC - 1) / DP_OZ_NC;
+    const size_t chunks = (size_t)natoms / DP_OZ_KC + m.ntypes;
+    switch (which) {
+    case 0: return chunks * nq * 8 * OZ_A_BLK;
+    case 1: return chunks * nn * 8 * OZ_B_BLK;
+    case 2: return (size_t)m.ntypes * (nq * DP_OZ_TILE + nn * DP_OZ_NC);
+    default: return 6 * (size_t)natoms * oz.fmax;
+    }
+}
+
+cudaError_t dp_launch_pgrad_fit_oz(cudaStream_t st, const DevModel &m, const OzModel &oz, const OzBuffers &ob,
+                                   const OzGradBuffers &og, const int32_t *types, int N, double cE,
+                                   const NlistBuffers &nb, EvalBuffers eb, PGradBuffers pb, int num_sms,
+                                   int32_t *status, double *grad, int64_t *launches)
+{
+    const OzRun r(st, m, oz, ob, N, nb, eb.Ei, num_sms, status, launches);
+    const int nf = r.nf, K1 = r.K1, T = r.T, ld = oz.fmax;
+    const size_t plane = r.plane;
+    cudaError_t e = r.init();
+    if (e != cudaSuccess) return e;
+    // per layer: tanh values, tangent pre-activations, outputs, their tangents
+    auto keep = [&](int kind, int l) { return pb.fit_scr + (size_t)(kind * nf + l) * plane; };
+    double *hb[2] = {og.x, og.x + plane}, *dhb[2] = {og.x + 2 * plane, og.x + 3 * plane};
+    double *zb = og.x + 4 * plane, *dzb = og.x + 5 * plane;
+
+    // forward, value and tangent
+    int kin = K1;
+    for (int l = 0; l < nf; ++l) {
+        const double *x = l == 0 ? eb.D : keep(2, l - 1), *dx = l == 0 ? pb.dD : keep(3, l - 1);
+        const int ldx = l == 0 ? K1 : ld, sk = dp_skip_kind(kin, m.fit[l]);
+        if ((e = r.split(0, x, ldx, nullptr, oz.fwd[l])) != cudaSuccess) return e;
+        if ((e = r.gemm(oz.fwd[l], 0, sk, kin, l, x, ldx, false, nullptr, keep(0, l), keep(2, l), ld)) != cudaSuccess)
+            return e;
+        if ((e = r.split(0, dx, ldx, nullptr, oz.fwd[l])) != cudaSuccess) return e;
+        if ((e = r.gemm(oz.fwd[l], 2, sk, kin, l, dx, ldx, false, keep(0, l), keep(1, l), keep(3, l), ld)) !=
+            cudaSuccess)
+            return e;
+        kin = m.fit[l];
+    }
+
+    // gradient of a layer's weights and, as the row after them, its bias
+    auto weights = [&](const double *x, const double *dx, int ldx, int K, int F, int64_t off) -> cudaError_t {
+        const int nq = K / DP_OZ_TILE + 1, nN = (F + DP_OZ_NC - 1) / DP_OZ_NC;  // K + 1 rows
+        const int splits = std::min(64, (N + 31) / 32);
+        for (int pass = 0; pass < 2; ++pass) {
+            OzColsPair c;
+            int32_t *expb = og.exp + (size_t)T * nq * DP_OZ_TILE;
+            c.c[0] = OzCols{pass == 0 ? x : dx, ldx, K, pass == 0 ? K : -1, DP_OZ_TILE, nq, og.a, og.exp, og.mx};
+            c.c[1] = OzCols{pass == 0 ? zb : dzb, ld, F, -1, DP_OZ_NC, nN, og.b, expb,
+                            og.mx + (size_t)T * nq * DP_OZ_TILE};
+            cudaError_t e2 = cudaMemsetAsync(og.mx, 0, 8 * (size_t)T * (nq * DP_OZ_TILE + nN * DP_OZ_NC), st);
+            if (e2 != cudaSuccess) return e2;
+            const int cols = std::max(K, F);
+            k_oz_colmax<<<dim3((cols + 127) / 128, splits, 2), 128, 0, st>>>(c, nb.type_perm, nb.type_start, N);
+            k_oz_tsplit<<<dim3(N / DP_OZ_KC + T, std::max(nq, (nN * DP_OZ_NC + 127) / 128), 2), 256, 0, st>>>(
+                c, nb.type_perm, nb.type_start, T);
+            *launches += 2;
+            OzGemmArgs a;
+            std::memset(&a, 0, sizeof(a));
+            a.a = og.a;
+            a.aexp = og.exp;
+            a.w = og.b;
+            a.wexp = expb;
+            a.g.N = F;
+            a.g.nN = nN;
+            a.g.beta = 7;
+            a.g.S = 8;
+            a.epi = 1;
+            a.skip = pass;  // the second product is added to the first
+            a.wg = 1;
+            a.rows = K + 1;
+            a.nq = nq;
+            a.hout = grad;
+            a.ldo = a.ldh = F;
+            for (int t = 0; t < T; ++t) a.out_off[t] = m.fit_base[t] + off;
+            a.units = T * nq * nN;
+            if ((e2 = r.launch(a)) != cudaSuccess) return e2;
+        }
+        return cudaSuccess;
+    };
+
+    // reverse mode of cE E - dE
+    const int Fl = m.fit[nf - 1];
+    auto blocks = [&](int F) { return (int)std::min<size_t>(((size_t)N * F + 255) / 256, 8192); };
+    k_oz_pg_out<<<blocks(Fl), 256, 0, st>>>(m, types, N, cE, Fl, ld, r.wo_off, hb[(nf - 1) & 1], dhb[(nf - 1) & 1], zb,
+                                            dzb);
+    *launches += 1;
+    if ((e = weights(keep(2, nf - 1), keep(3, nf - 1), ld, Fl, 1, r.wo_off)) != cudaSuccess) return e;
+    for (int l = nf - 1; l >= 0; --l) {
+        const int F = m.fit[l], kl = l == 0 ? K1 : m.fit[l - 1], sk = dp_skip_kind(kl, F);
+        double *h = hb[l & 1], *dh = dhb[l & 1];
+        k_oz_pg_z<<<blocks(F), 256, 0, st>>>(N, F, ld, keep(0, l), keep(1, l), h, dh, zb, dzb);
+        *launches += 1;
+        if ((e = weights(l == 0 ? eb.D : keep(2, l - 1), l == 0 ? pb.dD : keep(3, l - 1), l == 0 ? K1 : ld, kl, F,
+                         r.woff[l])) != cudaSuccess)
+            return e;
+        double *out = l == 0 ? pb.Db : hb[(l - 1) & 1], *dout = l == 0 ? pb.dDb : dhb[(l - 1) & 1];
+        const int ldo = l == 0 ? K1 : ld;
+        if ((e = r.split(0, zb, ld, nullptr, oz.bwd[l])) != cudaSuccess) return e;
+        if ((e = r.gemm(oz.bwd[l], 1, sk, kl, l, h, ld, false, nullptr, nullptr, out, ldo)) != cudaSuccess) return e;
+        if ((e = r.split(0, dzb, ld, nullptr, oz.bwd[l])) != cudaSuccess) return e;
+        if ((e = r.gemm(oz.bwd[l], 1, sk, kl, l, dh, ld, false, nullptr, nullptr, dout, ldo)) != cudaSuccess) return e;
+    }
+    return cudaGetLastError();
 }

@@ -22,7 +22,10 @@
 // and k_pg_emb are replaced by the series' kernels, which work on moments and
 // at the series' nodes instead of on every row through the net; they stay for
 // nets that are not resolved and, launched behind a device flag (`gate`), for
-// frames with a row beyond the series' domain.
+// frames with a row beyond the series' domain.  k_pg_fit runs in contexts that
+// keep the fitting net on the FP64 units; the others take fit_oz.cu.
+#include <algorithm>
+
 #include "cheb.cuh"
 #include "dp_internal.cuh"
 
@@ -658,12 +661,23 @@ __global__ void __launch_bounds__(NT, 1) k_pg_emb(DevModel m, const double *__re
     }
 }
 
-// The embedding parameters (p < nemb) come from the series' kernels unless the gate is set.
-__global__ void k_pg_reduce(const double *__restrict__ slices, int nslices, int64_t nparams, int64_t nemb,
-                            const int32_t *gate, double *__restrict__ grad)
+// Parameters [0, nemb) are the embedding nets' and come from the series' kernels
+// unless the gate is set; [nemb, last) are in the slices where k_pg_fit ran.
+__global__ void k_pg_zero(double *__restrict__ slices, int nslices, int64_t nparams, int64_t nemb, int64_t last,
+                          const int32_t *gate)
 {
     const int64_t first = gate != nullptr && *gate == 0 ? nemb : 0;
-    for (int64_t p = first + blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < nparams; p += (int64_t)gridDim.x * blockDim.x) {
+    for (int c = blockIdx.y; c < nslices; c += gridDim.y)
+        for (int64_t p = first + blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < last;
+             p += (int64_t)gridDim.x * blockDim.x)
+            slices[(size_t)c * nparams + p] = 0.0;
+}
+
+__global__ void k_pg_reduce(const double *__restrict__ slices, int nslices, int64_t nparams, int64_t nemb,
+                            int64_t last, const int32_t *gate, double *__restrict__ grad)
+{
+    const int64_t first = gate != nullptr && *gate == 0 ? nemb : 0;
+    for (int64_t p = first + blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < last; p += (int64_t)gridDim.x * blockDim.x) {
         double acc = 0.0;
         for (int c = 0; c < nslices; ++c) acc += slices[(size_t)c * nparams + p];
         grad[p] = acc;
@@ -679,7 +693,8 @@ size_t dp_pgrad_row_scratch(int num_sms) { return (size_t)num_sms * 6 * ROWS * (
 cudaError_t dp_launch_pgrad(cudaStream_t st, const DevModel &m, int64_t nparams, const double *x, const int32_t *types,
                             Box3 box, int N, const double *lam, double cE, const FormatBuffers &fb,
                             const NlistBuffers &nb, EvalBuffers eb, PGradBuffers pb, int num_sms,
-                            const ChebModel *cm, const ChebGradBuffers *cg, const double *trig, double *grad,
+                            const ChebModel *cm, const ChebGradBuffers *cg, const double *trig, const OzModel *oz,
+                            const OzBuffers *ob, const OzGradBuffers *og, int32_t *status, double *grad,
                             int64_t *launches)
 {
     const int32_t *gate = cm ? cg->far : nullptr;
@@ -693,8 +708,7 @@ cudaError_t dp_launch_pgrad(cudaStream_t st, const DevModel &m, int64_t nparams,
     const int grid_emb = num_sms < N ? num_sms : (N > 0 ? N : 1);
     cudaError_t e;
     // slices: one per CTA of k_pg_fit / k_pg_emb (both use num_sms CTAs)
-    e = cudaMemsetAsync(pb.slices, 0, sizeof(double) * (size_t)num_sms * nparams, st);
-    if (e != cudaSuccess) return e;
+    const int64_t nemb = (int64_t)m.ntypes * m.ntypes * m.emb_net_size, last = oz ? nemb : nparams;
     if (cm && (e = dp_launch_chebpg_fwd(st, m, *cm, x, types, box, N, lam, fb, nb, eb, pb, *cg, launches)) != cudaSuccess)
         return e;
     {
@@ -704,7 +718,15 @@ cudaError_t dp_launch_pgrad(cudaStream_t st, const DevModel &m, int64_t nparams,
         k_pg_tan<<<grid_emb, NT, smem, st>>>(m, x, types, box, N, lam, fb.nlist, fb.nreal, eb.T, pb.dT, eb.D, pb.dD,
                                              LD, wsz, gate);
     }
-    {
+    // after k_pg_tan: the series' forward has set the gate
+    const int zgrid = (int)std::min<int64_t>((last + 255) / 256, 64);
+    k_pg_zero<<<dim3(zgrid, num_sms), 256, 0, st>>>(pb.slices, num_sms, nparams, nemb, last, gate);
+    *launches += 1;
+    if (oz) {
+        if ((e = dp_launch_pgrad_fit_oz(st, m, *oz, *ob, *og, types, N, cE, nb, eb, pb, num_sms, status, grad,
+                                        launches)) != cudaSuccess)
+            return e;
+    } else {
         const size_t smem = sizeof(double) * 4 * FRT * (FW + 1);
         e = cudaFuncSetAttribute(k_pg_fit, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
@@ -721,9 +743,9 @@ cudaError_t dp_launch_pgrad(cudaStream_t st, const DevModel &m, int64_t nparams,
                                             pb.slices, nparams, pb.rowscr, LD, wsz, gate);
     }
     if (cm && (e = dp_launch_chebpg_bwd(st, m, *cm, N, nb, eb, pb, *cg, trig, grad, launches)) != cudaSuccess) return e;
-    k_pg_reduce<<<(int)((nparams + 255) / 256 < 4096 ? (nparams + 255) / 256 : 4096), 256, 0, st>>>(
-        pb.slices, num_sms, nparams, (int64_t)m.ntypes * m.ntypes * m.emb_net_size, gate, grad);
-    *launches += 4;
+    k_pg_reduce<<<(int)std::min<int64_t>((last + 255) / 256, 4096), 256, 0, st>>>(pb.slices, num_sms, nparams, nemb,
+                                                                                  last, gate, grad);
+    *launches += oz ? 3 : 4;
     (void)maxw;
     (void)grid_emb;
     return cudaGetLastError();
