@@ -15,11 +15,12 @@ struct ChebModel {
     int n;             // terms used by every net (0: not resolved, the series is not used)
     const double *C;   // [T T][NN][M]: G_f(s) = sum_n C[net][n][f] T_n(t)
     const double *Ct;  // [T][M][T NN]: the same values, the nets of centre type a side by side
+    const double *V;   // [T T][NN][M]: dG_f/ds = sum_n V[net][n][f] T_n(t)
 };
 
 // Device scratch of the construction; bytes of one context's buffers.
 struct ChebBuffers {
-    double *C, *Ct;
+    double *C, *Ct, *V;
     double *y;      // node values, [T T][NN][M][2] (high and low part)
     double *mx;     // [T T][NN] max_f |C|
     double *trig;   // [4 NN][2] cos(pi j / (2 NN)), then [DP_CHEB_NTANH][2] tanh(k / 32)
@@ -27,7 +28,7 @@ struct ChebBuffers {
 constexpr int DP_CHEB_NTANH = 705;
 
 bool dp_cheb_supported(const DevModel &m);
-size_t dp_cheb_elems(const DevModel &m, int which);  // doubles of C, Ct, y, mx, trig (which = 0..4)
+size_t dp_cheb_elems(const DevModel &m, int which);  // doubles of C, Ct, V, y, mx, trig (which = 0..5)
 cudaError_t dp_launch_cheb_setup(cudaStream_t st, ChebBuffers cb, int64_t *launches);
 // Coefficients of every net from the device parameters.
 cudaError_t dp_launch_cheb_build(cudaStream_t st, const DevModel &m, ChebBuffers cb, int64_t *launches);
@@ -44,12 +45,12 @@ cudaError_t dp_launch_cheb_bwd(cudaStream_t st, const DevModel &m, const ChebMod
 // every atom with the moments kept, then, from dPhi/dD and dPhi/d(dD), the
 // gradient of the embedding nets' parameters by way of the coefficients.
 struct ChebGradBuffers {
-    double *mom;    // [N][T n][8] moments and their tangents
-    double *part;   // [DP_CHEB_SPLITS][T T][NN][M] partial coefficient adjoints
-    double *node;   // [T T][NN][2][sum of widths] layer outputs and z adjoints at the nodes
+    double *mom;    // [N][T n][12] moments (k_chebpg_fwd)
+    double *part;   // [dp_cheb_splits][2][T T][NN][M] partial adjoints of C and V
+    double *node;   // [T T][NN][4][sum of widths] layer outputs and z adjoints at the nodes, with tangents
     int32_t *far;   // set when a row lies beyond S: the caller's other kernels run instead
 };
-constexpr int DP_CHEB_SPLITS = 64;
+inline int dp_cheb_splits(int ntypes) { return ntypes > 8 ? 8 : 64 / ntypes; }  // atom shares of a centre type
 // Terms the gradient keeps: the parameter derivatives' series converge as the
 // nets' with a polynomial factor, which 8 more terms cover.
 inline int dp_cheb_grad_terms(int n) { return n + 8 < DP_CHEB_NN ? n + 8 : DP_CHEB_NN; }

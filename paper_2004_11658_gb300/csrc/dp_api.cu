@@ -564,12 +564,13 @@ dp_status ensure_cheb(dp_ctx *c)
     if (c->cheb_version < 0) e = dp_launch_cheb_setup(c->stream, c->cb, &c->launches);
     if (e == cudaSuccess) e = dp_launch_cheb_build(c->stream, c->m, c->cb, &c->launches);
     if (e != cudaSuccess) return cuda_fail(e, "embedding series");
-    const size_t bytes = sizeof(double) * dp_cheb_elems(c->m, 3);
+    const size_t bytes = sizeof(double) * dp_cheb_elems(c->m, 4);
     DP_CUDA(cudaMemcpyAsync(c->h_cheb_mx, c->cb.mx, bytes, cudaMemcpyDeviceToHost, c->stream), "embedding series");
     DP_CUDA(cudaStreamSynchronize(c->stream), "embedding series");
     c->cheb.n = dp_cheb_terms(c->m, c->h_cheb_mx);
     c->cheb.C = c->cb.C;
     c->cheb.Ct = c->cb.Ct;
+    c->cheb.V = c->cb.V;
     c->cheb_version = c->model->version;
     return DP_OK;
 }
@@ -954,7 +955,7 @@ void dp_ctx_free(dp_ctx *c)
                     c->eb.fit_t, c->eb.fit_h, c->d_p32, c->d_emb_ops, c->d_fit_fwd, c->d_fit_bwd,
                     c->pb.dT, c->pb.dD, c->pb.Db, c->pb.dDb, c->pb.fit_scr, c->pb.rowscr, c->pb.slices,
                     c->d_oz_w, c->d_oz_e, c->ob.a, c->ob.aexp, c->ob.t, c->ob.h, c->ob.g, c->d_dtile, c->d_ex_w,
-                    c->eb.Gst, c->eb.Gmx, c->cb.C, c->cb.Ct, c->cb.y, c->cb.mx, c->cb.trig, c->cg.mom,
+                    c->eb.Gst, c->eb.Gmx, c->cb.C, c->cb.Ct, c->cb.V, c->cb.y, c->cb.mx, c->cb.trig, c->cg.mom,
                     c->cg.part, c->cg.node, c->cg.far, c->og.a, c->og.b, c->og.exp, c->og.mx, c->og.x};
     for (void *p : bufs) dev_free(p);
     delete c;
@@ -1046,9 +1047,9 @@ dp_status dp_ctx_create(const dp_model *model, int64_t natoms_max, int32_t cand_
     }
     c->cheb_version = -1;
     if (precision == DP_PREC_FP64 && dp_cheb_supported(c->m)) {
-        double **bufs[] = {&c->cb.C, &c->cb.Ct, &c->cb.y, &c->cb.mx, &c->cb.trig};
-        for (int q = 0; q < 5; ++q) ALLOC(*bufs[q], dp_cheb_elems(c->m, q));
-        if (!s && cudaMallocHost((void **)&c->h_cheb_mx, sizeof(double) * dp_cheb_elems(c->m, 3)) != cudaSuccess) {
+        double **bufs[] = {&c->cb.C, &c->cb.Ct, &c->cb.V, &c->cb.y, &c->cb.mx, &c->cb.trig};
+        for (int q = 0; q < 6; ++q) ALLOC(*bufs[q], dp_cheb_elems(c->m, q));
+        if (!s && cudaMallocHost((void **)&c->h_cheb_mx, sizeof(double) * dp_cheb_elems(c->m, 4)) != cudaSuccess) {
             c->h_cheb_mx = nullptr;
             cudaGetLastError();
             s = fail(DP_ERR_NOMEM, "pinned allocation failed");

@@ -224,6 +224,17 @@ __global__ void __launch_bounds__(CT) k_cheb_coef(DevModel m, const double *__re
     }
 }
 
+// Coefficients of the derivative, V_n = (2 / S) (2 - [n = 0]) sum_{m = n+1, n+3, ..} m C_m
+// (the terms decrease geometrically: smallest first).
+__global__ void __launch_bounds__(CT) k_cheb_deriv(DevModel m, const double *__restrict__ C, double *__restrict__ V)
+{
+    const int net = blockIdx.x / NN, n = blockIdx.x % NN, f = threadIdx.x;
+    if (f >= m.M) return;
+    double v = 0.0;
+    for (int q = NN - 1 - (NN - n) % 2; q > n; q -= 2) v = fma((double)q, C[(size_t)(net * NN + q) * m.M + f], v);
+    V[(size_t)blockIdx.x * m.M + f] = v * ((n == 0 ? 1.0 : 2.0) * DP_CHEB_SCALE);
+}
+
 // ---------------------------------------------------------- rows beyond S ---
 
 // The net with its s-derivative at s, by the whole CTA (rows with s > S only):
@@ -672,13 +683,18 @@ __global__ void __launch_bounds__(CT) k_cheb_bwd(DevModel m, ChebModel cm, const
 // ------------------------------------------------- parameter gradient ------
 //
 // Phi = sum_i (cE E_i - dE_i) with dE_i the tangent of E_i along
-// delta r_ij = lambda_j - lambda_i (csrc/pgrad.cu).  With P the moments and dP
-// their tangents, T = scale P C and dT = scale dP C, so the adjoint of the
-// coefficients is sum_atoms (P Tb + dP dTb); it goes back through the discrete
-// transform to the net's values at the NN nodes, and reverse mode runs through
-// the net at NN points instead of at every row.  12,288 water atoms, student
-// widths: 70 -> 5.3 ms (the net, its tangent and its reverse mode at every row
-// before); 648 atoms, full width: 13.8 -> 0.5 ms.
+// delta r_ij = lambda_j - lambda_i (csrc/pgrad.cu).  With the moments
+//   P_n = sum_rows R~ T_n,  dP_n = sum_rows dR~ T_n,  Q_n = sum_rows R~ ds T_n,
+// T = scale P C and dT = scale (dP C + Q V).  The adjoints of C and V are sums
+// over the atoms, sum (P Tb + dP dTb) and sum Q dTb; both go back through the
+// discrete transform to the net's values and derivatives at the NN nodes, and
+// reverse mode runs through the net with its s-tangent at NN points instead of
+// at every row.  (Folding V's adjoint into C's would multiply it by n^2 and
+// lose two digits to the cancellation over the nodes.)  12,288 water atoms,
+// student widths: 70 -> 5.0 ms (the net, its tangent and its reverse mode at
+// every row before); 648 atoms, full width: 13.8 -> 0.6 ms.
+
+constexpr int PM = 12;  // moments per term: P, dP, Q (4 components each)
 
 // T, dT, D, dD and the moments of one atom per CTA, as k_cheb_fwd with the tangent.
 __global__ void __launch_bounds__(CT) k_chebpg_fwd(DevModel m, ChebModel cm, const double *__restrict__ x,
@@ -693,12 +709,11 @@ __global__ void __launch_bounds__(CT) k_chebpg_fwd(DevModel m, ChebModel cm, con
 {
     extern __shared__ __align__(16) double sm[];
     const int nc = cm.n, M = m.M, T = m.ntypes, nm = m.nm, tid = threadIdx.x;
-    double *R8 = sm;                       // [CT][8] R~ and dR~
-    double *part = R8 + CT * 8;            // [CT][8]
-    double *Mom = part + CT * 8;           // [T nc][8]
-    double *Ts = Mom + T * nc * 8;         // [8][M] T, dT
+    double *RM = sm;                       // [CT][PM] R~, dR~, R~ ds
+    double *part = RM + CT * PM;           // [CT][PM]
+    double *Mom = part + CT * PM;          // [T nc][PM]
+    double *Ts = Mom + T * nc * PM;        // [8][M] T, dT
     double *Tch = Ts + 8 * M;              // [nc][LDT] T_n(t)
-    double *dTch = Tch + nc * LDT;         // [nc][LDT] d/dtau T_n(t)
     __shared__ int start[DP_MAX_TYPES + 1];
     const int i = type_perm[blockIdx.x];
     const int a = types[i];
@@ -711,7 +726,7 @@ __global__ void __launch_bounds__(CT) k_chebpg_fwd(DevModel m, ChebModel cm, con
         }
         start[T] = r;
     }
-    for (int p = tid; p < T * nc * 8; p += CT) Mom[p] = 0.0;
+    for (int p = tid; p < T * nc * PM; p += CT) Mom[p] = 0.0;
     __syncthreads();
     const int R = start[T];
     const double xi[3] = {x[3 * i], x[3 * i + 1], x[3 * i + 2]};
@@ -731,27 +746,26 @@ __global__ void __launch_bounds__(CT) k_chebpg_fwd(DevModel m, ChebModel cm, con
             const double u[3] = {d[0] * inv, d[1] * inv, d[2] * inv};
             const double dr[3] = {lam[3 * j] - li[0], lam[3 * j + 1] - li[1], lam[3 * j + 2] - li[2]};
             const double udr = u[0] * dr[0] + u[1] * dr[1] + u[2] * dr[2];
-            double *Rq = R8 + tid * 8;
+            double *Rq = RM + tid * PM;
+            const double dst = ds * udr;  // the tangent of s
             Rq[0] = s;
-            Rq[4] = ds * udr;
+            Rq[4] = dst;
+            Rq[8] = s * dst;
 #pragma unroll
             for (int e = 0; e < 3; ++e) {
                 Rq[1 + e] = s * u[e];
-                Rq[5 + e] = ds * u[e] * udr + s * inv * (dr[e] - u[e] * udr);
+                Rq[5 + e] = dst * u[e] + s * inv * (dr[e] - u[e] * udr);
+                Rq[9 + e] = s * u[e] * dst;
             }
             any_far |= !(s <= DP_CHEB_S);
-            const double t = fma(s, DP_CHEB_SCALE, -1.0), t2 = t + t, dt = DP_CHEB_SCALE * Rq[4];
-            double p0 = 1.0, p1 = t, q0 = 0.0, q1 = dt;
+            const double t = fma(s, DP_CHEB_SCALE, -1.0), t2 = t + t;
+            double p0 = 1.0, p1 = t;
             Tch[tid] = 1.0;
-            dTch[tid] = 0.0;
             for (int n = 1; n < nc; ++n) {
                 Tch[n * LDT + tid] = p1;
-                dTch[n * LDT + tid] = q1;
-                const double p2 = fma(t2, p1, -p0), q2 = fma(t2, q1, fma(2.0 * dt, p1, -q0));
+                const double p2 = fma(t2, p1, -p0);
                 p0 = p1;
                 p1 = p2;
-                q0 = q1;
-                q1 = q2;
             }
         }
         __syncthreads();
@@ -759,42 +773,46 @@ __global__ void __launch_bounds__(CT) k_chebpg_fwd(DevModel m, ChebModel cm, con
             const int lo = max(start[b] - c0, 0), hi = min(start[b + 1] - c0, CT);
             if (lo >= hi) continue;
             if (msl < ns) {
-                double acc[8];
+                double acc[PM];
 #pragma unroll
-                for (int c = 0; c < 8; ++c) acc[c] = 0.0;
+                for (int c = 0; c < PM; ++c) acc[c] = 0.0;
                 for (int r = lo + msl; r < hi; r += ns) {
-                    const double tv = Tch[mn * LDT + r], dv = dTch[mn * LDT + r];
-                    const double *Rq = R8 + r * 8;
+                    const double tv = Tch[mn * LDT + r];
+                    const double *Rq = RM + r * PM;
 #pragma unroll
-                    for (int c = 0; c < 4; ++c) {
-                        acc[c] = fma(tv, Rq[c], acc[c]);
-                        acc[4 + c] = fma(tv, Rq[4 + c], fma(dv, Rq[c], acc[4 + c]));
-                    }
+                    for (int c = 0; c < PM; ++c) acc[c] = fma(tv, Rq[c], acc[c]);
                 }
 #pragma unroll
-                for (int c = 0; c < 8; ++c) part[tid * 8 + c] = acc[c];
+                for (int c = 0; c < PM; ++c) part[tid * PM + c] = acc[c];
             }
             __syncthreads();
-            for (int p = tid; p < nc * 8; p += CT) {
-                double v = Mom[b * nc * 8 + p];
-                for (int u = 0; u < ns; ++u) v += part[u * nc * 8 + p];
-                Mom[b * nc * 8 + p] = v;
+            for (int p = tid; p < nc * PM; p += CT) {
+                double v = Mom[b * nc * PM + p];
+                for (int u = 0; u < ns; ++u) v += part[u * nc * PM + p];
+                Mom[b * nc * PM + p] = v;
             }
             __syncthreads();
         }
     }
     if (any_far) atomicOr(far_flag, 1);
-    for (int p = tid; p < T * nc * 8; p += CT) momout[(size_t)i * T * nc * 8 + p] = Mom[p];
+    for (int p = tid; p < T * nc * PM; p += CT) momout[(size_t)i * T * nc * PM + p] = Mom[p];
     {
-        const double *C = cm.C + (size_t)(a_ok ? a : 0) * T * NN * M;
+        const size_t net0 = (size_t)(a_ok ? a : 0) * T * NN * M;
         for (int p = tid; p < 8 * M; p += CT) {
             const int c = p / M, f = p - c * M;
             double acc = 0.0;
             for (int b = 0; b < T; ++b) {
                 if (start[b] == start[b + 1]) continue;
-                const double *Cb = C + (size_t)b * NN * M + f, *mo = Mom + b * nc * 8 + c;
+                const double *Cb = cm.C + net0 + (size_t)b * NN * M + f, *Vb = cm.V + net0 + (size_t)b * NN * M + f;
+                const double *mo = Mom + b * nc * PM + c;
+                if (c < 4) {
 #pragma unroll 4
-                for (int n = 0; n < nc; ++n) acc = fma(mo[n * 8], Cb[n * M], acc);
+                    for (int n = 0; n < nc; ++n) acc = fma(mo[n * PM], Cb[n * M], acc);
+                } else {
+#pragma unroll 4
+                    for (int n = 0; n < nc; ++n)
+                        acc = fma(mo[n * PM], Cb[n * M], fma(mo[n * PM + 4], Vb[n * M], acc));
+                }
             }
             Ts[p] = acc * m.desc_scale;
         }
@@ -885,11 +903,11 @@ __global__ void __launch_bounds__(CT) k_chebpg_tb(DevModel m, double *__restrict
     }
 }
 
-// Partial coefficient adjoints: CTA (split, centre type, 16 terms of the type's
-// nets side by side) sums P Tb + dP dTb over its share of the type's atoms;
-// thread = (4 terms, features u, u + 32, ...).
+// Partial adjoints of C and V: CTA (split, centre type, 16 terms of the type's
+// nets side by side) sums P Tb + dP dTb and Q dTb over its share of the type's
+// atoms; thread = (4 terms, features u, u + 32, ...).
 constexpr int CBK = 16;
-constexpr int CBA = 8;  // atoms staged at once
+constexpr int CBA = 4;  // atoms staged at once
 __global__ void __launch_bounds__(CT) k_chebpg_cb(DevModel m, int nc, const int32_t *__restrict__ type_perm,
                                                   const int32_t *__restrict__ type_start,
                                                   const double *__restrict__ mom, const double *__restrict__ Tb,
@@ -900,23 +918,23 @@ __global__ void __launch_bounds__(CT) k_chebpg_cb(DevModel m, int nc, const int3
     extern __shared__ __align__(16) double sm[];
     const int M = m.M, T = m.ntypes, Kt = T * nc, tid = threadIdx.x;
     const int a = blockIdx.y, k0 = blockIdx.z * CBK;
-    double *ms = sm;               // [CBA][8][CBK]
-    double *ts = ms + CBA * 8 * CBK;  // [CBA][8][M]
+    double *ms = sm;                   // [CBA][PM][CBK]
+    double *ts = ms + CBA * PM * CBK;  // [CBA][8][M]: Tb, dTb
     const int s0 = type_start[a], cnt = type_start[a + 1] - s0;
     const int lo = (int)((long long)blockIdx.x * cnt / gridDim.x), hi = (int)((long long)(blockIdx.x + 1) * cnt / gridDim.x);
     const int kq = (tid >> 5) * 4, fl = tid & 31;
-    double acc[4][4];
+    double acc[4][4], accv[4][4];
 #pragma unroll
     for (int u = 0; u < 4; ++u)
 #pragma unroll
-        for (int v = 0; v < 4; ++v) acc[u][v] = 0.0;
+        for (int v = 0; v < 4; ++v) acc[u][v] = accv[u][v] = 0.0;
     for (int b0 = lo; b0 < hi; b0 += CBA) {
         const int n = min(CBA, hi - b0);
         __syncthreads();
-        for (int p = tid; p < n * 8 * CBK; p += CT) {
-            const int at = p / (8 * CBK), k = (p / 8) % CBK, c = p % 8;
+        for (int p = tid; p < n * PM * CBK; p += CT) {
+            const int at = p / (PM * CBK), k = (p / PM) % CBK, c = p % PM;
             const size_t i = type_perm[s0 + b0 + at];
-            ms[(at * 8 + c) * CBK + k] = k0 + k < Kt ? mom[(i * Kt + k0 + k) * 8 + c] : 0.0;
+            ms[(at * PM + c) * CBK + k] = k0 + k < Kt ? mom[(i * Kt + k0 + k) * PM + c] : 0.0;
         }
         for (int p = tid; p < n * 8 * M; p += CT) {
             const int at = p / (8 * M), r = p - at * 8 * M;
@@ -924,28 +942,42 @@ __global__ void __launch_bounds__(CT) k_chebpg_cb(DevModel m, int nc, const int3
             ts[p] = r < 4 * M ? Tb[i * 4 * M + r] : dTb[i * 4 * M + r - 4 * M];
         }
         __syncthreads();
-        for (int e = 0; e < 8 * n; ++e) {
-            double mv[4];
+        for (int at = 0; at < n; ++at)
+#pragma unroll 2
+            for (int c = 0; c < 4; ++c) {
+                const double *mp = ms + (at * PM + c) * CBK + kq;
+                double mv[3][4];
 #pragma unroll
-            for (int u = 0; u < 4; ++u) mv[u] = ms[e * CBK + kq + u];
-#pragma unroll
-            for (int v = 0; v < 4; ++v)
-                if (fl + 32 * v < M) {
-                    const double tv = ts[e * M + fl + 32 * v];
-#pragma unroll
-                    for (int u = 0; u < 4; ++u) acc[u][v] = fma(mv[u], tv, acc[u][v]);
+                for (int u = 0; u < 4; ++u) {
+                    mv[0][u] = mp[u];
+                    mv[1][u] = mp[4 * CBK + u];
+                    mv[2][u] = mp[8 * CBK + u];
                 }
-        }
+#pragma unroll
+                for (int v = 0; v < 4; ++v)
+                    if (fl + 32 * v < M) {
+                        const double tv = ts[(at * 8 + c) * M + fl + 32 * v], dv = ts[(at * 8 + 4 + c) * M + fl + 32 * v];
+#pragma unroll
+                        for (int u = 0; u < 4; ++u) {
+                            acc[u][v] = fma(mv[0][u], tv, fma(mv[1][u], dv, acc[u][v]));
+                            accv[u][v] = fma(mv[2][u], dv, accv[u][v]);
+                        }
+                    }
+            }
     }
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
         const int k = k0 + kq + u;
         if (k >= Kt) continue;
         const int b = k / nc, n = k - b * nc;
+        const size_t nets = (size_t)T * T;
+        double *pc = part + ((2 * (size_t)blockIdx.x * nets + a * T + b) * NN + n) * M, *pv = pc + nets * NN * M;
 #pragma unroll
         for (int v = 0; v < 4; ++v)
-            if (fl + 32 * v < M)
-                part[(((size_t)blockIdx.x * T * T + a * T + b) * NN + n) * M + fl + 32 * v] = acc[u][v];
+            if (fl + 32 * v < M) {
+                pc[fl + 32 * v] = acc[u][v];
+                pv[fl + 32 * v] = accv[u][v];
+            }
     }
 }
 
@@ -960,73 +992,109 @@ __global__ void k_chebpg_sum(double *__restrict__ part, size_t elems, int splits
     }
 }
 
-// One CTA per (net, node): the adjoint of the net's value there, Gb_f = sum_n
-// (2 - [n = 0]) / NN cos(pi n (2k+1) / (2 NN)) Cb_nf, and reverse mode through
-// the layers; layer outputs h and z adjoints go to node[net][k][0 / 1][.].
+// One CTA per (net, node): the adjoints of the net's value and derivative there,
+// Gb_f = sum_n w_nk Cb_nf and G'b_f = sum_n w_nk Vb_nf with w_nk = (2 - [n = 0]) / NN
+// cos(pi n (2k+1) / (2 NN)), and reverse mode through the layers with their
+// s-tangents; h, dh, zb and dzb of every layer go to node[net][k][0 .. 3][.].
 __global__ void __launch_bounds__(CT) k_chebpg_node(DevModel m, int nc, const double *__restrict__ trig,
-                                                    const double *__restrict__ Cb, double *__restrict__ node, int se,
-                                                    const int32_t *far_flag)
+                                                    const double *__restrict__ Cb, const double *__restrict__ Vb,
+                                                    double *__restrict__ node, int se, const int32_t *far_flag)
 {
     if (*far_flag) return;
-    __shared__ double h[DP_MAX_LAYERS][DP_MAX_EMB_W], t[DP_MAX_LAYERS][DP_MAX_EMB_W], g[DP_MAX_EMB_W], zb[DP_MAX_EMB_W];
+    __shared__ double h[DP_MAX_LAYERS][DP_MAX_EMB_W], dh[DP_MAX_LAYERS][DP_MAX_EMB_W], t[DP_MAX_LAYERS][DP_MAX_EMB_W],
+        dz[DP_MAX_LAYERS][DP_MAX_EMB_W];
+    __shared__ double g[DP_MAX_EMB_W], dg[DP_MAX_EMB_W], zb[DP_MAX_EMB_W], dzb[DP_MAX_EMB_W];
     const int net = blockIdx.x / NN, k = blockIdx.x % NN, o = threadIdx.x, M = m.M;
     const double *P = m.params + m.emb_base[net];
     const double s = (1.0 + trig[2 * (2 * k + 1)]) / DP_CHEB_SCALE;
-    if (o < m.emb[0]) h[0][o] = t[0][o] = dp_tanh64(fma(s, P[o], P[m.emb[0] + o]), m.tanh_tab);
+    if (o < m.emb[0]) {
+        const double tv = dp_tanh64(fma(s, P[o], P[m.emb[0] + o]), m.tanh_tab);
+        h[0][o] = t[0][o] = tv;
+        dz[0][o] = P[o];
+        dh[0][o] = fma(-tv, tv, 1.0) * P[o];
+    }
     int off = 2 * m.emb[0];
     for (int l = 1; l < m.n_emb; ++l) {
         __syncthreads();
         const int win = m.emb[l - 1], wout = m.emb[l], sk = dp_skip_kind(win, wout);
         if (o < wout) {
-            double z = P[off + win * wout + o];
-            for (int p = 0; p < win; ++p) z = fma(h[l - 1][p], P[off + p * wout + o], z);
-            t[l][o] = dp_tanh64(z, m.tanh_tab);
-            h[l][o] = t[l][o] + (sk ? h[l - 1][o < win ? o : o - win] : 0.0);
+            double z = P[off + win * wout + o], d = 0.0;
+            for (int p = 0; p < win; ++p) {
+                const double w = P[off + p * wout + o];
+                z = fma(h[l - 1][p], w, z);
+                d = fma(dh[l - 1][p], w, d);
+            }
+            const double tv = dp_tanh64(z, m.tanh_tab);
+            const int os = o < win ? o : o - win;
+            t[l][o] = tv;
+            dz[l][o] = d;
+            h[l][o] = tv + (sk ? h[l - 1][os] : 0.0);
+            dh[l][o] = fma(fma(-tv, tv, 1.0), d, sk ? dh[l - 1][os] : 0.0);
         }
         off += win * wout + wout;
     }
     if (o < M) {
-        double v = 0.0;
-        for (int n = 0; n < nc; ++n)
-            v = fma(trig[2 * ((n * (2 * k + 1)) % (4 * NN))] * (n == 0 ? 1.0 / NN : 2.0 / NN),
-                    Cb[((size_t)net * NN + n) * M + o], v);
+        double v = 0.0, dv = 0.0;
+        for (int n = nc - 1; n >= 0; --n) {
+            const double w = trig[2 * ((n * (2 * k + 1)) % (4 * NN))] * (n == 0 ? 1.0 / NN : 2.0 / NN);
+            v = fma(w, Cb[((size_t)net * NN + n) * M + o], v);
+            dv = fma(w, Vb[((size_t)net * NN + n) * M + o], dv);
+        }
         g[o] = v;
+        dg[o] = dv;
     }
-    double *hn = node + (size_t)blockIdx.x * 2 * se, *zn = hn + se;
+    double *nd = node + (size_t)blockIdx.x * 4 * se;
     int lo = se;
     for (int l = m.n_emb - 1; l >= 0; --l) {
         __syncthreads();
         const int out = m.emb[l], in = l > 0 ? m.emb[l - 1] : 0;
         lo -= out;
         if (o < out) {
-            zb[o] = fma(-t[l][o], t[l][o], 1.0) * g[o];
-            hn[lo + o] = h[l][o];
-            zn[lo + o] = zb[o];
+            const double one = fma(-t[l][o], t[l][o], 1.0), d = dg[o];
+            dzb[o] = one * d;
+            zb[o] = one * fma(-2.0 * t[l][o] * dz[l][o], d, g[o]);
+            nd[lo + o] = h[l][o];
+            nd[se + lo + o] = dh[l][o];
+            nd[2 * se + lo + o] = zb[o];
+            nd[3 * se + lo + o] = dzb[o];
         }
         __syncthreads();
         if (l > 0) {
             off -= in * out + out;
             const int sk = dp_skip_kind(in, out);
-            double v = 0.0;
+            double v = 0.0, d = 0.0;
             if (o < in) {
-                for (int p = 0; p < out; ++p) v = fma(P[off + o * out + p], zb[p], v);
-                if (sk) v += g[o];
-                if (sk == 2) v += g[o + in];
+                for (int p = 0; p < out; ++p) {
+                    const double w = P[off + o * out + p];
+                    v = fma(w, zb[p], v);
+                    d = fma(w, dzb[p], d);
+                }
+                if (sk) {
+                    v += g[o];
+                    d += dg[o];
+                }
+                if (sk == 2) {
+                    v += g[o + in];
+                    d += dg[o + in];
+                }
             }
             __syncthreads();
-            if (o < in) g[o] = v;
+            if (o < in) {
+                g[o] = v;
+                dg[o] = d;
+            }
         }
     }
 }
 
-// Gradient of every embedding parameter from the nodes' layer outputs and z
-// adjoints: dW[q][o] = sum_k h_k[q] zb_k[o], db[o] = sum_k zb_k[o].
+// Gradient of every embedding parameter from the nodes: dW[q][o] = sum_k h_k[q]
+// zb_k[o] + dh_k[q] dzb_k[o] (layer 0: h = s, dh = 1), db[o] = sum_k zb_k[o].
 __global__ void k_chebpg_grad(DevModel m, const double *__restrict__ trig, const double *__restrict__ node, int se,
                               double *__restrict__ grad, const int32_t *far_flag)
 {
     if (*far_flag) return;
     const int net = blockIdx.y;
-    const double *nd = node + (size_t)net * NN * 2 * se;
+    const double *nd = node + (size_t)net * NN * 4 * se;
     for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < m.emb_net_size; p += gridDim.x * blockDim.x) {
         int l = 0, lo = 0, r = p, in = 1;  // layer, its offset in the node arrays, index in the layer
         while (r >= (in + 1) * m.emb[l]) {
@@ -1036,19 +1104,24 @@ __global__ void k_chebpg_grad(DevModel m, const double *__restrict__ trig, const
             ++l;
         }
         const int out = m.emb[l], q = r / out, o = r - q * out;
-        double v = 0.0;
+        double v = 0.0, w = 0.0;
         for (int k = 0; k < NN; ++k) {
-            const double *hk = nd + (size_t)k * 2 * se, *zk = hk + se;
-            const double hv = q == in ? 1.0 : l == 0 ? (1.0 + trig[2 * (2 * k + 1)]) / DP_CHEB_SCALE : hk[lo - in + q];
-            v = fma(hv, zk[lo + o], v);
+            const double *n = nd + (size_t)k * 4 * se;
+            double hv = 1.0, dv = 0.0;
+            if (q < in) {
+                hv = l == 0 ? (1.0 + trig[2 * (2 * k + 1)]) / DP_CHEB_SCALE : n[lo - in + q];
+                dv = l == 0 ? 1.0 : n[se + lo - in + q];
+            }
+            v = fma(hv, n[2 * se + lo + o], v);
+            w = fma(dv, n[3 * se + lo + o], w);
         }
-        grad[m.emb_base[net] + p] = v;
+        grad[m.emb_base[net] + p] = v + w;
     }
 }
 
 size_t pg_fwd_smem(const DevModel &m, int nc)
 {
-    return sizeof(double) * (2 * CT * 8 + (size_t)m.ntypes * nc * 8 + 8 * m.M + 2 * (size_t)nc * LDT);
+    return sizeof(double) * (2 * CT * PM + (size_t)m.ntypes * nc * PM + 8 * m.M + (size_t)nc * LDT);
 }
 
 size_t pg_tb_smem(const DevModel &m) { return sizeof(double) * (8 * (size_t)m.M + 8 * m.m2 + (size_t)m.m2 * (m.M | 1)); }
@@ -1076,9 +1149,10 @@ size_t dp_cheb_elems(const DevModel &m, int which)
     const size_t nets = (size_t)m.ntypes * m.ntypes;
     switch (which) {
     case 0:
-    case 1: return nets * NN * m.M;
-    case 2: return nets * NN * m.M * 2;
-    case 3: return nets * NN;
+    case 1:
+    case 2: return nets * NN * m.M;
+    case 3: return nets * NN * m.M * 2;
+    case 4: return nets * NN;
     default: return 2 * (4 * NN + DP_CHEB_NTANH);
     }
 }
@@ -1095,7 +1169,8 @@ cudaError_t dp_launch_cheb_build(cudaStream_t st, const DevModel &m, ChebBuffers
     const int grid = m.ntypes * m.ntypes * NN;
     k_cheb_nodes<<<grid, CT, 0, st>>>(m, cb.trig, cb.y);
     k_cheb_coef<<<grid, CT, 0, st>>>(m, cb.trig, cb.y, cb.C, cb.Ct, cb.mx);
-    *launches += 2;
+    k_cheb_deriv<<<grid, CT, 0, st>>>(m, cb.C, cb.V);
+    *launches += 3;
     return cudaGetLastError();
 }
 
@@ -1154,9 +1229,9 @@ size_t dp_cheb_grad_elems(const DevModel &m, int n, int64_t natoms, int which)
     size_t se = 0;
     for (int l = 0; l < m.n_emb; ++l) se += m.emb[l];
     switch (which) {
-    case 0: return (size_t)natoms * m.ntypes * n * 8;
-    case 1: return DP_CHEB_SPLITS * nets * NN * m.M;
-    default: return nets * NN * 2 * se;
+    case 0: return (size_t)natoms * m.ntypes * n * PM;
+    case 1: return (size_t)dp_cheb_splits(m.ntypes) * 2 * nets * NN * m.M;
+    default: return nets * NN * 4 * se;
     }
 }
 
@@ -1183,16 +1258,16 @@ cudaError_t dp_launch_chebpg_bwd(cudaStream_t st, const DevModel &m, const ChebM
     int se = 0;
     for (int l = 0; l < m.n_emb; ++l) se += m.emb[l];
     cudaError_t e = cudaFuncSetAttribute(k_chebpg_tb, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_MAX);
-    const size_t csm = sizeof(double) * CBA * 8 * (CBK + (size_t)m.M);
+    const size_t csm = sizeof(double) * CBA * (PM * CBK + 8 * (size_t)m.M);
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(k_chebpg_cb, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)csm);
     if (e != cudaSuccess) return e;
     k_chebpg_tb<<<N, CT, pg_tb_smem(m), st>>>(m, eb.T, pb.dT, pb.Db, pb.dDb, gb.far);
-    k_chebpg_cb<<<dim3(DP_CHEB_SPLITS, T, (Kt + CBK - 1) / CBK), CT, csm, st>>>(
+    k_chebpg_cb<<<dim3(dp_cheb_splits(T), T, (Kt + CBK - 1) / CBK), CT, csm, st>>>(
         m, cm.n, nb.type_perm, nb.type_start, gb.mom, eb.T, pb.dT, gb.part, gb.far);
-    const size_t elems = (size_t)T * T * NN * m.M;
-    k_chebpg_sum<<<(int)((elems + 255) / 256), 256, 0, st>>>(gb.part, elems, DP_CHEB_SPLITS, gb.far);
-    k_chebpg_node<<<T * T * NN, CT, 0, st>>>(m, cm.n, trig, gb.part, gb.node, se, gb.far);
+    const size_t elems = 2 * (size_t)T * T * NN * m.M;
+    k_chebpg_sum<<<(int)((elems + 255) / 256), 256, 0, st>>>(gb.part, elems, dp_cheb_splits(T), gb.far);
+    k_chebpg_node<<<T * T * NN, CT, 0, st>>>(m, cm.n, trig, gb.part, gb.part + elems / 2, gb.node, se, gb.far);
     k_chebpg_grad<<<dim3((m.emb_net_size + 255) / 256, T * T), 256, 0, st>>>(m, trig, gb.node, se, grad, gb.far);
     *launches += 5;
     return cudaGetLastError();
