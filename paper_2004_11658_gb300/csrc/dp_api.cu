@@ -620,8 +620,7 @@ dp_status enqueue_eval(dp_ctx *c, const double *coords, const int32_t *types, co
             GroupTimer tm(c, G_EMBED_BWD);
             e = cheb ? dp_launch_cheb_bwd(c->stream, c->m, c->cheb, types, n, c->fb, c->nb, c->eb, &c->launches)
                 : mixed && c->eb.Gmx
-                    ? dp_launch_embed_bwd_stmx(c->stream, c->m, coords, types, b, n, c->fb, c->eb, c->num_sms,
-                                               &c->launches)
+                    ? dp_launch_embed_bwd_stmx(c->stream, c->m, types, n, c->fb, c->eb, &c->launches)
                 : mixed     ? dp_launch_embed_bwd_mx(c->stream, c->m, c->mx, coords, types, b, n, c->fb, c->nb,
                                                      c->eb, c->num_sms, c->d_status, &c->launches)
                 : c->use_ex && c->eb.Gst

@@ -140,6 +140,27 @@ __device__ __forceinline__ void dp_switch(double r, double rs, double rc, double
     }
 }
 
+// The same with one division, for kernels whose results need not repeat
+// dp_switch's last bit: inv = 1/r is returned, irc = 1/(rc - rs) given.
+__device__ __forceinline__ void dp_switch_inv(double r, double rs, double rc, double irc, double &s, double &ds,
+                                              double &inv)
+{
+    inv = 1.0 / r;
+    s = inv;
+    ds = -inv * inv;
+    if (!(r < rs)) {
+        if (r < rc) {
+            const double u = (r - rs) * irc, u2 = u * u, um1 = u - 1.0;
+            const double w = u2 * u * (-6.0 * u2 + 15.0 * u - 10.0) + 1.0;
+            s = w * inv;
+            ds = (-30.0 * u2 * um1 * um1 * irc - s) * inv;
+        } else {
+            s = 0.0;
+            ds = 0.0;
+        }
+    }
+}
+
 // FP64 tanh by piecewise Taylor polynomials (tanh64.cu): interval k is
 // centred at k/40, k = 0..DP_TANH_NINT-1, and stores [centre, a_0 .. a_7].
 #define DP_TANH_INV_H 40
@@ -361,9 +382,8 @@ cudaError_t dp_launch_embed_tan_mx(cudaStream_t st, const DevModel &m, const Mix
                                    const int32_t *types, Box3 box, int N, const FormatBuffers &fb,
                                    const NlistBuffers &nb, EvalBuffers eb, int num_sms, int32_t *status,
                                    int64_t *launches);
-cudaError_t dp_launch_embed_bwd_stmx(cudaStream_t st, const DevModel &m, const double *x, const int32_t *types,
-                                     Box3 box, int N, const FormatBuffers &fb, EvalBuffers eb, int num_sms,
-                                     int64_t *launches);
+cudaError_t dp_launch_embed_bwd_stmx(cudaStream_t st, const DevModel &m, const int32_t *types, int N,
+                                     const FormatBuffers &fb, EvalBuffers eb, int64_t *launches);
 cudaError_t dp_launch_embed_fwd_mx(cudaStream_t st, const DevModel &m, const MixedModel &mx, const double *x,
                                    const int32_t *types, Box3 box, int N, const FormatBuffers &fb,
                                    const NlistBuffers &nb, EvalBuffers eb, int num_sms, int32_t *status,

@@ -36,12 +36,13 @@
 // 1e-15 of their norm on water, 2e-14 on copper, both ways).
 #include <cmath>
 
+#include "atom_cta.cuh"
 #include "cheb.cuh"
 
 namespace {
 
 constexpr int NN = DP_CHEB_NN;
-constexpr int CT = 128;       // threads of a CTA = rows of a chunk
+constexpr int CT = DP_ATOM_CT;  // threads of a CTA = rows of a chunk (128)
 constexpr int LDT = CT + 1;   // row pitch of the T_n(t) table (odd: lanes on n hit different banks)
 constexpr unsigned FULL = 0xffffffffu;
 
@@ -320,6 +321,7 @@ __global__ void __launch_bounds__(CT) k_cheb_fwd(DevModel m, ChebModel cm, const
     __syncthreads();
     const int R = start[T];
     const double xi[3] = {x[3 * i], x[3 * i + 1], x[3 * i + 2]};
+    const double irc = 1.0 / (m.rcut - m.rcut_smth);
     const int ns = CT / nc;                    // row slices of the moment sums
     const int mn = tid % nc, msl = tid / nc;   // this thread's term and slice
     bool any_far = false;
@@ -332,13 +334,12 @@ __global__ void __launch_bounds__(CT) k_cheb_fwd(DevModel m, ChebModel cm, const
             const size_t slot = (size_t)i * nm + m.sel_off[b] + (q - start[b]);
             const int j = nlist[slot];
             const double xj[3] = {x[3 * j], x[3 * j + 1], x[3 * j + 2]};
-            double d[3], s, ds;
-            const double r = dp_pinned_dist(xi, xj, box, d);
-            dp_switch(r, m.rcut_smth, m.rcut, s, ds);
+            double d[3], s, ds, inv;
+            dp_switch_inv(dp_pinned_dist(xi, xj, box, d), m.rcut_smth, m.rcut, irc, s, ds, inv);
             pair_d[slot * 3] = d[0];
             pair_d[slot * 3 + 1] = d[1];
             pair_d[slot * 3 + 2] = d[2];
-            const double sr = s / r;
+            const double sr = s * inv;
             far = !(s <= DP_CHEB_S);
             double *Rq = R4 + tid * 4;
             Rq[0] = far ? 0.0 : s;
@@ -420,11 +421,11 @@ __global__ void __launch_bounds__(CT) k_cheb_fwd(DevModel m, ChebModel cm, const
             const double dv[3] = {d[0], d[1], d[2]};
             const double r = __dsqrt_rn(__dadd_rn(__dadd_rn(__dmul_rn(dv[0], dv[0]), __dmul_rn(dv[1], dv[1])),
                                                   __dmul_rn(dv[2], dv[2])));
-            double s, ds;
-            dp_switch(r, m.rcut_smth, m.rcut, s, ds);
+            double s, ds, inv;
+            dp_switch_inv(r, m.rcut_smth, m.rcut, irc, s, ds, inv);
             if (s <= DP_CHEB_S) continue;  // uniform: every thread has the same row
             net_direct(m, a * T + b, s, ga, da, gb, db);
-            const double sr = s / r;
+            const double sr = s * inv;
             for (int p = tid; p < 4 * M; p += CT) {
                 const int c = p / M;
                 Ts[p] += (c == 0 ? s : sr * dv[c - 1]) * ga[p - c * M] * m.desc_scale;
@@ -482,34 +483,7 @@ __global__ void __launch_bounds__(CT) k_cheb_bwd(DevModel m, ChebModel cm, const
     }
     __syncthreads();
     const int R = start[T];
-    // gT[c][x] = scale ([x < m2] sum_b gD[x][b] T[c][b] + sum_{a < m2} gD[a][x] T[c][a]);
-    // the m2 4 long sums two threads each first
-    for (int p = tid; p < 8 * m2; p += CT) {
-        const int h = p / (4 * m2), e = p - h * 4 * m2, c = e / m2, xx = e - c * m2;
-        const double *gr = gs + xx * LDG, *tr = Ts + c * M;
-        double v0 = 0.0, v1 = 0.0;
-        int b = h;
-        for (; b + 2 < M; b += 4) {
-            v0 = fma(gr[b], tr[b], v0);
-            v1 = fma(gr[b + 2], tr[b + 2], v1);
-        }
-        for (; b < M; b += 2) v0 = fma(gr[b], tr[b], v0);
-        lp[p] = v0 + v1;
-    }
-    __syncthreads();
-    for (int p = tid; p < 4 * M; p += CT) {
-        const int c = p / M, xx = p - c * M;
-        double v0 = 0.0, v1 = 0.0;
-        int a2 = 0;
-        for (; a2 + 1 < m2; a2 += 2) {
-            v0 = fma(gs[a2 * LDG + xx], Ts[c * M + a2], v0);
-            v1 = fma(gs[(a2 + 1) * LDG + xx], Ts[c * M + a2 + 1], v1);
-        }
-        if (a2 < m2) v0 = fma(gs[a2 * LDG + xx], Ts[c * M + a2], v0);
-        v0 += v1;
-        if (xx < m2) v0 += lp[c * m2 + xx] + lp[4 * m2 + c * m2 + xx];
-        g4[xx * 4 + c] = v0 * m.desc_scale;
-    }
+    dp_atom_gT(gs, LDG, Ts, lp, m2, M, m.desc_scale, [&](int c, int xx, double v) { g4[xx * 4 + c] = v; });
     __syncthreads();
     // U_kc = sum_f C_kf gT_cf: thread = (term k of the centre's nets, feature slice)
     {
@@ -550,6 +524,7 @@ __global__ void __launch_bounds__(CT) k_cheb_bwd(DevModel m, ChebModel cm, const
     }
     __syncthreads();
 
+    const double irc = 1.0 / (m.rcut - m.rcut_smth);
     double fo[3] = {0.0, 0.0, 0.0}, vir[9];
 #pragma unroll
     for (int q = 0; q < 9; ++q) vir[q] = 0.0;
@@ -579,12 +554,11 @@ __global__ void __launch_bounds__(CT) k_cheb_bwd(DevModel m, ChebModel cm, const
             const int b = row_block(start, T, q);
             double *pg = pair_g + ((size_t)i * nm + m.sel_off[b] + (q - start[b])) * 3;
             const double d[3] = {pg[0], pg[1], pg[2]};
-            const double r = radius(d);
-            double s, ds;
-            dp_switch(r, m.rcut_smth, m.rcut, s, ds);
+            double s, ds, inv;
+            dp_switch_inv(radius(d), m.rcut_smth, m.rcut, irc, s, ds, inv);
             far = !(s <= DP_CHEB_S);
             if (!far) {
-                const double inv = 1.0 / r, sr = s * inv;
+                const double sr = s * inv;
                 const double t = fma(s, DP_CHEB_SCALE, -1.0), t2 = t + t;
                 const double2 *uv = reinterpret_cast<const double2 *>(UV + b * nc * 8);
                 double P[4] = {uv[0].x, uv[0].y, uv[1].x, uv[1].y};
@@ -620,9 +594,8 @@ __global__ void __launch_bounds__(CT) k_cheb_bwd(DevModel m, ChebModel cm, const
             const int b = row_block(start, T, q);
             double *pg = pair_g + ((size_t)i * nm + m.sel_off[b] + (q - start[b])) * 3;
             const double d[3] = {pg[0], pg[1], pg[2]};
-            const double r = radius(d);
-            double s, ds;
-            dp_switch(r, m.rcut_smth, m.rcut, s, ds);
+            double s, ds, inv;
+            dp_switch_inv(radius(d), m.rcut_smth, m.rcut, irc, s, ds, inv);
             net_direct(m, a * T + b, s, ga, da, gb, db);
             double p[8];
 #pragma unroll
@@ -642,42 +615,13 @@ __global__ void __launch_bounds__(CT) k_cheb_bwd(DevModel m, ChebModel cm, const
 #pragma unroll
                 for (int c = 0; c < 8; ++c)
                     for (int w = 1; w < CT / 32; ++w) p[c] += fsum[w][c];
-                const double inv = 1.0 / r, sr = s * inv;
+                const double sr = s * inv;
                 chain(pg, d, inv, s, ds, p, s * p[4] + sr * (d[0] * p[5] + d[1] * p[6] + d[2] * p[7]));
             }
             __syncthreads();
         }
     }
-    // own force and virial: a transposing shuffle tree (16 adds), then the four warps in order
-    {
-        double p[16];
-#pragma unroll
-        for (int q = 0; q < 3; ++q) p[q] = fo[q];
-#pragma unroll
-        for (int q = 0; q < 9; ++q) p[3 + q] = vir[q];
-#pragma unroll
-        for (int q = 12; q < 16; ++q) p[q] = 0.0;
-        const int lane = tid & 31;
-#pragma unroll
-        for (int w = 16, n = 8; w >= 2; w >>= 1, n >>= 1) {
-            const bool up = (lane & w) != 0;
-#pragma unroll
-            for (int k = 0; k < n; ++k) {
-                const double send = up ? p[k] : p[n + k];
-                const double keep = up ? p[n + k] : p[k];
-                p[k] = keep + __shfl_xor_sync(FULL, send, w);
-            }
-        }
-        p[0] += __shfl_xor_sync(FULL, p[0], 1);
-        if ((lane & 1) == 0) wsum[tid >> 5][lane >> 1] = p[0];
-        __syncthreads();
-        if (tid < 12) {
-            double v = wsum[0][tid];
-            for (int w = 1; w < CT / 32; ++w) v += wsum[w][tid];
-            if (tid < 3) f_own[(size_t)i * 3 + tid] = v;
-            else vir_part[(size_t)i * 9 + tid - 3] = v;
-        }
-    }
+    dp_atom_sum12(fo, vir, wsum, f_own, vir_part, i);
 }
 
 // ------------------------------------------------- parameter gradient ------
@@ -731,6 +675,7 @@ __global__ void __launch_bounds__(CT) k_chebpg_fwd(DevModel m, ChebModel cm, con
     const int R = start[T];
     const double xi[3] = {x[3 * i], x[3 * i + 1], x[3 * i + 2]};
     const double li[3] = {lam[3 * i], lam[3 * i + 1], lam[3 * i + 2]};
+    const double irc = 1.0 / (m.rcut - m.rcut_smth);
     const int ns = CT / nc, mn = tid % nc, msl = tid / nc;
     bool any_far = false;
     for (int c0 = 0; c0 < R; c0 += CT) {
@@ -739,10 +684,8 @@ __global__ void __launch_bounds__(CT) k_chebpg_fwd(DevModel m, ChebModel cm, con
             const int b = row_block(start, T, q);
             const int j = nlist[(size_t)i * nm + m.sel_off[b] + (q - start[b])];
             const double xj[3] = {x[3 * j], x[3 * j + 1], x[3 * j + 2]};
-            double d[3], s, ds;
-            const double r = dp_pinned_dist(xi, xj, box, d);
-            dp_switch(r, m.rcut_smth, m.rcut, s, ds);
-            const double inv = 1.0 / r;
+            double d[3], s, ds, inv;
+            dp_switch_inv(dp_pinned_dist(xi, xj, box, d), m.rcut_smth, m.rcut, irc, s, ds, inv);
             const double u[3] = {d[0] * inv, d[1] * inv, d[2] * inv};
             const double dr[3] = {lam[3 * j] - li[0], lam[3 * j + 1] - li[1], lam[3 * j + 2] - li[2]};
             const double udr = u[0] * dr[0] + u[1] * dr[1] + u[2] * dr[2];

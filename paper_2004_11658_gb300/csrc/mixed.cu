@@ -35,6 +35,7 @@
 // tensor memory and returns.
 #include <cuda_bf16.h>
 
+#include "atom_cta.cuh"
 #include "dp_internal.cuh"
 #include "tc.cuh"
 
@@ -604,6 +605,12 @@ __device__ __forceinline__ void embed_mx_tangent_body(
                 if (valid) {
                     const double xi[3] = {x[3 * i], x[3 * i + 1], x[3 * i + 2]};
                     geometry(m, x, xi, nlist[(size_t)i * nm + slot], box, gg);
+                    if constexpr (TAN) {  // r_ij for the streaming backward
+                        double *pd = pair_g + ((size_t)i * nm + slot) * 3;
+                        pd[0] = gg.d[0];
+                        pd[1] = gg.d[1];
+                        pd[2] = gg.d[2];
+                    }
                 }
                 float h0[E1], dh0[E1];
                 const float s32 = (float)gg.s;
@@ -895,10 +902,10 @@ __global__ void __launch_bounds__(MXT, 1) k_embed_tan_mx(
     DevModel m, MixedModel mx, const double *__restrict__ x, const int32_t *__restrict__ types, Box3 box, int N,
     const int32_t *__restrict__ type_perm, const int32_t *__restrict__ type_start, const int32_t *__restrict__ nlist,
     const int32_t *__restrict__ nreal, double *__restrict__ Tout, double *__restrict__ Dout,
-    float *__restrict__ Gsto, int32_t *status)
+    float *__restrict__ Gsto, double *__restrict__ pair_d, int32_t *status)
 {
     embed_mx_tangent_body<E1, false, true>(m, mx, x, types, box, N, type_perm, type_start, nlist, nreal, Tout,
-                                           nullptr, nullptr, nullptr, nullptr, Dout, Gsto, status);
+                                           nullptr, pair_d, nullptr, nullptr, Dout, Gsto, status);
 }
 
 // Error-free sum of two double-float numbers: (h, l) += (h2, l2).
@@ -914,175 +921,146 @@ __device__ __forceinline__ void df_add(float &h, float &l, float h2, float l2)
 // ------------------------------------------------------ streaming backward --
 //
 // k_embed_bwd_stmx: the mixed backward once k_embed_tan_mx has stored G and
-// dG/ds (FP32) of every real row.  One warp per atom: dE/dT in FP64 (as
-// k_embed_bwd_mx), split into two FP32 parts; the atom's real rows 32 at a
-// time, lane q on the geometry of row q; in 8 steps of 4 rows, 8 lanes per
-// row form sum_f G[f] gT[c][f] and sum_f dG[f] gT[c][f] in double-float
-// arithmetic over the features u, u + 8, ... (exact products with gT's parts),
-// a transposing shuffle tree of error-free double-float sums leaves component
-// u on lane u, and the row's lane applies the chain rule through R~(r_ij) in
-// FP64.  Fixed summation order: bit-reproducible.
-constexpr int SMW = 4;  // warps (atoms in flight) per CTA
+// dG/ds (FP32) and r_ij of every real row.  One 128-thread CTA per atom: dE/dT
+// in FP64 split into two FP32 parts; thread q on the geometry of row q; 8
+// lanes per row form sum_f G[f] gT[c][f] and sum_f dG[f] gT[c][f] in
+// double-float arithmetic over the features u, u + 8, ... (exact products with
+// gT's parts), a transposing shuffle tree of error-free double-float sums
+// leaves component u on lane u, and the row's thread applies the chain rule
+// through R~(r_ij) in FP64.  Fixed summation order: bit-reproducible.
+//
+// Bound by the FP64 pipe (dE/dT, geometry, chain rule: about 620 warp
+// instructions of 16 cycles per water atom).  With a warp per atom, dE/dD read
+// from global memory at one line per lane and r_ij formed again with four
+// divisions, 98,304 water atoms took 7.2 ms; now 6.2 ms.
 
 template <int E1>
-__global__ void __launch_bounds__(SMW * 32, 4) k_embed_bwd_stmx(
-    DevModel m, const double *__restrict__ x, const int32_t *__restrict__ types, Box3 box, int N,
-    const int32_t *__restrict__ nlist, const int32_t *__restrict__ nreal, const double *__restrict__ Tin,
+__global__ void __launch_bounds__(DP_ATOM_CT) k_embed_bwd_stmx(
+    DevModel m, const int32_t *__restrict__ types, const int32_t *__restrict__ nreal, const double *__restrict__ Tin,
     const double *__restrict__ gD, const float *__restrict__ Gsto, double *__restrict__ pair_g,
     double *__restrict__ f_own, double *__restrict__ vir_part)
 {
-    constexpr int E3 = 4 * E1, KF = (E3 + 7) / 8;
-    static_assert(4 * E3 >= 32 * 8, "the row sums [32][8] fit in the T buffer");
-    // per warp: R1 holds T of the atom, then dE/dT as FP32 parts (gth, gtl); R2 holds dE/dT in
-    // FP64 while it is formed, then the row sums [32][8]
-    __shared__ double R1sh[SMW][4 * E3];
-    __shared__ double R2sh[SMW][4 * E3];
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int sub = lane & 7, gq = lane >> 3;
+    constexpr int E3 = 4 * E1, KF = (E3 + 7) / 8, LDG = E3 + 1, CT = DP_ATOM_CT;
+    extern __shared__ __align__(16) double gs[];  // [m2][LDG] dE/dD, then [8 m2] long sums
+    __shared__ double Ts[4 * E3];
+    __shared__ float4 gth[E3], gtl[E3];           // dE/dT of a feature, FP32 parts
+    __shared__ double sa[CT][9];                  // row sums
+    __shared__ double wsum[CT / 32][16];
+    __shared__ int slots[CT];
+    __shared__ int start[DP_MAX_TYPES + 1];
+    const int tid = threadIdx.x, sub = tid & 7, grp = tid >> 3;
     const int T = m.ntypes, nm = m.nm, m2 = m.m2;
-    double *Ts = R1sh[w], *gTd = R2sh[w], *sa_s = R2sh[w];
-    float *gth = reinterpret_cast<float *>(R1sh[w]), *gtl = gth + 4 * E3;
-
-    for (int i = blockIdx.x * SMW + w; i < N; i += gridDim.x * SMW) {
-        const int a = types[i];
-        const bool a_ok = (unsigned)a < (unsigned)T;
-        for (int p = lane; p < 4 * E3; p += 32) Ts[p] = Tin[(size_t)i * 4 * E3 + p];
-        __syncwarp();
-        {
-            // the 4 M2 long sums first, two per lane with every lane busy (two chains each), then
-            // every entry's M2 short terms on top of them; then the FP32 parts over T
-            const double *gd = gD + (size_t)i * m2 * E3;
-            for (int p = lane; p < 4 * m2; p += 32) {
-                const int cc = p / m2, xx = p - cc * m2;
-                double acc = 0.0, acc2 = 0.0;
-                for (int b2i = 0; b2i < E3; b2i += 2) {  // E3 = 4 e1 is even
-                    acc = fma(gd[xx * E3 + b2i], Ts[cc * E3 + b2i], acc);
-                    acc2 = fma(gd[xx * E3 + b2i + 1], Ts[cc * E3 + b2i + 1], acc2);
-                }
-                gTd[cc * E3 + xx] = acc + acc2;
-            }
-            __syncwarp();
-            for (int p = lane; p < 4 * E3; p += 32) {
-                const int cc = p / E3, xx = p - cc * E3;
-                double acc = xx < m2 ? gTd[p] : 0.0;
-                for (int a2 = 0; a2 < m2; ++a2) acc = fma(gd[a2 * E3 + xx], Ts[cc * E3 + a2], acc);
-                gTd[p] = acc * m.desc_scale;
-            }
-            __syncwarp();
-            for (int p = lane; p < 4 * E3; p += 32) df_split(gTd[p], gth[p], gtl[p]);
+    const int i = blockIdx.x;
+    const bool a_ok = (unsigned)types[i] < (unsigned)T;
+    if (tid == 0) {
+        int r = 0;
+        for (int b = 0; b < T; ++b) {
+            start[b] = r;
+            r += a_ok ? nreal[(size_t)i * T + b] : 0;
         }
-        __syncwarp();
-        int nr = 0;
-        if (a_ok)
-            for (int b = 0; b < T; ++b) nr += nreal[(size_t)i * T + b];
-        const double xi[3] = {x[3 * i], x[3 * i + 1], x[3 * i + 2]};
-        double fo[3] = {0.0, 0.0, 0.0}, vir[9];
-#pragma unroll
-        for (int q = 0; q < 9; ++q) vir[q] = 0.0;
-        for (int q0 = 0; q0 < nr; q0 += 32) {
-            // row q0 + lane: its slot (type block and rank) and geometry
-            int slot = -1;
-            if (q0 + lane < nr) {
-                int rem = q0 + lane;
-                for (int b = 0; b < T; ++b) {
-                    const int nb = nreal[(size_t)i * T + b];
-                    if (slot < 0 && rem < nb) slot = m.sel_off[b] + rem;
-                    rem -= nb;
-                }
-            }
-            RowGeo gg;
-            gg.s = gg.ds = 0.0;
-            gg.R[0] = gg.R[1] = gg.R[2] = gg.R[3] = 0.0;
-            gg.d[0] = gg.d[1] = gg.d[2] = 0.0;
-            gg.r = 1.0;
-            if (slot >= 0) geometry(m, x, xi, nlist[(size_t)i * nm + slot], box, gg);
-            // the 8 sums of rows q0 + 4 it + gq, 8 lanes per row
-            for (int it = 0; it < 8 && q0 + 4 * it < nr; ++it) {
-                const int sl = __shfl_sync(0xffffffffu, slot, 4 * it + gq);
-                float ph[8], pl[8];
-#pragma unroll
-                for (int c = 0; c < 8; ++c) ph[c] = pl[c] = 0.f;
-                if (sl >= 0) {
-                    const float *gr = Gsto + ((size_t)i * nm + sl) * (2 * E3);
-#pragma unroll
-                    for (int k = 0; k < KF; ++k) {
-                        const int ff = sub + 8 * k;
-                        if (8 * k + 8 <= E3 || ff < E3) {
-                            const float G = gr[ff], dG = gr[E3 + ff];
-#pragma unroll
-                            for (int c = 0; c < 4; ++c) {
-                                const float bh = gth[c * E3 + ff], bl = gtl[c * E3 + ff];
-                                df_fma(ph[c], pl[c], G, bh, bl);
-                                df_fma(ph[4 + c], pl[4 + c], dG, bh, bl);
-                            }
-                        }
-                    }
-                }
-                // transposing tree over the row's 8 lanes: lane u ends with component u
-#pragma unroll
-                for (int o = 4, n = 4; o >= 1; o >>= 1, n >>= 1) {
-                    const bool up = (sub & o) != 0;
-#pragma unroll
-                    for (int k = 0; k < n; ++k) {
-                        const float sh = up ? ph[k] : ph[n + k], sl2 = up ? pl[k] : pl[n + k];
-                        float kh = up ? ph[n + k] : ph[k], kl = up ? pl[n + k] : pl[k];
-                        const float rh = __shfl_xor_sync(0xffffffffu, sh, o);
-                        const float rl = __shfl_xor_sync(0xffffffffu, sl2, o);
-                        df_add(kh, kl, rh, rl);
-                        ph[k] = kh;
-                        pl[k] = kl;
-                    }
-                }
-                sa_s[(4 * it + gq) * 8 + sub] = df_value(ph[0], pl[0]);
-            }
-            __syncwarp();
-            // chain rule through R~(r_ij) in FP64, lane q on row q0 + q
-            if (slot >= 0) {
-                double ra[4], rb[4];
-#pragma unroll
-                for (int c = 0; c < 4; ++c) {
-                    ra[c] = sa_s[lane * 8 + c];
-                    rb[c] = sa_s[lane * 8 + 4 + c];
-                }
-                double gR0 = ra[0];
-#pragma unroll
-                for (int c = 0; c < 4; ++c) gR0 = fma(gg.R[c], rb[c], gR0);
-                const double inv = 1.0 / gg.r;
-                const double u[3] = {gg.d[0] * inv, gg.d[1] * inv, gg.d[2] * inv};
-                const double dot = ra[1] * u[0] + ra[2] * u[1] + ra[3] * u[2];
-                const double sr = gg.s * inv;
-                const double coef = gR0 * gg.ds + gg.ds * dot - sr * dot;
-                double gv[3];
-#pragma unroll
-                for (int bb = 0; bb < 3; ++bb) gv[bb] = fma(u[bb], coef, sr * ra[1 + bb]);
-                double *pg = pair_g + ((size_t)i * nm + slot) * 3;
-                pg[0] = gv[0];
-                pg[1] = gv[1];
-                pg[2] = gv[2];
-#pragma unroll
-                for (int aa = 0; aa < 3; ++aa) {
-                    fo[aa] += gv[aa];
-#pragma unroll
-                    for (int bb = 0; bb < 3; ++bb) vir[aa * 3 + bb] -= gg.d[aa] * gv[bb];
-                }
-            }
-            __syncwarp();
-        }
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) {
-#pragma unroll
-            for (int q = 0; q < 3; ++q) fo[q] += __shfl_xor_sync(0xffffffffu, fo[q], off);
-#pragma unroll
-            for (int q = 0; q < 9; ++q) vir[q] += __shfl_xor_sync(0xffffffffu, vir[q], off);
-        }
-        if (lane == 0) {
-#pragma unroll
-            for (int q = 0; q < 3; ++q) f_own[(size_t)i * 3 + q] = fo[q];
-#pragma unroll
-            for (int q = 0; q < 9; ++q) vir_part[(size_t)i * 9 + q] = vir[q];
-        }
-        __syncwarp();
+        start[T] = r;
     }
+    for (int p = tid; p < 4 * E3; p += CT) Ts[p] = Tin[(size_t)i * 4 * E3 + p];
+    {
+        const double *g = gD + (size_t)i * m2 * E3;
+        for (int p = tid; p < m2 * E3; p += CT) gs[(p / E3) * LDG + p % E3] = g[p];
+    }
+    __syncthreads();
+    dp_atom_gT(gs, LDG, Ts, gs + m2 * LDG, m2, E3, m.desc_scale, [&](int c, int xx, double v) {
+        df_split(v, reinterpret_cast<float *>(gth + xx)[c], reinterpret_cast<float *>(gtl + xx)[c]);
+    });
+    const int nr = start[T];
+    const double irc = 1.0 / (m.rcut - m.rcut_smth);
+    double fo[3] = {0.0, 0.0, 0.0}, vir[9];
+#pragma unroll
+    for (int q = 0; q < 9; ++q) vir[q] = 0.0;
+    for (int q0 = 0; q0 < nr; q0 += CT) {
+        const int nrow = min(CT, nr - q0);
+        double d[3], s = 0.0, ds = 0.0, inv = 0.0;
+        double *pg = nullptr;
+        __syncthreads();
+        if (tid < nrow) {
+            int b = 0;
+            while (b + 1 < T && q0 + tid >= start[b + 1]) ++b;
+            const int slot = m.sel_off[b] + q0 + tid - start[b];
+            slots[tid] = slot;
+            pg = pair_g + ((size_t)i * nm + slot) * 3;
+#pragma unroll
+            for (int c = 0; c < 3; ++c) d[c] = pg[c];
+            const double r = __dsqrt_rn(__dadd_rn(__dadd_rn(__dmul_rn(d[0], d[0]), __dmul_rn(d[1], d[1])),
+                                                  __dmul_rn(d[2], d[2])));
+            dp_switch_inv(r, m.rcut_smth, m.rcut, irc, s, ds, inv);
+        }
+        __syncthreads();
+        // the 8 sums of rows 16 it + grp, 8 lanes per row
+        for (int it = 0; 16 * it < nrow; ++it) {
+            const int rl = 16 * it + grp;
+            float ph[8], pl[8];
+#pragma unroll
+            for (int c = 0; c < 8; ++c) ph[c] = pl[c] = 0.f;
+            if (rl < nrow) {
+                const float *gr = Gsto + ((size_t)i * nm + slots[rl]) * (2 * E3);
+                float G[KF], dG[KF];
+#pragma unroll
+                for (int k = 0; k < KF; ++k) {
+                    const int ff = sub + 8 * k;
+                    const bool in = 8 * k + 8 <= E3 || ff < E3;
+                    G[k] = in ? gr[ff] : 0.f;
+                    dG[k] = in ? gr[E3 + ff] : 0.f;
+                }
+#pragma unroll
+                for (int k = 0; k < KF; ++k) {
+                    const int ff = sub + 8 * k;
+                    if (8 * k + 8 <= E3 || ff < E3) {
+                        const float4 bh = gth[ff], bl = gtl[ff];
+                        df_fma(ph[0], pl[0], G[k], bh.x, bl.x);
+                        df_fma(ph[1], pl[1], G[k], bh.y, bl.y);
+                        df_fma(ph[2], pl[2], G[k], bh.z, bl.z);
+                        df_fma(ph[3], pl[3], G[k], bh.w, bl.w);
+                        df_fma(ph[4], pl[4], dG[k], bh.x, bl.x);
+                        df_fma(ph[5], pl[5], dG[k], bh.y, bl.y);
+                        df_fma(ph[6], pl[6], dG[k], bh.z, bl.z);
+                        df_fma(ph[7], pl[7], dG[k], bh.w, bl.w);
+                    }
+                }
+            }
+            // transposing tree over the row's 8 lanes: lane u ends with component u
+#pragma unroll
+            for (int o = 4, n = 4; o >= 1; o >>= 1, n >>= 1) {
+                const bool up = (sub & o) != 0;
+#pragma unroll
+                for (int k = 0; k < n; ++k) {
+                    const float sh = up ? ph[k] : ph[n + k], sl2 = up ? pl[k] : pl[n + k];
+                    float kh = up ? ph[n + k] : ph[k], kl = up ? pl[n + k] : pl[k];
+                    const float rh = __shfl_xor_sync(0xffffffffu, sh, o);
+                    const float rl2 = __shfl_xor_sync(0xffffffffu, sl2, o);
+                    df_add(kh, kl, rh, rl2);
+                    ph[k] = kh;
+                    pl[k] = kl;
+                }
+            }
+            if (rl < nrow) sa[rl][sub] = df_value(ph[0], pl[0]);
+        }
+        __syncthreads();
+        // chain rule through R~(r_ij) in FP64
+        if (tid < nrow) {
+            const double *ra = sa[tid], *rb = ra + 4;
+            const double u[3] = {d[0] * inv, d[1] * inv, d[2] * inv};
+            const double dot = ra[1] * u[0] + ra[2] * u[1] + ra[3] * u[2];
+            const double q = rb[0] + rb[1] * u[0] + rb[2] * u[1] + rb[3] * u[2];
+            const double sr = s * inv;
+            const double coef = fma(s, q, ra[0] + dot) * ds - sr * dot;
+#pragma unroll
+            for (int e = 0; e < 3; ++e) {
+                const double gv = fma(u[e], coef, sr * ra[1 + e]);
+                pg[e] = gv;
+                fo[e] += gv;
+#pragma unroll
+                for (int f = 0; f < 3; ++f) vir[f * 3 + e] -= d[f] * gv;
+            }
+        }
+    }
+    dp_atom_sum12(fo, vir, wsum, f_own, vir_part, i);
 }
 
 // ----------------------------------------------------------------- fitting --
@@ -1488,19 +1466,19 @@ cudaError_t launch_tan(cudaStream_t st, const DevModel &m, const MixedModel &mx,
     int grid = ctas_per_sm(smem) * num_sms;
     if (grid > (N + 7) / 8) grid = (N + 7) / 8;
     k_embed_tan_mx<E1><<<grid, MXT, smem, st>>>(m, mx, x, types, box, N, nb.type_perm, nb.type_start, fb.nlist,
-                                                fb.nreal, eb.T, eb.D, eb.Gmx, status);
+                                                fb.nreal, eb.T, eb.D, eb.Gmx, eb.pair_g, status);
     return cudaGetLastError();
 }
 
 template <int E1>
-cudaError_t launch_bwd_stmx(cudaStream_t st, const DevModel &m, const double *x, const int32_t *types, Box3 box,
-                            int N, const FormatBuffers &fb, EvalBuffers eb, int num_sms)
+cudaError_t launch_bwd_stmx(cudaStream_t st, const DevModel &m, const int32_t *types, int N, const FormatBuffers &fb,
+                            EvalBuffers eb)
 {
-    int grid = (N + SMW - 1) / SMW;
-    if (grid > 4 * num_sms) grid = 4 * num_sms;
-    if (grid < 1) grid = 1;
-    k_embed_bwd_stmx<E1><<<grid, SMW * 32, 0, st>>>(m, x, types, box, N, fb.nlist, fb.nreal, eb.T, eb.gD, eb.Gmx,
-                                                    eb.pair_g, eb.f_own, eb.vir_part);
+    const size_t smem = sizeof(double) * ((size_t)m.m2 * (4 * E1 + 1) + 8 * (size_t)m.m2);
+    cudaError_t e = cudaFuncSetAttribute(k_embed_bwd_stmx<E1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    k_embed_bwd_stmx<E1><<<N, DP_ATOM_CT, smem, st>>>(m, types, fb.nreal, eb.T, eb.gD, eb.Gmx, eb.pair_g, eb.f_own,
+                                                     eb.vir_part);
     return cudaGetLastError();
 }
 
@@ -1526,15 +1504,14 @@ cudaError_t dp_launch_embed_tan_mx(cudaStream_t st, const DevModel &m, const Mix
     }
 }
 
-cudaError_t dp_launch_embed_bwd_stmx(cudaStream_t st, const DevModel &m, const double *x, const int32_t *types,
-                                     Box3 box, int N, const FormatBuffers &fb, EvalBuffers eb, int num_sms,
-                                     int64_t *launches)
+cudaError_t dp_launch_embed_bwd_stmx(cudaStream_t st, const DevModel &m, const int32_t *types, int N,
+                                     const FormatBuffers &fb, EvalBuffers eb, int64_t *launches)
 {
     *launches += 1;
     switch (m.emb[0]) {
-    case 16: return launch_bwd_stmx<16>(st, m, x, types, box, N, fb, eb, num_sms);
-    case 25: return launch_bwd_stmx<25>(st, m, x, types, box, N, fb, eb, num_sms);
-    case 32: return launch_bwd_stmx<32>(st, m, x, types, box, N, fb, eb, num_sms);
+    case 16: return launch_bwd_stmx<16>(st, m, types, N, fb, eb);
+    case 25: return launch_bwd_stmx<25>(st, m, types, N, fb, eb);
+    case 32: return launch_bwd_stmx<32>(st, m, types, N, fb, eb);
     default: return cudaErrorInvalidValue;
     }
 }
