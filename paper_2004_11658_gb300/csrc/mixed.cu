@@ -133,6 +133,25 @@ __device__ __forceinline__ void df_split(double v, float &h, float &l)
 
 __device__ __forceinline__ double df_value(float h, float l) { return (double)h + (double)l; }
 
+// Conversions between FP32 and FP64 on the integer pipe (the FP64 pipe takes 16
+// cycles per warp instruction, conversions included): exact, and rounded to
+// nearest even, for normal FP32 results; zero, subnormal and non-finite values
+// take the instruction.
+__device__ __forceinline__ double f2d(float v)
+{
+    const uint32_t u = __float_as_uint(v), e = (u >> 23) & 0xff;
+    if (e == 0 || e == 0xff) return (u << 1) == 0 ? __hiloint2double((int)u, 0) : (double)v;
+    return __hiloint2double((int)((u & 0x80000000u) | (((u >> 3) & 0x0fffffffu) + 0x38000000u)), (int)(u << 29));
+}
+__device__ __forceinline__ float d2f(double v)
+{
+    const unsigned long long b = (unsigned long long)__double_as_longlong(v);
+    const unsigned long long r = b + 0x0fffffffull + ((b >> 29) & 1ull);
+    const uint32_t e = (uint32_t)(r >> 52) & 0x7ff;
+    if (e < 897 || e > 1150) return (b << 1) == 0 ? __uint_as_float((uint32_t)(b >> 32)) : (float)v;
+    return __uint_as_float(((uint32_t)(b >> 32) & 0x80000000u) | ((e - 896) << 23) | ((uint32_t)(r >> 29) & 0x7fffffu));
+}
+
 __device__ __forceinline__ void copy16(unsigned char *dst, const unsigned char *__restrict__ src, int bytes)
 {
     for (int q = threadIdx.x * 16; q < bytes; q += blockDim.x * 16)
@@ -1118,8 +1137,12 @@ __global__ void __launch_bounds__(256) k_d2bf(const double *__restrict__ D, int 
     }
 }
 
-// One CTA = one tile of up to 128 atoms of one type.
-__global__ void __launch_bounds__(MXT, 1) k_fit_mx(DevModel m, MixedModel mx, int N,
+// One CTA = one tile of up to 128 atoms of one type; 16 warps, warp w on the rows
+// 32 (w % 4) .. + 31 and every fourth 16-column slice: the epilogues are chains of
+// tensor-memory, tanh and L2 accesses, with 4 warps 510 us per tile
+// (98,304 water atoms: k_d2bf and k_fit_mx 3.40 ms, now 1.4 ms).
+constexpr int FIT_TH = 512;
+__global__ void __launch_bounds__(FIT_TH, 1) k_fit_mx(DevModel m, MixedModel mx, int N,
                                                    const int32_t *__restrict__ type_perm,
                                                    const int32_t *__restrict__ type_start,
                                                    const double *__restrict__ D, double *__restrict__ Ei,
@@ -1130,14 +1153,15 @@ __global__ void __launch_bounds__(MXT, 1) k_fit_mx(DevModel m, MixedModel mx, in
     unsigned char *Ab = smraw;                               // [FIT_NS][128][64] bf16 (layer-1 input chunks)
     unsigned char *Bb = Ab + FIT_NS * MXT * FIT_KC * 2;      // [FIT_NS][256][64] bf16 (weight chunks)
     unsigned char *Hb = Bb + FIT_NS * 256 * FIT_KC * 2;      // [128][256] bf16 (activation / gradient)
-    static_assert(MXT * 17 * sizeof(double) <= FIT_NS * MXT * FIT_KC * 2, "the dE/dD staging fits in the A ring");
+    static_assert(FIT_TH * 17 * sizeof(float) <= FIT_NS * MXT * FIT_KC * 2, "the dE/dD staging fits in the A ring");
     __shared__ __align__(8) uint64_t full[FIT_NS], empty[FIT_NS], dbar;
     __shared__ uint32_t tslot;
     __shared__ int pfail;
     __shared__ int rows_atom[MXT];
     constexpr int HK = 256;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    (void)lane;
+    __shared__ double epart[4][MXT];
+    const int tid = threadIdx.x, lane = tid & 31, warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
+    const int row = 32 * (warp & 3) + lane, slice = warp >> 2;  // this thread's row and column slice
     const int M = m.M, K1 = m.m2 * M, nf = m.n_fit;
 
     int bid = blockIdx.x, a = -1, first = 0, cnt = 0;
@@ -1163,25 +1187,25 @@ __global__ void __launch_bounds__(MXT, 1) k_fit_mx(DevModel m, MixedModel mx, in
         tc::mbar_init(&dbar, 1);
         pfail = 0;
     }
-    int ctr = 0;         // chunks issued so far (thread 0)
+    int ctr = 0;         // chunks issued so far (warp 0)
     uint32_t dph = 0;    // parity of the next completion of dbar
-    rows_atom[tid] = tid < cnt ? type_perm[first + tid] : -1;
+    if (tid < MXT) rows_atom[tid] = tid < cnt ? type_perm[first + tid] : -1;
     tc_sync();
-    const uint32_t tbase = tslot;
-    const uint32_t tlane = tbase + ((uint32_t)(32 * warp) << 16);
-    const int my = rows_atom[tid];
-    const bool warp_live = 32 * warp < cnt;
+    const uint32_t tbase = __shfl_sync(0xffffffffu, tslot, 0);
+    const uint32_t tlane = tbase + ((uint32_t)(32 * (warp & 3)) << 16);
+    const int my = rows_atom[row];
+    const bool warp_live = 32 * (warp & 3) < cnt;
     bool alive = true;
     const float *P32 = mx.p32 + m.fit_base[a];
     // per-tile activation buffers, column-major over the tile's 128 rows so that a warp's
     // accesses are contiguous: t of layer l, feature n at tb[(l HK + n) MXT]; h at hb[n MXT]
-    float *tb = tbuf + (size_t)tile_id * nf * HK * MXT + tid;
-    float *hb = hbuf + (size_t)tile_id * HK * MXT + tid;
+    float *tb = tbuf + (size_t)tile_id * nf * HK * MXT + row;
+    float *hb = hbuf + (size_t)tile_id * HK * MXT + row;
 
     // Streamed GEMM into TMEM columns [0, Np): K-chunks of FIT_KC.  B (weights,
     // K-chunked, chunk kc at Bsrc + kc * chunk_bytes + row_off_bytes) always comes
     // by bulk copy; A is the layer-1 input (the descriptor's BF16 tile, bulk
-    // copy) or the resident activation Hb.  One thread runs a FIT_NS-stage ring:
+    // copy) or the resident activation Hb.  Warp 0 (one elected lane issues) runs a FIT_NS-stage ring:
     // wait for the chunk, issue its MMAs, release the stage by commit, refill the
     // stage of the previous chunk.  Chunks are numbered across calls (ctr) so the
     // barrier parities stay consistent; every call ends with all MMAs complete.
@@ -1191,28 +1215,30 @@ __global__ void __launch_bounds__(MXT, 1) k_fit_mx(DevModel m, MixedModel mx, in
         const uint32_t idesc = tc::make_idesc_bf16(MXT, Np);
         const uint32_t bbytes = (uint32_t)Np * FIT_KC * 2;
         const uint32_t abytes = from_D ? (uint32_t)MXT * FIT_KC * 2 : 0u;
-        if (tid == 0) {
+        if (warp == 0) {
             const int c0 = ctr;
             int issued = 0, consumed = 0;
             auto load = [&](int c) {
                 const int s = c % FIT_NS, kc = c - c0;
-                mbar_expect_tx_mx(&full[s], abytes + bbytes);
-                bulk_g2s_mx(Bb + (size_t)s * 256 * FIT_KC * 2, Bsrc + kc * chunk_bytes + row_off_bytes, bbytes,
-                            &full[s]);
-                if (from_D)
-                    bulk_g2s_mx(Ab + (size_t)s * MXT * FIT_KC * 2, dtile + (size_t)kc * MXT * FIT_KC * 2, abytes,
+                __syncwarp();
+                if (tc::elect_one()) {
+                    mbar_expect_tx_mx(&full[s], abytes + bbytes);
+                    bulk_g2s_mx(Bb + (size_t)s * 256 * FIT_KC * 2, Bsrc + kc * chunk_bytes + row_off_bytes, bbytes,
                                 &full[s]);
+                    if (from_D)
+                        bulk_g2s_mx(Ab + (size_t)s * MXT * FIT_KC * 2, dtile + (size_t)kc * MXT * FIT_KC * 2, abytes,
+                                    &full[s]);
+                }
                 ++issued;
             };
             for (int c = c0; c < c0 + FIT_NS && c < c0 + nK; ++c) load(c);
             bool ok = true;
             for (int c = c0; c < c0 + nK; ++c) {
                 const int s = c % FIT_NS, kc = c - c0;
-                if (!tc::mbar_wait(&full[s], (c / FIT_NS) & 1)) {
-                    ok = false;
-                    break;
-                }
+                ok = __all_sync(0xffffffffu, tc::mbar_wait(&full[s], (c / FIT_NS) & 1));
+                if (!ok) break;
                 ++consumed;
+                if (tc::elect_one()) {
 #pragma unroll
                 for (int kk = 0; kk < FIT_KC / 16; ++kk) {
                     const uint64_t ad =
@@ -1223,17 +1249,18 @@ __global__ void __launch_bounds__(MXT, 1) k_fit_mx(DevModel m, MixedModel mx, in
                     tc::mma_bf16(tbase, ad, bd, idesc, kc > 0 || kk > 0);
                 }
                 tc::mma_commit(&empty[s]);
+                }
+                __syncwarp();
                 if (c - 1 >= c0 && c - 1 + FIT_NS < c0 + nK) {
                     const int ps = (c - 1) % FIT_NS;
-                    if (!tc::mbar_wait(&empty[ps], ((c - 1) / FIT_NS) & 1)) {
-                        ok = false;
-                        break;
-                    }
+                    ok = __all_sync(0xffffffffu, tc::mbar_wait(&empty[ps], ((c - 1) / FIT_NS) & 1));
+                    if (!ok) break;
                     load(c - 1 + FIT_NS);
                 }
             }
-            tc::mma_commit(&dbar);
-            if (!ok) {
+            if (tc::elect_one()) tc::mma_commit(&dbar);
+            __syncwarp();
+            if (!ok && lane == 0) {
                 atomicOr(status, DPF_MMA_TIMEOUT);
                 for (int c = c0 + consumed; c < c0 + issued; ++c) tc::mbar_wait(&full[c % FIT_NS], (c / FIT_NS) & 1);
                 pfail = 1;
@@ -1269,8 +1296,15 @@ __global__ void __launch_bounds__(MXT, 1) k_fit_mx(DevModel m, MixedModel mx, in
         }
         const float *bias = P32 + boff;
         if (warp_live) {
-            for (int cc = 0; cc < Np; cc += 16) {
-                float v[16];
+            for (int cc = 16 * slice; cc < Np; cc += 64) {
+                float v[16], hp[16];
+                if (my >= 0 && l > 0) {  // equal-width skip after the first layer (widths are multiples of 16)
+#pragma unroll
+                    for (int q = 0; q < 16; ++q) hp[q] = hb[(cc + q) * MXT];
+                } else {
+#pragma unroll
+                    for (int q = 0; q < 16; ++q) hp[q] = 0.f;
+                }
                 tc::tmem_ld16(tlane + cc, v);
                 if (my >= 0) {
 #pragma unroll
@@ -1279,19 +1313,21 @@ __global__ void __launch_bounds__(MXT, 1) k_fit_mx(DevModel m, MixedModel mx, in
                         if (n < F) {
                             const float t = tanhf(v[q] + bias[n]);
                             tb[(l * HK + n) * MXT] = t;
-                            hb[n * MXT] = (l > 0 ? hb[n * MXT] : 0.f) + t;  // equal-width skip after the first layer
+                            hb[n * MXT] = hp[q] + t;
                         }
                     }
                 }
+                __syncwarp();
             }
         }
         __syncthreads();
         // next layer's A operand (bf16, zero-padded to 256)
-        for (int k8 = 0; k8 < HK; k8 += 8) {
+#pragma unroll 2
+        for (int k8 = 8 * slice; k8 < HK; k8 += 32) {
             float v[8];
 #pragma unroll
             for (int q = 0; q < 8; ++q) v[q] = (my >= 0 && k8 + q < F) ? hb[(k8 + q) * MXT] : 0.f;
-            st8(Hb, tid, k8, HK, v);
+            st8(Hb, row, k8, HK, v);
         }
         tc_sync();
         Kin = F;
@@ -1307,19 +1343,25 @@ __global__ void __launch_bounds__(MXT, 1) k_fit_mx(DevModel m, MixedModel mx, in
         }
         wo = P32 + off;
     }
-    if (alive && my >= 0) {
-        double e = (double)wo[Kin];
-        for (int n = 0; n < Kin; ++n) e = fma((double)hb[n * MXT], (double)wo[n], e);
-        Ei[my] = e;
+    {
+        double e = 0.0;
+        if (alive && my >= 0)
+            for (int n = slice; n < Kin; n += 4) e = fma(f2d(hb[n * MXT]), f2d(wo[n]), e);
+        epart[slice][row] = e;
+        __syncthreads();
+        if (alive && my >= 0 && slice == 0)
+            Ei[my] = ((f2d(wo[Kin]) + e) + epart[1][row]) + (epart[2][row] + epart[3][row]);
     }
 
     // ---------------- backward: gh = w_out; gz_l = gh * (1 - t_l^2)
     if (my >= 0)
-        for (int n = 0; n < Kin; ++n) hb[n * MXT] = wo[n];
+        for (int n = slice; n < Kin; n += 4) hb[n * MXT] = wo[n];
+    __syncthreads();
     for (int l = nf - 1; l >= 0 && alive; --l) {
         const int F = m.fit[l];
         const int Kl = (l == 0) ? K1 : m.fit[l - 1];
-        for (int k8 = 0; k8 < HK; k8 += 8) {
+#pragma unroll 2
+        for (int k8 = 8 * slice; k8 < HK; k8 += 32) {
             float v[8];
 #pragma unroll
             for (int q = 0; q < 8; ++q) {
@@ -1331,7 +1373,7 @@ __global__ void __launch_bounds__(MXT, 1) k_fit_mx(DevModel m, MixedModel mx, in
                 }
                 v[q] = gz;
             }
-            st8(Hb, tid, k8, HK, v);
+            st8(Hb, row, k8, HK, v);
         }
         tc_sync();
         const int nK = mx.fit_fp[l] / FIT_KC;
@@ -1344,35 +1386,39 @@ __global__ void __launch_bounds__(MXT, 1) k_fit_mx(DevModel m, MixedModel mx, in
             alive = gemm(false, nK, Bsrc, (int64_t)Kinp * 128, (int64_t)(n0 / 8) * 1024, nb);
             if (!alive) break;
             if (l == 0) {
-                // dE/dD through shared memory (the A ring is idle in the backward), 16 columns at
-                // a time, so that each half-warp stores 128 contiguous bytes of one atom's row
-                double *stage = reinterpret_cast<double *>(Ab);  // [MXT][17]
-                for (int cc = 0; cc < nb; cc += 16) {
-                    if (warp_live) {
+                // dE/dD through the warp's share of the A ring (idle in the backward), 16
+                // columns at a time, so that each half-warp stores 128 contiguous bytes of one
+                // atom's row
+                float *stage = reinterpret_cast<float *>(Ab) + warp * 32 * 17;
+                if (warp_live)
+                    for (int cc = 16 * slice; cc < nb; cc += 64) {
                         float v[16];
                         tc::tmem_ld16(tlane + cc, v);
 #pragma unroll
-                        for (int q = 0; q < 16; ++q) stage[tid * 17 + q] = (double)v[q];
+                        for (int q = 0; q < 16; ++q) stage[lane * 17 + q] = v[q];
+                        __syncwarp();
+                        const int n = n0 + cc + (lane & 15);
+#pragma unroll 4
+                        for (int r2 = lane >> 4; r2 < 32; r2 += 2) {
+                            const int at = rows_atom[32 * (warp & 3) + r2];
+                            if (at >= 0 && n < Kl) gD[(size_t)at * K1 + n] = f2d(stage[r2 * 17 + (lane & 15)]);
+                        }
+                        __syncwarp();
                     }
-                    __syncthreads();
-                    for (int p = tid; p < MXT * 16; p += MXT) {
-                        const int row = p >> 4, q = p & 15, n = n0 + cc + q;
-                        const int at = rows_atom[row];
-                        if (at >= 0 && n < Kl) gD[(size_t)at * K1 + n] = stage[row * 17 + q];
-                    }
-                    __syncthreads();
-                }
             } else if (warp_live) {
-                for (int cc = 0; cc < nb; cc += 16) {
-                    float v[16];
+                for (int cc = 16 * slice; cc < nb; cc += 64) {
+                    float v[16], hp[16];
+#pragma unroll
+                    for (int q = 0; q < 16; ++q) hp[q] = my >= 0 && n0 + cc + q < Kl ? hb[(n0 + cc + q) * MXT] : 0.f;
                     tc::tmem_ld16(tlane + cc, v);
                     if (my >= 0) {
 #pragma unroll
                         for (int q = 0; q < 16; ++q) {
                             const int n = n0 + cc + q;
-                            if (n < Kl) hb[n * MXT] = v[q] + hb[n * MXT];  // equal widths: the skip passes gh through
+                            if (n < Kl) hb[n * MXT] = v[q] + hp[q];  // equal widths: the skip passes gh through
                         }
                     }
+                    __syncwarp();
                 }
             }
             tc_sync();
@@ -1580,7 +1626,7 @@ cudaError_t dp_launch_fit_mx(cudaStream_t st, const DevModel &m, const MixedMode
     k_d2bf<<<(grid * MXT * 32 + 255) / 256, 256, 0, st>>>(eb.D, K1, mx.fit_kp[0] / FIT_KC, nb.type_perm,
                                                           nb.type_start, m.ntypes, mx.dtile);
     *launches += 1;
-    k_fit_mx<<<grid, MXT, smem, st>>>(m, mx, N, nb.type_perm, nb.type_start, eb.D, eb.Ei, eb.gD, eb.fit_t,
+    k_fit_mx<<<grid, FIT_TH, smem, st>>>(m, mx, N, nb.type_perm, nb.type_start, eb.D, eb.Ei, eb.gD, eb.fit_t,
                                       eb.fit_h, status);
     *launches += 1;
     return cudaGetLastError();
