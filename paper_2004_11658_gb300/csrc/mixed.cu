@@ -124,15 +124,6 @@ __device__ __forceinline__ void df_fma(float &sh, float &sl, float a, float bh, 
     sl = __fadd_rn(sl, __fadd_rn(err, __fmaf_rn(a, bl, e)));
 }
 
-// v = h + l to about 2^-48 relative (h = v rounded to FP32, l = the rest rounded)
-__device__ __forceinline__ void df_split(double v, float &h, float &l)
-{
-    h = __double2float_rn(v);
-    l = __double2float_rn(v - (double)h);
-}
-
-__device__ __forceinline__ double df_value(float h, float l) { return (double)h + (double)l; }
-
 // Conversions between FP32 and FP64 on the integer pipe (the FP64 pipe takes 16
 // cycles per warp instruction, conversions included): exact, and rounded to
 // nearest even, for normal FP32 results; zero, subnormal and non-finite values
@@ -151,6 +142,15 @@ __device__ __forceinline__ float d2f(double v)
     if (e < 897 || e > 1150) return (b << 1) == 0 ? __uint_as_float((uint32_t)(b >> 32)) : (float)v;
     return __uint_as_float(((uint32_t)(b >> 32) & 0x80000000u) | ((e - 896) << 23) | ((uint32_t)(r >> 29) & 0x7fffffu));
 }
+
+// v = h + l to about 2^-48 relative (h = v rounded to FP32, l = the rest rounded)
+__device__ __forceinline__ void df_split(double v, float &h, float &l)
+{
+    h = d2f(v);
+    l = d2f(v - f2d(h));
+}
+
+__device__ __forceinline__ double df_value(float h, float l) { return f2d(h) + f2d(l); }
 
 __device__ __forceinline__ void copy16(unsigned char *dst, const unsigned char *__restrict__ src, int bytes)
 {
@@ -375,7 +375,7 @@ __global__ void __launch_bounds__(MXT, 1) k_embed_fwd_mx(
                     st8_op<SPLIT>(A0, S::A0B, tid, k8, K1p, v);
                 }
                 tc_sync();
-                if (tid == 0) {
+                if (warp == 0 && tc::elect_one()) {
 #pragma unroll
                     for (int kk = 0; kk < K1p / 16; ++kk)
                         mma_op<SPLIT>(tbase, tc::smem_u32(A0) + kk * 256, S::A0B, tc::smem_u32(B1) + kk * 256, S::B1B,
@@ -407,7 +407,7 @@ __global__ void __launch_bounds__(MXT, 1) k_embed_fwd_mx(
                 }
                 tc_sync();
                 if (!alive) break;
-                if (tid == 0) {
+                if (warp == 0 && tc::elect_one()) {
 #pragma unroll
                     for (int kk = 0; kk < K2p / 16; ++kk)
                         mma_op<SPLIT>(tbase, tc::smem_u32(A1) + kk * 256, S::A1B, tc::smem_u32(B2) + kk * 256, S::B2B,
@@ -432,15 +432,19 @@ __global__ void __launch_bounds__(MXT, 1) k_embed_fwd_mx(
                             Gw[lane * 17 + q] = G2;
                         }
                         __syncwarp();
-#pragma unroll
-                        for (int u = 0; u < 2; ++u) {
-                            const int p = lane + 32 * u, c = p >> 4, q = p & 15, o = cc + q;
+                        {
+                            // lane: feature cc + lane % 16, components lane / 16 and lane / 16 + 2
+                            const int q = lane & 15, c = lane >> 4, o = cc + q;
                             if (o < E3) {
-                                float sh = 0.f, sl = 0.f;
+                                float sh = 0.f, sl = 0.f, sh2 = 0.f, sl2 = 0.f;
 #pragma unroll 8
-                                for (int rr = 0; rr < 32; ++rr)
-                                    df_fma(sh, sl, Gw[rr * 17 + q], Rwh[rr * 4 + c], Rwl[rr * 4 + c]);
+                                for (int rr = 0; rr < 32; ++rr) {
+                                    const float g = Gw[rr * 17 + q];
+                                    df_fma(sh, sl, g, Rwh[rr * 4 + c], Rwl[rr * 4 + c]);
+                                    df_fma(sh2, sl2, g, Rwh[rr * 4 + c + 2], Rwl[rr * 4 + c + 2]);
+                                }
                                 Tww[c * E3 + o] = df_value(sh, sl);
+                                Tww[(c + 2) * E3 + o] = df_value(sh2, sl2);
                             }
                         }
                         __syncwarp();
@@ -651,7 +655,7 @@ __device__ __forceinline__ void embed_mx_tangent_body(
                     st8_op<SPLIT>(dA0, S::A0B, tid, k8, K1p, dv);
                 }
                 tc_sync();
-                if (tid == 0) {
+                if (warp == 0 && tc::elect_one()) {
 #pragma unroll
                     for (int kk = 0; kk < K1p / 16; ++kk) {
                         const uint32_t bb = tc::smem_u32(B1) + kk * 256;
@@ -696,7 +700,7 @@ __device__ __forceinline__ void embed_mx_tangent_body(
                 }
                 tc_sync();
                 if (!alive) break;
-                if (tid == 0) {
+                if (warp == 0 && tc::elect_one()) {
 #pragma unroll
                     for (int kk = 0; kk < K2p / 16; ++kk) {
                         const uint32_t bb = tc::smem_u32(B2) + kk * 256;
@@ -747,15 +751,19 @@ __device__ __forceinline__ void embed_mx_tangent_body(
                                 }
                         }
                         __syncwarp();
-#pragma unroll
-                        for (int u = 0; u < 2; ++u) {
-                            const int p = lane + 32 * u, c = p >> 4, q = p & 15, o = cc + q;
+                        {
+                            // lane: feature cc + lane % 16, components lane / 16 and lane / 16 + 2
+                            const int q = lane & 15, c = lane >> 4, o = cc + q;
                             if (o < E3) {
-                                float sh = 0.f, sl = 0.f;
+                                float sh = 0.f, sl = 0.f, sh2 = 0.f, sl2 = 0.f;
 #pragma unroll 8
-                                for (int rr = 0; rr < 32; ++rr)
-                                    df_fma(sh, sl, Gw[rr * 17 + q], Rwh[rr * 4 + c], Rwl[rr * 4 + c]);
+                                for (int rr = 0; rr < 32; ++rr) {
+                                    const float g = Gw[rr * 17 + q];
+                                    df_fma(sh, sl, g, Rwh[rr * 4 + c], Rwl[rr * 4 + c]);
+                                    df_fma(sh2, sl2, g, Rwh[rr * 4 + c + 2], Rwl[rr * 4 + c + 2]);
+                                }
                                 Tww[c * E3 + o] = df_value(sh, sl);
+                                Tww[(c + 2) * E3 + o] = df_value(sh2, sl2);
                             }
                         }
                         __syncwarp();
