@@ -949,7 +949,7 @@ void dp_ctx_free(dp_ctx *c)
     void *bufs[] = {c->nb.cand, c->nb.ncand, c->nb.xref, c->nb.cell_count, c->nb.cell_start,
                     c->nb.cell_cursor, c->nb.cell_atoms, c->nb.cell_sorted, c->nb.cell_pos, c->nb.atom_cell,
                     c->nb.type_perm, c->nb.type_start, c->fb.nlist, c->fb.keys, c->fb.nreal,
-                    c->eb.T, c->eb.D, c->eb.gD, c->eb.Ei, c->eb.pair_g, c->eb.f_own, c->eb.vir_part,
+                    c->eb.T, c->eb.D, c->eb.gD, c->eb.Ei, c->eb.pair_g, c->eb.f_own, c->eb.vir_part, c->eb.red_part, c->eb.red_count,
                     c->d_energy, c->d_virial, c->md_force, c->ke_part, c->d_inv_mass_conv, c->d_mass,
                     c->eb.fit_t, c->eb.fit_h, c->d_p32, c->d_emb_ops, c->d_fit_fwd, c->d_fit_bwd,
                     c->pb.dT, c->pb.dD, c->pb.Db, c->pb.dDb, c->pb.fit_scr, c->pb.rowscr, c->pb.slices,
@@ -1014,6 +1014,8 @@ dp_status dp_ctx_create(const dp_model *model, int64_t natoms_max, int32_t cand_
     ALLOC(c->eb.pair_g, N * nm * 3);
     ALLOC(c->eb.f_own, 3 * N);
     ALLOC(c->eb.vir_part, 9 * N);
+    ALLOC(c->eb.red_part, DP_REDUCE_CTAS * 16);
+    ALLOC(c->eb.red_count, 1);
     ALLOC(c->d_energy, 1);
     ALLOC(c->d_virial, 9);
     ALLOC(c->md_force, 3 * N);
@@ -1102,6 +1104,7 @@ dp_status dp_ctx_create(const dp_model *model, int64_t natoms_max, int32_t cand_
     if (!s) {
         cudaError_t e = cudaMemsetAsync(c->d_status, 0, sizeof(int32_t), c->stream);
         if (e == cudaSuccess) e = cudaMemsetAsync(c->d_gate, 0, sizeof(int32_t), c->stream);
+        if (e == cudaSuccess) e = cudaMemsetAsync(c->eb.red_count, 0, sizeof(int32_t), c->stream);
         if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
         if (e != cudaSuccess) s = cuda_fail(e, "dp_ctx_create");
     }

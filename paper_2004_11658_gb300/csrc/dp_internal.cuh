@@ -249,6 +249,7 @@ cudaError_t dp_launch_format(cudaStream_t st, const DevModel &m, const double *x
                              NlistBuffers nb, FormatBuffers fb, int32_t *status, int32_t *retry,
                              int64_t *launches);
 
+constexpr int DP_REDUCE_CTAS = 64;
 struct EvalBuffers {
     double *T;         // [N][4][M]
     double *D;         // [N][m2*M]
@@ -257,6 +258,8 @@ struct EvalBuffers {
     double *pair_g;    // [N][nm][3]
     double *f_own;     // [N][3]
     double *vir_part;  // [N][9]
+    double *red_part;  // [DP_REDUCE_CTAS][16] partial sums of E and the virial
+    int32_t *red_count;  // CTAs done (0 between launches)
     float *fit_t;      // mixed mode: tanh values of the fitting layers [tile][n_fit][256][128]
     float *fit_h;      // mixed mode: fitting activation / gradient [tile][256][128]
     double *Gst;       // FP64 mode, when it fits: G and dG/ds of every neighbour slot [N nm][2 M]
