@@ -36,8 +36,8 @@
 // DPF_MMA_TIMEOUT, waits for its copies and MMAs, frees tensor memory and
 // returns.
 //
-// Measured per evaluation (12,288 water atoms): the six GEMMs 2.8 -> 1.22 ms,
-// the six splits 0.74 -> 0.43 ms; 192 atoms: the whole fitting net 0.96 -> 0.33
+// Measured per evaluation (12,288 water atoms): the six GEMMs 2.8 -> 1.14 ms,
+// the six splits 0.74 -> 0.43 ms; 192 atoms: the whole fitting net 0.96 -> 0.29
 // ms.  One elected lane of a whole warp issues: behind `threadIdx.x == 0` the
 // same MMAs took 139 cycles each instead of 97 in the former kernel.
 #include <algorithm>
@@ -218,7 +218,6 @@ struct OzGemmArgs {
     OzGemm g;
     const int32_t *type_perm, *type_start;
     int ntypes;
-    int epi;      // 0: forward (bias, tanh, skip); 1: backward (skip gradient); 2: tangent forward
     int skip;     // skip kind of the layer
     int skip_in;  // input width of the layer
     const double *bias[DP_MAX_TYPES];
@@ -318,7 +317,7 @@ __device__ __forceinline__ bool oz_unit(const OzGemmArgs &p, int u, OzUnit &U)
 // 60 B/clk that large bulk copies reach = 10.3 k; with the FP64 tanh 20 k
 // cycles of FP64 pipe.  The tanh table sits in shared memory: its lookups by 32
 // lanes cost 32 wavefronts each through L1, and were 53 k cycles per unit.
-template <int S>
+template <int S, int EPI, bool SEG>
 __global__ void __launch_bounds__(OZ_THREADS, 1) k_oz_gemm(OzGemmArgs p)
 {
     extern __shared__ __align__(1024) unsigned char smraw[];
@@ -357,7 +356,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_oz_gemm(OzGemmArgs p)
         // copies: the tanh table, then the digit chunks of every unit
         int c = 0;
         bool ok = true;
-        if (p.epi == 0 && tc::elect_one()) {
+        if (EPI == 0 && tc::elect_one()) {
             mbar_expect_tx(&tabbar, OZ_TAB_BYTES);
             bulk_g2s(smraw + NST * stage_bytes, p.tanh_tab, OZ_TAB_BYTES, &tabbar);
         }
@@ -381,7 +380,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_oz_gemm(OzGemmArgs p)
         if (!ok) fail = 1;
         // no copy is in flight when the CTA leaves
         for (int q = c > NST ? c - NST : 0; q < c; ++q) tc::mbar_wait(&full[q % NST], (q / NST) & 1);
-        if (p.epi == 0) tc::mbar_wait(&tabbar, 0);
+        if (EPI == 0) tc::mbar_wait(&tabbar, 0);
     } else if (warp == 8) {
         const uint32_t idesc = tc::make_idesc_bf16(DP_OZ_TILE, DP_OZ_NC);
         // the MMAs of one chunk, then the commit that frees its stage; one copy of
@@ -457,7 +456,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_oz_gemm(OzGemmArgs p)
         const bool vec = !p.wg && (p.ldo & 1) == 0 && (p.ldh & 1) == 0;  // rows start on 16 bytes
         int sc = 0;
         bool ok = true;
-        if (p.epi == 0) ok = __all_sync(0xffffffffu, tc::mbar_wait(&tabbar, 0));
+        if (EPI == 0) ok = __all_sync(0xffffffffu, tc::mbar_wait(&tabbar, 0));
         for (int u = blockIdx.x; u < p.units && ok; u += gridDim.x) {
             OzUnit U;
             if (!oz_unit<S>(p, u, U)) break;
@@ -476,107 +475,142 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_oz_gemm(OzGemmArgs p)
             const int esc = (i >= 0 ? p.aexp[erow] : 0) - g.beta * (S + 1);
             double *hout = p.hout + (p.wg ? p.out_off[U.a] : 0);
             // the skip's operands, asked for before the MMAs are waited for
-            const bool bcast = p.epi == 1 && p.gbc[U.a] != nullptr;
+            const bool bcast = EPI == 1 && p.gbc[U.a] != nullptr;
             const double *hin = bcast ? p.gbc[U.a] : (p.wg ? hout : p.hin) + (size_t)(i < 0 ? 0 : i) * p.ldh;
-            double sk[16];
+            double sk[2][8];
 #pragma unroll
-            for (int n = 0; n < 16; ++n) sk[n] = 0.0;
-            if (i >= 0) {
-                if (p.skip == 1 && vec && !bcast && n0 + 16 <= g.N) {
+            for (int h = 0; h < 2; ++h) {
+                const int q0 = n0 + 8 * h;
 #pragma unroll
-                    for (int n = 0; n < 16; n += 2) {
-                        const double2 v = *reinterpret_cast<const double2 *>(hin + n0 + n);
-                        sk[n] = v.x;
-                        sk[n + 1] = v.y;
-                    }
-                } else if (p.skip != 0) {
+                for (int n = 0; n < 8; ++n) sk[h][n] = 0.0;
+                if (i >= 0 && p.skip != 0) {
+                    if (p.skip == 1 && vec && !bcast && q0 + 8 <= g.N) {
 #pragma unroll
-                    for (int n = 0; n < 16; ++n)
-                        if (n0 + n < g.N) {
-                            const int q = n0 + n;
-                            sk[n] = p.skip == 1 ? hin[q]
-                                    : p.epi != 1 ? hin[q % p.skip_in]
-                                                 : hin[q] + hin[q + p.skip_in];
+                        for (int n = 0; n < 8; n += 2) {
+                            const double2 v = *reinterpret_cast<const double2 *>(hin + q0 + n);
+                            sk[h][n] = v.x;
+                            sk[h][n + 1] = v.y;
                         }
-                }
-            }
-            long long hi[16], lo[16];
-#pragma unroll
-            for (int n = 0; n < 16; ++n) hi[n] = lo[n] = 0;
-            for (int sg = 0; sg < U.nseg; ++sg, ++sc) {
-                const int buf = sc & 1;
-                ok = tc::mbar_wait(&tfull[buf], (sc >> 1) & 1) && !fail;
-                ok = __all_sync(0xffffffffu, ok);
-                if (!ok) break;
-                tc::fence_after_sync();
-#pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    long long a[8], b[8];
-#pragma unroll
-                    for (int gg = 2; gg <= S + 1; ++gg) {
-                        float v[8];
-                        tc::tmem_ld8(tl_lane + buf * TBUF + (uint32_t)(gg - 2) * DP_OZ_NC + 8 * h, v);
+                    } else {
 #pragma unroll
                         for (int n = 0; n < 8; ++n) {
-                            const long long iv = (long long)__float2int_rn(v[n]);
-                            if (gg == 2) a[n] = iv;
-                            else if (gg <= H + 1) a[n] = (a[n] << g.beta) + iv;
-                            else if (gg == H + 2) b[n] = iv;
-                            else b[n] = (b[n] << g.beta) + iv;
+                            const int q = q0 + n;
+                            if (q < g.N)
+                                sk[h][n] = p.skip == 1 ? hin[q]
+                                           : EPI != 1  ? hin[q % p.skip_in]
+                                                       : hin[q] + hin[q + p.skip_in];
                         }
                     }
+                }
+            }
+            // group sums of 8 columns (half h of the 16) in buffer buf
+            auto groups = [&](int buf, int h, long long (&a)[8], long long (&b)[8]) {
+#pragma unroll
+                for (int gg = 2; gg <= S + 1; ++gg) {
+                    float v[8];
+                    tc::tmem_ld8(tl_lane + buf * TBUF + (uint32_t)(gg - 2) * DP_OZ_NC + 8 * h, v);
 #pragma unroll
                     for (int n = 0; n < 8; ++n) {
-                        hi[8 * h + n] += a[n];
-                        lo[8 * h + n] += b[n];
+                        const long long iv = (long long)__float2int_rn(v[n]);
+                        if (gg == 2) a[n] = iv;
+                        else if (gg <= H + 1) a[n] = (a[n] << g.beta) + iv;
+                        else if (gg == H + 2) b[n] = iv;
+                        else b[n] = (b[n] << g.beta) + iv;
                     }
                 }
-                tc::fence_before_sync();
-                __syncwarp();
-                if (lane == 0) tc::mbar_arrive(&tempty[buf]);
-            }
-            if (!ok) break;
-            if (i < 0) continue;
-            double *ho = hout + (size_t)i * p.ldo + n0;
-            double *to = p.epi != 1 ? p.tout + (size_t)i * p.ldo + n0 : nullptr;
-            const double *ti = p.epi == 2 ? p.tin + (size_t)i * p.ldo + n0 : nullptr;
+            };
+            auto finish = [&](int h, const long long (&hi)[8], const long long (&lo)[8], const double (&skh)[8]) {
+                if (i < 0) return;
+                const int q0 = n0 + 8 * h;
+                double *ho = hout + (size_t)i * p.ldo + q0;
+                double *to = EPI != 1 ? p.tout + (size_t)i * p.ldo + q0 : nullptr;
+                const double *ti = EPI == 2 ? p.tin + (size_t)i * p.ldo + q0 : nullptr;
+                const int4 f0 = fe4[2 * h], f1 = fe4[2 * h + 1];
+                const int fe[8] = {f0.x, f0.y, f0.z, f0.w, f1.x, f1.y, f1.z, f1.w};
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const int4 f4 = fe4[q];
-                const int fe[4] = {f4.x, f4.y, f4.z, f4.w};
-#pragma unroll
-                for (int n2 = 0; n2 < 4; n2 += 2) {
+                for (int n2 = 0; n2 < 8; n2 += 2) {
                     double y[2], t[2];
 #pragma unroll
                     for (int v = 0; v < 2; ++v) {
-                        const int n = 4 * q + n2 + v, e = esc + fe[n2 + v];
-                        y[v] = e > -900 && e < 900 ? oz_i64x2_scaled_w(hi[n], lo[n], w, e)
-                                                   : scale2(fma((double)hi[n], oz_pow2(w), (double)lo[n]), e);
-                        if (e > 5000) y[v] = __longlong_as_double(0x7ff8000000000000ll);
-                        const int col = n0 + n;
-                        if (p.epi == 0) {
-                            t[v] = dp_tanh64(y[v] + (col < g.N ? p.bias[U.a][col] : 0.0), tab);
+                        const int n = n2 + v, e = esc + fe[n];
+                        const bool in = q0 + n < g.N;
+                        if (e > -900 && e < 900) y[v] = oz_i64x2_round(hi[n], lo[n], w, e);
+                        else if (e > 5000) y[v] = __longlong_as_double(0x7ff8000000000000ll);
+                        else y[v] = scale2(fma((double)hi[n], oz_pow2(w), (double)lo[n]), e);
+                        if constexpr (EPI == 0) {
+                            t[v] = dp_tanh64(y[v] + (in ? p.bias[U.a][q0 + n] : 0.0), tab);
                             y[v] = t[v];
-                        } else if (p.epi == 2) {
-                            const double tv = col < g.N ? ti[n] : 0.0;
+                        } else if constexpr (EPI == 2) {
+                            const double tv = in ? ti[n] : 0.0;
                             t[v] = y[v];
                             y[v] *= fma(-tv, tv, 1.0);
                         }
-                        y[v] += sk[n];
+                        y[v] += skh[n];
                     }
-                    const int n = 4 * q + n2;
-                    if (vec && n0 + n + 2 <= g.N) {
-                        *reinterpret_cast<double2 *>(ho + n) = make_double2(y[0], y[1]);
-                        if (p.epi != 1) *reinterpret_cast<double2 *>(to + n) = make_double2(t[0], t[1]);
+                    if (vec && q0 + n2 + 2 <= g.N) {
+                        *reinterpret_cast<double2 *>(ho + n2) = make_double2(y[0], y[1]);
+                        if constexpr (EPI != 1) *reinterpret_cast<double2 *>(to + n2) = make_double2(t[0], t[1]);
                     } else {
 #pragma unroll
                         for (int v = 0; v < 2; ++v)
-                            if (n0 + n + v < g.N) {
-                                ho[n + v] = y[v];
-                                if (p.epi != 1) to[n + v] = t[v];
+                            if (q0 + n2 + v < g.N) {
+                                ho[n2 + v] = y[v];
+                                if constexpr (EPI != 1) to[n2 + v] = t[v];
                             }
                     }
                 }
+            };
+            auto wait = [&](int buf) {
+                ok = tc::mbar_wait(&tfull[buf], (sc >> 1) & 1) && !fail;
+                ok = __all_sync(0xffffffffu, ok);
+                tc::fence_after_sync();
+                return ok;
+            };
+            auto release = [&](int buf) {
+                tc::fence_before_sync();
+                __syncwarp();
+                if (lane == 0) tc::mbar_arrive(&tempty[buf]);
+                ++sc;
+            };
+            if constexpr (SEG) {
+                long long hi[2][8], lo[2][8];
+#pragma unroll
+                for (int h = 0; h < 2; ++h)
+#pragma unroll
+                    for (int n = 0; n < 8; ++n) hi[h][n] = lo[h][n] = 0;
+                for (int sg = 0; sg < U.nseg; ++sg) {
+                    const int buf = sc & 1;
+                    if (!wait(buf)) break;
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        long long a[8], b[8];
+                        groups(buf, h, a, b);
+#pragma unroll
+                        for (int n = 0; n < 8; ++n) {
+                            hi[h][n] += a[n];
+                            lo[h][n] += b[n];
+                        }
+                    }
+                    release(buf);
+                }
+                if (!ok) break;
+                finish(0, hi[0], lo[0], sk[0]);
+                finish(1, hi[1], lo[1], sk[1]);
+            } else {
+                // one segment: 8 columns at a time, half the code
+                const int buf = sc & 1;
+                if (!wait(buf)) break;
+#pragma unroll 1
+                for (int h = 0; h < 2; ++h) {
+                    long long a[8], b[8];
+                    double skh[8];
+#pragma unroll
+                    for (int n = 0; n < 8; ++n) skh[n] = h == 0 ? sk[0][n] : sk[1][n];
+                    __syncwarp();
+                    groups(buf, h, a, b);
+                    finish(h, a, b, skh);
+                }
+                release(buf);
             }
         }
         if (!ok) fail = 1;
@@ -894,14 +928,7 @@ struct OzRun {
 
     cudaError_t init() const
     {
-        if (tiles > ob.tiles) return cudaErrorInvalidValue;
-        cudaError_t e = cudaFuncSetAttribute(k_oz_gemm<8>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)gemm_smem(8));
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(k_oz_gemm<5>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gemm_smem(5));
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(k_oz_gemm<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gemm_smem(4));
-        return e;
+        return tiles > ob.tiles ? cudaErrorInvalidValue : cudaSuccess;
     }
 
     cudaError_t split(int mode, const double *src, int lds, const double *tv, const OzGemm &g) const
@@ -933,23 +960,42 @@ struct OzRun {
         return cudaGetLastError();
     }
 
-    cudaError_t launch(OzGemmArgs &a) const
+    template <int S, int EPI, bool SEG>
+    cudaError_t launch_as(const OzGemmArgs &a) const
+    {
+        const size_t smem = gemm_smem(S);
+        cudaError_t e = cudaFuncSetAttribute(k_oz_gemm<S, EPI, SEG>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             (int)smem);
+        if (e != cudaSuccess) return e;
+        k_oz_gemm<S, EPI, SEG><<<std::min(a.units, num_sms), OZ_THREADS, smem, st>>>(a);
+        *launches += 1;
+        return cudaGetLastError();
+    }
+
+    // epi 0: forward (bias, tanh, skip); 1: backward (skip gradient); 2: tangent forward
+    template <int S>
+    cudaError_t launch_epi(const OzGemmArgs &a, int epi) const
+    {
+        const bool seg = a.wg || a.g.seg < a.g.nK;
+        if (epi == 0) return seg ? launch_as<S, 0, true>(a) : launch_as<S, 0, false>(a);
+        if (epi == 1) return seg ? launch_as<S, 1, true>(a) : launch_as<S, 1, false>(a);
+        return seg ? launch_as<S, 2, true>(a) : launch_as<S, 2, false>(a);
+    }
+
+    cudaError_t launch(OzGemmArgs &a, int epi) const
     {
         a.type_perm = nb.type_perm;
         a.type_start = nb.type_start;
         a.ntypes = T;
         a.tanh_tab = m.tanh_tab;
         a.status = status;
-        const int grid = std::min(a.units, num_sms);
-        const size_t smem = gemm_smem(a.g.S);
-        if (a.g.S == 4) k_oz_gemm<4><<<grid, OZ_THREADS, smem, st>>>(a);
-        else if (a.g.S == 5) k_oz_gemm<5><<<grid, OZ_THREADS, smem, st>>>(a);
-        else k_oz_gemm<8><<<grid, OZ_THREADS, smem, st>>>(a);
-        *launches += 1;
-        return cudaGetLastError();
+        // plans of 4 and 5 digits have one segment and no tangent
+        if (a.g.S == 8) return launch_epi<8>(a, epi);
+        if (a.g.S == 5) return epi == 0 ? launch_as<5, 0, false>(a) : launch_as<5, 1, false>(a);
+        return epi == 0 ? launch_as<4, 0, false>(a) : launch_as<4, 1, false>(a);
     }
 
-    // epi as in OzGemmArgs; hin: the skip's operand (with bcast_wout the output weights)
+    // hin: the skip's operand (with bcast_wout the output weights)
     cudaError_t gemm(const OzGemm &g, int epi, int skip, int skip_in, int l, const double *hin, int ldh,
                      bool bcast_wout, const double *tin, double *tout, double *hout, int ldo) const
     {
@@ -961,7 +1007,6 @@ struct OzRun {
         a.w = oz.w;
         a.wexp = oz.wexp;
         a.g = g;
-        a.epi = epi;
         a.skip = skip;
         a.skip_in = skip_in;
         for (int t = 0; t < T; ++t) {
@@ -975,7 +1020,7 @@ struct OzRun {
         a.hout = hout;
         a.ldo = ldo;
         a.units = tiles * g.nN;
-        return launch(a);
+        return launch(a, epi);
     }
 };
 
@@ -1092,7 +1137,6 @@ cudaError_t dp_launch_pgrad_fit_oz(cudaStream_t st, const DevModel &m, const OzM
             a.g.nN = nN;
             a.g.beta = 7;
             a.g.S = 8;
-            a.epi = 1;
             a.skip = pass;  // the second product is added to the first
             a.wg = 1;
             a.rows = K + 1;
@@ -1101,7 +1145,7 @@ cudaError_t dp_launch_pgrad_fit_oz(cudaStream_t st, const DevModel &m, const OzM
             a.ldo = a.ldh = F;
             for (int t = 0; t < T; ++t) a.out_off[t] = m.fit_base[t] + off;
             a.units = T * nq * nN;
-            if ((e2 = r.launch(a)) != cudaSuccess) return e2;
+            if ((e2 = r.launch(a, 1)) != cudaSuccess) return e2;
         }
         return cudaSuccess;
     };

@@ -140,3 +140,45 @@ static __host__ __device__ __forceinline__ double oz_i64x2_scaled(long long hi, 
 {
     return oz_i64x2_scaled_w(hi, lo, 32, p);
 }
+
+// oz_i64x2_scaled_w for |hi| < 2^61, |lo| < 2^60, 1 <= w <= 32 and a result in the
+// normal range, in 64-bit arithmetic: hi is shifted up by k <= w as far as 62 bits
+// allow, lo's bits below 2^(w - k) are kept as a sticky bit (they matter only when
+// the sum has 62 bits, of which 53 are kept), and one rounding to nearest even
+// leaves the value of fma((double)hi, 2^w, (double)lo) * 2^p bit for bit.
+static __host__ __device__ __forceinline__ double oz_i64x2_round(long long hi, long long lo, int w, int p)
+{
+    const unsigned long long ah = (unsigned long long)(hi < 0 ? -hi : hi);
+#ifdef __CUDA_ARCH__
+    const int lzh = __clzll((long long)ah);
+#else
+    const int lzh = ah ? __builtin_clzll(ah) : 64;
+#endif
+    const int k = lzh - 2 < w ? lzh - 2 : w, d = w - k;  // |hi 2^k| < 2^62
+    const long long kept = lo >> d;
+    const long long m = (hi << k) + kept;
+    const unsigned long long sticky = (unsigned long long)(lo - (kept << d)) != 0ull ? 1ull : 0ull;
+    const unsigned long long u0 = (unsigned long long)m | sticky;
+    const bool neg = (long long)u0 < 0;
+    const unsigned long long u = neg ? 0ull - u0 : u0;
+    if (u == 0) return 0.0;
+#ifdef __CUDA_ARCH__
+    const int lz = __clzll((long long)u);
+#else
+    const int lz = __builtin_clzll(u);
+#endif
+    const int sh = 11 - lz;  // u has 64 - lz bits
+    unsigned long long r;    // 53 bits (or 2^53 after rounding up)
+    if (sh <= 0) r = u << -sh;
+    else r = (u + ((1ull << (sh - 1)) - 1ull) + ((u >> sh) & 1ull)) >> sh;
+    // r 2^sh 2^d 2^p; the hidden bit of r adds one to the exponent field
+    const unsigned long long bits =
+        ((unsigned long long)(sh + d + p + 1074) << 52) + r + (neg ? 0x8000000000000000ull : 0ull);
+#ifdef __CUDA_ARCH__
+    return __longlong_as_double((long long)bits);
+#else
+    double v;
+    std::memcpy(&v, &bits, 8);
+    return v;
+#endif
+}
