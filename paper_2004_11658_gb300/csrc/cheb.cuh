@@ -35,11 +35,16 @@ cudaError_t dp_launch_cheb_build(cudaStream_t st, const DevModel &m, ChebBuffers
 // Terms needed for the nets of the host copy of mx, 0 if not resolved.
 int dp_cheb_terms(const DevModel &m, const double *mx);
 
+// os: the products with the series on the tensor cores (dp_cheb_gemm), a_dig
+// their digit scratch; null: on the FP64 units, fused.
+bool dp_cheb_gemm(const DevModel &m, int n, int N);
 cudaError_t dp_launch_cheb_fwd(cudaStream_t st, const DevModel &m, const ChebModel &cm, const double *x,
                                const int32_t *types, Box3 box, int N, const FormatBuffers &fb,
-                               const NlistBuffers &nb, EvalBuffers eb, int64_t *launches);
+                               const NlistBuffers &nb, EvalBuffers eb, const OzSeries *os, uint16_t *a_dig, int num_sms,
+                               int32_t *status, int64_t *launches);
 cudaError_t dp_launch_cheb_bwd(cudaStream_t st, const DevModel &m, const ChebModel &cm, const int32_t *types, int N,
-                               const FormatBuffers &fb, const NlistBuffers &nb, EvalBuffers eb, int64_t *launches);
+                               const FormatBuffers &fb, const NlistBuffers &nb, EvalBuffers eb, const OzSeries *os,
+                               uint16_t *a_dig, int num_sms, int32_t *status, int64_t *launches);
 
 // Parameter gradient through the series (csrc/embed_cheb.cu): T, dT, D, dD of
 // every atom with the moments kept, then, from dPhi/dD and dPhi/d(dD), the

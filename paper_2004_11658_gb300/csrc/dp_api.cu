@@ -158,6 +158,8 @@ struct dp_ctx {
     ChebBuffers cb;
     double *h_cheb_mx;  // pinned host copy of cb.mx
     ChebGradBuffers cg; // parameter gradient (allocated on first use)
+    OzSeries os;        // digits of the series (os.w null: products on the FP64 units only)
+    bool os_ok;
     int64_t cheb_version;
     // mixed precision: BF16 / FP32 copies of the parameters
     MixedModel mx;
@@ -571,6 +573,11 @@ dp_status ensure_cheb(dp_ctx *c)
     c->cheb.C = c->cb.C;
     c->cheb.Ct = c->cb.Ct;
     c->cheb.V = c->cb.V;
+    c->os_ok = c->os.w && c->cheb.n > 0 && dp_oz_series_plan(c->m, c->cheb.n, c->os);
+    if (c->os_ok) {
+        e = dp_launch_oz_series(c->stream, c->m, c->os, DP_CHEB_NN, c->cheb.n, c->cb.C, &c->launches);
+        if (e != cudaSuccess) return cuda_fail(e, "series digits");
+    }
     c->cheb_version = c->model->version;
     return DP_OK;
 }
@@ -587,11 +594,15 @@ dp_status enqueue_eval(dp_ctx *c, const double *coords, const int32_t *types, co
         if ((s = enqueue_format(c, coords, types, b, nloc))) return s;
         if (c->use_cheb && (s = ensure_cheb(c))) return s;
         const bool cheb = c->use_cheb && c->cheb.n > 0;
+        if (cheb && c->use_oz && (s = ensure_oz(c))) return s;
+        const bool gemm = cheb && c->os_ok && c->use_oz && dp_cheb_gemm(c->m, c->cheb.n, n) &&
+                          dp_oz_series_fits(c->m, c->os, c->ob, n);
+        const OzSeries *os = gemm ? &c->os : nullptr;
         if (!mixed && !cheb && c->use_ex && (s = ensure_ex(c))) return s;
         {
             GroupTimer tm(c, G_EMBED_FWD);
-            e = cheb ? dp_launch_cheb_fwd(c->stream, c->m, c->cheb, coords, types, b, n, c->fb, c->nb, c->eb,
-                                          &c->launches)
+            e = cheb ? dp_launch_cheb_fwd(c->stream, c->m, c->cheb, coords, types, b, n, c->fb, c->nb, c->eb, os,
+                                          c->ob.a, c->num_sms, c->d_status, &c->launches)
                 : mixed && c->eb.Gmx
                     ? dp_launch_embed_tan_mx(c->stream, c->m, c->mx, coords, types, b, n, c->fb, c->nb, c->eb,
                                              c->num_sms, c->d_status, &c->launches)
@@ -618,7 +629,8 @@ dp_status enqueue_eval(dp_ctx *c, const double *coords, const int32_t *types, co
         }
         {
             GroupTimer tm(c, G_EMBED_BWD);
-            e = cheb ? dp_launch_cheb_bwd(c->stream, c->m, c->cheb, types, n, c->fb, c->nb, c->eb, &c->launches)
+            e = cheb ? dp_launch_cheb_bwd(c->stream, c->m, c->cheb, types, n, c->fb, c->nb, c->eb, os, c->ob.a,
+                                          c->num_sms, c->d_status, &c->launches)
                 : mixed && c->eb.Gmx
                     ? dp_launch_embed_bwd_stmx(c->stream, c->m, types, n, c->fb, c->eb, &c->launches)
                 : mixed     ? dp_launch_embed_bwd_mx(c->stream, c->m, c->mx, coords, types, b, n, c->fb, c->nb,
@@ -955,7 +967,8 @@ void dp_ctx_free(dp_ctx *c)
                     c->pb.dT, c->pb.dD, c->pb.Db, c->pb.dDb, c->pb.fit_scr, c->pb.rowscr, c->pb.slices,
                     c->d_oz_w, c->d_oz_e, c->ob.a, c->ob.aexp, c->ob.t, c->ob.h, c->ob.g, c->d_dtile, c->d_ex_w,
                     c->eb.Gst, c->eb.Gmx, c->cb.C, c->cb.Ct, c->cb.V, c->cb.y, c->cb.mx, c->cb.trig, c->cg.mom,
-                    c->cg.part, c->cg.node, c->cg.far, c->og.a, c->og.b, c->og.exp, c->og.mx, c->og.x};
+                    c->os.w, c->os.e, c->os.aexp, c->cg.part, c->cg.node, c->cg.far, c->og.a, c->og.b, c->og.exp,
+                    c->og.mx, c->og.x};
     for (void *p : bufs) dev_free(p);
     delete c;
 }
@@ -1056,6 +1069,12 @@ dp_status dp_ctx_create(const dp_model *model, int64_t natoms_max, int32_t cand_
             s = fail(DP_ERR_NOMEM, "pinned allocation failed");
         }
         c->use_cheb = true;
+        OzSeries &os = c->os;
+        if (dp_oz_series_plan(c->m, DP_CHEB_NN, os)) {
+            ALLOC(os.w, (size_t)os.w_elems);
+            ALLOC(os.e, (size_t)os.e_elems);
+            ALLOC(os.aexp, 4 * N + 128 * (T + 1));
+        }
     }
     // G and dG/ds (FP32) stored by the mixed forward (plain BF16 operands), on the same rule
     if (!s && precision == DP_PREC_MIXED) {

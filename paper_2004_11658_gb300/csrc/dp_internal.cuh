@@ -353,6 +353,23 @@ cudaError_t dp_launch_fit_oz(cudaStream_t st, const DevModel &m, const OzModel &
                              const NlistBuffers &nb, EvalBuffers eb, int num_sms, int32_t *status,
                              int64_t *launches);
 
+// Y = X W with four rows (components of R~) per centre and the series of the
+// embedding nets as W: T from the moments (gf) and U from dE/dT (gb).
+struct OzSeries {
+    OzGemm gf, gb;
+    uint16_t *w;       // digits of the series, per centre type
+    int32_t *e;        // their exponents
+    int32_t *aexp;     // row exponents, 4 N + 128 ntypes
+    int64_t w_elems, e_elems;
+};
+bool dp_oz_series_plan(const DevModel &m, int n, OzSeries &os);  // n terms per net
+cudaError_t dp_launch_oz_series(cudaStream_t st, const DevModel &m, const OzSeries &os, int nn, int n, const double *C,
+                                int64_t *launches);
+bool dp_oz_series_fits(const DevModel &m, const OzSeries &os, const OzBuffers &ob, int N);
+cudaError_t dp_launch_oz_rows(cudaStream_t st, const DevModel &m, const OzSeries &os, const OzGemm &g, uint16_t *a_dig,
+                              int N, const double *x, int ldx, double *y, int ldy, const NlistBuffers &nb, int num_sms,
+                              int32_t *status, int64_t *launches);
+
 // FP64 embedding forward with its last layer on the tensor cores by exact
 // splitting (csrc/embed_x.cu): 3-layer doubling nets with e1 in {16, 25, 32}.
 bool dp_ex_supported(const DevModel &m);

@@ -28,10 +28,11 @@
 // What bounds the kernels: the FP64 pipe (16 cycles per warp instruction and SM).
 // One 128-thread CTA per atom, several per SM, so that the phases of different
 // atoms overlap; rows one per thread, then the per-atom products over (term,
-// component) and (component, feature) items.  Measured per evaluation of 139,968
-// water atoms (20 terms): forward 159 -> 13.0 ms, backward 25.0 -> 16.7 ms against
-// the kernels of embed_x.cu that evaluate the nets and keep G and dG/ds; 32,000
-// copper atoms: 79 -> 3.0 and 12.8 -> 4.6 ms; 192 water atoms: 0.37 -> 0.04 and
+// component) and (component, feature) items, which large boxes take to the tensor
+// cores (dp_cheb_gemm).  Measured per evaluation of 139,968 water atoms (20
+// terms): forward 159 -> 6.9 ms, backward 25.0 -> 13.5 ms against the kernels of
+// embed_x.cu that evaluate the nets and keep G and dG/ds; 32,000 copper atoms: 79
+// -> 2.3 and 12.8 -> 4.2 ms; 192 water atoms: 0.37 -> 0.04 and
 // 0.17 -> 0.05 ms.  Errors against extended precision are the same (forces
 // 1e-15 of their norm on water, 2e-14 on copper, both ways).
 #include <cmath>
@@ -288,8 +289,52 @@ __device__ __forceinline__ int row_block(const int *start, int T, int q)
     return b;
 }
 
+// Adds the rows beyond S to T (Ts [4][M], scaled), in row order, by the whole CTA.
+__device__ __forceinline__ void far_rows_T(const DevModel &m, int a, int i, const int *start,
+                                           double (&fbuf)[4][DP_MAX_EMB_W], const double *pair_d, double *Ts)
+{
+    const int T = m.ntypes, M = m.M, tid = threadIdx.x;
+    const double irc = 1.0 / (m.rcut - m.rcut_smth);
+    double *ga = fbuf[0], *da = fbuf[1], *gb = fbuf[2], *db = fbuf[3];
+    for (int q = 0; q < start[T]; ++q) {
+        const int b = row_block(start, T, q);
+        const double *d = pair_d + ((size_t)i * m.nm + m.sel_off[b] + (q - start[b])) * 3;
+        const double dv[3] = {d[0], d[1], d[2]};
+        const double r = __dsqrt_rn(__dadd_rn(__dadd_rn(__dmul_rn(dv[0], dv[0]), __dmul_rn(dv[1], dv[1])),
+                                              __dmul_rn(dv[2], dv[2])));
+        double s, ds, inv;
+        dp_switch_inv(r, m.rcut_smth, m.rcut, irc, s, ds, inv);
+        if (s <= DP_CHEB_S) continue;  // uniform: every thread has the same row
+        net_direct(m, a * T + b, s, ga, da, gb, db);
+        const double sr = s * inv;
+        for (int p = tid; p < 4 * M; p += CT) {
+            const int c = p / M;
+            Ts[p] += (c == 0 ? s : sr * dv[c - 1]) * ga[p - c * M] * m.desc_scale;
+        }
+        __syncthreads();
+    }
+}
+
+// D = T_<^T T of one atom by the whole CTA.
+__device__ __forceinline__ void descriptor(const DevModel &m, int i, const double *Ts, double *__restrict__ Dout)
+{
+    const int M = m.M, nd = m.m2 * M;
+    for (int q = threadIdx.x; q < nd; q += CT) {
+        const int a2 = q / M, b2 = q - a2 * M;
+        double acc = Ts[a2] * Ts[b2];
+        acc = fma(Ts[M + a2], Ts[M + b2], acc);
+        acc = fma(Ts[2 * M + a2], Ts[2 * M + b2], acc);
+        acc = fma(Ts[3 * M + a2], Ts[3 * M + b2], acc);
+        Dout[(size_t)i * nd + q] = acc;
+    }
+}
+
 // ---------------------------------------------------------------- forward ---
 
+// MOM: the CTA stops at the scaled moments, written to Tout as [4][T nc] rows of
+// the atom, with a flag in Dout[i] when it has rows beyond S; T and D follow in
+// other kernels (dp_launch_cheb_fwd).
+template <bool MOM>
 __global__ void __launch_bounds__(CT) k_cheb_fwd(DevModel m, ChebModel cm, const double *__restrict__ x,
                                                  const int32_t *__restrict__ types, Box3 box,
                                                  const int32_t *__restrict__ type_perm,
@@ -386,6 +431,12 @@ __global__ void __launch_bounds__(CT) k_cheb_fwd(DevModel m, ChebModel cm, const
         }
         __syncthreads();
     }
+    if constexpr (MOM) {
+        for (int p = tid; p < T * nc * 4; p += CT)
+            Tout[((size_t)i * 4 + (p & 3)) * (T * nc) + (p >> 2)] = Mom[p] * m.desc_scale;
+        if (tid == 0) Dout[i] = any_far ? 1.0 : 0.0;
+        return;
+    }
     // T = scale sum_k P_k C_k, items (c, f)
     {
         const double *C = cm.C + (size_t)(a_ok ? a : 0) * T * NN * M;
@@ -413,40 +464,60 @@ __global__ void __launch_bounds__(CT) k_cheb_fwd(DevModel m, ChebModel cm, const
         }
     }
     __syncthreads();
-    if (any_far) {
-        double *ga = fbuf[0], *da = fbuf[1], *gb = fbuf[2], *db = fbuf[3];
-        for (int q = 0; q < R; ++q) {
-            const int b = row_block(start, T, q);
-            const double *d = pair_d + ((size_t)i * nm + m.sel_off[b] + (q - start[b])) * 3;
-            const double dv[3] = {d[0], d[1], d[2]};
-            const double r = __dsqrt_rn(__dadd_rn(__dadd_rn(__dmul_rn(dv[0], dv[0]), __dmul_rn(dv[1], dv[1])),
-                                                  __dmul_rn(dv[2], dv[2])));
-            double s, ds, inv;
-            dp_switch_inv(r, m.rcut_smth, m.rcut, irc, s, ds, inv);
-            if (s <= DP_CHEB_S) continue;  // uniform: every thread has the same row
-            net_direct(m, a * T + b, s, ga, da, gb, db);
-            const double sr = s * inv;
-            for (int p = tid; p < 4 * M; p += CT) {
-                const int c = p / M;
-                Ts[p] += (c == 0 ? s : sr * dv[c - 1]) * ga[p - c * M] * m.desc_scale;
-            }
-            __syncthreads();
-        }
-    }
+    if (any_far) far_rows_T(m, a, i, start, fbuf, pair_d, Ts);
     for (int p = tid; p < 4 * M; p += CT) Tout[(size_t)i * 4 * M + p] = Ts[p];
-    const int nd = m.m2 * M;
-    for (int q = tid; q < nd; q += CT) {
-        const int a2 = q / M, b2 = q - a2 * M;
-        double acc = Ts[a2] * Ts[b2];
-        acc = fma(Ts[M + a2], Ts[M + b2], acc);
-        acc = fma(Ts[2 * M + a2], Ts[2 * M + b2], acc);
-        acc = fma(Ts[3 * M + a2], Ts[3 * M + b2], acc);
-        Dout[(size_t)i * nd + q] = acc;
+    descriptor(m, i, Ts, Dout);
+}
+
+// T of one atom finished (rows beyond S added) and D = T_<^T T, one CTA per atom.
+__global__ void __launch_bounds__(CT) k_cheb_desc(DevModel m, const int32_t *__restrict__ types,
+                                                  const int32_t *__restrict__ type_perm,
+                                                  const int32_t *__restrict__ nreal, const double *__restrict__ flag,
+                                                  const double *__restrict__ pair_d, double *__restrict__ Tio,
+                                                  double *__restrict__ Dout)
+{
+    __shared__ double Ts[4 * DP_MAX_EMB_W];
+    __shared__ int start[DP_MAX_TYPES + 1];
+    __shared__ double fbuf[4][DP_MAX_EMB_W];
+    const int M = m.M, T = m.ntypes, tid = threadIdx.x;
+    const int i = type_perm[blockIdx.x];
+    for (int p = tid; p < 4 * M; p += CT) Ts[p] = Tio[(size_t)i * 4 * M + p];
+    const bool far = flag[i] != 0.0;
+    if (far && tid == 0) {
+        int r = 0;
+        for (int b = 0; b < T; ++b) {
+            start[b] = r;
+            r += nreal[(size_t)i * T + b];
+        }
+        start[T] = r;
     }
+    __syncthreads();
+    if (far) {
+        far_rows_T(m, types[i], i, start, fbuf, pair_d, Ts);
+        for (int p = tid; p < 4 * M; p += CT) Tio[(size_t)i * 4 * M + p] = Ts[p];
+    }
+    descriptor(m, i, Ts, Dout);
+}
+
+// dE/dT of one atom per CTA, as [4][M].
+__global__ void __launch_bounds__(CT) k_cheb_gT(DevModel m, const int32_t *__restrict__ type_perm,
+                                                const double *__restrict__ Tin, const double *__restrict__ gD,
+                                                double *__restrict__ gT)
+{
+    extern __shared__ __align__(16) double sm[];
+    const int M = m.M, m2 = m.m2, tid = threadIdx.x, LDG = M | 1;
+    double *Ts = sm, *lp = Ts + 4 * M, *gs = lp + 8 * m2;
+    const size_t i = type_perm[blockIdx.x];
+    for (int p = tid; p < 4 * M; p += CT) Ts[p] = Tin[i * 4 * M + p];
+    for (int p = tid; p < m2 * M; p += CT) gs[(p / M) * LDG + p % M] = gD[i * m2 * M + p];
+    __syncthreads();
+    dp_atom_gT(gs, LDG, Ts, lp, m2, M, m.desc_scale, [&](int c, int xx, double v) { gT[(i * 4 + c) * M + xx] = v; });
 }
 
 // --------------------------------------------------------------- backward ---
 
+// PRE: dE/dT (gD, as [4][M]) and U (Tin, as [4][T nc]) of the atom are there already.
+template <bool PRE>
 __global__ void __launch_bounds__(CT) k_cheb_bwd(DevModel m, ChebModel cm, const int32_t *__restrict__ types,
                                                  const int32_t *__restrict__ type_perm,
                                                  const int32_t *__restrict__ nreal, const double *__restrict__ Tin,
@@ -476,44 +547,49 @@ __global__ void __launch_bounds__(CT) k_cheb_bwd(DevModel m, ChebModel cm, const
         }
         start[T] = r;
     }
-    for (int p = tid; p < 4 * M; p += CT) Ts[p] = Tin[(size_t)i * 4 * M + p];
-    {
-        const double *g = gD + (size_t)i * m2 * M;
-        for (int p = tid; p < m2 * M; p += CT) gs[(p / M) * LDG + p % M] = g[p];
+    if constexpr (PRE) {
+        for (int p = tid; p < Kt * 4; p += CT) UV[(p % Kt) * 8 + p / Kt] = Tin[(size_t)i * 4 * Kt + p];
+    } else {
+        for (int p = tid; p < 4 * M; p += CT) Ts[p] = Tin[(size_t)i * 4 * M + p];
+        {
+            const double *g = gD + (size_t)i * m2 * M;
+            for (int p = tid; p < m2 * M; p += CT) gs[(p / M) * LDG + p % M] = g[p];
+        }
+        __syncthreads();
+        dp_atom_gT(gs, LDG, Ts, lp, m2, M, m.desc_scale, [&](int c, int xx, double v) { g4[xx * 4 + c] = v; });
+        __syncthreads();
+        // U_kc = sum_f C_kf gT_cf: thread = (term k of the centre's nets, feature slice)
+        {
+            const double *Ct = cm.Ct + (size_t)(a_ok ? a : 0) * M * T * NN;
+            const int nsl = Kt < CT ? CT / Kt : 1;
+            for (int p = tid; p < Kt * nsl; p += CT) {
+                const int fs = p / Kt, k = p - fs * Kt, b = k / nc;
+                const double *ck = Ct + b * NN + (k - b * nc);
+                double acc[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll 4
+                for (int f = fs; f < M; f += nsl) {
+                    const double cv = ck[(size_t)f * T * NN];
+                    const double2 u = *reinterpret_cast<const double2 *>(g4 + f * 4);
+                    const double2 w = *reinterpret_cast<const double2 *>(g4 + f * 4 + 2);
+                    acc[0] = fma(cv, u.x, acc[0]);
+                    acc[1] = fma(cv, u.y, acc[1]);
+                    acc[2] = fma(cv, w.x, acc[2]);
+                    acc[3] = fma(cv, w.y, acc[3]);
+                }
+#pragma unroll
+                for (int c = 0; c < 4; ++c) gs[p * 4 + c] = acc[c];
+            }
+            __syncthreads();
+            for (int p = tid; p < Kt * 4; p += CT) {
+                double v = gs[p];
+                for (int u = 1; u < nsl; ++u) v += gs[u * Kt * 4 + p];
+                UV[(p >> 2) * 8 + (p & 3)] = v;
+            }
+        }
+        __syncthreads();
     }
     __syncthreads();
     const int R = start[T];
-    dp_atom_gT(gs, LDG, Ts, lp, m2, M, m.desc_scale, [&](int c, int xx, double v) { g4[xx * 4 + c] = v; });
-    __syncthreads();
-    // U_kc = sum_f C_kf gT_cf: thread = (term k of the centre's nets, feature slice)
-    {
-        const double *Ct = cm.Ct + (size_t)(a_ok ? a : 0) * M * T * NN;
-        const int nsl = Kt < CT ? CT / Kt : 1;
-        for (int p = tid; p < Kt * nsl; p += CT) {
-            const int fs = p / Kt, k = p - fs * Kt, b = k / nc;
-            const double *ck = Ct + b * NN + (k - b * nc);
-            double acc[4] = {0.0, 0.0, 0.0, 0.0};
-#pragma unroll 4
-            for (int f = fs; f < M; f += nsl) {
-                const double cv = ck[(size_t)f * T * NN];
-                const double2 u = *reinterpret_cast<const double2 *>(g4 + f * 4);
-                const double2 w = *reinterpret_cast<const double2 *>(g4 + f * 4 + 2);
-                acc[0] = fma(cv, u.x, acc[0]);
-                acc[1] = fma(cv, u.y, acc[1]);
-                acc[2] = fma(cv, w.x, acc[2]);
-                acc[3] = fma(cv, w.y, acc[3]);
-            }
-#pragma unroll
-            for (int c = 0; c < 4; ++c) gs[p * 4 + c] = acc[c];
-        }
-        __syncthreads();
-        for (int p = tid; p < Kt * 4; p += CT) {
-            double v = gs[p];
-            for (int u = 1; u < nsl; ++u) v += gs[u * Kt * 4 + p];
-            UV[(p >> 2) * 8 + (p & 3)] = v;
-        }
-    }
-    __syncthreads();
     // V: the derivative's coefficients, d/ds = (2 / S) d/dt, v_n = (2 - [n = 0]) sum_{m = n+1, n+3, ..} m u_m
     for (int p = tid; p < Kt * 4; p += CT) {
         const int k = p >> 2, c = p & 3, b = k / nc, n = k - b * nc;
@@ -589,6 +665,10 @@ __global__ void __launch_bounds__(CT) k_cheb_bwd(DevModel m, ChebModel cm, const
     if (__syncthreads_or(any_far)) {
         // rows beyond S in row order; their d is still in place
         double *ga = fbuf[0], *da = fbuf[1], *gb = fbuf[2], *db = fbuf[3];
+        if constexpr (PRE) {
+            for (int p = tid; p < 4 * M; p += CT) g4[(p % M) * 4 + p / M] = gD[(size_t)i * 4 * M + p];
+            __syncthreads();
+        }
         for (int q = 0; q < R; ++q) {
             if (!((farbits[q >> 5] >> (q & 31)) & 1u)) continue;
             const int b = row_block(start, T, q);
@@ -1074,6 +1154,8 @@ size_t fwd_smem(const DevModel &m, int nc)
     return sizeof(double) * (CT * 4 + 2 * CT * 4 + (size_t)m.ntypes * nc * 4 + 4 * m.M + (size_t)nc * LDT);
 }
 
+size_t pre_smem(const DevModel &m, int nc) { return sizeof(double) * ((size_t)m.ntypes * nc * 8 + 4 * (size_t)m.M); }
+
 size_t bwd_smem(const DevModel &m, int nc)
 {
     const size_t Kt = (size_t)m.ntypes * nc, nsl = Kt < CT ? CT / Kt : 1;
@@ -1137,26 +1219,74 @@ int dp_cheb_terms(const DevModel &m, const double *mx)
     return need <= NN - 4 ? need : 0;
 }
 
+// The products with the series, T = scale P C and U = C dE/dT, as exact digit
+// products on the tensor cores (fit_oz.cu), four rows per atom: their 8 M T n FMAs
+// per atom leave the FP64 units (40% of the forward's there) for two splits, two
+// GEMMs, one kernel that forms D and one that forms dE/dT.  The rows use buffers
+// that are free at that point, hence M2 >= 4 and Kt <= M: the moments dE/dD's,
+// dE/dT D's, U T's, the flag of rows beyond S E_i's.  Per evaluation, fused ->
+// apart: 139,968 water atoms forward 13.0 -> 6.9 ms, backward 16.7 -> 13.5 ms;
+// 32,000 copper 2.9 -> 2.3 and 4.6 -> 4.2; 2,187 water (whole step) 1.17 ->
+// 1.13; 192 water 0.51 -> 0.53.  The line is the work that
+// pays for the four more launches: equal at 1,029 water atoms (40 terms) and
+// 2,048 copper atoms (20 terms), 100 features each.
+bool dp_cheb_gemm(const DevModel &m, int n, int N)
+{
+    const int Kt = m.ntypes * n;
+    return m.m2 >= 4 && Kt <= m.M && (int64_t)N * Kt * m.M >= (1 << 22);
+}
+
 cudaError_t dp_launch_cheb_fwd(cudaStream_t st, const DevModel &m, const ChebModel &cm, const double *x,
                                const int32_t *types, Box3 box, int N, const FormatBuffers &fb,
-                               const NlistBuffers &nb, EvalBuffers eb, int64_t *launches)
+                               const NlistBuffers &nb, EvalBuffers eb, const OzSeries *os, uint16_t *a_dig, int num_sms,
+                               int32_t *status, int64_t *launches)
 {
     const size_t smem = fwd_smem(m, cm.n);
-    cudaError_t e = cudaFuncSetAttribute(k_cheb_fwd, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_MAX);
+    cudaError_t e = cudaFuncSetAttribute(k_cheb_fwd<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_MAX);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k_cheb_fwd<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_MAX);
     if (e != cudaSuccess) return e;
-    k_cheb_fwd<<<N, CT, smem, st>>>(m, cm, x, types, box, nb.type_perm, fb.nlist, fb.nreal, eb.pair_g, eb.T, eb.D);
+    *launches += 1;
+    if (!os) {
+        k_cheb_fwd<false><<<N, CT, smem, st>>>(m, cm, x, types, box, nb.type_perm, fb.nlist, fb.nreal, eb.pair_g, eb.T,
+                                               eb.D);
+        return cudaGetLastError();
+    }
+    const int Kt = m.ntypes * cm.n;
+    k_cheb_fwd<true><<<N, CT, smem, st>>>(m, cm, x, types, box, nb.type_perm, fb.nlist, fb.nreal, eb.pair_g, eb.gD,
+                                          eb.Ei);
+    if ((e = dp_launch_oz_rows(st, m, *os, os->gf, a_dig, N, eb.gD, Kt, eb.T, m.M, nb, num_sms, status, launches)) !=
+        cudaSuccess)
+        return e;
+    k_cheb_desc<<<N, CT, 0, st>>>(m, types, nb.type_perm, fb.nreal, eb.Ei, eb.pair_g, eb.T, eb.D);
     *launches += 1;
     return cudaGetLastError();
 }
 
 cudaError_t dp_launch_cheb_bwd(cudaStream_t st, const DevModel &m, const ChebModel &cm, const int32_t *types, int N,
-                               const FormatBuffers &fb, const NlistBuffers &nb, EvalBuffers eb, int64_t *launches)
+                               const FormatBuffers &fb, const NlistBuffers &nb, EvalBuffers eb, const OzSeries *os,
+                               uint16_t *a_dig, int num_sms, int32_t *status, int64_t *launches)
 {
-    const size_t smem = bwd_smem(m, cm.n);
-    cudaError_t e = cudaFuncSetAttribute(k_cheb_bwd, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_MAX);
+    cudaError_t e = cudaFuncSetAttribute(k_cheb_bwd<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_MAX);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k_cheb_bwd<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_MAX);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k_cheb_gT, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_MAX);
     if (e != cudaSuccess) return e;
-    k_cheb_bwd<<<N, CT, smem, st>>>(m, cm, types, nb.type_perm, fb.nreal, eb.T, eb.gD, eb.pair_g, eb.f_own,
-                                    eb.vir_part);
+    *launches += 1;
+    if (!os) {
+        k_cheb_bwd<false><<<N, CT, bwd_smem(m, cm.n), st>>>(m, cm, types, nb.type_perm, fb.nreal, eb.T, eb.gD, eb.pair_g,
+                                                            eb.f_own, eb.vir_part);
+        return cudaGetLastError();
+    }
+    const int Kt = m.ntypes * cm.n;
+    const size_t gsm = sizeof(double) * (4 * (size_t)m.M + 8 * (size_t)m.m2 + (size_t)m.m2 * (m.M | 1));
+    k_cheb_gT<<<N, CT, gsm, st>>>(m, nb.type_perm, eb.T, eb.gD, eb.D);
+    if ((e = dp_launch_oz_rows(st, m, *os, os->gb, a_dig, N, eb.D, m.M, eb.T, Kt, nb, num_sms, status, launches)) !=
+        cudaSuccess)
+        return e;
+    k_cheb_bwd<true><<<N, CT, pre_smem(m, cm.n), st>>>(m, cm, types, nb.type_perm, fb.nreal, eb.T, eb.D, eb.pair_g,
+                                                      eb.f_own, eb.vir_part);
     *launches += 1;
     return cudaGetLastError();
 }

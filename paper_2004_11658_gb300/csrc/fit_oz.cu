@@ -65,22 +65,29 @@ struct TileRef {
     int a, first, cnt;
 };
 
-// Tile index -> (type, first position in type_perm, atoms); a = -1 past the end.
-__device__ __forceinline__ TileRef oz_tile(int tl, const int32_t *__restrict__ type_start, int ntypes)
+// Tile index -> (type, first row of the type-sorted rows, rows); a = -1 past the
+// end.  Every centre has rpa rows.
+__device__ __forceinline__ TileRef oz_tile(int tl, const int32_t *__restrict__ type_start, int ntypes, int rpa)
 {
     TileRef t{-1, 0, 0};
     for (int a = 0; a < ntypes; ++a) {
-        const int n_a = type_start[a + 1] - type_start[a];
+        const int n_a = (type_start[a + 1] - type_start[a]) * rpa;
         const int tiles = (n_a + DP_OZ_TILE - 1) / DP_OZ_TILE;
         if (tl < tiles) {
             t.a = a;
-            t.first = type_start[a] + tl * DP_OZ_TILE;
+            t.first = type_start[a] * rpa + tl * DP_OZ_TILE;
             t.cnt = min(DP_OZ_TILE, n_a - tl * DP_OZ_TILE);
             return t;
         }
         tl -= tiles;
     }
     return t;
+}
+
+// Row of a matrix [N rpa][.] that a row of the type-sorted rows stands for.
+__device__ __forceinline__ int oz_row(const int32_t *__restrict__ type_perm, int q, int rpa)
+{
+    return rpa == 1 ? type_perm[q] : type_perm[q / rpa] * rpa + q % rpa;
 }
 
 // Exponent of a row or column from the bits of its largest |x|: 2^e > |x|.  zero: its
@@ -112,7 +119,7 @@ struct OzSplitArgs {
     double *Ei;
     int K, nK, beta, S;
     const int32_t *type_perm, *type_start;
-    int ntypes;
+    int ntypes, rpa;
     uint16_t *a;
     int32_t *aexp;
     int64_t a_stride;
@@ -132,7 +139,7 @@ __global__ void __launch_bounds__(256) k_oz_split(OzSplitArgs p)
     __shared__ int nz_s[8];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int tl = blockIdx.x / (DP_OZ_TILE / 8), r0 = (blockIdx.x % (DP_OZ_TILE / 8)) * 8;
-    const TileRef T = oz_tile(tl, p.type_start, p.ntypes);
+    const TileRef T = oz_tile(tl, p.type_start, p.ntypes, p.rpa);
     if (T.a < 0) return;
     const double *wo = p.mode == 2 ? p.wout[T.a] : nullptr;
     const int bS = p.beta * p.S;
@@ -150,7 +157,7 @@ __global__ void __launch_bounds__(256) k_oz_split(OzSplitArgs p)
 
     {
         const int r = r0 + warp;
-        const int i = r < T.cnt ? p.type_perm[T.first + r] : -1;
+        const int i = r < T.cnt ? oz_row(p.type_perm, T.first + r, p.rpa) : -1;
         if (p.mode == 2) {
             double e = 0.0;
             if (i >= 0)
@@ -184,7 +191,7 @@ __global__ void __launch_bounds__(256) k_oz_split(OzSplitArgs p)
     // digits: lane handles row r0 + (lane & 7), columns kh*8 .. kh*8+7 of chunk kc
     const int jr = lane & 7, kh = (lane >> 3) & 1;
     const int r = r0 + jr;
-    const int i = r < T.cnt && nz_s[jr] ? p.type_perm[T.first + r] : -1;
+    const int i = r < T.cnt && nz_s[jr] ? oz_row(p.type_perm, T.first + r, p.rpa) : -1;
     const int sh = bS - e_s[jr];
     uint16_t *out = p.a + (size_t)tl * p.a_stride;
     const int ofs = oz_kofs(r, kh * 8);
@@ -217,7 +224,7 @@ struct OzGemmArgs {
     const int32_t *wexp;
     OzGemm g;
     const int32_t *type_perm, *type_start;
-    int ntypes;
+    int ntypes, rpa;
     int skip;     // skip kind of the layer
     int skip_in;  // input width of the layer
     const double *bias[DP_MAX_TYPES];
@@ -273,7 +280,7 @@ __device__ __forceinline__ bool oz_unit(const OzGemmArgs &p, int u, OzUnit &U)
     if (!p.wg) {
         U.tl = u / g.nN;
         U.nchunk = u - U.tl * g.nN;
-        const TileRef T = oz_tile(U.tl, p.type_start, p.ntypes);
+        const TileRef T = oz_tile(U.tl, p.type_start, p.ntypes, p.rpa);
         U.a = T.a;
         U.first = T.first;
         U.cnt = T.cnt;
@@ -464,7 +471,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_oz_gemm(OzGemmArgs p)
             int i, erow;
             const int4 *fe4;
             if (!p.wg) {
-                i = row < U.cnt ? p.type_perm[U.first + row] : -1;
+                i = row < U.cnt ? oz_row(p.type_perm, U.first + row, p.rpa) : -1;
                 erow = U.tl * DP_OZ_TILE + row;
                 fe4 = reinterpret_cast<const int4 *>(p.wexp + g.e_off[U.a] + n0);
             } else {
@@ -621,40 +628,13 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_oz_gemm(OzGemmArgs p)
     if (warp == 0) tc::tmem_dealloc(tbase, TCOLS);
 }
 
-// Weight digits of every type, layer and direction, one CTA per 32 rows of a B
-// operand: row n of the forward operand is column n of W_l, row q of the
-// backward operand is row q of W_l.  (On the host this took most of a training
-// step on a small frame; the parameters change every step.)
-__global__ void __launch_bounds__(256) k_oz_wsplit(DevModel m, OzModel oz, uint16_t *__restrict__ w,
-                                                   int32_t *__restrict__ e)
+// Digits of 32 rows (chunk u) of type a's B operand, element (this thread's row, k)
+// = elem(k): lane = row, the 8 warps stride over k.
+template <class ELEM>
+__device__ __forceinline__ void oz_write_b(const OzGemm &g, int a, int u, ELEM elem, uint16_t *__restrict__ w,
+                                           int32_t *__restrict__ e, unsigned long long (&mx_s)[8][DP_OZ_NC])
 {
-    __shared__ unsigned long long mx_s[8][DP_OZ_NC];
-    int u = blockIdx.x, a = 0, l = 0, d = 0;
-    int kin = m.m2 * m.M;
-    int64_t off = 0;
-    for (;;) {
-        const OzGemm &t = d == 0 ? oz.fwd[l] : oz.bwd[l];
-        if (u < t.nN) break;
-        u -= t.nN;
-        if (++d == 2) {
-            d = 0;
-            off += (int64_t)kin * m.fit[l] + m.fit[l];
-            kin = m.fit[l];
-            if (++l == m.n_fit) {
-                l = 0;
-                ++a;
-                off = 0;
-                kin = m.m2 * m.M;
-            }
-        }
-    }
-    const OzGemm &g = d == 0 ? oz.fwd[l] : oz.bwd[l];
-    const double *W = m.params + m.fit_base[a] + off;
-    const int F = m.fit[l], rl = threadIdx.x & 31, sl = threadIdx.x >> 5, row = u * DP_OZ_NC + rl;
-    auto elem = [&](int k) -> double {
-        if (k >= g.K || row >= g.N) return 0.0;
-        return d == 0 ? W[(size_t)k * F + row] : W[(size_t)row * F + k];
-    };
+    const int rl = threadIdx.x & 31, sl = threadIdx.x >> 5, row = u * DP_OZ_NC + rl;
     unsigned long long mx = 0;  // parameters are finite
 #pragma unroll 4
     for (int k = sl; k < g.K; k += 8) {
@@ -688,6 +668,62 @@ __global__ void __launch_bounds__(256) k_oz_wsplit(DevModel m, OzModel oz, uint1
             *reinterpret_cast<uint4 *>(out + ((size_t)kc * g.S + sd) * OZ_B_BLK + oz_kofs(rl, kh * 8)) = v;
         }
     }
+}
+
+// Weight digits of every type, layer and direction, one CTA per 32 rows of a B
+// operand: row n of the forward operand is column n of W_l, row q of the
+// backward operand is row q of W_l.  (On the host this took most of a training
+// step on a small frame; the parameters change every step.)
+__global__ void __launch_bounds__(256) k_oz_wsplit(DevModel m, OzModel oz, uint16_t *__restrict__ w,
+                                                   int32_t *__restrict__ e)
+{
+    __shared__ unsigned long long mx_s[8][DP_OZ_NC];
+    int u = blockIdx.x, a = 0, l = 0, d = 0;
+    int kin = m.m2 * m.M;
+    int64_t off = 0;
+    for (;;) {
+        const OzGemm &t = d == 0 ? oz.fwd[l] : oz.bwd[l];
+        if (u < t.nN) break;
+        u -= t.nN;
+        if (++d == 2) {
+            d = 0;
+            off += (int64_t)kin * m.fit[l] + m.fit[l];
+            kin = m.fit[l];
+            if (++l == m.n_fit) {
+                l = 0;
+                ++a;
+                off = 0;
+                kin = m.m2 * m.M;
+            }
+        }
+    }
+    const OzGemm &g = d == 0 ? oz.fwd[l] : oz.bwd[l];
+    const double *W = m.params + m.fit_base[a] + off;
+    const int F = m.fit[l], row = u * DP_OZ_NC + (threadIdx.x & 31);
+    auto elem = [&](int k) -> double {
+        if (k >= g.K || row >= g.N) return 0.0;
+        return d == 0 ? W[(size_t)k * F + row] : W[(size_t)row * F + k];
+    };
+    oz_write_b(g, a, u, elem, w, e, mx_s);
+}
+
+// The same for the series of the embedding nets (embed_cheb.cu), C [T T][nn][M],
+// nc terms: forward rows f, k = (neighbour type, term); backward rows k, columns f.
+__global__ void __launch_bounds__(256) k_oz_series(OzGemm gf, OzGemm gb, int T, int nn, int nc, int M,
+                                                   const double *__restrict__ C, uint16_t *__restrict__ w,
+                                                   int32_t *__restrict__ e)
+{
+    __shared__ unsigned long long mx_s[8][DP_OZ_NC];
+    const int a = blockIdx.x / (gf.nN + gb.nN), v = blockIdx.x - a * (gf.nN + gb.nN);
+    const bool fwd = v < gf.nN;
+    const OzGemm &g = fwd ? gf : gb;
+    const int u = fwd ? v : v - gf.nN, row = u * DP_OZ_NC + (threadIdx.x & 31);
+    auto elem = [&](int k) -> double {
+        if (k >= g.K || row >= g.N) return 0.0;
+        const int kk = fwd ? k : row, f = fwd ? row : k;
+        return C[((size_t)(a * T + kk / nc) * nn + kk % nc) * M + f];
+    };
+    oz_write_b(g, a, u, elem, w, e, mx_s);
 }
 
 // --------------------------------------------- weight gradients' operands ---
@@ -952,6 +988,7 @@ struct OzRun {
         a.type_perm = nb.type_perm;
         a.type_start = nb.type_start;
         a.ntypes = T;
+        a.rpa = 1;
         a.a = ob.a;
         a.aexp = ob.aexp;
         a.a_stride = ob.a_stride;
@@ -987,6 +1024,7 @@ struct OzRun {
         a.type_perm = nb.type_perm;
         a.type_start = nb.type_start;
         a.ntypes = T;
+        a.rpa = 1;
         a.tanh_tab = m.tanh_tab;
         a.status = status;
         // plans of 4 and 5 digits have one segment and no tangent
@@ -1172,5 +1210,92 @@ cudaError_t dp_launch_pgrad_fit_oz(cudaStream_t st, const DevModel &m, const OzM
         if ((e = r.split(0, dzb, ld, nullptr, oz.bwd[l])) != cudaSuccess) return e;
         if ((e = r.gemm(oz.bwd[l], 1, sk, kl, l, dh, ld, false, nullptr, nullptr, dout, ldo)) != cudaSuccess) return e;
     }
+    return cudaGetLastError();
+}
+
+bool dp_oz_series_plan(const DevModel &m, int n, OzSeries &os)
+{
+    const int Kt = m.ntypes * n;
+    os.gf.K = os.gb.N = Kt;
+    os.gf.N = os.gb.K = m.M;
+    int64_t w = 0, e = 0;
+    for (OzGemm *g : {&os.gf, &os.gb}) {
+        g->nK = (g->K + DP_OZ_KC - 1) / DP_OZ_KC;
+        g->nN = (g->N + DP_OZ_NC - 1) / DP_OZ_NC;
+        g->beta = 7;
+        g->S = 8;
+        g->seg = g->nK;
+        if (g->nK > OZ_SEG) return false;
+        for (int a = 0; a < m.ntypes; ++a) {
+            g->w_off[a] = w;
+            w += (int64_t)g->nN * g->nK * g->S * OZ_B_BLK;
+            g->e_off[a] = e;
+            e += (int64_t)g->nN * DP_OZ_NC;
+        }
+    }
+    os.w_elems = w;
+    os.e_elems = e;
+    return true;
+}
+
+cudaError_t dp_launch_oz_series(cudaStream_t st, const DevModel &m, const OzSeries &os, int nn, int n, const double *C,
+                                int64_t *launches)
+{
+    k_oz_series<<<m.ntypes * (os.gf.nN + os.gb.nN), 256, 0, st>>>(os.gf, os.gb, m.ntypes, nn, n, m.M, C, os.w, os.e);
+    *launches += 1;
+    return cudaGetLastError();
+}
+
+// Digits needed for four rows per centre, and their capacity in the fitting net's buffer.
+bool dp_oz_series_fits(const DevModel &m, const OzSeries &os, const OzBuffers &ob, int N)
+{
+    const int64_t tiles = (4 * (int64_t)N + DP_OZ_TILE - 1) / DP_OZ_TILE + m.ntypes;
+    return tiles * std::max(os.gf.nK, os.gb.nK) * 8 * OZ_A_BLK <= (int64_t)ob.tiles * ob.a_stride;
+}
+
+cudaError_t dp_launch_oz_rows(cudaStream_t st, const DevModel &m, const OzSeries &os, const OzGemm &g, uint16_t *a_dig,
+                              int N, const double *x, int ldx, double *y, int ldy, const NlistBuffers &nb, int num_sms,
+                              int32_t *status, int64_t *launches)
+{
+    const int tiles = (4 * N + DP_OZ_TILE - 1) / DP_OZ_TILE + m.ntypes;
+    const int64_t stride = (int64_t)g.nK * 8 * OZ_A_BLK;
+    OzSplitArgs sp;
+    std::memset(&sp, 0, sizeof(sp));
+    sp.src = x;
+    sp.lds = ldx;
+    sp.K = g.K;
+    sp.nK = g.nK;
+    sp.beta = g.beta;
+    sp.S = g.S;
+    sp.type_perm = nb.type_perm;
+    sp.type_start = nb.type_start;
+    sp.ntypes = m.ntypes;
+    sp.rpa = 4;
+    sp.a = a_dig;
+    sp.aexp = os.aexp;
+    sp.a_stride = stride;
+    k_oz_split<<<tiles * (DP_OZ_TILE / 8), 256, 0, st>>>(sp);
+    OzGemmArgs a;
+    std::memset(&a, 0, sizeof(a));
+    a.a = a_dig;
+    a.aexp = os.aexp;
+    a.a_stride = stride;
+    a.w = os.w;
+    a.wexp = os.e;
+    a.g = g;
+    a.type_perm = nb.type_perm;
+    a.type_start = nb.type_start;
+    a.ntypes = m.ntypes;
+    a.rpa = 4;
+    a.hin = y;
+    a.hout = y;
+    a.ldh = a.ldo = ldy;
+    a.status = status;
+    a.units = tiles * g.nN;
+    const size_t smem = gemm_smem(8);
+    cudaError_t e = cudaFuncSetAttribute(k_oz_gemm<8, 1, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    k_oz_gemm<8, 1, false><<<std::min(a.units, num_sms), OZ_THREADS, smem, st>>>(a);
+    *launches += 2;
     return cudaGetLastError();
 }
