@@ -536,6 +536,9 @@ dp_status ensure_oz(dp_ctx *c)
         if ((s = dev_alloc(&ob.t, (size_t)nf * plane, "fitting activations"))) return s;
         if ((s = dev_alloc(&ob.h, 2 * plane, "fitting activations"))) return s;
         if ((s = dev_alloc(&ob.g, 2 * plane, "fitting activations"))) return s;
+        ob.slots = 2 * c->num_sms;
+        if ((s = dev_alloc(&ob.part, (size_t)ob.slots * 32 * 256, "fitting sums"))) return s;
+        if ((s = dev_alloc(&ob.cnt, (size_t)ob.slots * 8, "fitting sums"))) return s;
     }
     if (c->oz_version != c->model->version) {
         GroupTimer tm(c, G_FIT);
@@ -965,7 +968,7 @@ void dp_ctx_free(dp_ctx *c)
                     c->d_energy, c->d_virial, c->md_force, c->ke_part, c->d_inv_mass_conv, c->d_mass,
                     c->eb.fit_t, c->eb.fit_h, c->d_p32, c->d_emb_ops, c->d_fit_fwd, c->d_fit_bwd,
                     c->pb.dT, c->pb.dD, c->pb.Db, c->pb.dDb, c->pb.fit_scr, c->pb.rowscr, c->pb.slices,
-                    c->d_oz_w, c->d_oz_e, c->ob.a, c->ob.aexp, c->ob.t, c->ob.h, c->ob.g, c->d_dtile, c->d_ex_w,
+                    c->d_oz_w, c->d_oz_e, c->ob.a, c->ob.aexp, c->ob.t, c->ob.h, c->ob.g, c->ob.part, c->ob.cnt, c->d_dtile, c->d_ex_w,
                     c->eb.Gst, c->eb.Gmx, c->cb.C, c->cb.Ct, c->cb.V, c->cb.y, c->cb.mx, c->cb.trig, c->cg.mom,
                     c->os.w, c->os.e, c->os.aexp, c->cg.part, c->cg.node, c->cg.far, c->og.a, c->og.b, c->og.exp,
                     c->og.mx, c->og.x};

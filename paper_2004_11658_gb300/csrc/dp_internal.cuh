@@ -341,6 +341,9 @@ struct OzBuffers {
     double *h;              // activations, 2 x [Nmax][fmax]
     double *g;              // gradients, 2 x [Nmax][fmax]
     int64_t nmax;
+    int slots;              // units of one GEMM whose contraction several CTAs may share
+    long long *part;        // their chain sums, [slots][32][256]
+    int32_t *cnt;           // arrivals, [slots][8]
 };
 // Host: shapes of the split GEMMs (returns false if the fitting net is not
 // supported: hidden widths must be <= DP_MAX_FIT_W); device: the weight digits.

@@ -123,6 +123,8 @@ struct OzSplitArgs {
     uint16_t *a;
     int32_t *aexp;
     int64_t a_stride;
+    int32_t *cnt;  // part counters of the GEMM that follows (zeroed here)
+    int ncnt;
 };
 
 // One CTA per group of 8 rows of a tile (a row group of the canonical layout):
@@ -139,6 +141,8 @@ __global__ void __launch_bounds__(256) k_oz_split(OzSplitArgs p)
     __shared__ int nz_s[8];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int tl = blockIdx.x / (DP_OZ_TILE / 8), r0 = (blockIdx.x % (DP_OZ_TILE / 8)) * 8;
+    if (blockIdx.x == 0)
+        for (int q = tid; q < p.ncnt; q += 256) p.cnt[q] = 0;
     const TileRef T = oz_tile(tl, p.type_start, p.ntypes, p.rpa);
     if (T.a < 0) return;
     const double *wo = p.mode == 2 ? p.wout[T.a] : nullptr;
@@ -241,6 +245,10 @@ struct OzGemmArgs {
     // weight gradients Y = X^T Z, contracted over the atoms of each type
     int wg, rows, nq;                 // 1; rows of Y and their tiles
     int64_t out_off[DP_MAX_TYPES];    // of a type's Y in hout
+    // contraction shared by `parts` CTAs: their chain sums [unit][32][256 threads], arrivals per (pair, warp)
+    int parts;
+    long long *part;
+    int32_t *cnt;
 };
 
 // One unit of k_oz_gemm: a 128-row tile of the A operand and a 32-column chunk of Y.
@@ -277,6 +285,8 @@ template <int S>
 __device__ __forceinline__ bool oz_unit(const OzGemmArgs &p, int u, OzUnit &U)
 {
     const OzGemm &g = p.g;
+    const int ks = u % p.parts;
+    u /= p.parts;
     if (!p.wg) {
         U.tl = u / g.nN;
         U.nchunk = u - U.tl * g.nN;
@@ -305,6 +315,12 @@ __device__ __forceinline__ bool oz_unit(const OzGemmArgs &p, int u, OzUnit &U)
         U.bstep = (size_t)g.nN * S * OZ_B_BLK;
         U.as = p.a + kb * U.astep + (size_t)U.tl * S * OZ_A_BLK;
         U.bs = p.w + kb * U.bstep + (size_t)U.nchunk * S * OZ_B_BLK;
+    }
+    if (p.parts > 1) {
+        const int per = (U.nK + p.parts - 1) / p.parts, k0 = ks * per;
+        U.as += k0 * U.astep;
+        U.bs += k0 * U.bstep;
+        U.nK = max(0, min(U.nK - k0, per));
     }
     U.nseg = (U.nK + U.seg - 1) / U.seg;
     return U.a >= 0;
@@ -601,6 +617,35 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_oz_gemm(OzGemmArgs p)
                     release(buf);
                 }
                 if (!ok) break;
+                if (p.parts > 1) {
+                    // the last of the parts to arrive adds the others' sums (integers: in any order)
+                    const int ks = u % p.parts, ub = u - ks;
+                    auto slot = [&](int q, int v) { return p.part + ((size_t)(ub + q) * 32 + v) * 256 + tid; };
+#pragma unroll
+                    for (int h = 0; h < 2; ++h)
+#pragma unroll
+                        for (int n = 0; n < 8; ++n) {
+                            *slot(ks, 16 * h + n) = hi[h][n];
+                            *slot(ks, 16 * h + 8 + n) = lo[h][n];
+                        }
+                    __threadfence();
+                    __syncwarp();
+                    int old = 0;
+                    if (lane == 0) old = atomicAdd(&p.cnt[(u / p.parts) * 8 + warp], 1);
+                    old = __shfl_sync(0xffffffffu, old, 0);
+                    if (old != p.parts - 1) continue;
+                    __threadfence();
+                    for (int q = 0; q < p.parts; ++q) {
+                        if (q == ks) continue;
+#pragma unroll
+                        for (int h = 0; h < 2; ++h)
+#pragma unroll
+                            for (int n = 0; n < 8; ++n) {
+                                hi[h][n] += __ldcg(slot(q, 16 * h + n));
+                                lo[h][n] += __ldcg(slot(q, 16 * h + 8 + n));
+                            }
+                    }
+                }
                 finish(0, hi[0], lo[0], sk[0]);
                 finish(1, hi[1], lo[1], sk[1]);
             } else {
@@ -750,9 +795,12 @@ struct OzColsPair {
 
 // Column maxima: threads on columns, CTAs on shares of the type-sorted atoms.
 __global__ void __launch_bounds__(128) k_oz_colmax(OzColsPair pr, const int32_t *__restrict__ type_perm,
-                                                   const int32_t *__restrict__ type_start, int N)
+                                                   const int32_t *__restrict__ type_start, int N,
+                                                   int32_t *__restrict__ cnt, int ncnt)
 {
     const OzCols &o = pr.c[blockIdx.z];
+    if (blockIdx.x + blockIdx.y + blockIdx.z == 0)  // part counters of the GEMM that follows
+        for (int u = threadIdx.x; u < ncnt; u += 128) cnt[u] = 0;
     const int q = blockIdx.x * 128 + threadIdx.x;
     if (q >= o.K) return;
     const int lo = (int)((long long)blockIdx.y * N / gridDim.y), hi = (int)((long long)(blockIdx.y + 1) * N / gridDim.y);
@@ -870,6 +918,18 @@ void oz_plan_gemm(OzGemm &g, int bits)
     }
     g.beta = 0;
     g.S = 0;
+}
+
+// CTAs that share one long contraction (more than one segment) when the (tile,
+// column chunk) pairs would leave half of the SMs idle or more: exact integer
+// sums, so the result does not depend on the split.  A part keeps 8 chunks or
+// more, below which its fixed costs (sums written and read, 64 KB) outweigh the
+// MMAs (1.15 k cycles a chunk).  One CTA per pair took 88 us for the first layer
+// of 192 water atoms and 321 us for a weight gradient over 12,288; now 44 and 54 us
+// (95 us for the 240 x 240 weights, 321 before).
+int oz_parts(int pairs, int nK, int num_sms)
+{
+    return std::max(1, std::min(num_sms / std::max(pairs, 1), nK / 8));
 }
 
 size_t gemm_smem(int S) { return (size_t)OZ_NST * S * (OZ_A_BLK + OZ_B_BLK) * 2 + OZ_TAB_BYTES; }
@@ -992,6 +1052,8 @@ struct OzRun {
         a.a = ob.a;
         a.aexp = ob.aexp;
         a.a_stride = ob.a_stride;
+        a.cnt = ob.cnt;
+        a.ncnt = g.seg < g.nK ? ob.slots * 8 : 0;
         k_oz_split<<<tiles * (DP_OZ_TILE / 8), 256, 0, st>>>(a);
         *launches += 1;
         return cudaGetLastError();
@@ -1027,6 +1089,14 @@ struct OzRun {
         a.rpa = 1;
         a.tanh_tab = m.tanh_tab;
         a.status = status;
+        // the type partition makes at most T - 1 tiles more than the atoms fill
+        const int nK = a.wg ? N / (DP_OZ_KC * T) : a.g.nK;
+        const int pairs = a.wg ? a.units : (N + DP_OZ_TILE - 1) / DP_OZ_TILE * a.g.nN;
+        a.parts = 1;
+        if (a.wg || a.g.seg < a.g.nK) a.parts = std::max(1, std::min(oz_parts(pairs, nK, num_sms), ob.slots / a.units));
+        a.units *= a.parts;
+        a.part = ob.part;
+        a.cnt = ob.cnt;
         // plans of 4 and 5 digits have one segment and no tangent
         if (a.g.S == 8) return launch_epi<8>(a, epi);
         if (a.g.S == 5) return epi == 0 ? launch_as<5, 0, false>(a) : launch_as<5, 1, false>(a);
@@ -1161,7 +1231,8 @@ cudaError_t dp_launch_pgrad_fit_oz(cudaStream_t st, const DevModel &m, const OzM
             cudaError_t e2 = cudaMemsetAsync(og.mx, 0, 8 * (size_t)T * (nq * DP_OZ_TILE + nN * DP_OZ_NC), st);
             if (e2 != cudaSuccess) return e2;
             const int cols = std::max(K, F);
-            k_oz_colmax<<<dim3((cols + 127) / 128, splits, 2), 128, 0, st>>>(c, nb.type_perm, nb.type_start, N);
+            k_oz_colmax<<<dim3((cols + 127) / 128, splits, 2), 128, 0, st>>>(c, nb.type_perm, nb.type_start, N, ob.cnt,
+                                                                                 ob.slots * 8);
             k_oz_tsplit<<<dim3(N / DP_OZ_KC + T, std::max(nq, (nN * DP_OZ_NC + 127) / 128), 2), 256, 0, st>>>(
                 c, nb.type_perm, nb.type_start, T);
             *launches += 2;
@@ -1280,6 +1351,7 @@ cudaError_t dp_launch_oz_rows(cudaStream_t st, const DevModel &m, const OzSeries
     a.a = a_dig;
     a.aexp = os.aexp;
     a.a_stride = stride;
+    a.parts = 1;
     a.w = os.w;
     a.wexp = os.e;
     a.g = g;
