@@ -37,7 +37,7 @@
 // returns.
 //
 // Measured per evaluation (12,288 water atoms): the six GEMMs 2.8 -> 1.14 ms,
-// the six splits 0.74 -> 0.43 ms; 192 atoms: the whole fitting net 0.96 -> 0.29
+// the six splits 0.74 -> 0.33 ms; 192 atoms: the whole fitting net 0.96 -> 0.25
 // ms.  One elected lane of a whole warp issues: behind `threadIdx.x == 0` the
 // same MMAs took 139 cycles each instead of 97 in the former kernel.
 #include <algorithm>
@@ -125,7 +125,24 @@ struct OzSplitArgs {
     int64_t a_stride;
     int32_t *cnt;  // part counters of the GEMM that follows (zeroed here)
     int ncnt;
+    int vec;       // rows start on 16 bytes
 };
+
+// Digits sd of 8 values (with their bias, oz_digit_bias) as 8 BF16: the digit
+// sits in a float's mantissa and one subtraction makes it the float's value.
+template <int S, int B>
+__device__ __forceinline__ uint4 oz_pack_digits(const long long (&J)[8], int sd)
+{
+    uint32_t f[8];
+#pragma unroll
+    for (int q = 0; q < 8; ++q)
+        f[q] = sd == 0 ? __float_as_uint(__uint_as_float(0x4B400000u + (uint32_t)(int)(J[q] >> (B * (S - 1)))) - 12582912.f)
+                       : __float_as_uint(__uint_as_float(0x4B000000u | ((uint32_t)(J[q] >> (B * (S - 1 - sd))) &
+                                                                        ((1u << B) - 1))) -
+                                         (8388608.f + (float)((1 << (B - 1)) - 1)));
+    return make_uint4(__byte_perm(f[0], f[1], 0x7632), __byte_perm(f[2], f[3], 0x7632),
+                      __byte_perm(f[4], f[5], 0x7632), __byte_perm(f[6], f[7], 0x7632));
+}
 
 // One CTA per group of 8 rows of a tile (a row group of the canonical layout):
 // warp w takes the exponent (and output-layer energy) of row w, then every
@@ -133,20 +150,26 @@ struct OzSplitArgs {
 // lane = row (0..7) + 8 * (column half) + 16 * (chunk parity), the warps
 // striding over the chunk pairs.  (One warp per row group, rows one after the
 // other, took 277 us for the descriptors of 12,288 water atoms and 181 us for
-// 192: a chain of dependent loads on few warps.)  The conversions run on the
-// integer pipe.
+// 192: a chain of dependent loads on few warps.)  When the row groups are few,
+// gridDim.y CTAs share one: each finds the exponents, and writes its share of the
+// chunks.  Bound by instruction issue: the value's bits are rounded to an integer
+// on the integer pipe, its digits read from their places without a carry chain
+// and converted by one FP32 subtraction.  With a chain, a conversion instruction
+// per digit and 8-byte loads the descriptors of 12,288 atoms took 175 us and
+// those of 192 atoms 32 us; now 113 and 15 us.
+template <int S, int B>
 __global__ void __launch_bounds__(256) k_oz_split(OzSplitArgs p)
 {
     __shared__ int e_s[8];
     __shared__ int nz_s[8];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int tl = blockIdx.x / (DP_OZ_TILE / 8), r0 = (blockIdx.x % (DP_OZ_TILE / 8)) * 8;
-    if (blockIdx.x == 0)
+    if (blockIdx.x + blockIdx.y == 0)
         for (int q = tid; q < p.ncnt; q += 256) p.cnt[q] = 0;
     const TileRef T = oz_tile(tl, p.type_start, p.ntypes, p.rpa);
     if (T.a < 0) return;
     const double *wo = p.mode == 2 ? p.wout[T.a] : nullptr;
-    const int bS = p.beta * p.S;
+    constexpr int bS = B * S;
 
     // value of column k of atom i (0 past the row's end or the tile's atoms)
     auto value = [&](int i, int k) -> double {
@@ -168,15 +191,27 @@ __global__ void __launch_bounds__(256) k_oz_split(OzSplitArgs p)
                 for (int k = lane; k < p.K; k += 32) e = fma(p.src[(size_t)i * p.lds + k], wo[k], e);
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) e += __shfl_xor_sync(0xffffffffu, e, o);
-            if (i >= 0 && lane == 0) p.Ei[i] = *p.bout[T.a] + e;
+            if (i >= 0 && lane == 0 && blockIdx.y == 0) p.Ei[i] = *p.bout[T.a] + e;
         }
         // largest |x| by its bits; a row with an infinity or NaN gives NaN
         unsigned long long mx = 0;
-#pragma unroll 4
-        for (int k = lane; k < p.K; k += 32) {
-            const unsigned long long b = (unsigned long long)__double_as_longlong(fabs(value(i, k)));
+        auto larger = [&](double v) {
+            const unsigned long long b = (unsigned long long)__double_as_longlong(fabs(v));
             mx = b > mx ? b : mx;
+        };
+        int k0 = 0;  // columns taken two at a time
+        if (p.mode == 0 && p.vec && i >= 0) {
+            const double *x = p.src + (size_t)i * p.lds;
+            k0 = p.K & ~1;
+#pragma unroll 8
+            for (int k = 2 * lane; k < k0; k += 64) {
+                const double2 v = *reinterpret_cast<const double2 *>(x + k);
+                larger(v.x);
+                larger(v.y);
+            }
         }
+#pragma unroll 4
+        for (int k = k0 + lane; k < p.K; k += 32) larger(value(i, k));
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) {
             const unsigned long long q = __shfl_xor_sync(0xffffffffu, mx, o);
@@ -187,7 +222,7 @@ __global__ void __launch_bounds__(256) k_oz_split(OzSplitArgs p)
             const int e = oz_exponent(mx, bS, zero);
             e_s[warp] = e;
             nz_s[warp] = !zero;
-            p.aexp[(size_t)tl * DP_OZ_TILE + r] = e;
+            if (blockIdx.y == 0) p.aexp[(size_t)tl * DP_OZ_TILE + r] = e;
         }
     }
     __syncthreads();
@@ -199,23 +234,56 @@ __global__ void __launch_bounds__(256) k_oz_split(OzSplitArgs p)
     const int sh = bS - e_s[jr];
     uint16_t *out = p.a + (size_t)tl * p.a_stride;
     const int ofs = oz_kofs(r, kh * 8);
-    for (int kc = 2 * warp + (lane >> 4); kc < p.nK; kc += 16) {
+    for (int kc = 2 * (warp + 8 * blockIdx.y) + (lane >> 4); kc < p.nK; kc += 16 * gridDim.y) {
         const int k8 = kc * DP_OZ_KC + kh * 8;
-        long long I[8];
+        long long J[8];
+        double v[8];
+        if (p.vec && i >= 0 && k8 + 8 <= p.K) {
+            const double *x = p.mode == 2 ? wo + k8 : p.src + (size_t)i * p.lds + k8;
+            if (p.mode == 2) {
 #pragma unroll
-        for (int q = 0; q < 8; ++q) I[q] = oz_rint_pow2(value(i, k8 + q), sh);
-        for (int sd = p.S - 1; sd >= 0; --sd) {
-            int d[8];
+                for (int q = 0; q < 8; ++q) v[q] = x[q];
+            } else {
 #pragma unroll
-            for (int q = 0; q < 8; ++q) d[q] = sd > 0 ? oz_digit_step(I[q], p.beta) : (int)I[q];
-            uint4 u;
-            u.x = (uint32_t)oz_bf16_int(d[0]) | ((uint32_t)oz_bf16_int(d[1]) << 16);
-            u.y = (uint32_t)oz_bf16_int(d[2]) | ((uint32_t)oz_bf16_int(d[3]) << 16);
-            u.z = (uint32_t)oz_bf16_int(d[4]) | ((uint32_t)oz_bf16_int(d[5]) << 16);
-            u.w = (uint32_t)oz_bf16_int(d[6]) | ((uint32_t)oz_bf16_int(d[7]) << 16);
-            *reinterpret_cast<uint4 *>(out + ((size_t)kc * p.S + sd) * OZ_A_BLK + ofs) = u;
+                for (int q = 0; q < 8; q += 2) {
+                    const double2 u = *reinterpret_cast<const double2 *>(x + q);
+                    v[q] = u.x;
+                    v[q + 1] = u.y;
+                }
+            }
+            if (p.mode != 0) {
+                const double *tv = p.tv + (size_t)i * p.ldt + k8;
+#pragma unroll
+                for (int q = 0; q < 8; q += 2) {
+                    const double2 t = *reinterpret_cast<const double2 *>(tv + q);
+                    v[q] *= fma(-t.x, t.x, 1.0);
+                    v[q + 1] *= fma(-t.y, t.y, 1.0);
+                }
+            }
+        } else {
+#pragma unroll
+            for (int q = 0; q < 8; ++q) v[q] = value(i, k8 + q);
         }
+#pragma unroll
+        for (int q = 0; q < 8; ++q) J[q] = oz_rint_pow2(v[q], sh) + oz_digit_bias(S, B);
+#pragma unroll
+        for (int sd = 0; sd < S; ++sd)
+            *reinterpret_cast<uint4 *>(out + ((size_t)kc * S + sd) * OZ_A_BLK + ofs) = oz_pack_digits<S, B>(J, sd);
     }
+}
+
+cudaError_t launch_split(cudaStream_t st, OzSplitArgs &a, int tiles, int num_sms)
+{
+    const auto odd = [](const void *p, int ld) { return ((uintptr_t)p & 15) != 0 || (ld & 1) != 0; };
+    a.vec = !((a.mode != 2 && odd(a.src, a.lds)) || (a.mode != 0 && odd(a.tv, a.ldt)));
+    const int groups = tiles * (DP_OZ_TILE / 8);
+    // up to 4 CTAs per SM; 16 chunks are one pass of a CTA
+    const dim3 grid(groups, std::max(1, std::min(4 * num_sms / groups, (a.nK + 15) / 16)));
+    if (a.S == 8 && a.beta == 7) k_oz_split<8, 7><<<grid, 256, 0, st>>>(a);
+    else if (a.S == 4 && a.beta == 7) k_oz_split<4, 7><<<grid, 256, 0, st>>>(a);
+    else if (a.S == 5 && a.beta == 6) k_oz_split<5, 6><<<grid, 256, 0, st>>>(a);
+    else return cudaErrorInvalidValue;
+    return cudaGetLastError();
 }
 
 // ------------------------------------------------------------------- gemm --
@@ -778,7 +846,7 @@ __global__ void __launch_bounds__(256) k_oz_series(OzGemm gf, OzGemm gb, int T, 
 // digits of the columns of X (rows of the A operand) and of Zb (rows of the B
 // operand), scaled per column and type by its largest magnitude over the atoms.
 // The whole fitting part on the FP64 units, with per-CTA gradient slices, took 63
-// ms for 12,288 water atoms with the student's widths, now 4.0 ms; 648 atoms at
+// ms for 12,288 water atoms with the student's widths, now 2.6 ms; 648 atoms at
 // full width: 23 -> 0.8 ms (24 GEMMs and 14 splits, bound as k_oz_gemm).
 
 struct OzCols {
@@ -838,26 +906,18 @@ __global__ void __launch_bounds__(256) k_oz_tsplit(OzColsPair pr, const int32_t 
     bool zero;
     const int ex = oz_exponent(q == o.one ? 0x3ff0000000000000ull : q < o.K ? o.mx[col] : 0, beta * S, zero);
     if (kc == 0 && kh == 0) o.exp[col] = ex;
-    long long I[8];
+    long long J[8];
 #pragma unroll
     for (int u = 0; u < 8; ++u) {
         const int p = type_start[a] + kc * DP_OZ_KC + kh * 8 + u;
         double v = 0.0;
         if (!zero && p < type_start[a + 1]) v = q == o.one ? 1.0 : o.src[(size_t)type_perm[p] * o.ld + q];
-        I[u] = oz_rint_pow2(v, beta * S - ex);
+        J[u] = oz_rint_pow2(v, beta * S - ex) + oz_digit_bias(S, beta);
     }
     uint16_t *out = o.out + ((size_t)blockIdx.x * o.nb + q / o.rb) * S * o.rb * DP_OZ_KC + oz_kofs(q % o.rb, kh * 8);
-    for (int sd = S - 1; sd >= 0; --sd) {
-        int d[8];
 #pragma unroll
-        for (int u = 0; u < 8; ++u) d[u] = sd > 0 ? oz_digit_step(I[u], beta) : (int)I[u];
-        uint4 v;
-        v.x = (uint32_t)oz_bf16_int(d[0]) | ((uint32_t)oz_bf16_int(d[1]) << 16);
-        v.y = (uint32_t)oz_bf16_int(d[2]) | ((uint32_t)oz_bf16_int(d[3]) << 16);
-        v.z = (uint32_t)oz_bf16_int(d[4]) | ((uint32_t)oz_bf16_int(d[5]) << 16);
-        v.w = (uint32_t)oz_bf16_int(d[6]) | ((uint32_t)oz_bf16_int(d[7]) << 16);
-        *reinterpret_cast<uint4 *>(out + (size_t)sd * o.rb * DP_OZ_KC) = v;
-    }
+    for (int sd = 0; sd < S; ++sd)
+        *reinterpret_cast<uint4 *>(out + (size_t)sd * o.rb * DP_OZ_KC) = oz_pack_digits<S, beta>(J, sd);
 }
 
 // Adjoints of the output layer: hb = cE w_out, dhb = -w_out of the atom's type,
@@ -1054,9 +1114,8 @@ struct OzRun {
         a.a_stride = ob.a_stride;
         a.cnt = ob.cnt;
         a.ncnt = g.seg < g.nK ? ob.slots * 8 : 0;
-        k_oz_split<<<tiles * (DP_OZ_TILE / 8), 256, 0, st>>>(a);
         *launches += 1;
-        return cudaGetLastError();
+        return launch_split(st, a, tiles, num_sms);
     }
 
     template <int S, int EPI, bool SEG>
@@ -1345,7 +1404,8 @@ cudaError_t dp_launch_oz_rows(cudaStream_t st, const DevModel &m, const OzSeries
     sp.a = a_dig;
     sp.aexp = os.aexp;
     sp.a_stride = stride;
-    k_oz_split<<<tiles * (DP_OZ_TILE / 8), 256, 0, st>>>(sp);
+    cudaError_t e = launch_split(st, sp, tiles, num_sms);
+    if (e != cudaSuccess) return e;
     OzGemmArgs a;
     std::memset(&a, 0, sizeof(a));
     a.a = a_dig;
@@ -1365,7 +1425,7 @@ cudaError_t dp_launch_oz_rows(cudaStream_t st, const DevModel &m, const OzSeries
     a.status = status;
     a.units = tiles * g.nN;
     const size_t smem = gemm_smem(8);
-    cudaError_t e = cudaFuncSetAttribute(k_oz_gemm<8, 1, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    e = cudaFuncSetAttribute(k_oz_gemm<8, 1, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     k_oz_gemm<8, 1, false><<<std::min(a.units, num_sms), OZ_THREADS, smem, st>>>(a);
     *launches += 2;

@@ -29,6 +29,21 @@ static __host__ __device__ __forceinline__ int oz_digit_step(long long &I, int b
     return (int)r;
 }
 
+// The same digits without the carry chain: with 2^(beta-1) - 1 added in every
+// place but the first, place q of I + bias holds digit + 2^(beta-1) - 1, between 0
+// and 2^beta - 1, and the first place the first digit.
+static __host__ __device__ constexpr long long oz_digit_bias(int S, int beta)
+{
+    long long c = 0;
+    for (int q = 0; q < S - 1; ++q) c += ((1ll << (beta - 1)) - 1) << (beta * q);
+    return c;
+}
+static __host__ __device__ __forceinline__ int oz_digit_at(long long J, int S, int beta, int sd)
+{
+    const long long r = J >> (beta * (S - 1 - sd));
+    return sd == 0 ? (int)r : (int)(r & ((1ll << beta) - 1)) - ((1 << (beta - 1)) - 1);
+}
+
 // BF16 bits of a small integer (|d| <= 256): exact.
 static __host__ __device__ __forceinline__ uint16_t oz_bf16_int(int d)
 {
