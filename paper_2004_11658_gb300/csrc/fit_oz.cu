@@ -60,6 +60,7 @@ constexpr uint32_t OZ_TAB_BYTES = DP_TANH_NINT * DP_TANH_STRIDE * 8;
 static_assert(OZ_TAB_BYTES % 16 == 0, "bulk copy of the tanh table");
 constexpr int OZ_A_BLK = DP_OZ_TILE * DP_OZ_KC;  // elements of one A digit chunk (128 x 16)
 constexpr int OZ_B_BLK = DP_OZ_NC * DP_OZ_KC;    // elements of one W digit chunk (32 x 16)
+constexpr int OZ_KEEP = 256;                     // columns of a row that k_oz_split may keep between its passes
 
 struct TileRef {
     int a, first, cnt;
@@ -126,6 +127,7 @@ struct OzSplitArgs {
     int32_t *cnt;  // part counters of the GEMM that follows (zeroed here)
     int ncnt;
     int vec;       // rows start on 16 bytes
+    int keep;      // columns of a row kept in shared memory (0: none)
 };
 
 // Digits sd of 8 values (with their bias, oz_digit_bias) as 8 BF16: the digit
@@ -154,7 +156,10 @@ __device__ __forceinline__ uint4 oz_pack_digits(const long long (&J)[8], int sd)
 // gridDim.y CTAs share one: each finds the exponents, and writes its share of the
 // chunks.  Bound by instruction issue: the value's bits are rounded to an integer
 // on the integer pipe, its digits read from their places without a carry chain
-// and converted by one FP32 subtraction.  With a chain, a conversion instruction
+// and converted by one FP32 subtraction.  Products (1 - t^2) x of up to 256
+// columns stay in shared memory between the passes (formed twice, 240 columns of
+// 12,288 atoms took 52 us, now 43; plain values are read again: keeping them took
+// 28 instead of 26 us).  With a chain, a conversion instruction
 // per digit and 8-byte loads the descriptors of 12,288 atoms took 175 us and
 // those of 192 atoms 32 us; now 113 and 15 us.
 template <int S, int B>
@@ -162,6 +167,8 @@ __global__ void __launch_bounds__(256) k_oz_split(OzSplitArgs p)
 {
     __shared__ int e_s[8];
     __shared__ int nz_s[8];
+    extern __shared__ __align__(16) double v_s[];  // kept rows
+    const bool keep = p.keep != 0;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int tl = blockIdx.x / (DP_OZ_TILE / 8), r0 = (blockIdx.x % (DP_OZ_TILE / 8)) * 8;
     if (blockIdx.x + blockIdx.y == 0)
@@ -200,7 +207,15 @@ __global__ void __launch_bounds__(256) k_oz_split(OzSplitArgs p)
             mx = b > mx ? b : mx;
         };
         int k0 = 0;  // columns taken two at a time
-        if (p.mode == 0 && p.vec && i >= 0) {
+        if (keep) {
+#pragma unroll 4
+            for (int k = lane; k < p.nK * DP_OZ_KC; k += 32) {
+                const double v = value(i, k);
+                v_s[warp * p.keep + k] = v;
+                larger(v);
+            }
+            k0 = p.K;
+        } else if (p.mode == 0 && p.vec && i >= 0) {
             const double *x = p.src + (size_t)i * p.lds;
             k0 = p.K & ~1;
 #pragma unroll 8
@@ -238,7 +253,14 @@ __global__ void __launch_bounds__(256) k_oz_split(OzSplitArgs p)
         const int k8 = kc * DP_OZ_KC + kh * 8;
         long long J[8];
         double v[8];
-        if (p.vec && i >= 0 && k8 + 8 <= p.K) {
+        if (keep) {
+#pragma unroll
+            for (int q = 0; q < 8; q += 2) {
+                const double2 u = *reinterpret_cast<const double2 *>(v_s + jr * p.keep + k8 + q);
+                v[q] = i < 0 ? 0.0 : u.x;
+                v[q + 1] = i < 0 ? 0.0 : u.y;
+            }
+        } else if (p.vec && i >= 0 && k8 + 8 <= p.K) {
             const double *x = p.mode == 2 ? wo + k8 : p.src + (size_t)i * p.lds + k8;
             if (p.mode == 2) {
 #pragma unroll
@@ -276,12 +298,15 @@ cudaError_t launch_split(cudaStream_t st, OzSplitArgs &a, int tiles, int num_sms
 {
     const auto odd = [](const void *p, int ld) { return ((uintptr_t)p & 15) != 0 || (ld & 1) != 0; };
     a.vec = !((a.mode != 2 && odd(a.src, a.lds)) || (a.mode != 0 && odd(a.tv, a.ldt)));
+    // rows 16 bytes apart in the banks
+    a.keep = a.mode != 0 && a.K <= OZ_KEEP ? a.nK * DP_OZ_KC + 2 : 0;
+    const size_t smem = (size_t)a.keep * 8 * sizeof(double);
     const int groups = tiles * (DP_OZ_TILE / 8);
     // up to 4 CTAs per SM; 16 chunks are one pass of a CTA
     const dim3 grid(groups, std::max(1, std::min(4 * num_sms / groups, (a.nK + 15) / 16)));
-    if (a.S == 8 && a.beta == 7) k_oz_split<8, 7><<<grid, 256, 0, st>>>(a);
-    else if (a.S == 4 && a.beta == 7) k_oz_split<4, 7><<<grid, 256, 0, st>>>(a);
-    else if (a.S == 5 && a.beta == 6) k_oz_split<5, 6><<<grid, 256, 0, st>>>(a);
+    if (a.S == 8 && a.beta == 7) k_oz_split<8, 7><<<grid, 256, smem, st>>>(a);
+    else if (a.S == 4 && a.beta == 7) k_oz_split<4, 7><<<grid, 256, smem, st>>>(a);
+    else if (a.S == 5 && a.beta == 6) k_oz_split<5, 6><<<grid, 256, smem, st>>>(a);
     else return cudaErrorInvalidValue;
     return cudaGetLastError();
 }
