@@ -19,8 +19,8 @@
 // every partial sum of every C_g is below 2^24: the FP32 tensor-core
 // accumulators hold C_g exactly, in any summation order.  A longer contraction
 // is cut into segments that satisfy this, added up in int64 (FP64 mode: 8 digits
-// of 7 bits throughout, 36 MMAs per 16 columns and 8 planes to read; 66 and 11
-// for the 1,600-long first layer when one segment had to hold it, with 5-bit
+// of 7 bits throughout, 36 products per 16 columns and 8 planes to read; 66 and
+// 11 for the 1,600-long first layer when one segment had to hold it, with 5-bit
 // digits).  The result is the exact product of the digit expansions, rounded
 // once into FP64, and is reproducible bit for bit.
 //
@@ -29,17 +29,17 @@
 // (16-column chunks); k_oz_wsplit: the weights', once per set of parameters.
 // k_oz_gemm: persistent over (tile, 32-column chunk of Y); a copy warp streams
 // the digit chunks of A and W (cp.async.bulk, a 4-stage ring on mbarriers), an
-// MMA warp issues S(S+1)/2 MMAs of 128 x 32 x 16 per chunk into S group
-// accumulators in tensor memory, and 8 warps combine the groups exactly, round
+// MMA warp issues the S(S+1)/2 digit products of 128 x 32 x 16 of a chunk as S
+// MMAs into S group accumulators in tensor memory, and 8 warps combine the groups exactly, round
 // once and apply the layer's bias, tanh and skip (forward) or the skip gradient
 // (backward).  Every wait is bounded; on a timeout the kernel sets
 // DPF_MMA_TIMEOUT, waits for its copies and MMAs, frees tensor memory and
 // returns.
 //
-// Measured per evaluation (12,288 water atoms): the six GEMMs 2.8 -> 1.14 ms,
-// the six splits 0.74 -> 0.33 ms; 192 atoms: the whole fitting net 0.96 -> 0.25
-// ms.  One elected lane of a whole warp issues: behind `threadIdx.x == 0` the
-// same MMAs took 139 cycles each instead of 97 in the former kernel.
+// Measured per evaluation (12,288 water atoms): the six GEMMs 2.8 -> 1.0 ms, the
+// six splits 0.74 -> 0.30 ms; 192 atoms: the whole fitting net 0.96 -> 0.24 ms.
+// One elected lane of a whole warp issues: behind `threadIdx.x == 0` the same MMAs
+// took 139 cycles each instead of 97 in the former kernel.
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -427,12 +427,16 @@ __device__ __forceinline__ bool oz_unit(const OzGemmArgs &p, int u, OzUnit &U)
 // of the next.  A contraction longer than the accumulators hold exactly is cut
 // into segments of g.seg chunks, which the epilogue adds up in int64.
 //
-// Bounds, per unit of a 240-long contraction at S = 8: 15 chunks x 36 MMAs of
-// 20 cycles with A held in the collector (40 without, and 40 when two CTAs of
-// one SM alternate: measured) = 10.8 k cycles, 40 KB of copies per chunk at the
-// 60 B/clk that large bulk copies reach = 10.3 k; with the FP64 tanh 20 k
-// cycles of FP64 pipe.  The tanh table sits in shared memory: its lookups by 32
-// lanes cost 32 wavefronts each through L1, and were 53 k cycles per unit.
+// Bounds, per unit of a 240-long contraction at S = 8: 15 chunks of 1,152
+// accumulator columns at half a cycle = 8.6 k cycles of MMAs; 40 KB of copies per
+// chunk, 10.3 k at the 60 B/clk that large bulk copies reach alone; with the FP64
+// tanh 20 k cycles of FP64 pipe.  As 36 MMAs of N = 32 per chunk (20 cycles each
+// with A in the collector, 40 without) the chunk took a fifth longer: the first
+// layer of 12,288 atoms 392 us, now 324, the gradient to the descriptor 332 and
+// 274.  What is left there is the copies: every SM reads a tile's digits again
+// for each of its column chunks, 3 GB in 274 us out of L2.  The tanh table sits
+// in shared memory: its lookups by 32 lanes cost 32 wavefronts each through L1,
+// and were 53 k cycles per unit.
 template <int S, int EPI, bool SEG>
 __global__ void __launch_bounds__(OZ_THREADS, 1) k_oz_gemm(OzGemmArgs p)
 {
@@ -498,30 +502,22 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_oz_gemm(OzGemmArgs p)
         for (int q = c > NST ? c - NST : 0; q < c; ++q) tc::mbar_wait(&full[q % NST], (q / NST) & 1);
         if (EPI == 0) tc::mbar_wait(&tabbar, 0);
     } else if (warp == 8) {
-        const uint32_t idesc = tc::make_idesc_bf16(DP_OZ_TILE, DP_OZ_NC);
         // the MMAs of one chunk, then the commit that frees its stage; one copy of
-        // the code per stage, so that every descriptor is a constant
+        // the code per stage, so that every descriptor is a constant.  Digit s of A
+        // meets the digits t = 1 .. S + 1 - s of W in one MMA of N = 32 (S + 1 - s):
+        // W's digit planes lie one after the other, 32 rows each, and so do the
+        // accumulators of the groups s + t
         auto issue = [&](auto stage, uint32_t dbase, bool acc0) {
             constexpr int st = decltype(stage)::value;
             // descriptors of digit plane 1; plane s is (s - 1) blocks further (the
             // address field holds bytes / 16 and stays below 2^14 inside shared memory)
             const uint32_t abase = tc::smem_u32(smraw) + st * stage_bytes;
             const uint64_t ad0 = tc::make_desc(abase, 128, 256);
-            const uint64_t bd0 = tc::make_desc(abase + a_bytes, 128, 256);
+            const uint64_t bd = tc::make_desc(abase + a_bytes, 128, 256);
 #pragma unroll
-            for (int s = 1; s <= S; ++s) {
-                const uint64_t ad = ad0 + (uint64_t)((s - 1) * OZ_A_BLK * 2 / 16);
-#pragma unroll
-                for (int t = 1; t + s <= S + 1; ++t) {
-                    const uint32_t dc = dbase + (uint32_t)(s + t - 2) * DP_OZ_NC;
-                    const uint64_t bd = bd0 + (uint64_t)((t - 1) * OZ_B_BLK * 2 / 16);
-                    const bool acc = acc0 || s > 1;
-                    if (s == S) tc::mma_bf16(dc, ad, bd, idesc, acc);
-                    else if (t == 1) tc::mma_bf16_a<0>(dc, ad, bd, idesc, acc);
-                    else if (t + s <= S) tc::mma_bf16_a<1>(dc, ad, bd, idesc, acc);
-                    else tc::mma_bf16_a<2>(dc, ad, bd, idesc, acc);
-                }
-            }
+            for (int s = 1; s <= S; ++s)
+                tc::mma_bf16(dbase + (uint32_t)(s - 1) * DP_OZ_NC, ad0 + (uint64_t)((s - 1) * OZ_A_BLK * 2 / 16), bd,
+                             tc::make_idesc_bf16(DP_OZ_TILE, DP_OZ_NC * (S + 1 - s)), acc0 || s > 1);
             tc::mma_commit(&empty[st]);
         };
         int c = 0, sc = 0;
@@ -1009,7 +1005,7 @@ void oz_plan_gemm(OzGemm &g, int bits)
 // column chunk) pairs would leave half of the SMs idle or more: exact integer
 // sums, so the result does not depend on the split.  A part keeps 8 chunks or
 // more, below which its fixed costs (sums written and read, 64 KB) outweigh the
-// MMAs (1.15 k cycles a chunk).  One CTA per pair took 88 us for the first layer
+// MMAs (1 k cycles a chunk).  One CTA per pair took 88 us for the first layer
 // of 192 water atoms and 321 us for a weight gradient over 12,288; now 44 and 54 us
 // (95 us for the 240 x 240 weights, 321 before).
 int oz_parts(int pairs, int nK, int num_sms)
