@@ -55,7 +55,14 @@ struct ChebGradBuffers {
     double *node;   // [T T][NN][4][sum of widths] layer outputs and z adjoints at the nodes, with tangents
     int32_t *far;   // set when a row lies beyond S: the caller's other kernels run instead
 };
-inline int dp_cheb_splits(int ntypes) { return ntypes > 8 ? 8 : 64 / ntypes; }  // atom shares of a centre type
+// Atom shares of a centre type: 24 atoms each, so that several CTAs share an SM
+// (64 shares in all took 2.0 ms for 12,288 water atoms with the student's widths,
+// 1.25 as now), between 64 and 256 in all (the buffer's size).
+inline int dp_cheb_splits(int ntypes, int64_t natoms)
+{
+    const int64_t s = natoms / (24 * ntypes), lo = ntypes > 8 ? 8 : 64 / ntypes, hi = 4 * lo;
+    return (int)(s < lo ? lo : s > hi ? hi : s);
+}
 // Terms the gradient keeps: the parameter derivatives' series converge as the
 // nets' with a polynomial factor, which 8 more terms cover.
 inline int dp_cheb_grad_terms(int n) { return n + 8 < DP_CHEB_NN ? n + 8 : DP_CHEB_NN; }

@@ -715,7 +715,7 @@ __global__ void __launch_bounds__(CT) k_cheb_bwd(DevModel m, ChebModel cm, const
 // reverse mode runs through the net with its s-tangent at NN points instead of
 // at every row.  (Folding V's adjoint into C's would multiply it by n^2 and
 // lose two digits to the cancellation over the nodes.)  12,288 water atoms,
-// student widths: 70 -> 5.0 ms (the net, its tangent and its reverse mode at
+// student widths: 70 -> 4.2 ms (the net, its tangent and its reverse mode at
 // every row before); 648 atoms, full width: 13.8 -> 0.6 ms.
 
 constexpr int PM = 12;  // moments per term: P, dP, Q (4 components each)
@@ -1010,6 +1010,7 @@ __global__ void k_chebpg_sum(double *__restrict__ part, size_t elems, int splits
     if (*far_flag) return;
     for (size_t p = blockIdx.x * (size_t)blockDim.x + threadIdx.x; p < elems; p += (size_t)gridDim.x * blockDim.x) {
         double v = part[p];
+#pragma unroll 8
         for (int q = 1; q < splits; ++q) v += part[q * elems + p];
         part[p] = v;
     }
@@ -1303,7 +1304,7 @@ size_t dp_cheb_grad_elems(const DevModel &m, int n, int64_t natoms, int which)
     for (int l = 0; l < m.n_emb; ++l) se += m.emb[l];
     switch (which) {
     case 0: return (size_t)natoms * m.ntypes * n * PM;
-    case 1: return (size_t)dp_cheb_splits(m.ntypes) * 2 * nets * NN * m.M;
+    case 1: return (size_t)dp_cheb_splits(m.ntypes, natoms) * 2 * nets * NN * m.M;
     default: return nets * NN * 4 * se;
     }
 }
@@ -1336,10 +1337,11 @@ cudaError_t dp_launch_chebpg_bwd(cudaStream_t st, const DevModel &m, const ChebM
         e = cudaFuncSetAttribute(k_chebpg_cb, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)csm);
     if (e != cudaSuccess) return e;
     k_chebpg_tb<<<N, CT, pg_tb_smem(m), st>>>(m, eb.T, pb.dT, pb.Db, pb.dDb, gb.far);
-    k_chebpg_cb<<<dim3(dp_cheb_splits(T), T, (Kt + CBK - 1) / CBK), CT, csm, st>>>(
+    const int splits = dp_cheb_splits(T, N);
+    k_chebpg_cb<<<dim3(splits, T, (Kt + CBK - 1) / CBK), CT, csm, st>>>(
         m, cm.n, nb.type_perm, nb.type_start, gb.mom, eb.T, pb.dT, gb.part, gb.far);
     const size_t elems = 2 * (size_t)T * T * NN * m.M;
-    k_chebpg_sum<<<(int)((elems + 255) / 256), 256, 0, st>>>(gb.part, elems, dp_cheb_splits(T), gb.far);
+    k_chebpg_sum<<<(int)((elems + 255) / 256), 256, 0, st>>>(gb.part, elems, splits, gb.far);
     k_chebpg_node<<<T * T * NN, CT, 0, st>>>(m, cm.n, trig, gb.part, gb.part + elems / 2, gb.node, se, gb.far);
     k_chebpg_grad<<<dim3((m.emb_net_size + 255) / 256, T * T), 256, 0, st>>>(m, trig, gb.node, se, grad, gb.far);
     *launches += 5;

@@ -867,7 +867,7 @@ __global__ void __launch_bounds__(256) k_oz_series(OzGemm gf, OzGemm gb, int T, 
 // digits of the columns of X (rows of the A operand) and of Zb (rows of the B
 // operand), scaled per column and type by its largest magnitude over the atoms.
 // The whole fitting part on the FP64 units, with per-CTA gradient slices, took 63
-// ms for 12,288 water atoms with the student's widths, now 2.6 ms; 648 atoms at
+// ms for 12,288 water atoms with the student's widths, now 3.7 ms; 648 atoms at
 // full width: 23 -> 0.8 ms (24 GEMMs and 14 splits, bound as k_oz_gemm).
 
 struct OzCols {
@@ -1301,7 +1301,6 @@ cudaError_t dp_launch_pgrad_fit_oz(cudaStream_t st, const DevModel &m, const OzM
     // gradient of a layer's weights and, as the row after them, its bias
     auto weights = [&](const double *x, const double *dx, int ldx, int K, int F, int64_t off) -> cudaError_t {
         const int nq = K / DP_OZ_TILE + 1, nN = (F + DP_OZ_NC - 1) / DP_OZ_NC;  // K + 1 rows
-        const int splits = std::min(64, (N + 31) / 32);
         for (int pass = 0; pass < 2; ++pass) {
             OzColsPair c;
             int32_t *expb = og.exp + (size_t)T * nq * DP_OZ_TILE;
@@ -1310,8 +1309,11 @@ cudaError_t dp_launch_pgrad_fit_oz(cudaStream_t st, const DevModel &m, const OzM
                             og.mx + (size_t)T * nq * DP_OZ_TILE};
             cudaError_t e2 = cudaMemsetAsync(og.mx, 0, 8 * (size_t)T * (nq * DP_OZ_TILE + nN * DP_OZ_NC), st);
             if (e2 != cudaSuccess) return e2;
-            const int cols = std::max(K, F);
-            k_oz_colmax<<<dim3((cols + 127) / 128, splits, 2), 128, 0, st>>>(c, nb.type_perm, nb.type_start, N, ob.cnt,
+            // column maxima: 16 CTAs per SM, 16 atoms each or more (on 64 shares of the
+            // atoms a pass over 240 columns of 12,288 took 82 us, now 21)
+            const int cb = (std::max(K, F) + 127) / 128;
+            const int splits = std::max(1, std::min(8 * num_sms / cb, N / 16));
+            k_oz_colmax<<<dim3(cb, splits, 2), 128, 0, st>>>(c, nb.type_perm, nb.type_start, N, ob.cnt,
                                                                                  ob.slots * 8);
             k_oz_tsplit<<<dim3(N / DP_OZ_KC + T, std::max(nq, (nN * DP_OZ_NC + 127) / 128), 2), 256, 0, st>>>(
                 c, nb.type_perm, nb.type_start, T);
