@@ -349,7 +349,8 @@ dp_status dp_md_kick(dp_ctx *ctx, double *vel, const double *force, const int32_
  * dp_model_nparams), overwritten.  FP64 contexts only (DP_ERR_UNSUPPORTED
  * otherwise).  Reproducible bit for bit.  Scratch of about
  * num_SMs * nparams doubles plus ~130 KB per atom is allocated on the first
- * call. */
+ * call, and ~50 KB per atom more for the tensor-core products and the series
+ * when it can be had (without it the kernels that need none run). */
 dp_status dp_param_grad(dp_ctx *ctx, const double *coords, const int32_t *types, const double box[9],
                         int64_t N, double cE, const double *lambda, double *grad);
 /* Replace the parameters of a model (host array, nparams doubles).  Contexts

@@ -5,6 +5,7 @@
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
+#include <initializer_list>
 #include <new>
 #include <string>
 #include <vector>
@@ -531,14 +532,18 @@ dp_status ensure_oz(dp_ctx *c)
         ob.a_stride = c->oz.in_w;
         ob.nmax = N;
         const size_t plane = (size_t)N * c->oz.fmax;
-        if ((s = dev_alloc(&ob.a, (size_t)ob.tiles * ob.a_stride, "fitting digits"))) return s;
-        if ((s = dev_alloc(&ob.aexp, (size_t)ob.tiles * DP_OZ_TILE, "fitting digits"))) return s;
-        if ((s = dev_alloc(&ob.t, (size_t)nf * plane, "fitting activations"))) return s;
-        if ((s = dev_alloc(&ob.h, 2 * plane, "fitting activations"))) return s;
-        if ((s = dev_alloc(&ob.g, 2 * plane, "fitting activations"))) return s;
         ob.slots = 2 * c->num_sms;
-        if ((s = dev_alloc(&ob.part, (size_t)ob.slots * 32 * 256, "fitting sums"))) return s;
-        if ((s = dev_alloc(&ob.cnt, (size_t)ob.slots * 8, "fitting sums"))) return s;
+#define ALLOCO(ptr, n, what) \
+    if (!s && !(ptr)) s = dev_alloc(&(ptr), (n), what)
+        ALLOCO(ob.aexp, (size_t)ob.tiles * DP_OZ_TILE, "fitting digits");
+        ALLOCO(ob.t, (size_t)nf * plane, "fitting activations");
+        ALLOCO(ob.h, 2 * plane, "fitting activations");
+        ALLOCO(ob.g, 2 * plane, "fitting activations");
+        ALLOCO(ob.part, (size_t)ob.slots * 32 * 256, "fitting sums");
+        ALLOCO(ob.cnt, (size_t)ob.slots * 8, "fitting sums");
+        ALLOCO(ob.a, (size_t)ob.tiles * ob.a_stride, "fitting digits");  // last: marks the set as complete
+#undef ALLOCO
+        if (s) return s;
     }
     if (c->oz_version != c->model->version) {
         GroupTimer tm(c, G_FIT);
@@ -1418,18 +1423,30 @@ dp_status dp_param_grad(dp_ctx *c, const double *coords, const int32_t *types, c
         ALLOCP(c->pb.dDb, Nmax * nd);
         ALLOCP(c->pb.fit_scr, dp_pgrad_fit_scratch((int)Nmax));
         ALLOCP(c->pb.rowscr, dp_pgrad_row_scratch(c->num_sms));
-        if (c->use_cheb && dp_cheb_grad_supported(c->m, DP_CHEB_NN)) {
+        // without room for either route's scratch, the kernels that need none run
+        auto optional = [&](std::initializer_list<void **> l) {
+            if (s != DP_ERR_NOMEM) return;
+            for (void **q : l) {
+                dev_free(*q);
+                *q = nullptr;
+            }
+            s = DP_OK;
+        };
+        if (c->use_cheb && !s && dp_cheb_grad_supported(c->m, DP_CHEB_NN)) {
             ALLOCP(c->cg.mom, dp_cheb_grad_elems(c->m, DP_CHEB_NN, c->natoms_max, 0));
             ALLOCP(c->cg.part, dp_cheb_grad_elems(c->m, DP_CHEB_NN, c->natoms_max, 1));
             ALLOCP(c->cg.node, dp_cheb_grad_elems(c->m, DP_CHEB_NN, c->natoms_max, 2));
             ALLOCP(c->cg.far, 1);
+            optional({(void **)&c->cg.mom, (void **)&c->cg.part, (void **)&c->cg.node, (void **)&c->cg.far});
         }
-        if (c->use_oz) {
+        if (c->use_oz && !s) {
             ALLOCP(c->og.a, dp_oz_grad_elems(c->m, c->oz, c->natoms_max, 0));
             ALLOCP(c->og.b, dp_oz_grad_elems(c->m, c->oz, c->natoms_max, 1));
             ALLOCP(c->og.exp, dp_oz_grad_elems(c->m, c->oz, c->natoms_max, 2));
             ALLOCP(c->og.mx, dp_oz_grad_elems(c->m, c->oz, c->natoms_max, 2));
             ALLOCP(c->og.x, dp_oz_grad_elems(c->m, c->oz, c->natoms_max, 3));
+            optional({(void **)&c->og.a, (void **)&c->og.b, (void **)&c->og.exp, (void **)&c->og.mx,
+                      (void **)&c->og.x});
         }
         ALLOCP(c->pb.slices, (size_t)c->num_sms * np);  // last: marks the set as complete
 #undef ALLOCP
@@ -1447,7 +1464,8 @@ dp_status dp_param_grad(dp_ctx *c, const double *coords, const int32_t *types, c
     }
     cudaError_t e = dp_launch_pgrad(c->stream, c->m, np, coords, types, b, (int)N, lambda, cE, c->fb, c->nb, c->eb,
                                     c->pb, c->num_sms, cheb ? &cm : nullptr, &c->cg, c->cb.trig,
-                                    c->use_oz ? &c->oz : nullptr, &c->ob, &c->og, c->d_status, grad, &c->launches);
+                                    c->use_oz && c->og.x ? &c->oz : nullptr, &c->ob, &c->og, c->d_status, grad,
+                                    &c->launches);
     if (e != cudaSuccess) return cuda_fail(e, "dp_param_grad");
     return finish(c);
 }
