@@ -86,32 +86,32 @@ TRAFFIC = {
                       "src_sha": "c2c89c84fd00c488"},
     "embed_bwd_st<25>": {"bytes_per_row": (1883.360000e6 + 28.511232e6) / PROFILE_ROWS, "file": "embed_x.cu",
                          "src_sha": "c2c89c84fd00c488"},
-    "embed_tan_mx<25>": {"bytes_per_row": (49.605120e6 + 1008.945408e6) / PROFILE_ROWS, "file": "mixed.cu",
-                         "src_sha": "bd0c7271cc3b2bf4"},
-    "embed_bwd_st_mx<25>": {"bytes_per_row": (1043.964160e6 + 26.513920e6) / PROFILE_ROWS, "file": "mixed.cu",
-                            "src_sha": "bd0c7271cc3b2bf4"},
-    "embed_bwd_mx<25, split>": {"bytes_per_row": (204.796928e6 + 17.978880e6) / PROFILE_ROWS, "file": "mixed.cu",
-                                "src_sha": "bd0c7271cc3b2bf4"},
-    "embed_tan_mx<16>": {"bytes_per_row": (7.999488e6 + 603.240704e6) / PROFILE_ROWS, "file": "mixed.cu",
-                         "src_sha": "bd0c7271cc3b2bf4"},
-    "embed_bwd_st_mx<16>": {"bytes_per_row": (669.597440e6 + 25.187072e6) / PROFILE_ROWS, "file": "mixed.cu",
-                            "src_sha": "bd0c7271cc3b2bf4"},
+    "embed_tan_mx<25>": {"bytes_per_row": (54.107136e6 + 1037.398528e6) / PROFILE_ROWS, "file": "mixed.cu",
+                         "src_sha": "be819dbaa370fed3"},
+    "embed_bwd_st_mx<25>": {"bytes_per_row": (1063.947264e6 + 36.366080e6) / PROFILE_ROWS, "file": "mixed.cu",
+                            "src_sha": "be819dbaa370fed3"},
+    "embed_bwd_mx<25, split>": {"bytes_per_row": (204.732928e6 + 17.787136e6) / PROFILE_ROWS, "file": "mixed.cu",
+                                "src_sha": "be819dbaa370fed3"},
+    "embed_tan_mx<16>": {"bytes_per_row": (9.171456e6 + 628.367104e6) / PROFILE_ROWS, "file": "mixed.cu",
+                         "src_sha": "be819dbaa370fed3"},
+    "embed_bwd_st_mx<16>": {"bytes_per_row": (689.640192e6 + 25.842432e6) / PROFILE_ROWS, "file": "mixed.cu",
+                            "src_sha": "be819dbaa370fed3"},
 }
 # Pipe shares of the mixed embedding kernels (ncu, one evaluation of the
 # 12,288-atom water box, --profile-precision mixed / split): active-cycle
 # busy fractions of the FP64, FP32 (fma), integer (alu) and tensor pipes and
 # the schedulers' issue-active share.
 MODE_PIPES = {
-    "embed_tan_mx<25>": {"fp64": 0.386, "fma": 0.196, "alu": 0.087, "tensor": 0.016, "issue_active": 0.333,
-                         "file": "mixed.cu", "src_sha": "bd0c7271cc3b2bf4"},
-    "embed_bwd_st_mx<25>": {"fp64": 0.689, "fma": 0.282, "alu": 0.041, "tensor": 0.0, "issue_active": 0.406,
-                            "file": "mixed.cu", "src_sha": "bd0c7271cc3b2bf4"},
-    "embed_bwd_mx<25, split>": {"fp64": 0.448, "fma": 0.180, "alu": 0.094, "tensor": 0.028, "issue_active": 0.302,
-                                "file": "mixed.cu", "src_sha": "bd0c7271cc3b2bf4"},
-    "embed_tan_mx<16>": {"fp64": 0.442, "fma": 0.168, "alu": 0.081, "tensor": 0.006, "issue_active": 0.300,
-                         "file": "mixed.cu", "src_sha": "bd0c7271cc3b2bf4"},
-    "embed_bwd_st_mx<16>": {"fp64": 0.754, "fma": 0.239, "alu": 0.048, "tensor": 0.0, "issue_active": 0.366,
-                            "file": "mixed.cu", "src_sha": "bd0c7271cc3b2bf4"},
+    "embed_tan_mx<25>": {"fp64": 0.322, "fma": 0.216, "alu": 0.111, "tensor": 0.017, "issue_active": 0.363,
+                         "file": "mixed.cu", "src_sha": "be819dbaa370fed3"},
+    "embed_bwd_st_mx<25>": {"fp64": 0.655, "fma": 0.345, "alu": 0.108, "tensor": 0.000, "issue_active": 0.498,
+                            "file": "mixed.cu", "src_sha": "be819dbaa370fed3"},
+    "embed_bwd_mx<25, split>": {"fp64": 0.367, "fma": 0.199, "alu": 0.117, "tensor": 0.031, "issue_active": 0.330,
+                                "file": "mixed.cu", "src_sha": "be819dbaa370fed3"},
+    "embed_tan_mx<16>": {"fp64": 0.375, "fma": 0.189, "alu": 0.110, "tensor": 0.007, "issue_active": 0.332,
+                         "file": "mixed.cu", "src_sha": "be819dbaa370fed3"},
+    "embed_bwd_st_mx<16>": {"fp64": 0.721, "fma": 0.307, "alu": 0.123, "tensor": 0.000, "issue_active": 0.476,
+                            "file": "mixed.cu", "src_sha": "be819dbaa370fed3"},
 }
 FP64_ISSUED = {
     # k_embed_tan_x<25>: dfma 2.257e9, dadd 0.818e9, dmul 0.106e9 thread
@@ -122,6 +122,21 @@ FP64_ISSUED = {
     "embed_bwd_st<25>": {"fp64_flop_per_row": (2 * 1.069532688e9 + 0.100726048e9 + 0.043622898e9) / PROFILE_ROWS,
                          "pipe_busy": 0.939, "file": "embed_x.cu", "src_sha": "c2c89c84fd00c488"},
 }
+
+# The FP64 path with the embedding nets as series (embed_cheb.cu) and the exact
+# digit products (fit_oz.cu), summed over the kernels of a group in one evaluation
+# of the 12,288-atom water box; same meaning as above (pipe_busy weighted by the
+# kernels' active cycles), keyed by their sources.  Parts of this box's per-atom
+# arrays stay in L2, so the bytes are a lower bound for larger ones.
+SERIES_COUNTERS = {
+    "embed_fwd<25>": {"bytes_per_row": 198.640896e6 / PROFILE_ROWS, "fp64_flop_per_row": 0.436443e9 / PROFILE_ROWS,
+                      "pipe_busy": 0.792, "src_sha": "bef972990c3595e4"},
+    "fit<25>": {"bytes_per_row": 1600.926464e6 / PROFILE_ROWS, "fp64_flop_per_row": 0.264720e9 / PROFILE_ROWS,
+                "pipe_busy": 0.306, "src_sha": "bef972990c3595e4"},
+    "embed_bwd<25>": {"bytes_per_row": 428.686592e6 / PROFILE_ROWS, "fp64_flop_per_row": 0.890842e9 / PROFILE_ROWS,
+                      "pipe_busy": 0.875, "src_sha": "bef972990c3595e4"},
+}
+SERIES_SOURCES = ("embed_cheb.cu", "fit_oz.cu", "cheb.cuh", "atom_cta.cuh")
 
 
 def parse():
@@ -258,10 +273,10 @@ def measured_peaks():
         return {}
 
 
-def source_sha(fn):
-    """Hash of a kernel source file together with the shared device header."""
+def source_sha(*files):
+    """Hash of kernel source files together with the shared device header."""
     h = hashlib.sha256()
-    for name in (fn, "dp_internal.cuh"):
+    for name in files + ("dp_internal.cuh",):
         with open(os.path.join(ROOT, "paper_2004_11658_gb300", "csrc", name), "rb") as f:
             h.update(f.read())
     return h.hexdigest()[:16]
@@ -653,6 +668,61 @@ def fp64_roofline(desc, groups, dom, rows, nreal, N, store=False):
     return roof
 
 
+def digit_mma_flops_fit(desc, natoms):
+    """Tensor-core FLOPs the FP64 fitting net issues per evaluation
+    (k_oz_gemm<8>): 36 digit pairs per 16 columns of the contraction and 32
+    columns of the output, both padded, for every GEMM forward and backward."""
+    def chunks(K, N):
+        return -(-K // 16) * -(-N // 32)
+    kin, n = desc["m2"] * desc["emb"][-1], 0
+    for F in desc["fit"]:
+        n += chunks(kin, F) + chunks(F, kin)
+        kin = F
+    return natoms * 36 * n * 2 * 16 * 32
+
+
+def series_roofline(desc, groups, dom, rows, N, evals):
+    """Roofline of the FP64 path's dominant kernel group (time per evaluation)
+    with the embedding nets as series, by unit: the FP64 pipe and HBM from the
+    ncu counts per row, the tensor cores from the digit-MMA FLOPs issued; the
+    busiest unit at the top level.  The other groups beside it."""
+    pk = measured_peaks()
+    bf16_peak = pk.get("bf16_tflops_sustained", pk.get("bf16_tflops", 1720.9))
+    hbm = pk.get("hbm_gbs", 6712.6)
+
+    def one(g):
+        sec = groups[g]["ms"] / evals / 1000.0
+        key = f"{g}<{desc['emb'][0]}>"
+        c = SERIES_COUNTERS.get(key)
+        if c and c["src_sha"] != source_sha(*SERIES_SOURCES):
+            c = None
+        out = {"kernel": key, "ms_per_evaluation": sec * 1e3, "traffic": c["bytes_per_row"] * rows if c else None}
+        units = {}
+        if c:
+            fp = c["fp64_flop_per_row"] * rows / sec / 1e12
+            units["fp64_pipe"] = {"achieved": fp, "peak": FP64_PEAK_TFLOPS, "frac": fp / FP64_PEAK_TFLOPS,
+                                  "unit": "TFLOP/s", "busy_ncu": c["pipe_busy"],
+                                  "what": "FP64 FLOPs issued (2 dfma + dadd + dmul, ncu count per row of the "
+                                          "12,288-atom box); busy_ncu: the pipe's share of the active cycles"}
+            units["hbm"] = {"achieved": out["traffic"] / sec / 1e9, "peak": hbm,
+                            "frac": out["traffic"] / sec / 1e9 / hbm, "unit": "GB/s"}
+        if g == "fit":
+            mma = digit_mma_flops_fit(desc, N) / sec / 1e12
+            units["tensor_bf16"] = {"achieved": mma, "peak": bf16_peak, "frac": mma / bf16_peak, "unit": "TFLOP/s",
+                                    "what": "BF16 digit-MMA FLOPs issued (padded shapes)",
+                                    "peak_source": "MEASURED_PEAKS bf16_tflops_sustained (of measured)"}
+        if units:
+            top = max(units, key=lambda u: units[u]["frac"])
+            out.update({"bound": {"fp64_pipe": "alu", "hbm": "hbm", "tensor_bf16": "tensor"}[top],
+                        **{k: units[top][k] for k in ("achieved", "peak", "frac", "unit")}})
+        out.update(units)
+        return out
+
+    roof = dict(one(dom), rows_per_launch=rows)
+    roof["groups"] = [one(g) for g in ("embed_fwd", "fit", "embed_bwd") if g in groups and g != dom]
+    return roof
+
+
 def run_ours(args, rank, world, local_rank):
     import torch
     import torch.distributed as dist
@@ -737,7 +807,10 @@ def run_ours(args, rank, world, local_rank):
     groups = {g: {"ms": ms, "launches": n} for g, (ms, n) in kt.items()}
     timed_groups = {g: d for g, d in groups.items() if d["launches"] > 0}
     dom = max(timed_groups, key=lambda g: timed_groups[g]["ms"])
-    roof = fp64_roofline(desc, groups, dom, rows, nreal, N, store=store)
+    if dom in ("embed_fwd", "fit", "embed_bwd"):
+        roof = series_roofline(desc, timed_groups, dom, rows, N, args.steps * wl["md_per_step"])
+    else:
+        roof = fp64_roofline(desc, groups, dom, rows, nreal, N, store=store)
     th_all = torch.stack(thermo_all).cpu().numpy().reshape(-1, 4)
     etot = th_all[:, 0] + th_all[:, 1]
 
@@ -808,8 +881,8 @@ def run_ours(args, rank, world, local_rank):
             "gpu_launches": launches,
             "roofline": roof,
             "embed_store": {"on": bool(store),
-                            "what": "G and dG/ds of every real row kept in HBM between the embedding forward "
-                                    "(k_embed_tan_x) and the streaming backward (k_embed_bwd_st)"},
+                            "what": "HBM held for G and dG/ds of every real row, which the embedding kernels use "
+                                    "when a net's series in s(r) does not resolve (k_embed_tan_x, k_embed_bwd_st)"},
             "kernels_ms_per_step": {g: d["ms"] / args.steps for g, d in timed_groups.items()},
             "nve": {"etot_first": float(etot[0]), "etot_last": float(etot[-1]),
                     "max_abs_drift_eV_per_atom": float(np.abs(etot - etot[0]).max() / N),
