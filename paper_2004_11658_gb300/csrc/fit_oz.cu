@@ -1307,7 +1307,10 @@ cudaError_t dp_launch_pgrad_fit_oz(cudaStream_t st, const DevModel &m, const OzM
             c.c[0] = OzCols{pass == 0 ? x : dx, ldx, K, pass == 0 ? K : -1, DP_OZ_TILE, nq, og.a, og.exp, og.mx};
             c.c[1] = OzCols{pass == 0 ? zb : dzb, ld, F, -1, DP_OZ_NC, nN, og.b, expb,
                             og.mx + (size_t)T * nq * DP_OZ_TILE};
-            cudaError_t e2 = cudaMemsetAsync(og.mx, 0, 8 * (size_t)T * (nq * DP_OZ_TILE + nN * DP_OZ_NC), st);
+            const size_t cols = (size_t)T * (nq * DP_OZ_TILE + nN * DP_OZ_NC);
+            cudaError_t e2 = cudaMemsetAsync(og.mx, 0, 8 * cols, st);
+            // the exponents too: a type without atoms in the frame has no chunk that writes them
+            if (e2 == cudaSuccess) e2 = cudaMemsetAsync(og.exp, 0, 4 * cols, st);
             if (e2 != cudaSuccess) return e2;
             // column maxima: 16 CTAs per SM, 16 atoms each or more (on 64 shares of the
             // atoms a pass over 240 columns of 12,288 took 82 us, now 21)
