@@ -976,7 +976,7 @@ void dp_ctx_free(dp_ctx *c)
                     c->d_oz_w, c->d_oz_e, c->ob.a, c->ob.aexp, c->ob.t, c->ob.h, c->ob.g, c->ob.part, c->ob.cnt, c->d_dtile, c->d_ex_w,
                     c->eb.Gst, c->eb.Gmx, c->cb.C, c->cb.Ct, c->cb.V, c->cb.y, c->cb.mx, c->cb.trig, c->cg.mom,
                     c->os.w, c->os.e, c->os.aexp, c->cg.part, c->cg.node, c->cg.far, c->og.a, c->og.b, c->og.exp,
-                    c->og.mx, c->og.x};
+                    c->og.x};
     for (void *p : bufs) dev_free(p);
     delete c;
 }
@@ -1443,10 +1443,8 @@ dp_status dp_param_grad(dp_ctx *c, const double *coords, const int32_t *types, c
             ALLOCP(c->og.a, dp_oz_grad_elems(c->m, c->oz, c->natoms_max, 0));
             ALLOCP(c->og.b, dp_oz_grad_elems(c->m, c->oz, c->natoms_max, 1));
             ALLOCP(c->og.exp, dp_oz_grad_elems(c->m, c->oz, c->natoms_max, 2));
-            ALLOCP(c->og.mx, dp_oz_grad_elems(c->m, c->oz, c->natoms_max, 2));
             ALLOCP(c->og.x, dp_oz_grad_elems(c->m, c->oz, c->natoms_max, 3));
-            optional({(void **)&c->og.a, (void **)&c->og.b, (void **)&c->og.exp, (void **)&c->og.mx,
-                      (void **)&c->og.x});
+            optional({(void **)&c->og.a, (void **)&c->og.b, (void **)&c->og.exp, (void **)&c->og.x});
         }
         ALLOCP(c->pb.slices, (size_t)c->num_sms * np);  // last: marks the set as complete
 #undef ALLOCP

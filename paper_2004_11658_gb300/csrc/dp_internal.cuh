@@ -436,11 +436,10 @@ struct PGradBuffers {
 // parameters' part of grad.
 struct OzGradBuffers {
     uint16_t *a, *b;         // digits of the columns of X and Zb over the atoms
-    int32_t *exp;            // their exponents
-    unsigned long long *mx;  // their largest magnitudes
+    int32_t *exp;            // their exponents and levels, per segment
     double *x;               // adjoints, 6 x [natoms][fmax]
 };
-size_t dp_oz_grad_elems(const DevModel &m, const OzModel &oz, int64_t natoms, int which);  // a, b, exp (= mx), x
+size_t dp_oz_grad_elems(const DevModel &m, const OzModel &oz, int64_t natoms, int which);  // a, b, exp, x
 cudaError_t dp_launch_pgrad_fit_oz(cudaStream_t st, const DevModel &m, const OzModel &oz, const OzBuffers &ob,
                                    const OzGradBuffers &og, const int32_t *types, int N, double cE,
                                    const NlistBuffers &nb, EvalBuffers eb, PGradBuffers pb, int num_sms,

@@ -60,6 +60,7 @@ constexpr uint32_t OZ_TAB_BYTES = DP_TANH_NINT * DP_TANH_STRIDE * 8;
 static_assert(OZ_TAB_BYTES % 16 == 0, "bulk copy of the tanh table");
 constexpr int OZ_A_BLK = DP_OZ_TILE * DP_OZ_KC;  // elements of one A digit chunk (128 x 16)
 constexpr int OZ_B_BLK = DP_OZ_NC * DP_OZ_KC;    // elements of one W digit chunk (32 x 16)
+constexpr int OZ_WSEG = 16;                      // chunks of a weight gradient's segment (256 atoms)
 constexpr int OZ_KEEP = 256;                     // columns of a row that k_oz_split may keep between its passes
 
 struct TileRef {
@@ -335,9 +336,11 @@ struct OzGemmArgs {
     int32_t *status;
     int units;  // (tile, column chunk) pairs, tiles past the last atom included
     const double *tin;  // epi 2: tanh values of the value pass
-    // weight gradients Y = X^T Z, contracted over the atoms of each type
+    // weight gradients Y = X^T Z, contracted over the atoms of each type (epi 3)
     int wg, rows, nq;                 // 1; rows of Y and their tiles
     int64_t out_off[DP_MAX_TYPES];    // of a type's Y in hout
+    const double *x, *z;              // X and Z
+    int ldx, ldz, one;                // one: the last row of Y is the sum of Z's rows (else 0)
     // contraction shared by `parts` CTAs: their chain sums [unit][32][256 threads], arrivals per (pair, warp)
     int parts;
     long long *part;
@@ -347,7 +350,8 @@ struct OzGemmArgs {
 // One unit of k_oz_gemm: a 128-row tile of the A operand and a 32-column chunk of Y.
 struct OzUnit {
     int a, tl, nchunk, nK, nseg, seg;
-    int first, cnt;             // atoms of the tile (not wg)
+    int first, cnt;             // atoms of the tile; wg: first atom, atoms (of the type's, in type order)
+    int sg0;                    // wg: first segment, counted over the types
     const uint16_t *as, *bs;    // digits of the first K-chunk
     size_t astep, bstep;        // ... to the next
 };
@@ -374,13 +378,13 @@ __device__ __forceinline__ double scale2(double y, int e)
     return (e >= -1022 && e <= 1023) ? y * oz_pow2(e) : ldexp(y, e);
 }
 
-template <int S>
+template <int S, bool WG>
 __device__ __forceinline__ bool oz_unit(const OzGemmArgs &p, int u, OzUnit &U)
 {
     const OzGemm &g = p.g;
     const int ks = u % p.parts;
     u /= p.parts;
-    if (!p.wg) {
+    if constexpr (!WG) {
         U.tl = u / g.nN;
         U.nchunk = u - U.tl * g.nN;
         const TileRef T = oz_tile(U.tl, p.type_start, p.ntypes, p.rpa);
@@ -400,23 +404,75 @@ __device__ __forceinline__ bool oz_unit(const OzGemmArgs &p, int u, OzUnit &U)
         U.tl = (u - U.a * per) / g.nN;
         U.nchunk = u - U.a * per - U.tl * g.nN;
         int kb = 0;
-        for (int a = 0; a < U.a; ++a) kb += (p.type_start[a + 1] - p.type_start[a] + DP_OZ_KC - 1) / DP_OZ_KC;
+        U.sg0 = 0;
+        for (int a = 0; a < U.a; ++a) {
+            const int nk = (p.type_start[a + 1] - p.type_start[a] + DP_OZ_KC - 1) / DP_OZ_KC;
+            kb += nk;
+            U.sg0 += (nk + OZ_WSEG - 1) / OZ_WSEG;
+        }
         U.nK = (p.type_start[U.a + 1] - p.type_start[U.a] + DP_OZ_KC - 1) / DP_OZ_KC;
-        U.seg = OZ_SEG;
-        U.first = U.cnt = 0;
+        U.seg = OZ_WSEG;
+        U.first = p.type_start[U.a];
+        U.cnt = p.type_start[U.a + 1] - U.first;
         U.astep = (size_t)p.nq * S * OZ_A_BLK;
         U.bstep = (size_t)g.nN * S * OZ_B_BLK;
         U.as = p.a + kb * U.astep + (size_t)U.tl * S * OZ_A_BLK;
         U.bs = p.w + kb * U.bstep + (size_t)U.nchunk * S * OZ_B_BLK;
     }
     if (p.parts > 1) {
-        const int per = (U.nK + p.parts - 1) / p.parts, k0 = ks * per;
+        int per = (U.nK + p.parts - 1) / p.parts;
+        if constexpr (WG) per = (per + OZ_WSEG - 1) / OZ_WSEG * OZ_WSEG;  // whole segments
+        const int k0 = ks * per;
+        if constexpr (WG) {
+            U.sg0 += k0 / OZ_WSEG;
+            U.first += k0 * DP_OZ_KC;
+            U.cnt -= k0 * DP_OZ_KC;
+        }
         U.as += k0 * U.astep;
         U.bs += k0 * U.bstep;
         U.nK = max(0, min(U.nK - k0, per));
     }
     U.nseg = (U.nK + U.seg - 1) / U.seg;
     return U.a >= 0;
+}
+
+// Entries of a weight gradient that the digits of a segment may not carry.  The
+// digit product of n atoms errs by about 2^-58 sqrt(n) of the two columns' powers
+// of two 2^e, 2^f (the groups left out); a chain of FP64 FMAs by 2^-54 or more of the
+// products' size, which is smaller than 2^(e+f) when the columns have their
+// outliers at different atoms.  A column's level l says that three quarters of its
+// values are at least 2^(e-l).  The digits stand where the two levels are at most
+// OZ_EVEN together (normal deviates have 4 or 5 each; two columns at the line with
+// one outlier each leave products of 2^-5 and more), or where the result itself is
+// at least an eighth of 2^(e+f) (an outlier in one column only).  The others are
+// summed from the FP64 values.
+constexpr int OZ_EVEN = 10;
+constexpr int OZ_LVL_BITS = 5;  // exponent and level in one word; level -16: zeros, NaN
+__device__ __forceinline__ bool oz_digits_stand(double y, int va, int vw)
+{
+    constexpr int sh = 32 - OZ_LVL_BITS;
+    if (((va << sh) >> sh) + ((vw << sh) >> sh) <= OZ_EVEN) return true;
+    const int ey = (int)((__double_as_longlong(y) >> 52) & 0x7ff) - 1023;  // |y| >= 2^ey
+    return ey >= (va >> OZ_LVL_BITS) + (vw >> OZ_LVL_BITS) - 3;
+}
+// One entry (row k, column f) over na atoms of a segment by the whole warp: lanes
+// on the atoms, then a fixed tree.  (One lane's chain of loads held its warp up
+// for 70 k cycles: a few entries in 10,000 took the GEMM from 250 to 640 us.)
+__device__ __noinline__ double oz_wdot(const OzGemmArgs &p, int at0, int na, int k, int f)
+{
+    const int lane = threadIdx.x & 31;
+    double v = 0.0;
+#pragma unroll
+    for (int u = 0; u < OZ_WSEG * DP_OZ_KC / 32; ++u) {
+        const int q = lane + 32 * u;
+        if (q < na) {
+            const size_t i = p.type_perm[at0 + q];
+            v = fma(k < p.rows - 1 ? p.x[i * p.ldx + k] : p.one ? 1.0 : 0.0, p.z[i * p.ldz + f], v);
+        }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
 }
 
 // Persistent, one CTA per SM over the units (tile, 32-column chunk of Y) in
@@ -446,6 +502,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_oz_gemm(OzGemmArgs p)
     __shared__ volatile int fail;
     const int tid = threadIdx.x, lane = tid & 31, warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
     const OzGemm &g = p.g;
+    constexpr bool WG = EPI == 3, OUT2 = EPI == 0 || EPI == 2;  // OUT2: tout beside hout
     constexpr uint32_t a_bytes = (uint32_t)S * OZ_A_BLK * 2, b_bytes = (uint32_t)S * OZ_B_BLK * 2;
     constexpr uint32_t stage_bytes = a_bytes + b_bytes;
     constexpr int NST = OZ_NST;
@@ -482,7 +539,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_oz_gemm(OzGemmArgs p)
         }
         for (int u = blockIdx.x; u < p.units && ok; u += gridDim.x) {
             OzUnit U;
-            if (!oz_unit<S>(p, u, U)) break;
+            if (!oz_unit<S, WG>(p, u, U)) break;
             for (int kc = 0; kc < U.nK; ++kc, ++c) {
                 const int st = c % NST;
                 if (c >= NST) ok = tc::mbar_wait(&empty[st], (c / NST - 1) & 1) && !fail;
@@ -524,7 +581,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_oz_gemm(OzGemmArgs p)
         bool ok = true;
         for (int u = blockIdx.x; u < p.units && ok; u += gridDim.x) {
             OzUnit U;
-            if (!oz_unit<S>(p, u, U)) break;
+            if (!oz_unit<S, WG>(p, u, U)) break;
             for (int sg = 0; sg < U.nseg && ok; ++sg, ++sc) {
                 const int buf = sc & 1;
                 if (sc >= 2) ok = tc::mbar_wait(&tempty[buf], ((sc >> 1) - 1) & 1) && !fail;
@@ -565,30 +622,28 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_oz_gemm(OzGemmArgs p)
         const int w = g.beta * (S - H);
         const int half = warp >> 2, row = 32 * (warp & 3) + lane;
         const uint32_t tl_lane = tbase + ((uint32_t)(32 * (warp & 3)) << 16) + 16 * half;
-        const bool vec = !p.wg && (p.ldo & 1) == 0 && (p.ldh & 1) == 0;  // rows start on 16 bytes
+        const bool vec = !WG && (p.ldo & 1) == 0 && (p.ldh & 1) == 0;  // rows start on 16 bytes
         int sc = 0;
         bool ok = true;
         if (EPI == 0) ok = __all_sync(0xffffffffu, tc::mbar_wait(&tabbar, 0));
         for (int u = blockIdx.x; u < p.units && ok; u += gridDim.x) {
             OzUnit U;
-            if (!oz_unit<S>(p, u, U)) break;
+            if (!oz_unit<S, WG>(p, u, U)) break;
             const int n0 = U.nchunk * DP_OZ_NC + 16 * half;   // first of this thread's 16 columns of Y
-            int i, erow;
-            const int4 *fe4;
-            if (!p.wg) {
+            const int erow = U.tl * DP_OZ_TILE + row;
+            int i, esc = 0;
+            const int4 *fe4 = nullptr;
+            if constexpr (!WG) {
                 i = row < U.cnt ? oz_row(p.type_perm, U.first + row, p.rpa) : -1;
-                erow = U.tl * DP_OZ_TILE + row;
                 fe4 = reinterpret_cast<const int4 *>(p.wexp + g.e_off[U.a] + n0);
+                esc = (i >= 0 ? p.aexp[erow] : 0) - g.beta * (S + 1);
             } else {
-                i = U.tl * DP_OZ_TILE + row < p.rows ? U.tl * DP_OZ_TILE + row : -1;
-                erow = U.a * p.nq * DP_OZ_TILE + U.tl * DP_OZ_TILE + row;
-                fe4 = reinterpret_cast<const int4 *>(p.wexp + U.a * g.nN * DP_OZ_NC + n0);
+                i = erow < p.rows ? erow : -1;
             }
-            const int esc = (i >= 0 ? p.aexp[erow] : 0) - g.beta * (S + 1);
-            double *hout = p.hout + (p.wg ? p.out_off[U.a] : 0);
+            double *hout = p.hout + (WG ? p.out_off[U.a] : 0);
             // the skip's operands, asked for before the MMAs are waited for
             const bool bcast = EPI == 1 && p.gbc[U.a] != nullptr;
-            const double *hin = bcast ? p.gbc[U.a] : (p.wg ? hout : p.hin) + (size_t)(i < 0 ? 0 : i) * p.ldh;
+            const double *hin = bcast ? p.gbc[U.a] : (WG ? hout : p.hin) + (size_t)(i < 0 ? 0 : i) * p.ldh;
             double sk[2][8];
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
@@ -631,11 +686,17 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_oz_gemm(OzGemmArgs p)
                     }
                 }
             };
+            // the value of the group sums (hi, lo) of an entry whose exponents add up to e
+            auto scaled = [&](long long hi, long long lo, int e) -> double {
+                if (e > -900 && e < 900) return oz_i64x2_round(hi, lo, w, e);
+                if (e > 5000) return __longlong_as_double(0x7ff8000000000000ll);
+                return scale2(fma((double)hi, oz_pow2(w), (double)lo), e);
+            };
             auto finish = [&](int h, const long long (&hi)[8], const long long (&lo)[8], const double (&skh)[8]) {
                 if (i < 0) return;
                 const int q0 = n0 + 8 * h;
                 double *ho = hout + (size_t)i * p.ldo + q0;
-                double *to = EPI != 1 ? p.tout + (size_t)i * p.ldo + q0 : nullptr;
+                double *to = OUT2 ? p.tout + (size_t)i * p.ldo + q0 : nullptr;
                 const double *ti = EPI == 2 ? p.tin + (size_t)i * p.ldo + q0 : nullptr;
                 const int4 f0 = fe4[2 * h], f1 = fe4[2 * h + 1];
                 const int fe[8] = {f0.x, f0.y, f0.z, f0.w, f1.x, f1.y, f1.z, f1.w};
@@ -644,11 +705,9 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_oz_gemm(OzGemmArgs p)
                     double y[2], t[2];
 #pragma unroll
                     for (int v = 0; v < 2; ++v) {
-                        const int n = n2 + v, e = esc + fe[n];
+                        const int n = n2 + v;
                         const bool in = q0 + n < g.N;
-                        if (e > -900 && e < 900) y[v] = oz_i64x2_round(hi[n], lo[n], w, e);
-                        else if (e > 5000) y[v] = __longlong_as_double(0x7ff8000000000000ll);
-                        else y[v] = scale2(fma((double)hi[n], oz_pow2(w), (double)lo[n]), e);
+                        y[v] = scaled(hi[n], lo[n], esc + fe[n]);
                         if constexpr (EPI == 0) {
                             t[v] = dp_tanh64(y[v] + (in ? p.bias[U.a][q0 + n] : 0.0), tab);
                             y[v] = t[v];
@@ -661,13 +720,13 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_oz_gemm(OzGemmArgs p)
                     }
                     if (vec && q0 + n2 + 2 <= g.N) {
                         *reinterpret_cast<double2 *>(ho + n2) = make_double2(y[0], y[1]);
-                        if constexpr (EPI != 1) *reinterpret_cast<double2 *>(to + n2) = make_double2(t[0], t[1]);
+                        if constexpr (OUT2) *reinterpret_cast<double2 *>(to + n2) = make_double2(t[0], t[1]);
                     } else {
 #pragma unroll
                         for (int v = 0; v < 2; ++v)
                             if (q0 + n2 + v < g.N) {
                                 ho[n2 + v] = y[v];
-                                if constexpr (EPI != 1) to[n2 + v] = t[v];
+                                if constexpr (OUT2) to[n2 + v] = t[v];
                             }
                     }
                 }
@@ -684,7 +743,86 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_oz_gemm(OzGemmArgs p)
                 if (lane == 0) tc::mbar_arrive(&tempty[buf]);
                 ++sc;
             };
-            if constexpr (SEG) {
+            if constexpr (WG) {
+                // every segment has its own exponents; its sum is rounded once and added in order
+                double acc[2][8];
+#pragma unroll
+                for (int h = 0; h < 2; ++h)
+#pragma unroll
+                    for (int n = 0; n < 8; ++n) acc[h][n] = 0.0;
+                for (int sg = 0; sg < U.nseg; ++sg) {
+                    const int buf = sc & 1;
+                    if (!wait(buf)) break;
+                    long long a[2][8], b[2][8];
+                    groups(buf, 0, a[0], b[0]);
+                    groups(buf, 1, a[1], b[1]);
+                    release(buf);
+                    const size_t wi = (size_t)(U.sg0 + sg) * g.nN * DP_OZ_NC + n0;
+                    const int va = i < 0 ? -16 & ((1 << OZ_LVL_BITS) - 1)
+                                         : p.aexp[(size_t)(U.sg0 + sg) * p.nq * DP_OZ_TILE + erow];
+                    unsigned bad = 0;  // entries the digits may not carry
+#pragma unroll
+                    for (int n4 = 0; n4 < 4; ++n4) {
+                        const int4 f = *reinterpret_cast<const int4 *>(p.wexp + wi + 4 * n4);
+                        const int vw[4] = {f.x, f.y, f.z, f.w};
+#pragma unroll
+                        for (int v = 0; v < 4; ++v) {
+                            const int q = 4 * n4 + v, h = q >> 3, n = q & 7;
+                            const double y = scaled(a[h][n], b[h][n],
+                                                    (va >> OZ_LVL_BITS) + (vw[v] >> OZ_LVL_BITS) - g.beta * (S + 1));
+                            if (oz_digits_stand(y, va, vw[v])) acc[h][n] += y;
+                            else bad |= 1u << q;
+                        }
+                    }
+                    for (unsigned who = __ballot_sync(0xffffffffu, bad != 0); who != 0; who &= who - 1) {
+                        const int src = __ffs(who) - 1, k = __shfl_sync(0xffffffffu, i, src);
+                        for (unsigned m = __shfl_sync(0xffffffffu, bad, src); m != 0; m &= m - 1) {
+                            const int q = __ffs(m) - 1;
+                            const double y = oz_wdot(p, U.first + sg * OZ_WSEG * DP_OZ_KC,
+                                                     min(U.cnt - sg * OZ_WSEG * DP_OZ_KC, OZ_WSEG * DP_OZ_KC), k, n0 + q);
+#pragma unroll
+                            for (int n = 0; n < 16; ++n)
+                                if (n == q && lane == src) acc[n >> 3][n & 7] += y;
+                        }
+                    }
+                    __syncwarp();
+                }
+                if (!ok) break;
+                if (p.parts > 1) {
+                    // the last of the parts to arrive adds all of them up in order
+                    const int ks = u % p.parts, ub = u - ks;
+                    auto slot = [&](int q, int v) { return p.part + ((size_t)(ub + q) * 32 + v) * 256 + tid; };
+#pragma unroll
+                    for (int h = 0; h < 2; ++h)
+#pragma unroll
+                        for (int n = 0; n < 8; ++n) *slot(ks, 8 * h + n) = __double_as_longlong(acc[h][n]);
+                    __threadfence();
+                    __syncwarp();
+                    int old = 0;
+                    if (lane == 0) old = atomicAdd(&p.cnt[(u / p.parts) * 8 + warp], 1);
+                    old = __shfl_sync(0xffffffffu, old, 0);
+                    if (old != p.parts - 1) continue;
+                    __threadfence();
+#pragma unroll
+                    for (int h = 0; h < 2; ++h)
+#pragma unroll
+                        for (int n = 0; n < 8; ++n) {
+                            const double own = acc[h][n];
+                            acc[h][n] = 0.0;
+                            for (int q = 0; q < p.parts; ++q)
+                                acc[h][n] += q == ks ? own : __longlong_as_double(__ldcg(slot(q, 8 * h + n)));
+                        }
+                }
+                if (i >= 0) {
+#pragma unroll
+                    for (int h = 0; h < 2; ++h)
+#pragma unroll
+                        for (int n = 0; n < 8; ++n)
+                            if (n0 + 8 * h + n < g.N)
+                                hout[(size_t)i * p.ldo + n0 + 8 * h + n] = acc[h][n] + sk[h][n];
+                }
+                __syncwarp();
+            } else if constexpr (SEG) {
                 long long hi[2][8], lo[2][8];
 #pragma unroll
                 for (int h = 0; h < 2; ++h)
@@ -865,9 +1003,15 @@ __global__ void __launch_bounds__(256) k_oz_series(OzGemm gf, OzGemm gb, int T, 
 // dPhi/dW_l = X^T Zb + dX^T dZb over the atoms of a type (the parameter gradient
 // of pgrad.cu: forward with tangent and reverse mode run on the same GEMMs):
 // digits of the columns of X (rows of the A operand) and of Zb (rows of the B
-// operand), scaled per column and type by its largest magnitude over the atoms.
+// operand), scaled per column and segment of 256 atoms by its largest magnitude
+// there, so that an outlier takes bits from its own segment only; where it takes
+// them from a result, that is summed in FP64 (oz_digits_stand).  With one scale per
+// column and type, a descriptor outlier at one atom and an adjoint outlier at
+// another left errors of 5e-12 to 1e-10 of the first layer's largest entry where
+// FP64 sums, and these, leave 1e-15; the first layer of 12,288 atoms took 257 us,
+// now 293 (the two kernels before it 169 us, now 127 in one).
 // The whole fitting part on the FP64 units, with per-CTA gradient slices, took 63
-// ms for 12,288 water atoms with the student's widths, now 3.7 ms; 648 atoms at
+// ms for 12,288 water atoms with the student's widths, now 3.8 ms; 648 atoms at
 // full width: 23 -> 0.8 ms (24 GEMMs and 14 splits, bound as k_oz_gemm).
 
 struct OzCols {
@@ -875,70 +1019,89 @@ struct OzCols {
     int ld, K, one;      // column `one` is 1 for every atom (-1: none)
     int rb, nb;          // rows per block of the operand (128 or 32), blocks
     uint16_t *out;       // [chunk of 16 atoms][nb][S][rb x 16]
-    int32_t *exp;        // [T][nb rb]
-    unsigned long long *mx;  // [T][nb rb] bits of the largest magnitude (zeroed)
+    int32_t *exp;        // [segment][nb rb] exponent and level (oz_digits_stand)
 };
 struct OzColsPair {
     OzCols c[2];
 };
 
-// Column maxima: threads on columns, CTAs on shares of the type-sorted atoms.
-__global__ void __launch_bounds__(128) k_oz_colmax(OzColsPair pr, const int32_t *__restrict__ type_perm,
-                                                   const int32_t *__restrict__ type_start, int N,
-                                                   int32_t *__restrict__ cnt, int ncnt)
+// Exponents, levels and digits of one segment x 32 columns per CTA
+// (thread: one column, 32 atoms, read once).
+__global__ void __launch_bounds__(256) k_oz_cols(OzColsPair pr, const int32_t *__restrict__ type_perm,
+                                                 const int32_t *__restrict__ type_start, int ntypes,
+                                                 int32_t *__restrict__ cnt, int ncnt)
 {
-    const OzCols &o = pr.c[blockIdx.z];
+    constexpr int S = 8, beta = 7, W = OZ_WSEG * DP_OZ_KC, H = W / 8;
+    __shared__ int perm[W];
+    __shared__ unsigned long long mx_s[8][32], lv_s[2][8][32];
+    const OzCols o = blockIdx.z == 0 ? pr.c[0] : pr.c[1];
+    const int tid = threadIdx.x, c = tid & 31, h = tid >> 5, q = blockIdx.y * 32 + c, ncol = o.nb * o.rb;
     if (blockIdx.x + blockIdx.y + blockIdx.z == 0)  // part counters of the GEMM that follows
-        for (int u = threadIdx.x; u < ncnt; u += 128) cnt[u] = 0;
-    const int q = blockIdx.x * 128 + threadIdx.x;
-    if (q >= o.K) return;
-    const int lo = (int)((long long)blockIdx.y * N / gridDim.y), hi = (int)((long long)(blockIdx.y + 1) * N / gridDim.y);
-    int a = 0;
-    for (int p = lo; p < hi;) {
-        while (p >= type_start[a + 1]) ++a;
-        const int e = min(hi, type_start[a + 1]);
-        unsigned long long mx = 0;
-#pragma unroll 4
-        for (; p < e; ++p) {
-            const unsigned long long b =
-                (unsigned long long)__double_as_longlong(fabs(o.src[(size_t)type_perm[p] * o.ld + q]));
-            mx = b > mx ? b : mx;
-        }
-        atomicMax(&o.mx[(size_t)a * o.nb * o.rb + q], mx);
-    }
-}
-
-// Digits of 16 atoms x 128 columns per CTA (thread: one column, 8 atoms).
-__global__ void __launch_bounds__(256) k_oz_tsplit(OzColsPair pr, const int32_t *__restrict__ type_perm,
-                                                   const int32_t *__restrict__ type_start, int ntypes)
-{
-    constexpr int S = 8, beta = 7;
-    const OzCols &o = pr.c[blockIdx.z];
-    const int q = blockIdx.y * 128 + (threadIdx.x & 127), kh = threadIdx.x >> 7;
-    if (q >= o.nb * o.rb) return;
-    int kc = blockIdx.x, a = 0;
+        for (int u = tid; u < ncnt; u += 256) cnt[u] = 0;
+    int sg = blockIdx.x, a = 0, kb = 0;
     for (;; ++a) {
         if (a == ntypes) return;
-        const int nk = (type_start[a + 1] - type_start[a] + DP_OZ_KC - 1) / DP_OZ_KC;
-        if (kc < nk) break;
-        kc -= nk;
+        const int n = type_start[a + 1] - type_start[a], ns = (n + W - 1) / W;
+        if (sg < ns) break;
+        sg -= ns;
+        kb += (n + DP_OZ_KC - 1) / DP_OZ_KC;
     }
-    const int col = a * o.nb * o.rb + q;
+    if (q >= ncol) return;  // whole CTAs: blocks are multiples of 32 columns
+    const int first = type_start[a] + sg * W, n = min(W, type_start[a + 1] - first);
+    static_assert(W == 256, "one atom per thread");
+    perm[tid] = tid < n ? type_perm[first + tid] : -1;
+    __syncthreads();
+    double v[H];
+    unsigned long long mx = 0;
+#pragma unroll
+    for (int u = 0; u < H; ++u) {
+        const int i = perm[h * H + u];
+        v[u] = i < 0 ? 0.0 : q < o.K ? o.src[(size_t)i * o.ld + q] : q == o.one ? 1.0 : 0.0;
+        const unsigned long long b = (unsigned long long)__double_as_longlong(fabs(v[u]));
+        mx = b > mx ? b : mx;
+    }
+    mx_s[h][c] = mx;
+    __syncthreads();
+#pragma unroll
+    for (int u = 0; u < 8; ++u) mx = mx_s[u][c] > mx ? mx_s[u][c] : mx;
     bool zero;
-    const int ex = oz_exponent(q == o.one ? 0x3ff0000000000000ull : q < o.K ? o.mx[col] : 0, beta * S, zero);
-    if (kc == 0 && kh == 0) o.exp[col] = ex;
-    long long J[8];
+    const int ex = oz_exponent(mx, beta * S, zero);
+    uint16_t *out = o.out + ((size_t)(kb + sg * OZ_WSEG) * o.nb + q / o.rb) * S * o.rb * DP_OZ_KC + oz_kofs(q % o.rb, 0);
+    // values of level l or less, l = 0 .. 15, a byte each
+    unsigned long long lo = 0, hi = 0;
+    constexpr unsigned long long ONES = 0x0101010101010101ull;
 #pragma unroll
-    for (int u = 0; u < 8; ++u) {
-        const int p = type_start[a] + kc * DP_OZ_KC + kh * 8 + u;
-        double v = 0.0;
-        if (!zero && p < type_start[a + 1]) v = q == o.one ? 1.0 : o.src[(size_t)type_perm[p] * o.ld + q];
-        J[u] = oz_rint_pow2(v, beta * S - ex) + oz_digit_bias(S, beta);
+    for (int k = 0; k < H / 8; ++k) {
+        const int at = h * H + 8 * k, kc = at / DP_OZ_KC;
+        long long J[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            const long long I = zero ? 0 : oz_rint_pow2(v[8 * k + u], beta * S - ex);
+            const int l = __clzll(I < 0 ? -I : I) - (63 - beta * S);  // |I| <= 2^56
+            if (l < 8) lo += ONES << (8 * l);
+            if (l < 16) hi += l < 8 ? ONES : ONES << (8 * (l - 8));
+            J[u] = I + oz_digit_bias(S, beta);
+        }
+        if (kc * DP_OZ_KC < n) {
+            uint16_t *ok = out + (size_t)kc * o.nb * S * o.rb * DP_OZ_KC + (at % DP_OZ_KC) / 8 * 64;
+#pragma unroll
+            for (int sd = 0; sd < S; ++sd)
+                *reinterpret_cast<uint4 *>(ok + (size_t)sd * o.rb * DP_OZ_KC) = oz_pack_digits<S, beta>(J, sd);
+        }
     }
-    uint16_t *out = o.out + ((size_t)blockIdx.x * o.nb + q / o.rb) * S * o.rb * DP_OZ_KC + oz_kofs(q % o.rb, kh * 8);
-#pragma unroll
-    for (int sd = 0; sd < S; ++sd)
-        *reinterpret_cast<uint4 *>(out + (size_t)sd * o.rb * DP_OZ_KC) = oz_pack_digits<S, beta>(J, sd);
+    lv_s[0][h][c] = lo;
+    lv_s[1][h][c] = hi;
+    __syncthreads();
+    if (h == 0) {
+        auto count = [&](int l) {  // values of level l or less
+            int v = 0;
+            for (int u = 0; u < 8; ++u) v += (int)(lv_s[l >> 3][u][c] >> (8 * (l & 7)) & 0xff);
+            return v;
+        };
+        int l = zero ? -16 : 0;  // zeros: every product with them is exact; NaN: the digits do not count
+        while (l >= 0 && l < 15 && 4 * count(l) < 3 * n) ++l;
+        o.exp[(size_t)blockIdx.x * ncol + q] = ex * (1 << OZ_LVL_BITS) + (l & ((1 << OZ_LVL_BITS) - 1));
+    }
 }
 
 // Adjoints of the output layer: hb = cE w_out, dhb = -w_out of the atom's type,
@@ -1151,11 +1314,12 @@ struct OzRun {
         return cudaGetLastError();
     }
 
-    // epi 0: forward (bias, tanh, skip); 1: backward (skip gradient); 2: tangent forward
+    // epi 0: forward (bias, tanh, skip); 1: backward (skip gradient); 2: tangent forward; 3: weight gradient
     template <int S>
     cudaError_t launch_epi(const OzGemmArgs &a, int epi) const
     {
-        const bool seg = a.wg || a.g.seg < a.g.nK;
+        const bool seg = a.g.seg < a.g.nK;
+        if (epi == 3) return launch_as<S, 3, true>(a);
         if (epi == 0) return seg ? launch_as<S, 0, true>(a) : launch_as<S, 0, false>(a);
         if (epi == 1) return seg ? launch_as<S, 1, true>(a) : launch_as<S, 1, false>(a);
         return seg ? launch_as<S, 2, true>(a) : launch_as<S, 2, false>(a);
@@ -1260,10 +1424,11 @@ size_t dp_oz_grad_elems(const DevModel &m, const OzModel &oz, int64_t natoms, in
     const size_t K = (size_t)m.m2 * m.M > (size_t)oz.fmax ? (size_t)m.m2 * m.M : (size_t)oz.fmax;
     const size_t nq = K / DP_OZ_TILE + 1, nn = (oz.fmax + DP_OZ_NC - 1) / DP_OZ_NC;
     const size_t chunks = (size_t)natoms / DP_OZ_KC + m.ntypes;
+    const size_t segs = (size_t)natoms / (OZ_WSEG * DP_OZ_KC) + m.ntypes;
     switch (which) {
     case 0: return chunks * nq * 8 * OZ_A_BLK;
     case 1: return chunks * nn * 8 * OZ_B_BLK;
-    case 2: return (size_t)m.ntypes * (nq * DP_OZ_TILE + nn * DP_OZ_NC);
+    case 2: return segs * (nq * DP_OZ_TILE + nn * DP_OZ_NC);
     default: return 6 * (size_t)natoms * oz.fmax;
     }
 }
@@ -1302,31 +1467,25 @@ cudaError_t dp_launch_pgrad_fit_oz(cudaStream_t st, const DevModel &m, const OzM
     auto weights = [&](const double *x, const double *dx, int ldx, int K, int F, int64_t off) -> cudaError_t {
         const int nq = K / DP_OZ_TILE + 1, nN = (F + DP_OZ_NC - 1) / DP_OZ_NC;  // K + 1 rows
         for (int pass = 0; pass < 2; ++pass) {
+            const int segs = N / (OZ_WSEG * DP_OZ_KC) + T;
             OzColsPair c;
-            int32_t *expb = og.exp + (size_t)T * nq * DP_OZ_TILE;
-            c.c[0] = OzCols{pass == 0 ? x : dx, ldx, K, pass == 0 ? K : -1, DP_OZ_TILE, nq, og.a, og.exp, og.mx};
-            c.c[1] = OzCols{pass == 0 ? zb : dzb, ld, F, -1, DP_OZ_NC, nN, og.b, expb,
-                            og.mx + (size_t)T * nq * DP_OZ_TILE};
-            const size_t cols = (size_t)T * (nq * DP_OZ_TILE + nN * DP_OZ_NC);
-            cudaError_t e2 = cudaMemsetAsync(og.mx, 0, 8 * cols, st);
-            // the exponents too: a type without atoms in the frame has no chunk that writes them
-            if (e2 == cudaSuccess) e2 = cudaMemsetAsync(og.exp, 0, 4 * cols, st);
-            if (e2 != cudaSuccess) return e2;
-            // column maxima: 16 CTAs per SM, 16 atoms each or more (on 64 shares of the
-            // atoms a pass over 240 columns of 12,288 took 82 us, now 21)
-            const int cb = (std::max(K, F) + 127) / 128;
-            const int splits = std::max(1, std::min(8 * num_sms / cb, N / 16));
-            k_oz_colmax<<<dim3(cb, splits, 2), 128, 0, st>>>(c, nb.type_perm, nb.type_start, N, ob.cnt,
-                                                                                 ob.slots * 8);
-            k_oz_tsplit<<<dim3(N / DP_OZ_KC + T, std::max(nq, (nN * DP_OZ_NC + 127) / 128), 2), 256, 0, st>>>(
-                c, nb.type_perm, nb.type_start, T);
-            *launches += 2;
+            int32_t *expb = og.exp + (size_t)segs * nq * DP_OZ_TILE;
+            c.c[0] = OzCols{pass == 0 ? x : dx, ldx, K, pass == 0 ? K : -1, DP_OZ_TILE, nq, og.a, og.exp};
+            c.c[1] = OzCols{pass == 0 ? zb : dzb, ld, F, -1, DP_OZ_NC, nN, og.b, expb};
+            k_oz_cols<<<dim3(segs, std::max(nq * DP_OZ_TILE, nN * DP_OZ_NC) / 32, 2), 256, 0, st>>>(
+                c, nb.type_perm, nb.type_start, T, ob.cnt, ob.slots * 8);
+            *launches += 1;
             OzGemmArgs a;
             std::memset(&a, 0, sizeof(a));
             a.a = og.a;
             a.aexp = og.exp;
             a.w = og.b;
             a.wexp = expb;
+            a.x = c.c[0].src;
+            a.z = c.c[1].src;
+            a.ldx = ldx;
+            a.ldz = ld;
+            a.one = pass == 0;
             a.g.N = F;
             a.g.nN = nN;
             a.g.beta = 7;
@@ -1339,7 +1498,8 @@ cudaError_t dp_launch_pgrad_fit_oz(cudaStream_t st, const DevModel &m, const OzM
             a.ldo = a.ldh = F;
             for (int t = 0; t < T; ++t) a.out_off[t] = m.fit_base[t] + off;
             a.units = T * nq * nN;
-            if ((e2 = r.launch(a, 1)) != cudaSuccess) return e2;
+            const cudaError_t e2 = r.launch(a, 3);
+            if (e2 != cudaSuccess) return e2;
         }
         return cudaSuccess;
     };
