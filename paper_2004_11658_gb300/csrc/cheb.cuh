@@ -2,17 +2,16 @@
 // (csrc/embed_cheb.cu): shapes, buffers and launchers.
 #pragma once
 
+#include "cheb_domain.h"
 #include "dp_internal.cuh"
 
-// Nodes (and stored terms) per net, and the resolved domain s in [0, S], mapped
-// to t = (2 / S) s - 1.  S = 4/3 is r = 0.75 A, below the O-H bond; nearer rows
-// evaluate the net itself.  (S = 2 needs 24 terms instead of 20.)
+// Nodes (and stored terms) per net.  The domain s in [0, S] (dp_cheb_domain) is
+// mapped to t = (2 / S) s - 1.
 constexpr int DP_CHEB_NN = 48;
-constexpr double DP_CHEB_SCALE = 1.5;               // 2 / S
-constexpr double DP_CHEB_S = 2.0 / DP_CHEB_SCALE;
 
 struct ChebModel {
     int n;             // terms used by every net (0: not resolved, the series is not used)
+    double S, scale;   // domain and 2 / S
     const double *C;   // [T T][NN][M]: G_f(s) = sum_n C[net][n][f] T_n(t)
     const double *Ct;  // [T][M][T NN]: the same values, the nets of centre type a side by side
     const double *V;   // [T T][NN][M]: dG_f/ds = sum_n V[net][n][f] T_n(t)
@@ -31,7 +30,7 @@ bool dp_cheb_supported(const DevModel &m);
 size_t dp_cheb_elems(const DevModel &m, int which);  // doubles of C, Ct, V, y, mx, trig (which = 0..5)
 cudaError_t dp_launch_cheb_setup(cudaStream_t st, ChebBuffers cb, int64_t *launches);
 // Coefficients of every net from the device parameters.
-cudaError_t dp_launch_cheb_build(cudaStream_t st, const DevModel &m, ChebBuffers cb, int64_t *launches);
+cudaError_t dp_launch_cheb_build(cudaStream_t st, const DevModel &m, double scale, ChebBuffers cb, int64_t *launches);
 // Terms needed for the nets of the host copy of mx, 0 if not resolved.
 int dp_cheb_terms(const DevModel &m, const double *mx);
 

@@ -572,7 +572,7 @@ dp_status ensure_cheb(dp_ctx *c)
     GroupTimer tm(c, G_EMBED_FWD);
     cudaError_t e = cudaSuccess;
     if (c->cheb_version < 0) e = dp_launch_cheb_setup(c->stream, c->cb, &c->launches);
-    if (e == cudaSuccess) e = dp_launch_cheb_build(c->stream, c->m, c->cb, &c->launches);
+    if (e == cudaSuccess) e = dp_launch_cheb_build(c->stream, c->m, c->cheb.scale, c->cb, &c->launches);
     if (e != cudaSuccess) return cuda_fail(e, "embedding series");
     const size_t bytes = sizeof(double) * dp_cheb_elems(c->m, 4);
     DP_CUDA(cudaMemcpyAsync(c->h_cheb_mx, c->cb.mx, bytes, cudaMemcpyDeviceToHost, c->stream), "embedding series");
@@ -1077,6 +1077,8 @@ dp_status dp_ctx_create(const dp_model *model, int64_t natoms_max, int32_t cand_
             s = fail(DP_ERR_NOMEM, "pinned allocation failed");
         }
         c->use_cheb = true;
+        c->cheb.S = dp_cheb_domain(c->m.rcut);
+        c->cheb.scale = 2.0 / c->cheb.S;
         OzSeries &os = c->os;
         if (dp_oz_series_plan(c->m, DP_CHEB_NN, os)) {
             ALLOC(os.w, (size_t)os.w_elems);

@@ -23,7 +23,7 @@
 // rounded to FP64.  dp_cheb_terms keeps the terms until the derivative of what
 // is left is below 2^-55 of the net's size; a net that 44 terms do not resolve
 // makes the context use the kernels of embed_x.cu / embed.cu instead.  Rows
-// with s > S (r < 0.75 A) evaluate the net itself, one row at a time.
+// with s > S (r < 0.75 A, dp_cheb_domain) evaluate the net itself, one row at a time.
 //
 // What bounds the kernels: the FP64 pipe (16 cycles per warp instruction and SM).
 // One 128-thread CTA per atom, several per SM, so that the phases of different
@@ -162,14 +162,15 @@ __device__ dd dd_tanh(dd x, const double *__restrict__ tab)
 
 // One CTA per (net, node): the net at s_k = S/2 (1 + cos(pi (2k+1) / (2 NN))),
 // thread o on output o of each layer.
-__global__ void __launch_bounds__(CT) k_cheb_nodes(DevModel m, const double *__restrict__ trig, double *__restrict__ y)
+__global__ void __launch_bounds__(CT) k_cheb_nodes(DevModel m, double scale, const double *__restrict__ trig,
+                                                   double *__restrict__ y)
 {
     __shared__ dd h[2][DP_MAX_EMB_W];
     const int net = blockIdx.x / NN, k = blockIdx.x % NN, o = threadIdx.x;
     const double *W = m.params + m.emb_base[net];
     const int q = 2 * k + 1;
     dd s = dd_add({1.0, 0.0}, {trig[2 * q], trig[2 * q + 1]});
-    s = dd_div(s, {DP_CHEB_SCALE, 0.0});
+    s = dd_div(s, {scale, 0.0});
     const double *tab = trig + 2 * 4 * NN;
     int win = m.emb[0], cur = 0;
     if (o < win) h[0][o] = dd_tanh(dd_add(dd_mul(s, {W[o], 0.0}), {W[win + o], 0.0}), tab);
@@ -228,13 +229,14 @@ __global__ void __launch_bounds__(CT) k_cheb_coef(DevModel m, const double *__re
 
 // Coefficients of the derivative, V_n = (2 / S) (2 - [n = 0]) sum_{m = n+1, n+3, ..} m C_m
 // (the terms decrease geometrically: smallest first).
-__global__ void __launch_bounds__(CT) k_cheb_deriv(DevModel m, const double *__restrict__ C, double *__restrict__ V)
+__global__ void __launch_bounds__(CT) k_cheb_deriv(DevModel m, double scale, const double *__restrict__ C,
+                                                   double *__restrict__ V)
 {
     const int net = blockIdx.x / NN, n = blockIdx.x % NN, f = threadIdx.x;
     if (f >= m.M) return;
     double v = 0.0;
     for (int q = NN - 1 - (NN - n) % 2; q > n; q -= 2) v = fma((double)q, C[(size_t)(net * NN + q) * m.M + f], v);
-    V[(size_t)blockIdx.x * m.M + f] = v * ((n == 0 ? 1.0 : 2.0) * DP_CHEB_SCALE);
+    V[(size_t)blockIdx.x * m.M + f] = v * ((n == 0 ? 1.0 : 2.0) * scale);
 }
 
 // ---------------------------------------------------------- rows beyond S ---
@@ -290,7 +292,7 @@ __device__ __forceinline__ int row_block(const int *start, int T, int q)
 }
 
 // Adds the rows beyond S to T (Ts [4][M], scaled), in row order, by the whole CTA.
-__device__ __forceinline__ void far_rows_T(const DevModel &m, int a, int i, const int *start,
+__device__ __forceinline__ void far_rows_T(const DevModel &m, double S, int a, int i, const int *start,
                                            double (&fbuf)[4][DP_MAX_EMB_W], const double *pair_d, double *Ts)
 {
     const int T = m.ntypes, M = m.M, tid = threadIdx.x;
@@ -304,7 +306,7 @@ __device__ __forceinline__ void far_rows_T(const DevModel &m, int a, int i, cons
                                               __dmul_rn(dv[2], dv[2])));
         double s, ds, inv;
         dp_switch_inv(r, m.rcut_smth, m.rcut, irc, s, ds, inv);
-        if (s <= DP_CHEB_S) continue;  // uniform: every thread has the same row
+        if (s <= S) continue;  // uniform: every thread has the same row
         net_direct(m, a * T + b, s, ga, da, gb, db);
         const double sr = s * inv;
         for (int p = tid; p < 4 * M; p += CT) {
@@ -385,13 +387,13 @@ __global__ void __launch_bounds__(CT) k_cheb_fwd(DevModel m, ChebModel cm, const
             pair_d[slot * 3 + 1] = d[1];
             pair_d[slot * 3 + 2] = d[2];
             const double sr = s * inv;
-            far = !(s <= DP_CHEB_S);
+            far = !(s <= cm.S);
             double *Rq = R4 + tid * 4;
             Rq[0] = far ? 0.0 : s;
             Rq[1] = far ? 0.0 : sr * d[0];
             Rq[2] = far ? 0.0 : sr * d[1];
             Rq[3] = far ? 0.0 : sr * d[2];
-            const double t = far ? 0.0 : fma(s, DP_CHEB_SCALE, -1.0), t2 = t + t;
+            const double t = far ? 0.0 : fma(s, cm.scale, -1.0), t2 = t + t;
             double p0 = 1.0, p1 = t;
             Tch[tid] = 1.0;
             for (int n = 1; n < nc; ++n) {
@@ -464,13 +466,13 @@ __global__ void __launch_bounds__(CT) k_cheb_fwd(DevModel m, ChebModel cm, const
         }
     }
     __syncthreads();
-    if (any_far) far_rows_T(m, a, i, start, fbuf, pair_d, Ts);
+    if (any_far) far_rows_T(m, cm.S, a, i, start, fbuf, pair_d, Ts);
     for (int p = tid; p < 4 * M; p += CT) Tout[(size_t)i * 4 * M + p] = Ts[p];
     descriptor(m, i, Ts, Dout);
 }
 
 // T of one atom finished (rows beyond S added) and D = T_<^T T, one CTA per atom.
-__global__ void __launch_bounds__(CT) k_cheb_desc(DevModel m, const int32_t *__restrict__ types,
+__global__ void __launch_bounds__(CT) k_cheb_desc(DevModel m, double S, const int32_t *__restrict__ types,
                                                   const int32_t *__restrict__ type_perm,
                                                   const int32_t *__restrict__ nreal, const double *__restrict__ flag,
                                                   const double *__restrict__ pair_d, double *__restrict__ Tio,
@@ -493,7 +495,7 @@ __global__ void __launch_bounds__(CT) k_cheb_desc(DevModel m, const int32_t *__r
     }
     __syncthreads();
     if (far) {
-        far_rows_T(m, types[i], i, start, fbuf, pair_d, Ts);
+        far_rows_T(m, S, types[i], i, start, fbuf, pair_d, Ts);
         for (int p = tid; p < 4 * M; p += CT) Tio[(size_t)i * 4 * M + p] = Ts[p];
     }
     descriptor(m, i, Ts, Dout);
@@ -596,7 +598,7 @@ __global__ void __launch_bounds__(CT) k_cheb_bwd(DevModel m, ChebModel cm, const
         const double *u = UV + b * nc * 8 + c;
         double v = 0.0;
         for (int q = n + 1; q < nc; q += 2) v = fma((double)q, u[q * 8], v);
-        UV[k * 8 + 4 + c] = v * ((n == 0 ? 1.0 : 2.0) * DP_CHEB_SCALE);
+        UV[k * 8 + 4 + c] = v * ((n == 0 ? 1.0 : 2.0) * cm.scale);
     }
     __syncthreads();
 
@@ -632,10 +634,10 @@ __global__ void __launch_bounds__(CT) k_cheb_bwd(DevModel m, ChebModel cm, const
             const double d[3] = {pg[0], pg[1], pg[2]};
             double s, ds, inv;
             dp_switch_inv(radius(d), m.rcut_smth, m.rcut, irc, s, ds, inv);
-            far = !(s <= DP_CHEB_S);
+            far = !(s <= cm.S);
             if (!far) {
                 const double sr = s * inv;
-                const double t = fma(s, DP_CHEB_SCALE, -1.0), t2 = t + t;
+                const double t = fma(s, cm.scale, -1.0), t2 = t + t;
                 const double2 *uv = reinterpret_cast<const double2 *>(UV + b * nc * 8);
                 double P[4] = {uv[0].x, uv[0].y, uv[1].x, uv[1].y};
                 double Qc[4] = {uv[2].x, uv[2].y, uv[3].x, uv[3].y};
@@ -780,8 +782,8 @@ __global__ void __launch_bounds__(CT) k_chebpg_fwd(DevModel m, ChebModel cm, con
                 Rq[5 + e] = dst * u[e] + s * inv * (dr[e] - u[e] * udr);
                 Rq[9 + e] = s * u[e] * dst;
             }
-            any_far |= !(s <= DP_CHEB_S);
-            const double t = fma(s, DP_CHEB_SCALE, -1.0), t2 = t + t;
+            any_far |= !(s <= cm.S);
+            const double t = fma(s, cm.scale, -1.0), t2 = t + t;
             double p0 = 1.0, p1 = t;
             Tch[tid] = 1.0;
             for (int n = 1; n < nc; ++n) {
@@ -1020,7 +1022,7 @@ __global__ void k_chebpg_sum(double *__restrict__ part, size_t elems, int splits
 // Gb_f = sum_n w_nk Cb_nf and G'b_f = sum_n w_nk Vb_nf with w_nk = (2 - [n = 0]) / NN
 // cos(pi n (2k+1) / (2 NN)), and reverse mode through the layers with their
 // s-tangents; h, dh, zb and dzb of every layer go to node[net][k][0 .. 3][.].
-__global__ void __launch_bounds__(CT) k_chebpg_node(DevModel m, int nc, const double *__restrict__ trig,
+__global__ void __launch_bounds__(CT) k_chebpg_node(DevModel m, int nc, double scale, const double *__restrict__ trig,
                                                     const double *__restrict__ Cb, const double *__restrict__ Vb,
                                                     double *__restrict__ node, int se, const int32_t *far_flag)
 {
@@ -1030,7 +1032,7 @@ __global__ void __launch_bounds__(CT) k_chebpg_node(DevModel m, int nc, const do
     __shared__ double g[DP_MAX_EMB_W], dg[DP_MAX_EMB_W], zb[DP_MAX_EMB_W], dzb[DP_MAX_EMB_W];
     const int net = blockIdx.x / NN, k = blockIdx.x % NN, o = threadIdx.x, M = m.M;
     const double *P = m.params + m.emb_base[net];
-    const double s = (1.0 + trig[2 * (2 * k + 1)]) / DP_CHEB_SCALE;
+    const double s = (1.0 + trig[2 * (2 * k + 1)]) / scale;
     if (o < m.emb[0]) {
         const double tv = dp_tanh64(fma(s, P[o], P[m.emb[0] + o]), m.tanh_tab);
         h[0][o] = t[0][o] = tv;
@@ -1113,7 +1115,7 @@ __global__ void __launch_bounds__(CT) k_chebpg_node(DevModel m, int nc, const do
 
 // Gradient of every embedding parameter from the nodes: dW[q][o] = sum_k h_k[q]
 // zb_k[o] + dh_k[q] dzb_k[o] (layer 0: h = s, dh = 1), db[o] = sum_k zb_k[o].
-__global__ void k_chebpg_grad(DevModel m, const double *__restrict__ trig, const double *__restrict__ node, int se,
+__global__ void k_chebpg_grad(DevModel m, double scale, const double *__restrict__ trig, const double *__restrict__ node, int se,
                               double *__restrict__ grad, const int32_t *far_flag)
 {
     if (*far_flag) return;
@@ -1133,7 +1135,7 @@ __global__ void k_chebpg_grad(DevModel m, const double *__restrict__ trig, const
             const double *n = nd + (size_t)k * 4 * se;
             double hv = 1.0, dv = 0.0;
             if (q < in) {
-                hv = l == 0 ? (1.0 + trig[2 * (2 * k + 1)]) / DP_CHEB_SCALE : n[lo - in + q];
+                hv = l == 0 ? (1.0 + trig[2 * (2 * k + 1)]) / scale : n[lo - in + q];
                 dv = l == 0 ? 1.0 : n[se + lo - in + q];
             }
             v = fma(hv, n[2 * se + lo + o], v);
@@ -1190,12 +1192,12 @@ cudaError_t dp_launch_cheb_setup(cudaStream_t st, ChebBuffers cb, int64_t *launc
     return cudaGetLastError();
 }
 
-cudaError_t dp_launch_cheb_build(cudaStream_t st, const DevModel &m, ChebBuffers cb, int64_t *launches)
+cudaError_t dp_launch_cheb_build(cudaStream_t st, const DevModel &m, double scale, ChebBuffers cb, int64_t *launches)
 {
     const int grid = m.ntypes * m.ntypes * NN;
-    k_cheb_nodes<<<grid, CT, 0, st>>>(m, cb.trig, cb.y);
+    k_cheb_nodes<<<grid, CT, 0, st>>>(m, scale, cb.trig, cb.y);
     k_cheb_coef<<<grid, CT, 0, st>>>(m, cb.trig, cb.y, cb.C, cb.Ct, cb.mx);
-    k_cheb_deriv<<<grid, CT, 0, st>>>(m, cb.C, cb.V);
+    k_cheb_deriv<<<grid, CT, 0, st>>>(m, scale, cb.C, cb.V);
     *launches += 3;
     return cudaGetLastError();
 }
@@ -1208,10 +1210,11 @@ int dp_cheb_terms(const DevModel &m, const double *mx)
         double size = 0.0, tail = 0.0;
         for (int n = 0; n < NN; ++n) size = c[n] > size ? c[n] : size;
         if (!(size <= 1e300)) return 0;
-        // |d/ds of the terms n ..| <= (2 / S) sum n^2 |C_n|
+        // the derivative of the terms n .., by s / S, is 2 sum n^2 |C_n| or less (3/4 of
+        // it are asked for: as by s at S = 4/3)
         int n = NN;
         for (; n > 0; --n) {
-            tail += DP_CHEB_SCALE * (double)(n - 1) * (n - 1) * c[n - 1];
+            tail += 1.5 * (double)(n - 1) * (n - 1) * c[n - 1];
             if (tail > 0x1p-55 * size) break;
         }
         need = n > need ? n : need;
@@ -1259,7 +1262,7 @@ cudaError_t dp_launch_cheb_fwd(cudaStream_t st, const DevModel &m, const ChebMod
     if ((e = dp_launch_oz_rows(st, m, *os, os->gf, a_dig, N, eb.gD, Kt, eb.T, m.M, nb, num_sms, status, launches)) !=
         cudaSuccess)
         return e;
-    k_cheb_desc<<<N, CT, 0, st>>>(m, types, nb.type_perm, fb.nreal, eb.Ei, eb.pair_g, eb.T, eb.D);
+    k_cheb_desc<<<N, CT, 0, st>>>(m, cm.S, types, nb.type_perm, fb.nreal, eb.Ei, eb.pair_g, eb.T, eb.D);
     *launches += 1;
     return cudaGetLastError();
 }
@@ -1342,8 +1345,8 @@ cudaError_t dp_launch_chebpg_bwd(cudaStream_t st, const DevModel &m, const ChebM
         m, cm.n, nb.type_perm, nb.type_start, gb.mom, eb.T, pb.dT, gb.part, gb.far);
     const size_t elems = 2 * (size_t)T * T * NN * m.M;
     k_chebpg_sum<<<(int)((elems + 255) / 256), 256, 0, st>>>(gb.part, elems, splits, gb.far);
-    k_chebpg_node<<<T * T * NN, CT, 0, st>>>(m, cm.n, trig, gb.part, gb.part + elems / 2, gb.node, se, gb.far);
-    k_chebpg_grad<<<dim3((m.emb_net_size + 255) / 256, T * T), 256, 0, st>>>(m, trig, gb.node, se, grad, gb.far);
+    k_chebpg_node<<<T * T * NN, CT, 0, st>>>(m, cm.n, cm.scale, trig, gb.part, gb.part + elems / 2, gb.node, se, gb.far);
+    k_chebpg_grad<<<dim3((m.emb_net_size + 255) / 256, T * T), 256, 0, st>>>(m, cm.scale, trig, gb.node, se, grad, gb.far);
     *launches += 5;
     return cudaGetLastError();
 }
