@@ -439,40 +439,52 @@ __device__ __forceinline__ bool oz_unit(const OzGemmArgs &p, int u, OzUnit &U)
 // Entries of a weight gradient that the digits of a segment may not carry.  The
 // digit product of n atoms errs by about 2^-58 sqrt(n) of the two columns' powers
 // of two 2^e, 2^f (the groups left out); a chain of FP64 FMAs by 2^-54 or more of the
-// products' size, which is smaller than 2^(e+f) when the columns have their
-// outliers at different atoms.  A column's level l says that three quarters of its
-// values are at least 2^(e-l).  The digits stand where the two levels are at most
-// OZ_EVEN together (normal deviates have 4 or 5 each; two columns at the line with
-// one outlier each leave products of 2^-5 and more), or where the result itself is
-// at least an eighth of 2^(e+f) (an outlier in one column only).  The others are
-// summed from the FP64 values.
-constexpr int OZ_EVEN = 10;
+// products' size, which is far below 2^(e+f) when the columns have their outliers
+// at different atoms.  A column's level l says that three quarters of its values
+// are at least 2^(e-l).  The digits stand where X's column is even (OZ_EVEN; normal
+// deviates have 4, a few per cent 5 or 6): Z's outliers then meet values of 2^(e-l);
+// where the two levels are small together; or where the result itself is at least
+// an eighth of 2^(e+f).  The others are summed from the FP64 values.  An even Z
+// alone is not enough: an atom with an outlier in X has saturated units, whose Z is 0.
+constexpr int OZ_EVEN = 5;
 constexpr int OZ_LVL_BITS = 5;  // exponent and level in one word; level -16: zeros, NaN
-__device__ __forceinline__ bool oz_digits_stand(double y, int va, int vw)
+__device__ __forceinline__ bool oz_digits_stand(double y, int vx, int vz)
 {
     constexpr int sh = 32 - OZ_LVL_BITS;
-    if (((va << sh) >> sh) + ((vw << sh) >> sh) <= OZ_EVEN) return true;
+    const int lx = (vx << sh) >> sh, lz = (vz << sh) >> sh;
+    if (lx <= OZ_EVEN || lx + lz <= 2 * OZ_EVEN) return true;
     const int ey = (int)((__double_as_longlong(y) >> 52) & 0x7ff) - 1023;  // |y| >= 2^ey
-    return ey >= (va >> OZ_LVL_BITS) + (vw >> OZ_LVL_BITS) - 3;
+    return ey >= (vx >> OZ_LVL_BITS) + (vz >> OZ_LVL_BITS) - 3;
 }
-// One entry (row k, column f) over na atoms of a segment by the whole warp: lanes
-// on the atoms, then a fixed tree.  (One lane's chain of loads held its warp up
-// for 70 k cycles: a few entries in 10,000 took the GEMM from 250 to 640 us.)
+// Row k, columns f .. f + 15, over na atoms of a segment by the whole warp: lanes on
+// the atoms, then a transposing tree that leaves column f + n on lanes 2n, 2n + 1.
+// (An entry at a time on its own lane held the warp up for 70 k cycles of dependent
+// loads, and a few entries in 10,000 took the GEMM from 290 to 640 us.)
 __device__ __noinline__ double oz_wdot(const OzGemmArgs &p, int at0, int na, int k, int f)
 {
     const int lane = threadIdx.x & 31;
-    double v = 0.0;
+    double v[16];
 #pragma unroll
-    for (int u = 0; u < OZ_WSEG * DP_OZ_KC / 32; ++u) {
-        const int q = lane + 32 * u;
-        if (q < na) {
-            const size_t i = p.type_perm[at0 + q];
-            v = fma(k < p.rows - 1 ? p.x[i * p.ldx + k] : p.one ? 1.0 : 0.0, p.z[i * p.ldz + f], v);
-        }
+    for (int n = 0; n < 16; ++n) v[n] = 0.0;
+#pragma unroll 2
+    for (int q = lane; q < na; q += 32) {
+        const size_t i = p.type_perm[at0 + q];
+        const double x = k < p.rows - 1 ? p.x[i * p.ldx + k] : p.one ? 1.0 : 0.0;
+        const double *z = p.z + i * p.ldz + f;
+#pragma unroll
+        for (int n = 0; n < 16; ++n)
+            if (f + n < p.g.N) v[n] = fma(x, z[n], v[n]);
     }
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    return v;
+    for (int w = 16, m = 8; w >= 2; w >>= 1, m >>= 1) {
+        const bool up = (lane & w) != 0;
+#pragma unroll
+        for (int n = 0; n < m; ++n) {
+            const double send = up ? v[n] : v[m + n], keep = up ? v[m + n] : v[n];
+            v[n] = keep + __shfl_xor_sync(0xffffffffu, send, w);
+        }
+    }
+    return v[0] + __shfl_xor_sync(0xffffffffu, v[0], 1);
 }
 
 // Persistent, one CTA per SM over the units (tile, 32-column chunk of Y) in
@@ -776,13 +788,12 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_oz_gemm(OzGemmArgs p)
                     }
                     for (unsigned who = __ballot_sync(0xffffffffu, bad != 0); who != 0; who &= who - 1) {
                         const int src = __ffs(who) - 1, k = __shfl_sync(0xffffffffu, i, src);
-                        for (unsigned m = __shfl_sync(0xffffffffu, bad, src); m != 0; m &= m - 1) {
-                            const int q = __ffs(m) - 1;
-                            const double y = oz_wdot(p, U.first + sg * OZ_WSEG * DP_OZ_KC,
-                                                     min(U.cnt - sg * OZ_WSEG * DP_OZ_KC, OZ_WSEG * DP_OZ_KC), k, n0 + q);
+                        const double y = oz_wdot(p, U.first + sg * OZ_WSEG * DP_OZ_KC,
+                                                 min(U.cnt - sg * OZ_WSEG * DP_OZ_KC, OZ_WSEG * DP_OZ_KC), k, n0);
 #pragma unroll
-                            for (int n = 0; n < 16; ++n)
-                                if (n == q && lane == src) acc[n >> 3][n & 7] += y;
+                        for (int n = 0; n < 16; ++n) {
+                            const double yn = __shfl_sync(0xffffffffu, y, 2 * n);
+                            if (lane == src && (bad >> n & 1u)) acc[n >> 3][n & 7] += yn;
                         }
                     }
                     __syncwarp();
