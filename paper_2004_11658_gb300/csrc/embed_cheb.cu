@@ -21,8 +21,8 @@
 // double-double arithmetic (Dekker 1971, Knuth's two-sum), k_cheb_coef the discrete
 // transform, also in double-double, so the stored coefficients are the series'
 // rounded to FP64.  dp_cheb_terms keeps the terms until the derivative of what
-// is left is below 2^-55 of the net's size; a net that 44 terms do not resolve
-// makes the context use the kernels of embed_x.cu / embed.cu instead.  Rows
+// is left is below 2^-55 of the net's size; a net that 44 terms do not resolve,
+// or that the series misses between its nodes (k_cheb_check), makes the context use the kernels of embed_x.cu / embed.cu instead.  Rows
 // with s > S (r < 0.75 A, dp_cheb_domain) evaluate the net itself, one row at a time.
 //
 // What bounds the kernels: the FP64 pipe (16 cycles per warp instruction and SM).
@@ -289,6 +289,40 @@ __device__ __forceinline__ int row_block(const int *start, int T, int q)
     int b = 0;
     while (b + 1 < T && q >= start[b + 1]) ++b;
     return b;
+}
+
+// The series (all NN terms) against the net in FP64 at the points between the nodes
+// and the ends of the domain, s = S/2 (1 + cos(pi j / NN)): a unit that turns between
+// two nodes (at s = 0 the first node is at S / 3734) leaves coefficients that look
+// resolved.  Where they differ by more than 2^-40 of the net's size, mx marks the net
+// as not resolved.  One CTA per (net, point).
+__global__ void __launch_bounds__(CT) k_cheb_check(DevModel m, double scale, const double *__restrict__ trig,
+                                                   const double *__restrict__ C, double *__restrict__ mx)
+{
+    __shared__ double fbuf[4][DP_MAX_EMB_W];
+    __shared__ double wm[CT / 32];
+    const int net = blockIdx.x / (NN + 1), j = blockIdx.x % (NN + 1), f = threadIdx.x, M = m.M;
+    const double t = trig[4 * j], t2 = t + t;
+    double *ga = fbuf[0], *da = fbuf[1], *gb = fbuf[2], *db = fbuf[3];
+    net_direct(m, net, (1.0 + t) / scale, ga, da, gb, db);
+    double diff = 0.0, size = 0.0;
+    if (f < M) {
+        double v = 0.0, p0 = 1.0, p1 = t;
+#pragma unroll 8
+        for (int n = 0; n < NN; ++n) {
+            const double c = C[(size_t)(net * NN + n) * M + f], p2 = fma(t2, p1, -p0);
+            v = fma(c, p0, v);
+            size = fmax(size, fabs(c));
+            p0 = p1;
+            p1 = p2;
+        }
+        diff = fabs(v - ga[f]);
+    }
+    for (int s = 16; s > 0; s >>= 1) size = fmax(size, __shfl_xor_sync(FULL, size, s));
+    if ((f & 31) == 0) wm[f >> 5] = size;
+    __syncthreads();
+    for (int w = 0; w < CT / 32; ++w) size = fmax(size, wm[w]);
+    if (__syncthreads_or(!(diff <= 0x1p-40 * size)) && f == 0) mx[net * NN] = 1e301;
 }
 
 // Adds the rows beyond S to T (Ts [4][M], scaled), in row order, by the whole CTA.
@@ -1198,7 +1232,8 @@ cudaError_t dp_launch_cheb_build(cudaStream_t st, const DevModel &m, double scal
     k_cheb_nodes<<<grid, CT, 0, st>>>(m, scale, cb.trig, cb.y);
     k_cheb_coef<<<grid, CT, 0, st>>>(m, cb.trig, cb.y, cb.C, cb.Ct, cb.mx);
     k_cheb_deriv<<<grid, CT, 0, st>>>(m, scale, cb.C, cb.V);
-    *launches += 3;
+    k_cheb_check<<<m.ntypes * m.ntypes * (NN + 1), CT, 0, st>>>(m, scale, cb.trig, cb.C, cb.mx);
+    *launches += 4;
     return cudaGetLastError();
 }
 
