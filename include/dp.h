@@ -187,7 +187,9 @@ void dp_ctx_free(dp_ctx *ctx);
  * net a second time; off, the backward recomputes them.  Both give the same
  * atomic energies, and forces and virial equal up to the order of the sums
  * over the M features.  dp_ctx_create turns the store on when it takes at most
- * half of the device memory free at that moment.  on = 1 allocates it
+ * half of the device memory free at that moment; an FP64 context then takes the
+ * memory in the first evaluation whose nets are not resolved, and turns the
+ * store off if it is not to be had there.  on = 1 allocates it at once
  * (DP_ERR_NOMEM if that fails, the context unchanged), on = 0 frees it;
  * DP_ERR_UNSUPPORTED for other contexts when on = 1.  Synchronises the
  * context's stream.  dp_ctx_embed_store returns 1 when the store is on, 0

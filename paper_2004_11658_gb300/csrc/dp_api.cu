@@ -152,6 +152,7 @@ struct dp_ctx {
     bool use_ex;
     unsigned char *d_ex_w;
     int64_t ex_version;
+    bool store;  // G and dG/ds of the FP64 rows are to be kept (eb.Gst, allocated when a net needs it)
     // FP64 embedding nets as Chebyshev series in s (cheb.n == 0: not resolved,
     // the kernels above run): made from the parameters of version cheb_version
     bool use_cheb;
@@ -556,6 +557,12 @@ dp_status ensure_oz(dp_ctx *c)
 
 dp_status ensure_ex(dp_ctx *c)
 {
+    if (c->store && !c->eb.Gst &&
+        cudaMalloc((void **)&c->eb.Gst, dp_ex_store_bytes(c->m, c->natoms_max)) != cudaSuccess) {
+        c->eb.Gst = nullptr;  // without room for it the rows are evaluated twice
+        c->store = false;
+        cudaGetLastError();
+    }
     if (c->ex_version == c->model->version) return DP_OK;
     std::vector<unsigned char> w(dp_ex_bytes(c->m), 0);
     dp_ex_split_weights(c->m, c->model->h_params, w.data());
@@ -1056,15 +1063,11 @@ dp_status dp_ctx_create(const dp_model *model, int64_t natoms_max, int32_t cand_
     if (precision == DP_PREC_FP64 && dp_ex_supported(c->m)) {
         ALLOC(c->d_ex_w, dp_ex_bytes(c->m));
         c->use_ex = true;
-        // G and dG/ds stored by the forward, when that takes at most half of the free memory
+        // G and dG/ds stored by the forward, when that takes at most half of the free
+        // memory.  It is taken by the first evaluation whose nets need it (ensure_ex):
+        // while the series runs, no kernel uses it
         size_t fr = 0, tot = 0;
-        const size_t gb = dp_ex_store_bytes(c->m, (int64_t)N);
-        if (!s && cudaMemGetInfo(&fr, &tot) == cudaSuccess && gb <= fr / 2) {
-            if (cudaMalloc((void **)&c->eb.Gst, gb) != cudaSuccess) {
-                c->eb.Gst = nullptr;
-                cudaGetLastError();
-            }
-        }
+        c->store = !s && cudaMemGetInfo(&fr, &tot) == cudaSuccess && dp_ex_store_bytes(c->m, (int64_t)N) <= fr / 2;
         cudaGetLastError();
     }
     c->cheb_version = -1;
@@ -1153,23 +1156,23 @@ dp_status dp_ctx_set_embed_store(dp_ctx *c, int32_t on)
         return fail(DP_ERR_UNSUPPORTED, "the store needs an FP64 context of the tensor-core embedding kernels "
                                         "or a mixed-precision context with plain BF16 operands");
     const bool have = c->eb.Gst != nullptr || c->eb.Gmx != nullptr;
-    if ((on != 0) == have) return DP_OK;
+    if (on ? have : !have && !c->store) return DP_OK;
     DP_CUDA(cudaStreamSynchronize(c->stream), "dp_ctx_set_embed_store");
     if (!on) {
         dev_free(c->eb.Gst);
         dev_free(c->eb.Gmx);
         c->eb.Gst = nullptr;
         c->eb.Gmx = nullptr;
+        c->store = false;
         return DP_OK;
     }
     if (mx) return dev_alloc(&c->eb.Gmx, dp_mx_store_bytes(c->m, c->natoms_max) / sizeof(float), "G and dG/ds rows");
-    return dev_alloc(&c->eb.Gst, dp_ex_store_bytes(c->m, c->natoms_max) / sizeof(double), "G and dG/ds rows");
+    dp_status s = dev_alloc(&c->eb.Gst, dp_ex_store_bytes(c->m, c->natoms_max) / sizeof(double), "G and dG/ds rows");
+    if (!s) c->store = true;
+    return s;
 }
 
-int32_t dp_ctx_embed_store(const dp_ctx *c)
-{
-    return c ? ((c->eb.Gst != nullptr || c->eb.Gmx != nullptr) ? 1 : 0) : -1;
-}
+int32_t dp_ctx_embed_store(const dp_ctx *c) { return c ? (c->store || c->eb.Gmx != nullptr ? 1 : 0) : -1; }
 
 dp_status dp_ctx_set_sync(dp_ctx *c, int32_t sync)
 {
