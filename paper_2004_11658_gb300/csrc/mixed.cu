@@ -1325,6 +1325,7 @@ __global__ void __launch_bounds__(FIT_TH, 1) k_fit_mx(DevModel m, MixedModel mx,
 #pragma unroll
                     for (int q = 0; q < 16; ++q) hp[q] = 0.f;
                 }
+                __syncwarp();  // rows past the last atom branch off above; the load takes the whole warp
                 tc::tmem_ld16(tlane + cc, v);
                 if (my >= 0) {
 #pragma unroll
@@ -1430,6 +1431,7 @@ __global__ void __launch_bounds__(FIT_TH, 1) k_fit_mx(DevModel m, MixedModel mx,
                     float v[16], hp[16];
 #pragma unroll
                     for (int q = 0; q < 16; ++q) hp[q] = my >= 0 && n0 + cc + q < Kl ? hb[(n0 + cc + q) * MXT] : 0.f;
+                    __syncwarp();
                     tc::tmem_ld16(tlane + cc, v);
                     if (my >= 0) {
 #pragma unroll
