@@ -131,18 +131,13 @@ struct OzSplitArgs {
     int keep;      // columns of a row kept in shared memory (0: none)
 };
 
-// Digits sd of 8 values (with their bias, oz_digit_bias) as 8 BF16: the digit
-// sits in a float's mantissa and one subtraction makes it the float's value.
+// Digits sd of 8 values (with their bias, oz_digit_bias) as 8 BF16.
 template <int S, int B>
 __device__ __forceinline__ uint4 oz_pack_digits(const long long (&J)[8], int sd)
 {
     uint32_t f[8];
 #pragma unroll
-    for (int q = 0; q < 8; ++q)
-        f[q] = sd == 0 ? __float_as_uint(__uint_as_float(0x4B400000u + (uint32_t)(int)(J[q] >> (B * (S - 1)))) - 12582912.f)
-                       : __float_as_uint(__uint_as_float(0x4B000000u | ((uint32_t)(J[q] >> (B * (S - 1 - sd))) &
-                                                                        ((1u << B) - 1))) -
-                                         (8388608.f + (float)((1 << (B - 1)) - 1)));
+    for (int q = 0; q < 8; ++q) f[q] = __float_as_uint(oz_digit_f32(J[q], S, B, sd));
     return make_uint4(__byte_perm(f[0], f[1], 0x7632), __byte_perm(f[2], f[3], 0x7632),
                       __byte_perm(f[4], f[5], 0x7632), __byte_perm(f[6], f[7], 0x7632));
 }

@@ -38,10 +38,24 @@ static __host__ __device__ constexpr long long oz_digit_bias(int S, int beta)
     for (int q = 0; q < S - 1; ++q) c += ((1ll << (beta - 1)) - 1) << (beta * q);
     return c;
 }
+// Digit sd as a float, without a conversion: the place's bits are put into the
+// mantissa of 2^23 (the first digit, signed, into that of 1.5 2^23) and one
+// subtraction leaves the digit.  Its upper 16 bits are the digit's BF16.
+static __host__ __device__ __forceinline__ float oz_digit_f32(long long J, int S, int beta, int sd)
+{
+    const uint32_t r = (uint32_t)(J >> (beta * (S - 1 - sd)));
+    const uint32_t u = sd == 0 ? 0x4B400000u + r : 0x4B000000u | (r & ((1u << beta) - 1));
+#ifdef __CUDA_ARCH__
+    const float f = __uint_as_float(u);
+#else
+    float f;
+    std::memcpy(&f, &u, 4);
+#endif
+    return f - (sd == 0 ? 12582912.f : 8388608.f + (float)((1 << (beta - 1)) - 1));
+}
 static __host__ __device__ __forceinline__ int oz_digit_at(long long J, int S, int beta, int sd)
 {
-    const long long r = J >> (beta * (S - 1 - sd));
-    return sd == 0 ? (int)r : (int)(r & ((1ll << beta) - 1)) - ((1 << (beta - 1)) - 1);
+    return (int)oz_digit_f32(J, S, beta, sd);
 }
 
 // BF16 bits of a small integer (|d| <= 256): exact.
