@@ -36,6 +36,7 @@
 #include <cuda_bf16.h>
 
 #include "atom_cta.cuh"
+#include "conv.cuh"
 #include "dp_internal.cuh"
 #include "tc.cuh"
 
@@ -122,25 +123,6 @@ __device__ __forceinline__ void df_fma(float &sh, float &sl, float a, float bh, 
     const float err = __fadd_rn(__fsub_rn(sh, __fsub_rn(s, z)), __fsub_rn(p, z));
     sh = s;
     sl = __fadd_rn(sl, __fadd_rn(err, __fmaf_rn(a, bl, e)));
-}
-
-// Conversions between FP32 and FP64 on the integer pipe (the FP64 pipe takes 16
-// cycles per warp instruction, conversions included): exact, and rounded to
-// nearest even, for normal FP32 results; zero, subnormal and non-finite values
-// take the instruction.
-__device__ __forceinline__ double f2d(float v)
-{
-    const uint32_t u = __float_as_uint(v), e = (u >> 23) & 0xff;
-    if (e == 0 || e == 0xff) return (u << 1) == 0 ? __hiloint2double((int)u, 0) : (double)v;
-    return __hiloint2double((int)((u & 0x80000000u) | (((u >> 3) & 0x0fffffffu) + 0x38000000u)), (int)(u << 29));
-}
-__device__ __forceinline__ float d2f(double v)
-{
-    const unsigned long long b = (unsigned long long)__double_as_longlong(v);
-    const unsigned long long r = b + 0x0fffffffull + ((b >> 29) & 1ull);
-    const uint32_t e = (uint32_t)(r >> 52) & 0x7ff;
-    if (e < 897 || e > 1150) return (b << 1) == 0 ? __uint_as_float((uint32_t)(b >> 32)) : (float)v;
-    return __uint_as_float(((uint32_t)(b >> 32) & 0x80000000u) | ((e - 896) << 23) | ((uint32_t)(r >> 29) & 0x7fffffu));
 }
 
 // v = h + l to about 2^-48 relative (h = v rounded to FP32, l = the rest rounded)
