@@ -622,9 +622,10 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_oz_gemm(OzGemmArgs p)
     } else {
         // y = sum_{g=2}^{S+1} C_g 2^(beta (S + 1 - g)): the group sums are integers
         // below 2^24, combined exactly in two int64 Horner chains (the H groups of
-        // largest scale, then the rest; each chain, summed over the segments, below
-        // 2^53 for every plan of oz_plan_gemm) and rounded once to FP64 with its
-        // scale, on the integer pipe: y 2^escale = sum_g C_g 2^(-beta g).
+        // largest scale, then the rest; each chain, summed over the segments of a
+        // plan of oz_plan_gemm, below 2^53; a weight gradient rounds every segment)
+        // and rounded once to FP64 with its scale, on the integer pipe:
+        // y 2^escale = sum_g C_g 2^(-beta g).
         constexpr int H = (S + 1) / 2;
         const int w = g.beta * (S - H);
         const int half = warp >> 2, row = 32 * (warp & 3) + lane;
@@ -809,15 +810,17 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_oz_gemm(OzGemmArgs p)
                     old = __shfl_sync(0xffffffffu, old, 0);
                     if (old != p.parts - 1) continue;
                     __threadfence();
+                    double own[16];
 #pragma unroll
-                    for (int h = 0; h < 2; ++h)
+                    for (int n = 0; n < 16; ++n) {
+                        own[n] = acc[n >> 3][n & 7];
+                        acc[n >> 3][n & 7] = 0.0;
+                    }
+#pragma unroll 2
+                    for (int q = 0; q < p.parts; ++q)
 #pragma unroll
-                        for (int n = 0; n < 8; ++n) {
-                            const double own = acc[h][n];
-                            acc[h][n] = 0.0;
-                            for (int q = 0; q < p.parts; ++q)
-                                acc[h][n] += q == ks ? own : __longlong_as_double(__ldcg(slot(q, 8 * h + n)));
-                        }
+                        for (int n = 0; n < 16; ++n)
+                            acc[n >> 3][n & 7] += q == ks ? own[n] : __longlong_as_double(__ldcg(slot(q, n)));
                 }
                 if (i >= 0) {
 #pragma unroll
@@ -1148,8 +1151,9 @@ __global__ void k_oz_pg_z(int N, int F, int ld, const double *__restrict__ t, co
 // Digit width, digit count and segment length of a GEMM of contraction length
 // K (nK chunks) at `bits` bits per operand.  From 55 bits on: 8 digits of 7
 // bits, the widest for which one 16-column chunk is exact, and as many chunks
-// per segment as stay exact, spread evenly (400 columns: 400 4^6 10 < 2^24); the
-// int64 chains hold 2^8 segments.  Below: one segment and the widest digits
+// per segment as stay exact, spread evenly (400 columns: 400 4^6 10 < 2^24); a
+// segment adds less than 2^45.1 to an int64 chain, and the widest descriptor (128 x
+// 128) has 41.  Below: one segment and the widest digits
 // that the whole contraction allows.
 void oz_plan_gemm(OzGemm &g, int bits)
 {
@@ -1172,11 +1176,12 @@ void oz_plan_gemm(OzGemm &g, int bits)
 
 // CTAs that share one long contraction (more than one segment) when the (tile,
 // column chunk) pairs would leave half of the SMs idle or more: exact integer
-// sums, so the result does not depend on the split.  A part keeps 8 chunks or
-// more, below which its fixed costs (sums written and read, 64 KB) outweigh the
-// MMAs (1 k cycles a chunk).  One CTA per pair took 88 us for the first layer
-// of 192 water atoms and 321 us for a weight gradient over 12,288; now 44 and 54 us
-// (95 us for the 240 x 240 weights, 321 before).
+// sums, so the result does not depend on the split; a weight gradient's parts hold
+// whole segments and their FP64 sums are added in order, the same on the same GPU.
+// A part keeps 8 chunks or more, below which its fixed costs (sums written and
+// read, 64 KB) outweigh the MMAs (1 k cycles a chunk).  One CTA per pair took 88 us
+// for the first layer of 192 water atoms and 321 us for a weight gradient over
+// 12,288; now 44 and 60 us (85 us for the 240 x 240 weights, 321 before).
 int oz_parts(int pairs, int nK, int num_sms)
 {
     return std::max(1, std::min(num_sms / std::max(pairs, 1), nK / 8));
