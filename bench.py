@@ -29,6 +29,7 @@ import hashlib
 import json
 import os
 import platform
+import re
 import statistics
 import subprocess
 import sys
@@ -71,7 +72,7 @@ FORCE_RMSE_TARGET = 1e-3   # eV/A, against the FP64 full model
 # Per-kernel counters from one ncu capture of one evaluation of the 12,288-atom
 # water box (bench.py --workload water12288 --profile-eval 1, 1,046,154 real
 # neighbour rows), reported only while the kernel source is the one captured
-# (hash of the .cu file and the shared header):
+# (hash of the .cu file and the headers it includes):
 #   bytes_per_row     (dram__bytes_read.sum + dram__bytes_write.sum) / rows: the
 #                     traffic of a launch grows with its rows (G and dG/ds rows,
 #                     per-atom T, D and dE/dD at ~91 rows per atom), so the bench
@@ -136,7 +137,7 @@ SERIES_COUNTERS = {
     "embed_bwd<25>": {"bytes_per_row": 428.686592e6 / PROFILE_ROWS, "fp64_flop_per_row": 0.890842e9 / PROFILE_ROWS,
                       "pipe_busy": 0.875, "src_sha": "bef972990c3595e4"},
 }
-SERIES_SOURCES = ("embed_cheb.cu", "fit_oz.cu", "cheb.cuh", "atom_cta.cuh")
+SERIES_SOURCES = ("embed_cheb.cu", "fit_oz.cu")
 
 
 def parse():
@@ -273,11 +274,29 @@ def measured_peaks():
         return {}
 
 
+CSRC = os.path.join(ROOT, "paper_2004_11658_gb300", "csrc")
+
+
+def source_files(*files):
+    """Kernel source files and the headers of csrc/ that they include, directly
+    or through one another, each once."""
+    todo, seen = list(files), []
+    while todo:
+        name = todo.pop(0)
+        if name in seen:
+            continue
+        seen.append(name)
+        with open(os.path.join(CSRC, name)) as f:
+            found = re.findall(r'^#include "([^"]+)"', f.read(), re.M)
+        todo += [h for h in found if os.path.exists(os.path.join(CSRC, h)) and not h.startswith("..")]
+    return seen
+
+
 def source_sha(*files):
-    """Hash of kernel source files together with the shared device header."""
+    """Hash of kernel source files together with their headers."""
     h = hashlib.sha256()
-    for name in files + ("dp_internal.cuh",):
-        with open(os.path.join(ROOT, "paper_2004_11658_gb300", "csrc", name), "rb") as f:
+    for name in sorted(source_files(*files)):
+        with open(os.path.join(CSRC, name), "rb") as f:
             h.update(f.read())
     return h.hexdigest()[:16]
 
