@@ -63,7 +63,8 @@ inline int dp_cheb_splits(int ntypes, int64_t natoms)
     return (int)(s < lo ? lo : s > hi ? hi : s);
 }
 // Terms the gradient keeps: the parameter derivatives' series converge as the
-// nets' with a polynomial factor, which 8 more terms cover.
+// nets' with a polynomial factor, which 8 more terms cover (nets of 29 to 46 terms
+// needed at most 2 more, in 40-digit arithmetic), and the last 4 for nets of 44.
 inline int dp_cheb_grad_terms(int n) { return n + 8 < DP_CHEB_NN ? n + 8 : DP_CHEB_NN; }
 size_t dp_cheb_grad_elems(const DevModel &m, int n, int64_t natoms, int which);  // doubles of mom, part, node
 bool dp_cheb_grad_supported(const DevModel &m, int n);
