@@ -83,45 +83,46 @@ FORCE_RMSE_TARGET = 1e-3   # eV/A, against the FP64 full model
 #   pipe_busy         sm__inst_executed_pipe_fp64 share of the active cycles
 PROFILE_ROWS = 1046154
 TRAFFIC = {
-    "embed_tan<25>": {"bytes_per_row": (10.468352e6 + 1811.331840e6) / PROFILE_ROWS, "file": "embed_x.cu",
-                      "src_sha": "c2c89c84fd00c488"},
-    "embed_bwd_st<25>": {"bytes_per_row": (1883.360000e6 + 28.511232e6) / PROFILE_ROWS, "file": "embed_x.cu",
-                         "src_sha": "c2c89c84fd00c488"},
-    "embed_tan_mx<25>": {"bytes_per_row": (54.107136e6 + 1037.398528e6) / PROFILE_ROWS, "file": "mixed.cu",
-                         "src_sha": "be819dbaa370fed3"},
-    "embed_bwd_st_mx<25>": {"bytes_per_row": (1063.947264e6 + 36.366080e6) / PROFILE_ROWS, "file": "mixed.cu",
-                            "src_sha": "be819dbaa370fed3"},
-    "embed_bwd_mx<25, split>": {"bytes_per_row": (204.732928e6 + 17.787136e6) / PROFILE_ROWS, "file": "mixed.cu",
-                                "src_sha": "be819dbaa370fed3"},
-    "embed_tan_mx<16>": {"bytes_per_row": (9.171456e6 + 628.367104e6) / PROFILE_ROWS, "file": "mixed.cu",
-                         "src_sha": "be819dbaa370fed3"},
-    "embed_bwd_st_mx<16>": {"bytes_per_row": (689.640192e6 + 25.842432e6) / PROFILE_ROWS, "file": "mixed.cu",
-                            "src_sha": "be819dbaa370fed3"},
+    "embed_tan<25>": {"bytes_per_row": (8.802048e6 + 1810.711296e6) / PROFILE_ROWS, "file": "embed_x.cu",
+                      "src_sha": "05ef0f1dff99fba4"},
+    "embed_bwd_st<25>": {"bytes_per_row": (1883.315200e6 + 28.983808e6) / PROFILE_ROWS, "file": "embed_x.cu",
+                         "src_sha": "05ef0f1dff99fba4"},
+    "embed_tan_mx<25>": {"bytes_per_row": (54.977536e6 + 1038.135040e6) / PROFILE_ROWS, "file": "mixed.cu",
+                         "src_sha": "146a7f922a31a1d9"},
+    "embed_bwd_st_mx<25>": {"bytes_per_row": (1063.892992e6 + 36.098816e6) / PROFILE_ROWS, "file": "mixed.cu",
+                            "src_sha": "146a7f922a31a1d9"},
+    "embed_bwd_mx<25, split>": {"bytes_per_row": (205.012992e6 + 18.074368e6) / PROFILE_ROWS, "file": "mixed.cu",
+                                "src_sha": "146a7f922a31a1d9"},
+    "embed_tan_mx<16>": {"bytes_per_row": (9.192960e6 + 628.519680e6) / PROFILE_ROWS, "file": "mixed.cu",
+                         "src_sha": "146a7f922a31a1d9"},
+    "embed_bwd_st_mx<16>": {"bytes_per_row": (689.644032e6 + 25.815296e6) / PROFILE_ROWS, "file": "mixed.cu",
+                            "src_sha": "146a7f922a31a1d9"},
 }
 # Pipe shares of the mixed embedding kernels (ncu, one evaluation of the
 # 12,288-atom water box, --profile-precision mixed / split): active-cycle
 # busy fractions of the FP64, FP32 (fma), integer (alu) and tensor pipes and
 # the schedulers' issue-active share.
 MODE_PIPES = {
-    "embed_tan_mx<25>": {"fp64": 0.322, "fma": 0.216, "alu": 0.111, "tensor": 0.017, "issue_active": 0.363,
-                         "file": "mixed.cu", "src_sha": "be819dbaa370fed3"},
-    "embed_bwd_st_mx<25>": {"fp64": 0.655, "fma": 0.345, "alu": 0.108, "tensor": 0.000, "issue_active": 0.498,
-                            "file": "mixed.cu", "src_sha": "be819dbaa370fed3"},
+    "embed_tan_mx<25>": {"fp64": 0.322, "fma": 0.215, "alu": 0.111, "tensor": 0.017, "issue_active": 0.362,
+                         "file": "mixed.cu", "src_sha": "146a7f922a31a1d9"},
+    "embed_bwd_st_mx<25>": {"fp64": 0.654, "fma": 0.344, "alu": 0.108, "tensor": 0.000, "issue_active": 0.497,
+                            "file": "mixed.cu", "src_sha": "146a7f922a31a1d9"},
     "embed_bwd_mx<25, split>": {"fp64": 0.367, "fma": 0.199, "alu": 0.117, "tensor": 0.031, "issue_active": 0.330,
-                                "file": "mixed.cu", "src_sha": "be819dbaa370fed3"},
-    "embed_tan_mx<16>": {"fp64": 0.375, "fma": 0.189, "alu": 0.110, "tensor": 0.007, "issue_active": 0.332,
-                         "file": "mixed.cu", "src_sha": "be819dbaa370fed3"},
-    "embed_bwd_st_mx<16>": {"fp64": 0.721, "fma": 0.307, "alu": 0.123, "tensor": 0.000, "issue_active": 0.476,
-                            "file": "mixed.cu", "src_sha": "be819dbaa370fed3"},
+                                "file": "mixed.cu", "src_sha": "146a7f922a31a1d9"},
+    "embed_tan_mx<16>": {"fp64": 0.374, "fma": 0.188, "alu": 0.109, "tensor": 0.007, "issue_active": 0.332,
+                         "file": "mixed.cu", "src_sha": "146a7f922a31a1d9"},
+    "embed_bwd_st_mx<16>": {"fp64": 0.720, "fma": 0.307, "alu": 0.123, "tensor": 0.000, "issue_active": 0.477,
+                            "file": "mixed.cu", "src_sha": "146a7f922a31a1d9"},
 }
 FP64_ISSUED = {
-    # k_embed_tan_x<25>: dfma 2.257e9, dadd 0.818e9, dmul 0.106e9 thread
-    # instructions; FP64 pipe busy 41.2% (issue active 24.3%)
-    "embed_tan<25>": {"fp64_flop_per_row": (2 * 2.257052574e9 + 0.817909986e9 + 0.105703644e9) / PROFILE_ROWS,
-                      "pipe_busy": 0.412, "file": "embed_x.cu", "src_sha": "c2c89c84fd00c488"},
-    # k_embed_bwd_st<25>: dfma 1.070e9, dadd 0.101e9, dmul 0.044e9; FP64 pipe busy 93.9%
-    "embed_bwd_st<25>": {"fp64_flop_per_row": (2 * 1.069532688e9 + 0.100726048e9 + 0.043622898e9) / PROFILE_ROWS,
-                         "pipe_busy": 0.939, "file": "embed_x.cu", "src_sha": "c2c89c84fd00c488"},
+    # k_embed_tan_x<25>: dfma 2.234e9, dadd 0.818e9, dmul 0.099e9 thread
+    # instructions; FP64 pipe busy 40.9% (issue active 24.7%); captured with first
+    # layers 100 times the seeded ones, whose series do not resolve
+    "embed_tan<25>": {"fp64_flop_per_row": (2 * 2.234264396e9 + 0.817792994e9 + 0.099426720e9) / PROFILE_ROWS,
+                      "pipe_busy": 0.409, "file": "embed_x.cu", "src_sha": "05ef0f1dff99fba4"},
+    # k_embed_bwd_st<25>: dfma 1.048e9, dadd 0.101e9, dmul 0.037e9; FP64 pipe busy 94.0%
+    "embed_bwd_st<25>": {"fp64_flop_per_row": (2 * 1.047563454e9 + 0.100726048e9 + 0.037345974e9) / PROFILE_ROWS,
+                         "pipe_busy": 0.940, "file": "embed_x.cu", "src_sha": "05ef0f1dff99fba4"},
 }
 
 # The FP64 path with the embedding nets as series (embed_cheb.cu) and the exact
@@ -130,12 +131,12 @@ FP64_ISSUED = {
 # kernels' active cycles), keyed by their sources.  Parts of this box's per-atom
 # arrays stay in L2, so the bytes are a lower bound for larger ones.
 SERIES_COUNTERS = {
-    "embed_fwd<25>": {"bytes_per_row": 198.640896e6 / PROFILE_ROWS, "fp64_flop_per_row": 0.436443e9 / PROFILE_ROWS,
-                      "pipe_busy": 0.792, "src_sha": "bef972990c3595e4"},
-    "fit<25>": {"bytes_per_row": 1600.926464e6 / PROFILE_ROWS, "fp64_flop_per_row": 0.264720e9 / PROFILE_ROWS,
-                "pipe_busy": 0.306, "src_sha": "bef972990c3595e4"},
-    "embed_bwd<25>": {"bytes_per_row": 428.686592e6 / PROFILE_ROWS, "fp64_flop_per_row": 0.890842e9 / PROFILE_ROWS,
-                      "pipe_busy": 0.875, "src_sha": "bef972990c3595e4"},
+    "embed_fwd<25>": {"bytes_per_row": 198.249216e6 / PROFILE_ROWS, "fp64_flop_per_row": 0.436443e9 / PROFILE_ROWS,
+                      "pipe_busy": 0.797, "src_sha": "b80d7fc59796fec4"},
+    "fit<25>": {"bytes_per_row": 1596.846336e6 / PROFILE_ROWS, "fp64_flop_per_row": 0.264720e9 / PROFILE_ROWS,
+                "pipe_busy": 0.309, "src_sha": "b80d7fc59796fec4"},
+    "embed_bwd<25>": {"bytes_per_row": 428.711424e6 / PROFILE_ROWS, "fp64_flop_per_row": 0.865608e9 / PROFILE_ROWS,
+                      "pipe_busy": 0.876, "src_sha": "b80d7fc59796fec4"},
 }
 SERIES_SOURCES = ("embed_cheb.cu", "fit_oz.cu")
 
