@@ -901,8 +901,8 @@ def run_ours(args, rank, world, local_rank):
             "gpu_launches": launches,
             "roofline": roof,
             "embed_store": {"on": bool(store),
-                            "what": "HBM held for G and dG/ds of every real row, which the embedding kernels use "
-                                    "when a net's series in s(r) does not resolve (k_embed_tan_x, k_embed_bwd_st)"},
+                            "what": "G and dG/ds of every real row kept in HBM when a net's series in s(r) does not "
+                                    "resolve (k_embed_tan_x, k_embed_bwd_st); the memory is taken only then"},
             "kernels_ms_per_step": {g: d["ms"] / args.steps for g, d in timed_groups.items()},
             "nve": {"etot_first": float(etot[0]), "etot_last": float(etot[-1]),
                     "max_abs_drift_eV_per_atom": float(np.abs(etot - etot[0]).max() / N),

@@ -85,8 +85,8 @@ typedef struct dp_ctx dp_ctx;
                              series in s made on the device (in double-double
                              arithmetic) whenever the parameters change: the
                              terms kept leave less than 2^-55 of the net's size.
-                             Nets that 44 terms do not resolve are evaluated as
-                             written, for 3-layer doubling nets with s_1 in
+                             Nets that 44 terms do not resolve, or that the series
+                             misses between its nodes, are evaluated as written, for 3-layer doubling nets with s_1 in
                              {16, 25, 32} with their last two layers and the
                              s-tangents as exact products (below).  The
                              fitting-net GEMMs run on the tensor cores as exact

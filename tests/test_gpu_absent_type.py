@@ -45,7 +45,8 @@ def test_absent_type_has_no_gradient(oracle, synth, ntypes, absent, fit):
         return dp.dp_param_grad(ctx, x, ty, b, 0.37, torch.tensor(lm, device="cuda"))
 
     used = dp.Context(model, len(c))
-    grad(used, t_all, lam * np.nan)
+    spoilt = blocks(synth, desc, grad(used, t_all, lam * np.nan).cpu().numpy())
+    assert all(np.isnan(spoilt[f"fit{a}.W1"]).any() for a in range(ntypes))
     for ctx in (used, dp.Context(model, len(c))):
         got = blocks(synth, desc, grad(ctx, t_some, lam).cpu().numpy())
         for name, g in got.items():
