@@ -86,14 +86,14 @@ typedef struct dp_ctx dp_ctx;
                              arithmetic) whenever the parameters change: the
                              terms kept leave less than 2^-55 of the net's size.
                              Nets that 44 terms do not resolve, or that the series
-                             misses between its nodes, are evaluated as written, for 3-layer doubling nets with s_1 in
-                             {16, 25, 32} with their last two layers and the
-                             s-tangents as exact products (below).  The
-                             fitting-net GEMMs run on the tensor cores as exact
-                             products of BF16 digit expansions of the FP64
-                             operands (every partial sum an integer below 2^24,
-                             held exactly by the FP32 accumulators), the rest
-                             on the FP64 units. */
+                             misses between its nodes, are evaluated as written,
+                             for 3-layer doubling nets with s_1 in {16, 25, 32}
+                             with their last two layers and the s-tangents as
+                             exact products (below).  The fitting-net GEMMs run
+                             on the tensor cores as exact products of BF16 digit
+                             expansions of the FP64 operands (every partial sum
+                             an integer below 2^24, held exactly by the FP32
+                             accumulators), the rest on the FP64 units. */
 #define DP_PREC_FP64_SIMT 2  /* every step in float64 on the FP64 units */
 #define DP_PREC_MIXED 1   /* embedding- and fitting-net GEMMs on the tensor cores
                              (BF16 operands, FP32 accumulation, FP32 tanh); the
